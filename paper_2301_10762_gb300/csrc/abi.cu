@@ -339,6 +339,7 @@ extern "C" void helm_factor_destroy(helm_factor_t *f) {
     dev_free(f->r32, st);
     dev_free(f->y, st);
     dev_free(f->norms, st);
+    dev_free(f->maxima, st);
     dev_free(f->state, st);
     bcr_free(f);
     delete f;
@@ -356,10 +357,12 @@ helm_status factor_reserve(helm_factor_t *f, int nrhs) {
     dev_free(f->r32, st);
     dev_free(f->y, st);
     dev_free(f->norms, st);
+    dev_free(f->maxima, st);
     dev_free(f->state, st);
     f->bd = f->xa = f->xb = nullptr;
     f->r32 = f->y = nullptr;
     f->norms = nullptr;
+    f->maxima = nullptr;
     f->state = nullptr;
     f->cap = 0;
     helm_status s;
@@ -371,6 +374,9 @@ helm_status factor_reserve(helm_factor_t *f, int nrhs) {
          (s = dev_alloc((void **)&f->y, cols * N * sizeof(float2), "allocate(work)", st)) != HELM_OK ||
          (s = dev_alloc((void **)&f->state, refine_state_bytes(op->n_omega), "allocate(refinement state)", st)) !=
              HELM_OK))
+        return s;
+    if (f->use_bcr &&
+        (s = dev_alloc((void **)&f->maxima, bcr_maxima_elems(op->g, cols) * sizeof(float), "allocate(maxima)", st)) != HELM_OK)
         return s;
     if ((s = dev_alloc((void **)&f->norms, cols * 2 * sizeof(double), "allocate(norms)", st)) != HELM_OK) return s;
     f->norms_host.assign(cols * 2, 0.0);
@@ -425,7 +431,7 @@ helm_status mixed_refine(const helm_factor_t *f, int nrhs, const double2 *B, dou
     auto sweep = [&](const int *skip_flag) -> cudaError_t {
         const int *frozen = skip_flag ? refine_sys(w.state) + 1 : nullptr;
         if (f->use_bcr) {
-            const helm_status bs = bcr_solve(f, nrhs, w.r32, w.y, skip_flag, frozen);
+            const helm_status bs = bcr_solve(f, nrhs, w.r32, w.y, w.maxima, skip_flag, frozen);
             return bs == HELM_OK ? cudaSuccess : cudaErrorLaunchFailure;
         }
         return launch_line_sweep<float>(g, n_sys, nrhs, (const float2 *)f->G, w.r32, nullptr, w.y, 0, rchunk,
@@ -515,7 +521,7 @@ helm_status solve_impl(helm_factor_t *f, int nrhs, const double2 *B, double2 *X,
         return HELM_OK;
     }
     if ((s = factor_reserve(f, nrhs)) != HELM_OK) return s;
-    const MixedWork w{f->bd, f->xa, f->xb, f->r32, f->y, f->norms, f->norms_host.data(), f->state};
+    const MixedWork w{f->bd, f->xa, f->xb, f->r32, f->y, f->norms, f->norms_host.data(), f->state, f->maxima};
     int it = 0;
     double rel = INFINITY;
     if ((s = mixed_refine(f, nrhs, B, X, conj, rtol, max_iter, w, &it, &rel)) != HELM_OK) return s;

@@ -5,6 +5,7 @@
 #include <vector>
 #include <cuda_runtime.h>
 #include "helm.h"
+#include "bcr_solve.h"
 #include "common.cuh"
 
 struct helm_op {
@@ -28,20 +29,21 @@ struct RefineState;   // device-side refinement control (kernels.h)
 
 // Block-cyclic-reduction factor (bcr.cu): the inverse of every line's block at the level it was
 // eliminated, the back-substitution blocks P_j, Q_j and the forward blocks W_j, V_j of the lines
-// eliminated at levels >= 1 (slot j / 2), and the solve's GEMM task lists on the device.
+// eliminated at levels >= 1 (slot j / 2), all in the solve kernel's operand layout (bcr_solve.h),
+// and the solve's steps.
 struct BcrData {
-    int levels = 0, half = 0;
-    float2 *Dinv = nullptr, *P = nullptr, *Q = nullptr, *W = nullptr, *V = nullptr;
-    int *tasks = nullptr;
-    float2 *split = nullptr;     // partial tiles of the solve's split-K GEMM launches
-    size_t split_cap = 0;        // (complex elements)
-    struct List {
-        int first = 0, count = 0;   // tasks of one GEMM launch of the solve
-        long long terms = 0;        // product terms over those tasks
-    };
-    std::vector<List> fwd, bwd;     // per level
-    List last;
+    int half = 0;
+    unsigned char *img = nullptr;   // blocks: [n_omega][nx] inverses, then [n_omega][half] of W, V, P, Q
+    float *scl = nullptr;           // row scales of the blocks
+    int *tasks = nullptr;           // the solve's tasks on the device
+    unsigned *ctl = nullptr;        // the solve's tile and step counters
+    float *gsmall = nullptr;        // vector maxima of the no-allocation solve (kSmallMaxima)
+    std::vector<helm::BsStep> steps;
+    long long terms = 0;            // products of one solve per system
 };
+// maxima of every call that fits the no-allocation solve's array: at most 2^19 entries per vector,
+// one maximum per 16 of them or more, two vectors
+constexpr size_t kSmallMaxima = (size_t)1 << 16;
 
 struct helm_factor {
     helm_op *op = nullptr;
@@ -60,6 +62,7 @@ struct helm_factor {
     float2 *r32 = nullptr, *y = nullptr;                  // mixed: correction right-hand side and result
     double *norms = nullptr;
     std::vector<double> norms_host;   // host copy of the norms (pageable: no pinned allocation)
+    float *maxima = nullptr;                  // mixed, block cyclic reduction: the solve's vector maxima
     helm::RefineState *state = nullptr;       // mixed: device-side refinement control
     mutable std::atomic<int> last_iters{3};   // correction sweeps the previous mixed solve took
 };
@@ -71,6 +74,7 @@ struct MixedWork {
     double *norms;        // device [cols][2]
     double *norms_host;   // host [cols][2]
     helm::RefineState *state;   // device
+    float *maxima;        // device, block cyclic reduction only (bcr_maxima_elems)
 };
 
 // acquisition on the device
@@ -111,7 +115,8 @@ bool factor_picks_bcr(const GridGeom &g, helm_prec prec, int method);
 helm_status bcr_factor(helm_factor_t *f);
 void bcr_free(helm_factor_t *f);
 // frozen: NULL, or the refinement's per-system flags (stride 2): columns of a set flag are skipped
-helm_status bcr_solve(const helm_factor_t *f, int nrhs, float2 *r, float2 *x, const int *skip,
+size_t bcr_maxima_elems(const GridGeom &g, size_t cols);   // floats of scratch of a solve of cols columns
+helm_status bcr_solve(const helm_factor_t *f, int nrhs, float2 *r, float2 *x, float *maxima, const int *skip,
                       const int *frozen = nullptr);
 helm_status blas_zgemm(int batch, int M, int N, int K, const float2 *A, long long sa, int lda, const float2 *Bt,
                        long long sb, int ldb, float sign, const float2 *C0, float2 *C, long long sc, int ldc,

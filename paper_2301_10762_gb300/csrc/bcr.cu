@@ -21,12 +21,13 @@
 // and the back substitution takes P_j = V_j^T = Dinv_j L_j, Q_j = W_j^T = Dinv_j U_j.
 // Level 0 has the diagonal couplings C: its products are elementwise scalings.
 //
-// The solve of A x = b (all right-hand sides of a system as the GEMM N dimension):
-//     forward, level 0:  y_j = Dinv_j b_j;  b_k -= C (y_a + y_c)
+// The solve of A x = b (all right-hand sides of a system as the products' N dimension) takes the
+// blocks W, V, P, Q and the inverses in the layout of bcr_solve.cu, which runs it:
+//     forward, level 0:  b_k -= C (Dinv_a b_a + Dinv_c b_c)
 //     forward, level l:  b_k -= W_a b_a + V_c b_c
 //     last line:         x_0 = Dinv_0 b_0
 //     backward, level l: x_j = Dinv_j b_j - P_j x_{j-s} - Q_j x_{j+s}
-//     backward, level 0: x_j = y_j - Dinv_j C (x_{j-1} + x_{j+1}).
+//     backward, level 0: x_j = Dinv_j (b_j - C (x_{j-1} + x_{j+1})).
 // Everything is complex FP32 (3xTF32 tensor products): the factor is the preconditioner of
 // the FP64-residual refinement of the mixed path, exactly as the line factor is.
 //
@@ -41,9 +42,12 @@
 
 #include <algorithm>
 #include <functional>
+#include <initializer_list>
+#include <utility>
 #include <vector>
 
 #include "abi_internal.h"
+#include "bcr_solve.h"
 #include "kernels.h"
 #include "pivot16.cuh"
 #include "tcgen05.cuh"
@@ -491,66 +495,6 @@ __global__ void __launch_bounds__(512) tri_rank1_kernel(int n, int n1, TriIn tri
     }
 }
 
-// out[idx_out] = in[idx_in]^T for n x n complex blocks (32 x 32 tiles through shared memory)
-__global__ void ztranspose_kernel(int n, const float2 *in, float2 *out, long long stride_in, long long stride_out,
-                                  const int *idx) {
-    __shared__ float2 t[32][33];
-    const int *ix = idx + 2 * (size_t)blockIdx.z;
-    const float2 *A = in + (long long)ix[0] * stride_in;
-    float2 *B = out + (long long)ix[1] * stride_out;
-    const int nt = (n + 31) / 32;
-    const int bi = blockIdx.x / nt, bj = blockIdx.x % nt;
-    for (int y = threadIdx.y; y < 32; y += blockDim.y) {
-        const int r = bi * 32 + y, c = bj * 32 + threadIdx.x;
-        if (r < n && c < n) t[y][threadIdx.x] = A[(size_t)r * n + c];
-    }
-    __syncthreads();
-    for (int y = threadIdx.y; y < 32; y += blockDim.y) {
-        const int r = bj * 32 + y, c = bi * 32 + threadIdx.x;
-        if (r < n && c < n) B[(size_t)r * n + c] = t[threadIdx.x][y];
-    }
-}
-
-// solve, level 0 of the forward pass: b_k -= C (y_{k-1} + y_{k+1}) for even k, y in x.  Thread:
-// two rows (one float4) of the line, for L0_COLS columns (frequency x right-hand side).
-constexpr int L0_COLS = 8;
-__global__ void bcr_solve_l0_fwd_kernel(GridGeom g, Coup cp, int cols, float2 *b, const float2 *x, const int *skip,
-                                        const int *frozen, int nrhs) {
-    if (skip && *skip) return;
-    const int nz = g.nz, nx = g.nx, N = nx * nz;
-    const int k = 2 * blockIdx.y, r = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
-    if (r >= nz) return;
-    const float c0 = cp.cx(r, nz), c1 = cp.cx(r + 1, nz);
-    for (int col = blockIdx.z * L0_COLS; col < min(cols, (int)(blockIdx.z + 1) * L0_COLS); ++col) {
-        if (frozen && frozen[2 * (col / nrhs)]) continue;   // a converged system's correction is not needed
-        const size_t off = (size_t)col * N + (size_t)k * nz + r;
-        float4 t = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (k >= 1) { const float4 v = *reinterpret_cast<const float4 *>(x + off - nz); t.x += v.x; t.y += v.y; t.z += v.z; t.w += v.w; }
-        if (k + 1 < nx) { const float4 v = *reinterpret_cast<const float4 *>(x + off + nz); t.x += v.x; t.y += v.y; t.z += v.z; t.w += v.w; }
-        float4 *bp = reinterpret_cast<float4 *>(b + off);
-        float4 v = *bp;
-        v.x -= c0 * t.x; v.y -= c0 * t.y; v.z -= c1 * t.z; v.w -= c1 * t.w;
-        *bp = v;
-    }
-}
-
-// solve, level 0 of the backward pass: b_j = C (x_{j-1} + x_{j+1}) for odd j
-__global__ void bcr_solve_l0_bwd_kernel(GridGeom g, Coup cp, int cols, float2 *b, const float2 *x, const int *skip,
-                                        const int *frozen, int nrhs) {
-    if (skip && *skip) return;
-    const int nz = g.nz, nx = g.nx, N = nx * nz;
-    const int j = 2 * blockIdx.y + 1, r = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
-    if (r >= nz) return;
-    const float c0 = cp.cx(r, nz), c1 = cp.cx(r + 1, nz);
-    for (int col = blockIdx.z * L0_COLS; col < min(cols, (int)(blockIdx.z + 1) * L0_COLS); ++col) {
-        if (frozen && frozen[2 * (col / nrhs)]) continue;
-        const size_t off = (size_t)col * N + (size_t)j * nz + r;
-        float4 t = *reinterpret_cast<const float4 *>(x + off - nz);
-        if (j + 1 < nx) { const float4 v = *reinterpret_cast<const float4 *>(x + off + nz); t.x += v.x; t.y += v.y; t.z += v.z; t.w += v.w; }
-        *reinterpret_cast<float4 *>(b + off) = make_float4(c0 * t.x, c0 * t.y, c1 * t.z, c1 * t.w);
-    }
-}
-
 // ----------------------------------------------------------------- host side
 
 struct TaskBuf {   // device copy of host-built task lists (freed on the stream when done)
@@ -572,8 +516,8 @@ helm_status upload_ints(const std::vector<int> &h, TaskBuf &b, cudaStream_t st) 
 // single copy before the launches are enqueued (a copy from pageable host memory waits for the
 // stream, so one copy per launch would serialise the host with the GPU at every launch).
 // partial tiles of split-K GEMM launches: 64 MB for a factorisation (its deep levels: 8 tasks of
-// 256 x 256 split 16 ways), 32 MB kept with a factor for its solves (64 tasks of 256 x 64 split 8 ways)
-constexpr size_t kFactorSplitElems = (size_t)8 << 20, kSolveSplitElems = (size_t)4 << 20;
+// 256 x 256 split 16 ways)
+constexpr size_t kFactorSplitElems = (size_t)8 << 20;
 
 struct Plan {
     cudaStream_t st;
@@ -798,18 +742,15 @@ helm_status invert_tridiag_blocks(int n, Fam in, Fam out, const std::vector<int>
     return HELM_OK;
 }
 
-helm_status transpose_blocks(int n, const float2 *in, float2 *out, long long stride, const std::vector<int> &pairs,
-                             Plan &pl) {
-    const int count = (int)(pairs.size() / 2);
-    if (count == 0) return HELM_OK;
-    const int off = pl.add(pairs);
+// images (bcr_solve.cu) of the blocks base + pairs[.][0] * n^2 as matrices pairs[.][1]
+helm_status image_blocks(int n, const float2 *base, bool trans, const std::vector<int> &pairs, unsigned char *img,
+                         float *scl, Plan &pl) {
+    if (pairs.empty()) return HELM_OK;
+    const int off = pl.add(pairs), count = (int)(pairs.size() / 2);
     const cudaStream_t st = pl.st;
     pl.ops.push_back([=](const int *dev) -> helm_status {
-        const int nt = (n + 31) / 32;
-        HELM_TRACED(K_ZTRANS, st, (ztranspose_kernel<<<dim3(nt * nt, 1, count), dim3(32, 8), 0, st>>>(
-                                      n, in, out, stride, stride, dev + off)));
-        const cudaError_t e = cudaGetLastError();
-        if (e != cudaSuccess) { helm_set_error("bcr: transpose", e); return HELM_ECUDA; }
+        const cudaError_t e = launch_bcr_image(n, base, (long long)n * n, trans, dev + off, count, img, scl, st);
+        if (e != cudaSuccess) { helm_set_error("bcr: images", e); return HELM_ECUDA; }
         return HELM_OK;
     });
     return HELM_OK;
@@ -826,34 +767,36 @@ helm_status bcr_factor(helm_factor_t *f) {
     const GridGeom &g = op->g;
     const int nx = g.nx, nz = g.nz, ns = op->n_omega;
     const long long nz2 = (long long)nz * nz;
-    const int half = nx / 2 + 1;
+    const int half = nx / 2 + 1, quart = nx / 4 + 1;
     const cudaStream_t st = op->st;
     BcrData &b = f->bcr;
     b.half = half;
     helm_status s;
     const size_t blk = (size_t)nz2 * sizeof(float2);
-    if ((s = dev_alloc((void **)&b.Dinv, (size_t)ns * nx * blk, "bcr: inverses", st)) != HELM_OK ||
-        (s = dev_alloc((void **)&b.P, (size_t)ns * half * blk, "bcr: P", st)) != HELM_OK ||
-        (s = dev_alloc((void **)&b.Q, (size_t)ns * half * blk, "bcr: Q", st)) != HELM_OK ||
-        (s = dev_alloc((void **)&b.W, (size_t)ns * half * blk, "bcr: W", st)) != HELM_OK ||
-        (s = dev_alloc((void **)&b.V, (size_t)ns * half * blk, "bcr: V", st)) != HELM_OK)
+    // kept: the image of every line's inverse and of W, V, P, Q of the lines eliminated at levels >= 1
+    const size_t n_mat = (size_t)ns * (nx + 4 * (size_t)half);
+    const BsLayout lay = bs_layout(nz);
+    if ((s = dev_alloc((void **)&b.img, n_mat * lay.mat_bytes, "bcr: blocks", st)) != HELM_OK ||
+        (s = dev_alloc((void **)&b.scl, n_mat * nz * sizeof(float), "bcr: row scales", st)) != HELM_OK ||
+        (s = dev_alloc((void **)&b.gsmall, kSmallMaxima * sizeof(float), "bcr: maxima", st)) != HELM_OK)
         return s;
-    // working blocks of the reduction: current diagonal blocks and couplings (ping-pong)
-    float2 *Dc = nullptr, *Lc = nullptr, *Ln = nullptr, *Uc = nullptr, *Un = nullptr;
+    // working blocks of the reduction: diagonal blocks (an eliminated line's is inverted in place),
+    // couplings L, U (ping-pong: line k of spacing sp at index k / sp), W and V of one level
+    float2 *D = nullptr, *LU[2][2] = {{nullptr, nullptr}, {nullptr, nullptr}}, *W = nullptr, *V = nullptr;
     struct Work {
-        float2 **p[5];
+        float2 **p[7];
         cudaStream_t st;
         ~Work() { for (auto q : p) dev_free(*q, st); }
-    } work{{&Dc, &Lc, &Ln, &Uc, &Un}, st};
-    if ((s = dev_alloc((void **)&Dc, (size_t)ns * nx * blk, "bcr: work", st)) != HELM_OK ||
-        (s = dev_alloc((void **)&Lc, (size_t)ns * half * blk, "bcr: work", st)) != HELM_OK ||
-        (s = dev_alloc((void **)&Ln, (size_t)ns * half * blk, "bcr: work", st)) != HELM_OK ||
-        (s = dev_alloc((void **)&Uc, (size_t)ns * half * blk, "bcr: work", st)) != HELM_OK ||
-        (s = dev_alloc((void **)&Un, (size_t)ns * half * blk, "bcr: work", st)) != HELM_OK)
+    } work{{&D, &LU[0][0], &LU[0][1], &LU[1][0], &LU[1][1], &W, &V}, st};
+    if ((s = dev_alloc((void **)&D, (size_t)ns * nx * blk, "bcr: work", st)) != HELM_OK ||
+        (s = dev_alloc((void **)&LU[0][0], (size_t)ns * half * blk, "bcr: work", st)) != HELM_OK ||
+        (s = dev_alloc((void **)&LU[0][1], (size_t)ns * half * blk, "bcr: work", st)) != HELM_OK ||
+        (s = dev_alloc((void **)&LU[1][0], (size_t)ns * quart * blk, "bcr: work", st)) != HELM_OK ||
+        (s = dev_alloc((void **)&LU[1][1], (size_t)ns * quart * blk, "bcr: work", st)) != HELM_OK ||
+        (s = dev_alloc((void **)&W, (size_t)ns * quart * blk, "bcr: work", st)) != HELM_OK ||
+        (s = dev_alloc((void **)&V, (size_t)ns * quart * blk, "bcr: work", st)) != HELM_OK)
         return s;
-    if ((s = dev_alloc((void **)&b.split, kSolveSplitElems * sizeof(float2), "bcr: split-K tiles", st)) != HELM_OK)
-        return s;
-    b.split_cap = kSolveSplitElems;
+    const int lu_stride[2] = {half, quart};
     cudaError_t e;
     Plan pl(st);
     if ((s = pl.with_split(kFactorSplitElems)) != HELM_OK) return s;
@@ -870,7 +813,7 @@ helm_status bcr_factor(helm_factor_t *f) {
     tri.cz_edge = coup_of(g).cz_edge;
     {
         const double2 *diag = op->diag;
-        float2 *D0 = Dc;
+        float2 *D0 = D;
         const Coup cp = coup_of(g);
         const int perq = (int)std::min<long long>(64, (nz2 / 2 + 255) / 256);
         if (!tri_level0) pl.ops.push_back([=](const int *) -> helm_status {
@@ -880,155 +823,158 @@ helm_status bcr_factor(helm_factor_t *f) {
             return HELM_OK;
         });
     }
-    const Fam fD{Dc, nz2, nz}, fDinv{b.Dinv, nz2, nz};
-    int levels = 0;
+    const Fam fD{D, nz2, nz};
+    auto mat = [&](int kind, int sy, int slot) { return (int)bs_matrix_index(nx, ns, half, kind << 24 | slot, sy); };
+    int cur = 0, levels = 0;   // L, U of the current spacing in LU[cur]
     for (int sp = 1; sp < nx; sp *= 2, ++levels) {
-        std::vector<int> inv_pairs, tv, tw, tp, tq, td, tl, tu;
+        std::vector<int> inv_pairs, tv, tw, td, tl, tu;
         for (int sy = 0; sy < ns; ++sy)
             for (int j = sp; j < nx; j += 2 * sp) inv_pairs.insert(inv_pairs.end(), {sy * nx + j, sy * nx + j});
         // level 0: the line blocks are still tridiagonal
-        s = (sp == 1 && tri_level0) ? invert_tridiag_blocks(nz, fD, fDinv, inv_pairs, op->status, pl, tri)
-                                    : invert_blocks(nz, fD, fDinv, inv_pairs, op->status, pl);
+        s = (sp == 1 && tri_level0) ? invert_tridiag_blocks(nz, fD, fD, inv_pairs, op->status, pl, tri)
+                                    : invert_blocks(nz, fD, fD, inv_pairs, op->status, pl);
         if (s != HELM_OK) return s;
         if (sp == 1) {
-            float2 *D0 = Dc, *Di = b.Dinv, *L1 = Ln, *U1 = Un;
+            float2 *D0 = D, *L1 = LU[0][0], *U1 = LU[0][1];
             const Coup cp = coup_of(g);
             pl.ops.push_back([=](const int *) -> helm_status {
                 HELM_TRACED(K_BCR_L0, st, (bcr_level0_kernel<<<dim3(per, (nx + 1) / 2, ns), 256, 0, st>>>(
-                                              g, cp, D0, Di, L1, U1, half, tri_diag)));
+                                              g, cp, D0, D0, L1, U1, half, tri_diag)));
                 const cudaError_t e2 = cudaGetLastError();
                 if (e2 != cudaSuccess) { helm_set_error("bcr: level 0", e2); return HELM_ECUDA; }
                 return HELM_OK;
             });
-        } else {
-            std::vector<int> vpairs, wpairs;
-            for (int sy = 0; sy < ns; ++sy) {
-                const int hb = sy * half, lb = sy * nx;
-                for (int j = sp; j < nx; j += 2 * sp) {
-                    // V_j = U_{j-s} Dinv_j;  W_j = L_{j+s} Dinv_j
-                    auto v = task8(hb + (j - sp) / 2, lb + j, 0, hb + j / 2);
-                    tv.insert(tv.end(), v.begin(), v.end());
-                    vpairs.insert(vpairs.end(), {hb + j / 2, hb + j / 2});
-                    if (j + sp < nx) {
-                        auto w = task8(hb + (j + sp) / 2, lb + j, 0, hb + j / 2);
-                        tw.insert(tw.end(), w.begin(), w.end());
-                        wpairs.insert(wpairs.end(), {hb + j / 2, hb + j / 2});
-                    }
-                }
-                for (int k = 0; k < nx; k += 2 * sp) {
-                    const bool ha = k >= sp, hc = k + sp < nx;
-                    if (!ha && !hc) continue;
-                    // D_k -= L_k W_a^T + U_k V_c^T
-                    auto d = task8(ha ? hb + k / 2 : -1, ha ? hb + (k - sp) / 2 : 0, lb + k, lb + k,
-                                   hc ? hb + k / 2 : -1, hc ? hb + (k + sp) / 2 : 0);
-                    td.insert(td.end(), d.begin(), d.end());
-                    if (k >= 2 * sp) {   // L_k <- -L_k V_a^T
-                        auto l = task8(hb + k / 2, hb + (k - sp) / 2, 0, hb + k / 2);
-                        tl.insert(tl.end(), l.begin(), l.end());
-                    }
-                    if (k + 2 * sp < nx) {   // U_k <- -U_k W_c^T
-                        auto u = task8(hb + k / 2, hb + (k + sp) / 2, 0, hb + k / 2);
-                        tu.insert(tu.end(), u.begin(), u.end());
-                    }
+            continue;   // (level 0 writes LU[0], which stays current)
+        }
+        const int nxt = cur ^ 1, cs = lu_stride[cur], nsd = lu_stride[nxt];
+        std::vector<int> vi, vt, wi, wt;   // images of V, P = V^T, W, Q = W^T
+        for (int sy = 0; sy < ns; ++sy) {
+            const int cb = sy * cs, nb = sy * nsd, lb = sy * nx, qb = sy * quart;
+            for (int j = sp; j < nx; j += 2 * sp) {
+                const int i = (j - sp) / (2 * sp);
+                // V_j = U_{j-s} Dinv_j;  W_j = L_{j+s} Dinv_j
+                auto v = task8(cb + (j - sp) / sp, lb + j, 0, qb + i);
+                tv.insert(tv.end(), v.begin(), v.end());
+                vi.insert(vi.end(), {qb + i, mat(BS_V, sy, j / 2)});
+                vt.insert(vt.end(), {qb + i, mat(BS_P, sy, j / 2)});
+                if (j + sp < nx) {
+                    auto w = task8(cb + (j + sp) / sp, lb + j, 0, qb + i);
+                    tw.insert(tw.end(), w.begin(), w.end());
+                    wi.insert(wi.end(), {qb + i, mat(BS_W, sy, j / 2)});
+                    wt.insert(wt.end(), {qb + i, mat(BS_Q, sy, j / 2)});
                 }
             }
-            ZGemmArgs ga;
-            ga.M = ga.N = ga.K = nz;
-            ga.status = op->status;
-            ga.nterms = 1;
-            ga.B[0] = zop(b.Dinv, nz2, nz);
-            ga.C = b.V; ga.c_stride = nz2; ga.ldc = nz;
-            ga.A[0] = zop(Uc, nz2, nz);
-            if ((s = gemm(ga, tv, pl)) != HELM_OK) return s;
-            ga.C = b.W;
-            ga.A[0] = zop(Lc, nz2, nz);
-            if ((s = gemm(ga, tw, pl)) != HELM_OK) return s;
-            if ((s = transpose_blocks(nz, b.V, b.P, nz2, vpairs, pl)) != HELM_OK) return s;
-            if ((s = transpose_blocks(nz, b.W, b.Q, nz2, wpairs, pl)) != HELM_OK) return s;
-            ZGemmArgs gd;
-            gd.M = gd.N = gd.K = nz;
-            gd.status = op->status;
-            gd.nterms = 2;
-            gd.A[0] = zop(Lc, nz2, nz); gd.B[0] = zop(b.W, nz2, nz); gd.sign[0] = -1.f;
-            gd.A[1] = zop(Uc, nz2, nz); gd.B[1] = zop(b.V, nz2, nz); gd.sign[1] = -1.f;
-            gd.C0 = zop(Dc, nz2, nz);
-            gd.C = Dc; gd.c_stride = nz2; gd.ldc = nz;
-            if ((s = gemm(gd, td, pl)) != HELM_OK) return s;
-            ZGemmArgs gl;
-            gl.M = gl.N = gl.K = nz;
-            gl.status = op->status;
-            gl.nterms = 1;
-            gl.sign[0] = -1.f;
-            gl.A[0] = zop(Lc, nz2, nz); gl.B[0] = zop(b.V, nz2, nz);
-            gl.C = Ln; gl.c_stride = nz2; gl.ldc = nz;
-            if ((s = gemm(gl, tl, pl)) != HELM_OK) return s;
-            gl.A[0] = zop(Uc, nz2, nz); gl.B[0] = zop(b.W, nz2, nz);
-            gl.C = Un;
-            if ((s = gemm(gl, tu, pl)) != HELM_OK) return s;
+            for (int k = 0; k < nx; k += 2 * sp) {
+                const bool ha = k >= sp, hc = k + sp < nx;
+                if (!ha && !hc) continue;
+                const int ck = cb + k / sp, nk = nb + k / (2 * sp), ia = qb + k / (2 * sp) - 1, ic = qb + k / (2 * sp);
+                // D_k -= L_k W_a^T + U_k V_c^T
+                auto d = task8(ha ? ck : -1, ha ? ia : 0, lb + k, lb + k, hc ? ck : -1, hc ? ic : 0);
+                td.insert(td.end(), d.begin(), d.end());
+                if (k >= 2 * sp) {   // L_k <- -L_k V_a^T
+                    auto l = task8(ck, ia, 0, nk);
+                    tl.insert(tl.end(), l.begin(), l.end());
+                }
+                if (k + 2 * sp < nx) {   // U_k <- -U_k W_c^T
+                    auto u = task8(ck, ic, 0, nk);
+                    tu.insert(tu.end(), u.begin(), u.end());
+                }
+            }
         }
-        std::swap(Lc, Ln);
-        std::swap(Uc, Un);
+        float2 *Lc = LU[cur][0], *Uc = LU[cur][1], *Ln = LU[nxt][0], *Un = LU[nxt][1];
+        ZGemmArgs ga;
+        ga.M = ga.N = ga.K = nz;
+        ga.status = op->status;
+        ga.nterms = 1;
+        ga.B[0] = zop(D, nz2, nz);
+        ga.C = V; ga.c_stride = nz2; ga.ldc = nz;
+        ga.A[0] = zop(Uc, nz2, nz);
+        if ((s = gemm(ga, tv, pl)) != HELM_OK) return s;
+        ga.C = W;
+        ga.A[0] = zop(Lc, nz2, nz);
+        if ((s = gemm(ga, tw, pl)) != HELM_OK) return s;
+        if ((s = image_blocks(nz, V, false, vi, b.img, b.scl, pl)) != HELM_OK ||
+            (s = image_blocks(nz, V, true, vt, b.img, b.scl, pl)) != HELM_OK ||
+            (s = image_blocks(nz, W, false, wi, b.img, b.scl, pl)) != HELM_OK ||
+            (s = image_blocks(nz, W, true, wt, b.img, b.scl, pl)) != HELM_OK)
+            return s;
+        ZGemmArgs gd;
+        gd.M = gd.N = gd.K = nz;
+        gd.status = op->status;
+        gd.nterms = 2;
+        gd.A[0] = zop(Lc, nz2, nz); gd.B[0] = zop(W, nz2, nz); gd.sign[0] = -1.f;
+        gd.A[1] = zop(Uc, nz2, nz); gd.B[1] = zop(V, nz2, nz); gd.sign[1] = -1.f;
+        gd.C0 = zop(D, nz2, nz);
+        gd.C = D; gd.c_stride = nz2; gd.ldc = nz;
+        if ((s = gemm(gd, td, pl)) != HELM_OK) return s;
+        ZGemmArgs gl;
+        gl.M = gl.N = gl.K = nz;
+        gl.status = op->status;
+        gl.nterms = 1;
+        gl.sign[0] = -1.f;
+        gl.A[0] = zop(Lc, nz2, nz); gl.B[0] = zop(V, nz2, nz);
+        gl.C = Ln; gl.c_stride = nz2; gl.ldc = nz;
+        if ((s = gemm(gl, tl, pl)) != HELM_OK) return s;
+        gl.A[0] = zop(Uc, nz2, nz); gl.B[0] = zop(W, nz2, nz);
+        gl.C = Un;
+        if ((s = gemm(gl, tu, pl)) != HELM_OK) return s;
+        cur = nxt;
     }
-    // the last line left: line 0
+    // the last line left: line 0; then every line's inverse is in its slot of D
     {
-        std::vector<int> last;
+        std::vector<int> last, di;
         for (int sy = 0; sy < ns; ++sy) last.insert(last.end(), {sy * nx, sy * nx});
-        if ((s = invert_blocks(nz, fD, fDinv, last, op->status, pl)) != HELM_OK) return s;
+        if ((s = invert_blocks(nz, fD, fD, last, op->status, pl)) != HELM_OK) return s;
+        for (int i = 0; i < ns * nx; ++i) di.insert(di.end(), {i, i});
+        if ((s = image_blocks(nz, D, false, di, b.img, b.scl, pl)) != HELM_OK) return s;
     }
     if ((s = pl.run()) != HELM_OK) return s;
-    b.levels = levels;
-    // the solve's task lists, built once: forward levels 1 .. L-1, last line, backward L-1 .. 1,
-    // level 0 both ways (vector operands indexed system * nx + line)
+    // the solve's steps and tasks (the same for every system), built once
     std::vector<int> all;
-    b.fwd.assign(levels, BcrData::List());
-    b.bwd.assign(levels, BcrData::List());
-    auto list_of = [&](int off, int nt) {
-        BcrData::List L;
-        L.first = off;
-        L.count = (int)all.size() / 8 - off;
-        L.terms = count_terms(all.data() + 8 * (size_t)off, (size_t)L.count, nt);
-        return L;
+    b.terms = 0;
+    auto step = [&](int first) {
+        const int n = (int)all.size() / 8 - first;
+        if (n > 0) b.steps.push_back(BsStep{first, n});
     };
-    auto add = [&](std::vector<int> &&v) { all.insert(all.end(), v.begin(), v.end()); };
-    for (int l = 0, sp = 1; l < levels; ++l, sp *= 2) {
-        const int off = (int)all.size() / 8;
-        for (int sy = 0; sy < ns; ++sy) {
-            const int hb = sy * half, lb = sy * nx;
-            if (l == 0) {
-                for (int j = 1; j < nx; j += 2) add(task8(lb + j, lb + j, 0, lb + j));   // y_j = Dinv_j b_j
-            } else {
-                for (int k = 0; k < nx; k += 2 * sp) {
-                    const bool ha = k >= sp, hc = k + sp < nx;
-                    if (!ha && !hc) continue;
-                    add(task8(ha ? hb + (k - sp) / 2 : -1, ha ? lb + k - sp : 0, lb + k, lb + k,
-                              hc ? hb + (k + sp) / 2 : -1, hc ? lb + k + sp : 0));
-                }
-            }
+    auto add = [&](int line, int type, std::initializer_list<std::pair<int, int>> terms) {
+        const size_t o = all.size();
+        all.resize(o + 8, 0);
+        all[o] = line;
+        all[o + 1] = type | (int)terms.size() << 4;
+        int q = 2;
+        for (auto &t : terms) { all[o + q++] = t.first; all[o + q++] = t.second; }
+        b.terms += (long long)terms.size();
+    };
+    auto blk_of = [](int kind, int slot) { return kind << 24 | slot; };
+    auto pair_step = [&](int sp, int type, int kind_a, int kind_c, int shift) {   // kept lines and their two neighbours
+        const int first = (int)all.size() / 8;
+        for (int k = 0; k < nx; k += 2 * sp) {
+            const int a = k - sp, c = k + sp;
+            if (a >= 0 && c < nx) add(k, type, {{blk_of(kind_a, a >> shift), a}, {blk_of(kind_c, c >> shift), c}});
+            else if (a >= 0) add(k, type, {{blk_of(kind_a, a >> shift), a}});
+            else if (c < nx) add(k, type, {{blk_of(kind_c, c >> shift), c}});
         }
-        b.fwd[l] = list_of(off, l == 0 ? 1 : 2);
-    }
-    {
-        const int off = (int)all.size() / 8;
-        for (int sy = 0; sy < ns; ++sy) add(task8(sy * nx, sy * nx, 0, sy * nx));
-        b.last = list_of(off, 1);
-    }
-    for (int l = 0, sp = 1; l < levels; ++l, sp *= 2) {
-        const int off = (int)all.size() / 8;
-        for (int sy = 0; sy < ns; ++sy) {
-            const int hb = sy * half, lb = sy * nx;
-            for (int j = sp; j < nx; j += 2 * sp) {
-                if (l == 0) {
-                    add(task8(lb + j, lb + j, lb + j, lb + j));   // x_j = y_j - Dinv_j t_j
-                } else {
-                    const bool hc = j + sp < nx;
-                    add(task8(lb + j, lb + j, 0, lb + j, hb + j / 2, lb + j - sp, hc ? hb + j / 2 : -1,
-                              hc ? lb + j + sp : 0));
-                }
-            }
+        step(first);
+    };
+    pair_step(1, BS_FWD0, BS_DINV, BS_DINV, 0);
+    for (int l = 1, sp = 2; l < levels; ++l, sp *= 2) pair_step(sp, BS_FWD, BS_W, BS_V, 1);
+    add(0, BS_LAST, {{blk_of(BS_DINV, 0), 0}});
+    step((int)all.size() / 8 - 1);
+    for (int l = levels - 1; l >= 0; --l) {
+        const int sp = 1 << l, first = (int)all.size() / 8;
+        for (int j = sp; j < nx; j += 2 * sp) {
+            if (l == 0) add(j, BS_BWD0, {{blk_of(BS_DINV, j), j}});
+            else if (j + sp < nx)
+                add(j, BS_BWD, {{blk_of(BS_DINV, j), j}, {blk_of(BS_P, j / 2), j - sp}, {blk_of(BS_Q, j / 2), j + sp}});
+            else add(j, BS_BWD, {{blk_of(BS_DINV, j), j}, {blk_of(BS_P, j / 2), j - sp}});
         }
-        b.bwd[l] = list_of(off, l == 0 ? 1 : 3);
+        step(first);
     }
-    if ((s = dev_alloc((void **)&b.tasks, all.size() * sizeof(int), "bcr: solve plan", st)) != HELM_OK) return s;
+    if ((int)b.steps.size() > BS_MAX_PHASE) { helm_set_msg("bcr: too many levels"); return HELM_EINVAL; }
+    if ((s = dev_alloc((void **)&b.tasks, all.size() * sizeof(int), "bcr: solve plan", st)) != HELM_OK ||
+        (s = dev_alloc((void **)&b.ctl, bs_ctl_words((int)b.steps.size(), ns) * sizeof(unsigned), "bcr: solve counters",
+                       st)) != HELM_OK)
+        return s;
     if ((e = cudaMemcpyAsync(b.tasks, all.data(), all.size() * sizeof(int), cudaMemcpyHostToDevice, st)) != cudaSuccess) {
         helm_set_error("bcr: solve plan", e);
         return HELM_ECUDA;
@@ -1040,115 +986,49 @@ helm_status bcr_factor(helm_factor_t *f) {
 void bcr_free(helm_factor_t *f) {
     const cudaStream_t st = f->op ? f->op->st : nullptr;
     BcrData &b = f->bcr;
-    dev_free(b.Dinv, st);
-    dev_free(b.P, st);
-    dev_free(b.Q, st);
-    dev_free(b.W, st);
-    dev_free(b.V, st);
+    dev_free(b.img, st);
+    dev_free(b.scl, st);
     dev_free(b.tasks, st);
-    dev_free(b.split, st);
+    dev_free(b.ctl, st);
+    dev_free(b.gsmall, st);
     b = BcrData();
 }
 
 // ------------------------------------------------------------------- solve
 
+size_t bcr_maxima_elems(const GridGeom &g, size_t cols) { return 2 * cols * g.nx * (size_t)bs_layout(g.nz).ng; }
+
 // x = A~^{-1} r for every system and right-hand side, complex FP32: r [n_sys][nrhs][N] is the
 // working vector (overwritten), x [n_sys][nrhs][N] the result.  skip: launches do nothing
-// while it is set (refinement finished).
-helm_status bcr_solve(const helm_factor_t *f, int nrhs, float2 *r, float2 *x, const int *skip, const int *frozen) {
+// while it is set (refinement finished).  maxima: bcr_maxima_elems floats of scratch.
+helm_status bcr_solve(const helm_factor_t *f, int nrhs, float2 *r, float2 *x, float *maxima, const int *skip,
+                      const int *frozen) {
     const helm_op *op = f->op;
     const GridGeom &g = op->g;
-    const int nx = g.nx, nz = g.nz, ns = op->n_omega, N = nx * nz;
-    const long long nz2 = (long long)nz * nz;
     const BcrData &b = f->bcr;
-    const cudaStream_t st = op->st;
-    const long long vhi = (long long)nrhs * N;   // vectors: index system * nx + line
-    auto vec = [&](const float2 *base) {   // ns groups of nx line vectors
-        ZOperand o = zop(base, nz, N, nx, vhi);
-        o.count = ns;
-        return o;
-    };
-    const long long n_lines = (long long)ns * nx, n_half = (long long)ns * b.half;
-    auto blocks = [&](const float2 *base, long long count) {
-        ZOperand o = zop(base, nz2, nz);
-        o.count = count;
-        return o;
-    };
-    ZGemmArgs ga;
-    ga.M = nz; ga.N = nrhs; ga.K = nz;
-    ga.c_col = 1;
-    ga.status = op->status;
-    ga.skip = skip;
-    ga.tries = wait_tries();
-    ga.part = b.split;
-    ga.part_cap = b.split_cap;
-    ga.sys_frozen = frozen;   // C index = system * nx + line
-    ga.sys_div = nx;
-    ga.c_stride = nz; ga.c_div = nx; ga.c_stride_hi = vhi; ga.ldc = N;
-    cudaError_t e;
-    auto launch = [&](ZGemmArgs a, const BcrData::List &lst) -> helm_status {
-        a.tasks = b.tasks + 8 * (size_t)lst.first;
-        a.flops = 8.0 * a.M * a.N * a.K * (double)lst.terms;
-        e = launch_zgemm(a, lst.count, st);
-        if (e != cudaSuccess) { helm_set_error("bcr solve: tensor-core GEMM", e); return HELM_ECUDA; }
-        return HELM_OK;
-    };
-    helm_status s;
-    const int nodd = nx / 2, neven = (nx + 1) / 2;
-    const Coup cp = coup_of(g);
-    const int cols = ns * nrhs, thr = std::min(128, nz / 2), per = (nz / 2 + thr - 1) / thr;
-    const int colb = (cols + L0_COLS - 1) / L0_COLS;
-    // forward, level 0: y_j = Dinv_j b_j into x, then b_k -= C (y_{k-1} + y_{k+1})
-    {
-        ZGemmArgs a = ga;
-        a.nterms = 1;
-        a.A[0] = blocks(b.Dinv, n_lines);
-        a.B[0] = vec(r);
-        a.C = x;
-        if ((s = launch(a, b.fwd[0])) != HELM_OK) return s;
-        HELM_TRACED(K_BCR_SOLVE_L0, st, (bcr_solve_l0_fwd_kernel<<<dim3(per, neven, colb), thr, 0, st>>>(
-                                            g, cp, cols, r, x, skip, frozen, nrhs)));
-        if ((e = cudaGetLastError()) != cudaSuccess) { helm_set_error("bcr solve: level 0", e); return HELM_ECUDA; }
-    }
-    for (int l = 1; l < b.levels; ++l) {   // b_k -= W_a b_a + V_c b_c
-        ZGemmArgs a = ga;
-        a.nterms = 2;
-        a.A[0] = blocks(b.W, n_half); a.B[0] = vec(r); a.sign[0] = -1.f;
-        a.A[1] = blocks(b.V, n_half); a.B[1] = vec(r); a.sign[1] = -1.f;
-        a.C0 = vec(r);
-        a.C = r;
-        if ((s = launch(a, b.fwd[l])) != HELM_OK) return s;
-    }
-    {   // x_0 = Dinv_0 b_0
-        ZGemmArgs a = ga;
-        a.nterms = 1;
-        a.A[0] = blocks(b.Dinv, n_lines);
-        a.B[0] = vec(r);
-        a.C = x;
-        if ((s = launch(a, b.last)) != HELM_OK) return s;
-    }
-    for (int l = b.levels - 1; l >= 1; --l) {   // x_j = Dinv_j b_j - P_j x_{j-s} - Q_j x_{j+s}
-        ZGemmArgs a = ga;
-        a.nterms = 3;
-        a.A[0] = blocks(b.Dinv, n_lines); a.B[0] = vec(r);
-        a.A[1] = blocks(b.P, n_half); a.B[1] = vec(x); a.sign[1] = -1.f;
-        a.A[2] = blocks(b.Q, n_half); a.B[2] = vec(x); a.sign[2] = -1.f;
-        a.C = x;
-        if ((s = launch(a, b.bwd[l])) != HELM_OK) return s;
-    }
-    {   // backward, level 0: t_j = C (x_{j-1} + x_{j+1}) into b_j, x_j = y_j - Dinv_j t_j
-        if (nodd > 0) {
-            HELM_TRACED(K_BCR_SOLVE_L0, st, (bcr_solve_l0_bwd_kernel<<<dim3(per, nodd, colb), thr, 0, st>>>(
-                                                g, cp, cols, r, x, skip, frozen, nrhs)));
-            if ((e = cudaGetLastError()) != cudaSuccess) { helm_set_error("bcr solve: level 0", e); return HELM_ECUDA; }
-        }
-        ZGemmArgs a = ga;
-        a.nterms = 1;
-        a.A[0] = blocks(b.Dinv, n_lines); a.B[0] = vec(r); a.sign[0] = -1.f;
-        a.C0 = vec(x);
-        a.C = x;
-        if ((s = launch(a, b.bwd[0])) != HELM_OK) return s;
-    }
+    BsArgs a{};
+    a.nx = g.nx;
+    a.nz = g.nz;
+    a.ns = op->n_omega;
+    a.nrhs = nrhs;
+    a.half = b.half;
+    a.r = r;
+    a.x = x;
+    a.gr = maxima;
+    a.gx = maxima + bcr_maxima_elems(g, (size_t)a.ns * nrhs) / 2;
+    a.img = b.img;
+    a.scl = b.scl;
+    a.tasks = b.tasks;
+    a.cx_in = (float)coup_x(g, 1);
+    a.cx_edge = (float)coup_x(g, 0);
+    a.ctl = b.ctl;
+    a.status = op->status;
+    a.skip = skip;
+    a.frozen = frozen;
+    a.tries = wait_tries();
+    const double flops = 8.0 * g.nz * g.nz * nrhs * (double)b.terms * a.ns;
+    const cudaError_t e = launch_bcr_solve(a, b.steps.data(), (int)b.steps.size(), flops, op->st);
+    if (e != cudaSuccess) { helm_set_error("bcr solve", e); return HELM_ECUDA; }
     return HELM_OK;
 }
 

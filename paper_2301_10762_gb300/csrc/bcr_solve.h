@@ -1,0 +1,71 @@
+// The persistent solve of a block-cyclic-reduction factor (bcr_solve.cu; internal header).
+#pragma once
+#include <cuda_runtime.h>
+#include <stdint.h>
+
+namespace helm {
+
+// Blocks of the factor in the solve's operand layout: n_chunk chunks of 32 columns, each the rows
+// (padded to 8) of the real and then of the imaginary part, 128 bytes a row (32 hi, 32 lo FP16)
+struct BsLayout {
+    int n_chunk, nzr, ng;   // ng: 32-row groups of a line (the vectors' maxima)
+    size_t mat_bytes;
+};
+__host__ __device__ inline BsLayout bs_layout(int nz) {
+    BsLayout l;
+    l.n_chunk = (nz + 31) / 32;
+    l.nzr = (nz + 7) & ~7;
+    l.ng = (nz + 31) / 32;
+    l.mat_bytes = (size_t)l.n_chunk * 2 * l.nzr * 128;
+    return l;
+}
+
+// Kinds of stored blocks: per system n_x inverses, then n_half of W, V, P and Q each (slot line / 2).
+// A block of a task is coded kind << 24 | slot; P and Q multiply x, the others r.
+enum { BS_DINV = 0, BS_W = 1, BS_V = 2, BS_P = 3, BS_Q = 4 };
+// steps (types of tasks): level 0 forward, level forward, last line, level backward, level 0 backward
+enum { BS_FWD0 = 0, BS_FWD = 1, BS_LAST = 2, BS_BWD = 3, BS_BWD0 = 4 };
+constexpr int BS_MAX_PHASE = 64;
+
+struct BsStep {   // one dependent step of the solve: its tasks (the same for every system)
+    int task0, tasks;
+};
+struct BsPhase {
+    int tile0, task0, tasks, mt, mrows, done;
+};
+struct BsArgs {
+    int nx, nz, ns, nrhs, half;
+    float2 *r, *x;          // [ns][nrhs][N]: right-hand sides (overwritten) and the result
+    float *gr, *gx;         // maxima of r and x: [ns][nx][ng][nrhs] each
+    const unsigned char *img;
+    const float *scl;       // [matrix][nz]: 2^-s of each row of the image
+    const int *tasks;       // [8] per task: line, type | terms << 4, then (block, line of the vector) per term
+    float cx_in, cx_edge;
+    unsigned *ctl;          // tile counter, abort word, tiles finished per step and system
+    int *status;
+    const int *skip, *frozen;
+    uint32_t tries;
+    // set by launch_bcr_solve
+    int N, n_chunk, nzr, ng, n_tiles, n_phase, n_tile_total;
+    size_t mat_bytes;
+    BsPhase ph[BS_MAX_PHASE];
+};
+inline size_t bs_ctl_words(int n_steps, int ns) { return 2 + (size_t)n_steps * ns; }
+__host__ __device__ inline int bs_kind(int code) { return code >> 24; }
+// matrix number of a coded block of system sys
+__host__ __device__ inline long long bs_matrix_index(int nx, int ns, int half, int code, int sys) {
+    const int kind = code >> 24, slot = code & 0xffffff;
+    return kind == BS_DINV ? (long long)sys * nx + slot
+                           : (long long)ns * nx + ((long long)(kind - 1) * ns + sys) * half + slot;
+}
+__device__ __forceinline__ long long bs_matrix(const BsArgs &a, int code, int sys) {
+    return bs_matrix_index(a.nx, a.ns, a.half, code, sys);
+}
+
+// dst matrices (pairs[.][1]) of the image from n x n row-major blocks src + pairs[.][0] * stride
+cudaError_t launch_bcr_image(int n, const float2 *src, long long stride, bool trans, const int *pairs_dev, int count,
+                             unsigned char *img, float *scl, cudaStream_t st);
+cudaError_t launch_bcr_solve(BsArgs a, const BsStep *steps, int n_steps, double flops, cudaStream_t st);
+int device_sms();   // streaming multiprocessors of the current device
+
+}  // namespace helm

@@ -88,14 +88,16 @@ struct helm_server {
         const helm::GridGeom geom{g.nx, g.nz, g.lx / (g.nx - 1), g.lz / (g.nz - 1), g.lumping};
         if (helm::factor_picks_bcr(geom, (helm_prec)prec, HELM_FACTOR_AUTO)) {
             // block cyclic reduction: the inverses of every line and P, Q, W, V of the eliminated
-            // ones, and as much again of working blocks while it factors (counted throughout)
-            const size_t kept = ((size_t)g.nx + 4 * ((size_t)g.nx / 2 + 1)) * blk;
-            return 2 * kept + 96 * N + 97 * kMiB;   // + the split-K tiles (32 MB kept, 64 MB while factoring)
+            // ones (rows padded to 32 columns), and as many working blocks while it factors
+            // (counted throughout)
+            const size_t kept = (size_t)g.nx + 4 * ((size_t)g.nx / 2 + 1);
+            return kept * (blk + helm::bs_layout(g.nz).mat_bytes + 4 * (size_t)g.nz) + 96 * N + 65 * kMiB;   // + the split-K tiles
         }
         return (size_t)g.nx * g.nz * g.nz * (prec == HELM_MIXED ? 8 : 16) + 96 * N + kMiB;
     }
     size_t scratch_bytes(const helm_grid &g, int prec, int nrhs) const {   // refinement scratch in the factor
-        return prec == HELM_MIXED ? (size_t)g.nx * g.nz * nrhs * 64 + (size_t)nrhs * 16 : (size_t)nrhs * 16;
+        return prec == HELM_MIXED ? (size_t)g.nx * (64 * g.nz + 8 * helm::bs_layout(g.nz).ng) * nrhs + (size_t)nrhs * 16
+                                  : (size_t)nrhs * 16;
     }
     size_t staging_bytes(const helm_grid &g, int nrhs) const {   // device B and X of a batch
         return (size_t)g.nx * g.nz * nrhs * 32;

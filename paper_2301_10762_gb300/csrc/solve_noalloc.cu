@@ -151,6 +151,7 @@ extern "C" helm_status helm_solve_noalloc(helm_factor_t *f, int32_t nrhs, const 
         w.norms = (double *)(p + 3 * p_bytes + 2 * v_bytes);
         w.norms_host = g_norms_host;
         w.state = (RefineState *)(p + 3 * p_bytes + 2 * v_bytes + n_bytes);
+        w.maxima = f->bcr.gsmall;   // (every call within the limits above fits it)
         if ((s = mixed_refine(f, nrhs, B, X, conj, rtol, max_iter, w, &it, &rel)) != HELM_OK) return s;
     }
     if (info) { info->iters = it; info->max_relres = rel; }

@@ -26,6 +26,11 @@ __host__ __device__ constexpr uint32_t idesc_tf32(int n_real) {
     return (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(n_real >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
 }
 
+// the same for FP16 operands; neg_b: the product with -B
+__host__ __device__ constexpr uint32_t idesc_f16(int n_real, bool neg_b) {
+    return (1u << 4) | (neg_b ? 1u << 14 : 0u) | ((uint32_t)(n_real >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
+}
+
 // x rounded to the TF32 grid (10 explicit mantissa bits), to nearest with ties away from zero:
 // add half a unit of the 11th bit to the magnitude bits and clear the 13 low bits.  Integer
 // operations at full rate (the conversion instruction runs on a low-rate pipe, and the operand
@@ -54,6 +59,14 @@ __device__ __forceinline__ void tc_mma(uint32_t tmem_d, uint64_t adesc, uint64_t
     asm volatile(
         "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
         " tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem_d),
+        "l"(adesc), "l"(bdesc), "r"(idesc), "r"(acc)
+        : "memory");
+}
+
+__device__ __forceinline__ void tc_mma_f16(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t acc) {
+    asm volatile(
+        "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
+        " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem_d),
         "l"(adesc), "l"(bdesc), "r"(idesc), "r"(acc)
         : "memory");
 }

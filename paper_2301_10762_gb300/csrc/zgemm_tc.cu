@@ -28,6 +28,7 @@
 
 #include <algorithm>
 
+#include "bcr_solve.h"
 #include "common.cuh"
 #include "kernels.h"
 #include "tcgen05.cuh"
@@ -465,18 +466,6 @@ __global__ void zsplit_reduce_kernel(ZGemmArgs a) {
     a.C[zop_off(task[7], a.c_div, a.c_stride, a.c_stride_hi) + (long long)i * a.ldc + o] = v;
 }
 
-// streaming multiprocessors of the current device (queried once)
-int num_sms() {
-    static const int n = []() {
-        int dev = 0, v = 0;
-        if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-            v = 0;
-        cudaGetLastError();
-        return v > 0 ? v : 148;
-    }();
-    return n;
-}
-
 using EncodeTiledFn = CUresult (*)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *,
                                    const cuuint64_t *, const cuuint32_t *, const cuuint32_t *, CUtensorMapInterleave,
                                    CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
@@ -546,7 +535,7 @@ template <int NT, bool RING> cudaError_t launch_nt(const ZGemmArgs &a, const ZMa
     ZGemmArgs b = a;
     b.ksplit = 1;
     const long long tiles = (long long)((a.M + ZG_BM - 1) / ZG_BM) * ((a.N + NT - 1) / NT) * n_tasks;
-    const int kNumSMs = num_sms();
+    const int kNumSMs = device_sms();
     if (a.part && tiles * 2 <= kNumSMs) {
         const int nkc = (a.K + ZG_KC - 1) / ZG_KC;
         long long ks = std::min<long long>(nkc, kNumSMs / tiles);
@@ -578,6 +567,18 @@ template <int NT> cudaError_t launch_narrow(const ZGemmArgs &a, int n_tasks, cud
 }
 
 }  // namespace
+
+// streaming multiprocessors of the current device (queried once)
+int device_sms() {
+    static const int n = []() {
+        int dev = 0, v = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+            v = 0;
+        cudaGetLastError();
+        return v > 0 ? v : 148;
+    }();
+    return n;
+}
 
 cudaError_t launch_zgemm(const ZGemmArgs &a, int n_tasks, cudaStream_t st) {
     if (n_tasks <= 0) return cudaSuccess;
