@@ -934,7 +934,7 @@ helm_status bcr_factor(helm_factor_t *f) {
     b.terms = 0;
     auto step = [&](int first) {
         const int n = (int)all.size() / 8 - first;
-        if (n > 0) b.steps.push_back(BsStep{first, n});
+        if (n > 0) b.steps.push_back(BsStep{first, n, all[8 * (size_t)first + 1] & 15});
     };
     auto add = [&](int line, int type, std::initializer_list<std::pair<int, int>> terms) {
         const size_t o = all.size();

@@ -44,19 +44,26 @@ namespace {
 
 constexpr int BS_WARPS = 14;                 // MMA, copy, 4 epilogue, 8 operand warps
 constexpr int BS_THREADS = 32 * BS_WARPS;
-constexpr int BS_EPI0 = 2, BS_OP0 = 6, BS_OPW = 8;
+constexpr int BS_OP0 = 6, BS_OPW = 8;        // (epilogue warps 2 .. 5)
 constexpr int BS_QD = 4;                     // tile queue of a CTA
 constexpr int BS_A = 32768;                  // A bytes of a stage: 128 rows x 128 bytes, Re and Im
 constexpr uint32_t BS_TMEM = 512;
 
+constexpr int BS_SLOTS = 4, BS_SLOT_COLS = 128;   // accumulators: one per product term, 128 columns
+
+// NT: widest tile of the launch (right-hand sides); a step with few lines takes narrower ones
 template <int NT> struct BsCfg {
     static constexpr int B = NT * 256;                   // B bytes of a stage: NT rows x 128 bytes, Re and Im
     static constexpr int STAGE = BS_A + B;
-    static constexpr int STAGES = NT == 64 ? 4 : 5;
-    static constexpr int SLOTS = NT == 64 ? 4 : 8;       // accumulators of 2 NT tensor-memory columns
+    static constexpr int STAGES = NT == 16 ? 5 : 3;
     static constexpr int PAIRS = NT / 16;                // row pairs of a chunk per operand warp
-    static constexpr size_t SMEM = (size_t)STAGES * STAGE + 1024;
+    // raw vector chunks on their way (NT rows x 256 bytes each): five, or three of three vectors in
+    // the last step, which takes tiles of at most 32 right-hand sides
+    static constexpr int RAW = NT == 64 ? 5 * B : 9 * B;
+    static constexpr size_t SMEM = (size_t)STAGES * STAGE + RAW + 1024;
 };
+constexpr int BS_AHEAD = 4, BS_AHEAD0 = 2;   // vector chunks in flight ahead of the one being split
+constexpr int BS_NT_BWD0 = 32;
 
 __device__ __forceinline__ void bulk_load(uint32_t dst, const void *src, uint32_t bytes, uint64_t *bar) {
     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
@@ -88,31 +95,43 @@ __device__ __forceinline__ void split_h2(float a, float b, uint32_t &hi, uint32_
 }
 
 struct Tile {
-    int phase, sys, task, n0, r0, rows;
+    int phase, sys, task, n0, r0, rows, nt;
 };
-__device__ __forceinline__ Tile decode(const BsArgs &a, int t, int nt_size) {
+__device__ __forceinline__ Tile decode(const BsArgs &a, int t) {
     int p = 0;
     while (p + 1 < a.n_phase && t >= a.ph[p + 1].tile0) ++p;
     const BsPhase &ph = a.ph[p];
     int q = t - ph.tile0;
     Tile o;
     o.phase = p;
+    o.nt = ph.nt;
     o.r0 = (q % ph.mt) * ph.mrows;
     q /= ph.mt;
-    o.n0 = (q % a.n_tiles) * nt_size;
-    q /= a.n_tiles;
+    o.n0 = (q % ph.n_tiles) * ph.nt;
+    q /= ph.n_tiles;
     o.sys = q / ph.tasks;
     o.task = ph.task0 + q % ph.tasks;
     o.rows = min(ph.mrows, a.nzr - o.r0);
     return o;
 }
 
-template <int NT, bool EVEN>
+// 16 bytes global -> shared through L2 (zeros if !in), asynchronous
+__device__ __forceinline__ void cp_async16_zfill(uint32_t dst, const void *src, bool in) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(in ? 16 : 0) : "memory");
+}
+__device__ __forceinline__ float4 ld_shared4(uint32_t addr) {
+    float4 v;
+    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr)
+                 : "memory");
+    return v;
+}
+
+template <int NT>
 __global__ void __launch_bounds__(BS_THREADS, 1) bcr_solve_kernel(const __grid_constant__ BsArgs a) {
     using Cfg = BsCfg<NT>;
-    constexpr int ST = Cfg::STAGES, SL = Cfg::SLOTS;
+    constexpr int ST = Cfg::STAGES, SL = BS_SLOTS, PR = Cfg::PAIRS;
     extern __shared__ uint8_t bs_smem[];
-    __shared__ __align__(8) uint64_t full_a[ST], full_b[ST], empty[ST];
+    __shared__ __align__(8) uint64_t full[ST], empty[ST];   // a stage written (the copy warp's bytes and the operand warps), read by its MMAs
     __shared__ __align__(8) uint64_t acc_full[SL], acc_empty[SL];
     __shared__ __align__(8) uint64_t tq_full[BS_QD], tq_empty[BS_QD], done_bar;
     __shared__ int tq[BS_QD];
@@ -123,8 +142,7 @@ __global__ void __launch_bounds__(BS_THREADS, 1) bcr_solve_kernel(const __grid_c
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     if (tid == 0) {
         for (int s = 0; s < ST; ++s) {
-            mbar_init(&full_a[s], 1);
-            mbar_init(&full_b[s], BS_OPW);
+            mbar_init(&full[s], 1 + BS_OPW);
             mbar_init(&empty[s], 1);
         }
         for (int s = 0; s < SL; ++s) {
@@ -157,9 +175,17 @@ __global__ void __launch_bounds__(BS_THREADS, 1) bcr_solve_kernel(const __grid_c
     };
     // bounded wait of a whole warp; false: give up (every lane takes the same decision)
     auto wait = [&](uint64_t *bar, int parity) -> bool {
-        const bool ok = mbar_wait_or_abort(bar, (uint32_t)(parity & 1), a.tries, &s_abort);
+        bool ok = a.tries > 0 && mbar_test_cta(bar, (uint32_t)(parity & 1));
+        if (__all_sync(0xffffffffu, ok)) return true;
+        ok = mbar_wait_cta(bar, (uint32_t)(parity & 1), a.tries, &s_abort);
         if (__all_sync(0xffffffffu, ok)) return true;
         if (lane == 0) give_up();
+        return false;
+    };
+    // the same for one thread on its own
+    auto wait1 = [&](uint64_t *bar, uint32_t parity) -> bool {
+        if (mbar_wait_cta(bar, parity, a.tries, &s_abort)) return true;
+        give_up();
         return false;
     };
     // next tile of the queue (i-th): its number, or -1 at the end or after a give-up
@@ -171,212 +197,180 @@ __global__ void __launch_bounds__(BS_THREADS, 1) bcr_solve_kernel(const __grid_c
         return t;
     };
 
+    // the step before tile tl's of the same system is complete (seen: the last one found complete)
+    auto step_wait = [&](const Tile &tl, int &seen) -> bool {
+        const int key = tl.phase * a.ns + tl.sys;
+        if (tl.phase == 0 || key == seen) return true;
+        const unsigned *cnt = a.ctl + 2 + (key - a.ns);
+        const unsigned want = (unsigned)a.ph[tl.phase - 1].done;
+        bool ok = false;
+        for (uint32_t q = 0; q < a.tries; ++q) {
+            if (ld_acquire(cnt) >= want) { ok = true; break; }
+            if (*(volatile int *)&s_abort || ((q & 63) == 63 && ld_acquire(a.ctl + 1))) break;
+            __nanosleep(20);
+        }
+        if (!__all_sync(0xffffffffu, ok)) {
+            if (lane == 0) give_up();
+            return false;
+        }
+        seen = key;
+        return true;
+    };
+
     if (warp == 1) {
-        // ---- copy warp: takes tiles, fills the queue, streams the blocks' chunks
-        int cc = 0;
-        bool go = true;
-        for (int i = 0; go; ++i) {
-            int t = 0;
-            if (lane == 0) {
+        // ---- copy warp (one thread): takes tiles, fills the queue, streams the blocks' chunks
+        if (elect_one()) {
+            int cs = 0, issued = 0;
+            uint32_t cph = 1;   // parity of the stage's previous release (the first round passes at once)
+            bool go = true;
+            for (int i = 0; go; ++i) {
+                int t;
                 for (;;) {   // the tiles of a converged system are passed over
                     t = (int)atomicAdd(a.ctl, 1u);
                     if (t >= a.n_tile_total) { t = -1; break; }
-                    if (!a.frozen || !a.frozen[2 * decode(a, t, NT).sys]) break;
+                    if (!a.frozen || !a.frozen[2 * decode(a, t).sys]) break;
                 }
-            }
-            t = __shfl_sync(0xffffffffu, t, 0);
-            if (i >= BS_QD && !wait(&tq_empty[i % BS_QD], i / BS_QD - 1)) break;
-            if (lane == 0) {
+                if (!wait1(&tq_empty[i % BS_QD], (uint32_t)((i / BS_QD) & 1) ^ 1u)) break;
                 tq[i % BS_QD] = t;
                 mbar_arrive(&tq_full[i % BS_QD]);
-            }
-            if (t < 0) break;
-            const Tile tl = decode(a, t, NT);
-            const int *task = a.tasks + 8 * tl.task;
-            const int nterms = task[1] >> 4;
-            const uint32_t bytes = (uint32_t)tl.rows * 128u;
-            for (int u = 0; go && u < nterms; ++u) {
-                const unsigned char *m = a.img + (size_t)bs_matrix(a, task[2 + 2 * u], tl.sys) * a.mat_bytes;
-                for (int c = 0; c < a.n_chunk; ++c, ++cc) {
-                    const int s = cc % ST;
-                    if (cc >= ST && !wait(&empty[s], cc / ST - 1)) { go = false; break; }
-                    if (lane == 0) {
-                        const uint32_t dst = smem0 + (uint32_t)(s * Cfg::STAGE);
-                        const unsigned char *src = m + ((size_t)(2 * c) * a.nzr + tl.r0) * 128;
-                        mbar_arrive_expect_tx(&full_a[s], 2 * bytes);
-                        bulk_load(dst, src, bytes, &full_a[s]);
-                        bulk_load(dst + 16384, src + (size_t)a.nzr * 128, bytes, &full_a[s]);
+                if (t < 0) break;
+                const Tile tl = decode(a, t);
+                const int *task = a.tasks + 8 * tl.task;
+                const int nterms = task[1] >> 4;
+                const uint32_t bytes = (uint32_t)tl.rows * 128u;
+                const size_t im_off = (size_t)a.nzr * 128;
+                for (int u = 0; go && u < nterms; ++u) {
+                    const unsigned char *src = a.img + (size_t)bs_matrix(a, task[2 + 2 * u], tl.sys) * a.mat_bytes +
+                                               (size_t)tl.r0 * 128;
+                    for (int c = 0; c < a.n_chunk; ++c, src += 2 * im_off) {
+                        if (!wait1(&empty[cs], cph)) { go = false; break; }
+                        const uint32_t dst = smem0 + (uint32_t)(cs * Cfg::STAGE);
+                        mbar_arrive_expect_tx(&full[cs], 2 * bytes);
+                        bulk_load(dst, src, bytes, &full[cs]);
+                        bulk_load(dst + 16384, src + im_off, bytes, &full[cs]);
+                        ++issued;
+                        if (++cs == ST) { cs = 0; cph ^= 1u; }
                     }
-                    __syncwarp();
                 }
             }
+            // no copy may land after the CTA has left.  (A stage's barrier completes with the operand
+            // warps' arrivals too, which an abort may leave out: then a fixed time is waited)
+            const int s0 = *(volatile int *)&s_abort;
+            if (s0) {
+                abort_drain();
+            } else {
+                for (int c = max(0, issued - ST); c < issued; ++c)
+                    mbar_wait_bounded(&full[c % ST], (uint32_t)((c / ST) & 1), kDefaultWaitTries);
+            }
         }
-        // no copy may land after the CTA has left
-        for (int c = max(0, cc - ST); c < cc; ++c) mbar_wait_bounded(&full_a[c % ST], (uint32_t)((c / ST) & 1), kDefaultWaitTries);
+        __syncwarp();
     } else if (warp == 0) {
-        // ---- MMA warp
-        int cc = 0, tt = 0;
-        bool go = true;
-        constexpr uint32_t id2 = idesc_f16(2 * NT, false), id1 = idesc_f16(NT, false), id1n = idesc_f16(NT, true);
-        for (int i = 0; go; ++i) {
-            const int t = next_tile(i);
-            if (t < 0) break;
-            const Tile tl = decode(a, t, NT);
-            const int nterms = a.tasks[8 * tl.task + 1] >> 4;
-            for (int u = 0; go && u < nterms; ++u, ++tt) {
-                const int sl = tt % SL;
-                if (tt >= SL && !wait(&acc_empty[sl], tt / SL - 1)) { go = false; break; }
-                const uint32_t dre = tmem + (uint32_t)(sl * 2 * NT), dim = dre + NT;
-                for (int c = 0; c < a.n_chunk; ++c, ++cc) {
-                    const int s = cc % ST;
-                    if (!wait(&full_a[s], cc / ST) || !wait(&full_b[s], cc / ST)) { go = false; break; }
-                    tc_fence_after();
-                    if (lane == 0) {
-                        const uint32_t ar = smem0 + (uint32_t)(s * Cfg::STAGE), ai = ar + 16384, br = ar + BS_A,
-                                       bi = br + (uint32_t)(NT * 128);
+        // ---- MMA warp (one thread; its instruction stream paces the whole CTA: a warp-wide vote per
+        // wait and two barriers per chunk cost 0.5 us a chunk)
+        if (elect_one()) {
+            int s = 0, sl = 0;
+            uint32_t ph = 0, slph = 1;
+            bool go = true;
+            const uint64_t dstage0 = desc_sw128(smem0);
+            for (int i = 0; go; ++i) {
+                if (!wait1(&tq_full[i % BS_QD], (uint32_t)((i / BS_QD) & 1))) break;
+                const int t = tq[i % BS_QD];
+                mbar_arrive(&tq_empty[i % BS_QD]);
+                if (t < 0) break;
+                const Tile tl = decode(a, t);
+                const int nterms = a.tasks[8 * tl.task + 1] >> 4, nt = tl.nt;
+                const uint32_t id2 = idesc_f16(2 * nt, false), id1 = idesc_f16(nt, false), id1n = idesc_f16(nt, true);
+                const bool narrow = nt <= 32;
+                for (int u = 0; go && u < nterms; ++u) {
+                    if (!wait1(&acc_empty[sl], slph)) { go = false; break; }
+                    const uint32_t d0 = tmem + (uint32_t)(sl * BS_SLOT_COLS), d1 = d0 + (uint32_t)(narrow ? 2 * nt : nt);
+                    for (int c = 0; c < a.n_chunk; ++c) {
+                        if (!wait1(&full[s], ph)) { go = false; break; }
+                        fence_proxy_async_smem();   // the operand warps' stores, ordered by the barrier
+                        tc_fence_after();
+                        const uint64_t dar = dstage0 + (uint64_t)(s * (Cfg::STAGE / 16)), dai = dar + 1024, dbr = dar + BS_A / 16,
+                                       dbi = dbr + (uint64_t)(nt * 8);
+                        // products hi*hi, hi*lo, lo*hi (lo 64 bytes into the row), each two steps of
+                        // K = 16 FP16 (32 bytes; 2 in descriptor units)
+                        if (narrow) {   // Ar [Br | Bi] and Ai [Br | Bi] side by side
 #pragma unroll
-                        for (int p = 0; p < 3; ++p) {   // hi*hi, hi*lo, lo*hi (lo 64 bytes into the row)
-                            const uint32_t oa = p == 2 ? 64u : 0u, ob = p == 1 ? 64u : 0u;
+                            for (int p = 0; p < 6; ++p) {
+                                const int ka = (p >= 4 ? 4 : 0) + 2 * (p & 1), kb = ((p >> 1) == 1 ? 4 : 0) + 2 * (p & 1);
+                                const uint32_t acc = p > 0 ? 1u : (c > 0 ? 1u : 0u);
+                                tc_mma_f16(d0, dar + ka, dbr + kb, id2, acc);
+                                tc_mma_f16(d1, dai + ka, dbr + kb, id2, acc);
+                            }
+                        } else {        // [Re | Im] += Ar [Br | Bi];  Re -= Ai Bi;  Im += Ai Br
 #pragma unroll
-                            for (int kk = 0; kk < 2; ++kk) {   // K = 16 FP16 (32 bytes) per instruction
-                                const uint32_t acc = (c > 0 || p > 0 || kk > 0) ? 1u : 0u;
-                                const uint32_t ka = oa + 32 * kk, kb = ob + 32 * kk;
-                                // [Re | Im] += Ar [Br | Bi];  Re -= Ai Bi;  Im += Ai Br
-                                tc_mma_f16(dre, desc_sw128(ar + ka), desc_sw128(br + kb), id2, acc);
-                                tc_mma_f16(dre, desc_sw128(ai + ka), desc_sw128(bi + kb), id1n, 1u);
-                                tc_mma_f16(dim, desc_sw128(ai + ka), desc_sw128(br + kb), id1, 1u);
+                            for (int p = 0; p < 6; ++p) {
+                                const int ka = (p >= 4 ? 4 : 0) + 2 * (p & 1), kb = ((p >> 1) == 1 ? 4 : 0) + 2 * (p & 1);
+                                const uint32_t acc = p > 0 ? 1u : (c > 0 ? 1u : 0u);
+                                tc_mma_f16(d0, dar + ka, dbr + kb, id2, acc);
+                                tc_mma_f16(d0, dai + ka, dbi + kb, id1n, 1u);
+                                tc_mma_f16(d1, dai + ka, dbr + kb, id1, 1u);
                             }
                         }
                         tc_commit(&empty[s]);
-                        if (c == a.n_chunk - 1) tc_commit(&acc_full[sl]);
+                        if (++s == ST) { s = 0; ph ^= 1u; }
                     }
-                    __syncwarp();
+                    if (go) tc_commit(&acc_full[sl]);
+                    if (++sl == SL) { sl = 0; slph ^= 1u; }
                 }
             }
+            tc_commit(&done_bar);   // every MMA issued
+            mbar_wait_bounded(&done_bar, 0, kDefaultWaitTries);
         }
-        if (lane == 0) tc_commit(&done_bar);   // every MMA issued
         __syncwarp();
-        mbar_wait_bounded(&done_bar, 0, kDefaultWaitTries);
     } else if (warp >= BS_OP0) {
-        // ---- operand warps: lane half h of row pair i holds right-hand side row(i, h), complex
-        // columns 2 j, 2 j + 1 of the chunk (j = lane & 15); rows 4 apart keep the 4-byte stores of
-        // the two halves on distinct banks
+        // ---- operand warps: lane half h of row pair q holds right-hand side row0 + 16 q (row0 with
+        // 4 h), complex columns 2 j, 2 j + 1 of the chunk (j = lane & 15); rows 4 apart keep the
+        // 4-byte stores of the two halves on distinct banks.  The vectors come from L2 or HBM, 1 to
+        // 3 us off: every lane copies its own 16 bytes per row into a raw slot asynchronously,
+        // BS_AHEAD chunks ahead of the one it splits (loads into registers ran at one latency per
+        // chunk whatever the number of sets: their scoreboards are shared)
         const int ow = warp - BS_OP0, h = lane >> 4, j = lane & 15;
         const size_t N = (size_t)a.N;
+        const uint32_t raw0 = smem0 + (uint32_t)(ST * Cfg::STAGE);
         int cc = 0, tt = 0, seen = -1;
         bool go = true;
         for (int i = 0; go; ++i) {
             const int t = next_tile(i);
             if (t < 0) break;
-            const Tile tl = decode(a, t, NT);
+            const Tile tl = decode(a, t);
             const int *task = a.tasks + 8 * tl.task;
-            const int type = task[1] & 15, nterms = task[1] >> 4;
-            // the previous step of this system
-            const int key = tl.phase * a.ns + tl.sys;
-            if (tl.phase > 0 && key != seen) {
-                const unsigned *cnt = a.ctl + 2 + (key - a.ns);
-                const unsigned want = (unsigned)a.ph[tl.phase - 1].done;
-                bool ok = false;
-                for (uint32_t q = 0; q < a.tries; ++q) {
-                    if (ld_acquire(cnt) >= want) { ok = true; break; }
-                    if (*(volatile int *)&s_abort || ((q & 63) == 63 && ld_acquire(a.ctl + 1))) break;
-                    __nanosleep(40);
-                }
-                if (!__all_sync(0xffffffffu, ok)) {
-                    if (lane == 0) give_up();
-                    break;
-                }
-                seen = key;
-            }
-            int rowi[Cfg::PAIRS];
-            bool val[Cfg::PAIRS];
-            size_t off[Cfg::PAIRS];
+            const int type = task[1] & 15, nterms = task[1] >> 4, np = tl.nt / 16;
+            if (!step_wait(tl, seen)) break;
+            const int row0 = 8 * (ow >> 2) + (ow & 3) + 4 * h;   // row of pair q: row0 + 16 q
+            const float2 *r0p = a.r + ((size_t)tl.sys * a.nrhs + tl.n0 + row0) * N;
+            const float2 *x0p = a.x + ((size_t)tl.sys * a.nrhs + tl.n0 + row0) * N;
+            const int nval = a.nrhs - tl.n0 - row0;
+            auto val = [&](int q) { return q < np && 16 * q < nval; };
+            // largest entry of line bl of the warp's rows (from the maxima its writer left)
+            auto line_max = [&](const float *g, int bl, int q) -> uint32_t {
+                uint32_t mx = 0;
+                for (int e = j; e < a.ng; e += 16)
+                    if (val(q))
+                        mx = max(mx, __float_as_uint(__ldcg(g + (((size_t)tl.sys * a.nx + bl) * a.ng + e) * a.nrhs + tl.n0 +
+                                                              row0 + 16 * q)));
+                return mx;
+            };
+            auto over_lanes = [&](uint32_t m) {
+                for (int o = 8; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+                return m;
+            };
+            float sc[PR];
+            auto set_scale = [&](int q, int sh, int sl) {
+                sc[q] = pow2(sh);
+                if (j == 0 && q < np) s_bscale[sl][row0 + 16 * q] = pow2(-sh);
+            };
+            // split and store one chunk's pairs into stage s
+            auto put = [&](int s, const float4 (&v)[PR]) {
+                const uint32_t br = smem0 + (uint32_t)(s * Cfg::STAGE + BS_A), bi = br + (uint32_t)(tl.nt * 128);
 #pragma unroll
-            for (int q = 0; q < Cfg::PAIRS; ++q) {
-                const int p = ow * Cfg::PAIRS + q;
-                rowi[q] = 8 * (p >> 2) + (p & 3) + 4 * h;
-                val[q] = tl.n0 + rowi[q] < a.nrhs;
-                off[q] = ((size_t)tl.sys * a.nrhs + (val[q] ? tl.n0 + rowi[q] : 0)) * N;
-            }
-            for (int u = 0; go && u < nterms; ++u, ++tt) {
-                const int bl = task[3 + 2 * u], sl = tt % SL;
-                const bool is_x = bs_kind(task[2 + 2 * u]) >= BS_P;
-                const float2 *vec = is_x ? a.x : a.r;
-                // type 4 (level 0, backward): r_j - C (x_{j-1} + x_{j+1})
-                const bool l0b = type == BS_BWD0, two = l0b && bl + 1 < a.nx;
-                const float *gm = is_x ? a.gx : a.gr;
-                auto load1 = [&](const float2 *p, int k) -> float4 {   // entries k, k + 1 of a line slice
-                    if constexpr (EVEN) return __ldcg(reinterpret_cast<const float4 *>(p + k));
-                    const float2 v0 = __ldcg(p + k), v1 = k + 1 < a.nz ? __ldcg(p + k + 1) : make_float2(0.f, 0.f);
-                    return make_float4(v0.x, v0.y, v1.x, v1.y);
-                };
-                float4 nb[Cfg::PAIRS], na[Cfg::PAIRS], nc[Cfg::PAIRS];
-                auto fetch = [&](int c) {
-                    const int k = 32 * c + 2 * j;
-#pragma unroll
-                    for (int q = 0; q < Cfg::PAIRS; ++q) {
-                        const bool in = val[q] && k < a.nz;
-                        const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
-                        nb[q] = in ? load1(vec + off[q] + (size_t)bl * a.nz, k) : z;
-                        if (l0b) {
-                            na[q] = in ? load1(a.x + off[q] + (size_t)(bl - 1) * a.nz, k) : z;
-                            nc[q] = in && two ? load1(a.x + off[q] + (size_t)(bl + 1) * a.nz, k) : z;
-                        }
-                    }
-                };
-                fetch(0);
-                // the slice's maximum (a bound of it on level 0, backward) and its scale
-                float sc[Cfg::PAIRS];
-                if (tt >= SL && !wait(&acc_empty[sl], tt / SL - 1)) { go = false; break; }
-#pragma unroll
-                for (int q = 0; q < Cfg::PAIRS; ++q) {
-                    auto line_max = [&](const float *g, int line) -> uint32_t {
-                        uint32_t mx = 0;
-                        for (int e = j; e < a.ng; e += 16)
-                            if (val[q])
-                                mx = max(mx, __float_as_uint(__ldcg(g + (((size_t)tl.sys * a.nx + line) * a.ng + e) * a.nrhs +
-                                                                      tl.n0 + rowi[q])));
-                        return mx;
-                    };
-                    uint32_t mx = line_max(gm, bl);
-                    if (l0b) {
-                        uint32_t ma = line_max(a.gx, bl - 1), mc = two ? line_max(a.gx, bl + 1) : 0u;
-                        for (int o = 8; o > 0; o >>= 1) {
-                            ma = max(ma, __shfl_xor_sync(0xffffffffu, ma, o));
-                            mc = max(mc, __shfl_xor_sync(0xffffffffu, mc, o));
-                        }
-                        for (int o = 8; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-                        mx = abs_bits(__uint_as_float(mx) +
-                                      fabsf(a.cx_in) * (__uint_as_float(ma) + __uint_as_float(mc)));
-                    } else {
-                        for (int o = 8; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-                    }
-                    const int sh = scale_shift(mx);
-                    sc[q] = pow2(sh);
-                    if (j == 0) s_bscale[sl][rowi[q]] = pow2(-sh);
-                }
-                for (int c = 0; c < a.n_chunk; ++c, ++cc) {
-                    const int s = cc % ST, k = 32 * c + 2 * j;
-                    float4 v[Cfg::PAIRS];
-#pragma unroll
-                    for (int q = 0; q < Cfg::PAIRS; ++q) {
-                        v[q] = nb[q];
-                        if (l0b) {
-                            const float c0 = (k == 0 || k == a.nz - 1) ? a.cx_edge : a.cx_in;
-                            const float c1 = k + 1 == a.nz - 1 ? a.cx_edge : a.cx_in;
-                            v[q].x -= c0 * (na[q].x + nc[q].x);
-                            v[q].y -= c0 * (na[q].y + nc[q].y);
-                            v[q].z -= c1 * (na[q].z + nc[q].z);
-                            v[q].w -= c1 * (na[q].w + nc[q].w);
-                        }
-                    }
-                    if (c + 1 < a.n_chunk) fetch(c + 1);
-                    if (cc >= ST && !wait(&empty[s], cc / ST - 1)) { go = false; break; }
-                    const uint32_t br = smem0 + (uint32_t)(s * Cfg::STAGE + BS_A), bi = br + (uint32_t)(NT * 128);
-#pragma unroll
-                    for (int q = 0; q < Cfg::PAIRS; ++q) {
+                for (int q = 0; q < PR; ++q) {
+                    if (q < np) {
                         uint32_t hi, lo;
-                        const int r = rowi[q];
+                        const int r = row0 + 16 * q;
                         const uint32_t in16 = (uint32_t)(j & 3) * 4;
                         const uint32_t oh = sw128(r, j >> 2) + in16, ol = sw128(r, 4 + (j >> 2)) + in16;
                         split_h2(v[q].x * sc[q], v[q].z * sc[q], hi, lo);
@@ -386,54 +380,181 @@ __global__ void __launch_bounds__(BS_THREADS, 1) bcr_solve_kernel(const __grid_c
                         asm volatile("st.shared.b32 [%0], %1;" ::"r"(bi + oh), "r"(hi) : "memory");
                         asm volatile("st.shared.b32 [%0], %1;" ::"r"(bi + ol), "r"(lo) : "memory");
                     }
-                    fence_proxy_async_smem();
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(&full_b[s]);
+                }
+                // (the fence that makes these stores visible to the tensor core stands in the MMA
+                // warp: here it would also wait for every load the warp has in flight)
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&full[s]);
+            };
+            // this lane's 16 bytes of row pair q in raw slot e
+            auto raw = [&](int e, int q) { return raw0 + (uint32_t)((e * tl.nt + row0 + 16 * q) * 256 + 16 * j); };
+            // copy chunk c of a line (base: its entry of this warp's first row) into raw slot e
+            auto fetch = [&](int e, const float2 *base, int c, bool on) {
+                const int k = 32 * c + 2 * j;
+#pragma unroll
+                for (int q = 0; q < PR; ++q) {
+                    if (q < np) {
+                        const bool in = on && val(q) && k < a.nz;
+                        cp_async16_zfill(raw(e, q), in ? base + (size_t)(16 * q) * N + k : a.r, in);
+                    }
+                }
+            };
+            if (type == BS_BWD0) {
+                // level 0, backward: v = r_j - C (x_{j-1} + x_{j+1}); its maximum is bounded by the parts'
+                const int bl = task[3], sl = tt % SL;
+                const bool two = bl + 1 < a.nx;
+                const size_t lo = (size_t)bl * a.nz;
+                auto fetch3 = [&](int c) {
+                    if (c < a.n_chunk) {
+                        const int e = 3 * (c % (BS_AHEAD0 + 1));
+                        fetch(e, r0p + lo, c, true);
+                        fetch(e + 1, x0p + lo - a.nz, c, true);
+                        fetch(e + 2, x0p + lo + a.nz, c, two);
+                    }
+                    cp_async_commit();
+                };
+#pragma unroll
+                for (int c = 0; c < BS_AHEAD0; ++c) fetch3(c);
+                int sh[PR];
+#pragma unroll
+                for (int q = 0; q < PR; ++q) {
+                    const uint32_t mr = over_lanes(line_max(a.gr, bl, q)), ma = over_lanes(line_max(a.gx, bl - 1, q));
+                    const uint32_t mc = two ? over_lanes(line_max(a.gx, bl + 1, q)) : 0u;
+                    sh[q] = scale_shift(abs_bits(__uint_as_float(mr) +
+                                                 fabsf(a.cx_in) * (__uint_as_float(ma) + __uint_as_float(mc))));
+                }
+                if (tt >= SL && !wait(&acc_empty[sl], tt / SL - 1)) break;
+#pragma unroll
+                for (int q = 0; q < PR; ++q) set_scale(q, sh[q], sl);
+                for (int c = 0; c < a.n_chunk; ++c, ++cc) {
+                    const int s = cc % ST, k = 32 * c + 2 * j, e = 3 * (c % (BS_AHEAD0 + 1));
+                    const float c0 = (k == 0 || k == a.nz - 1) ? a.cx_edge : a.cx_in;
+                    const float c1 = k + 1 == a.nz - 1 ? a.cx_edge : a.cx_in;
+                    fetch3(c + BS_AHEAD0);
+                    cp_async_wait<BS_AHEAD0>();
+                    float4 v[PR];
+#pragma unroll
+                    for (int q = 0; q < PR; ++q) {
+                        if (q < np) {
+                            const float4 nb = ld_shared4(raw(e, q)), na = ld_shared4(raw(e + 1, q)), nc = ld_shared4(raw(e + 2, q));
+                            v[q] = make_float4(nb.x - c0 * (na.x + nc.x), nb.y - c0 * (na.y + nc.y),
+                                               nb.z - c1 * (na.z + nc.z), nb.w - c1 * (na.w + nc.w));
+                        }
+                    }
+                    if (cc >= ST && !wait(&empty[s], cc / ST - 1)) { go = false; break; }
+                    put(s, v);
+                }
+                ++tt;
+                continue;
+            }
+            // the chunks of all terms as one sequence
+            int fu = 0, fc = 0, fe = 0;
+            const float2 *fv = r0p;
+            auto fetch_next = [&]() {
+                if (fu < nterms) {
+                    if (fc == 0) fv = (bs_kind(task[2 + 2 * fu]) >= BS_P ? x0p : r0p) + (size_t)task[3 + 2 * fu] * a.nz;
+                    fetch(fe, fv, fc, true);
+                    if (++fc == a.n_chunk) { fc = 0; ++fu; }
+                    if (++fe == BS_AHEAD + 1) fe = 0;
+                }
+                cp_async_commit();
+            };
+            for (int d = 0; d < BS_AHEAD; ++d) fetch_next();
+            int sh[PR];   // the terms' shifts, ten bits each
+#pragma unroll
+            for (int q = 0; q < PR; ++q) sh[q] = 0;
+            for (int u = 0; u < nterms; ++u) {
+                const float *gm = bs_kind(task[2 + 2 * u]) >= BS_P ? a.gx : a.gr;
+                uint32_t mx[PR];
+#pragma unroll
+                for (int q = 0; q < PR; ++q) mx[q] = line_max(gm, task[3 + 2 * u], q);
+#pragma unroll
+                for (int q = 0; q < PR; ++q) sh[q] |= (scale_shift(over_lanes(mx[q])) + 512) << (10 * u);
+            }
+            int e = 0;
+            for (int u = 0; go && u < nterms; ++u, ++tt) {
+                const int sl = tt % SL;
+                if (tt >= SL && !wait(&acc_empty[sl], tt / SL - 1)) { go = false; break; }
+#pragma unroll
+                for (int q = 0; q < PR; ++q) set_scale(q, ((sh[q] >> (10 * u)) & 1023) - 512, sl);
+                for (int c = 0; c < a.n_chunk; ++c, ++cc) {
+                    const int s = cc % ST;
+                    fetch_next();
+                    cp_async_wait<BS_AHEAD>();
+                    float4 v[PR];
+#pragma unroll
+                    for (int q = 0; q < PR; ++q)
+                        if (q < np) v[q] = ld_shared4(raw(e, q));
+                    if (cc >= ST && !wait(&empty[s], cc / ST - 1)) { go = false; break; }
+                    put(s, v);
+                    if (++e == BS_AHEAD + 1) e = 0;
                 }
             }
         }
+        cp_async_wait<0>();
     } else {
         // ---- epilogue warps: tensor-memory lanes 32 q .. + 31 = rows r0 + 32 q + lane of the line
         const int q = warp & 3;
         const size_t N = (size_t)a.N;
-        int tt = 0;
+        int tt = 0, seen = -1;
         bool go = true;
         for (int i = 0; go; ++i) {
             const int t = next_tile(i);
             if (t < 0) break;
-            const Tile tl = decode(a, t, NT);
+            const Tile tl = decode(a, t);
             const int *task = a.tasks + 8 * tl.task;
-            const int line = task[0], type = task[1] & 15, nterms = task[1] >> 4;
+            const int line = task[0], type = task[1] & 15, nterms = task[1] >> 4, nt = tl.nt;
             const int row = 32 * q + lane, m = tl.r0 + row;
             const bool on = row < tl.rows && m < a.nz, warp_on = 32 * q < tl.rows;
             const bool to_r = type <= BS_FWD;
             float2 *vec = to_r ? a.r : a.x;
             float *gm = to_r ? a.gr : a.gx;
             float f[3] = {0.f, 0.f, 0.f};   // row scale and sign of each term
-            if (on)
-                for (int u = 0; u < nterms; ++u) {
+#pragma unroll
+            for (int u = 0; u < 3; ++u)
+                if (on && u < nterms) {
                     f[u] = __ldg(a.scl + (size_t)bs_matrix(a, task[2 + 2 * u], tl.sys) * a.nz + m);
                     if (type == BS_FWD0) f[u] *= -((m == 0 || m == a.nz - 1) ? a.cx_edge : a.cx_in);
                     if (type == BS_FWD || (type == BS_BWD && u > 0)) f[u] = -f[u];
                 }
+            float2 *out = vec + ((size_t)tl.sys * a.nrhs + tl.n0) * N + (size_t)line * a.nz + m;
+            float *gout = gm + (((size_t)tl.sys * a.nx + line) * a.ng + (tl.r0 >> 5) + q) * a.nrhs + tl.n0;
+            const int ncol = min(nt, a.nrhs - tl.n0);
+            // the old line, ahead of the products that are added to it
+            float2 old[16];
+            auto fetch_old = [&](int c0) {
+#pragma unroll
+                for (int e = 0; e < 16; ++e)
+                    old[e] = on && to_r && c0 + e < ncol ? __ldcg(out + (size_t)(c0 + e) * N) : make_float2(0.f, 0.f);
+            };
+            if (to_r && !step_wait(tl, seen)) break;
+            if (warp_on) fetch_old(0);
             for (int u = 0; u < nterms && go; ++u) go = wait(&acc_full[(tt + u) % SL], (tt + u) / SL);
             if (!go) break;
             tc_fence_after();
-            float2 *out = vec + ((size_t)tl.sys * a.nrhs + tl.n0) * N + (size_t)line * a.nz + m;
-            float *gout = gm + (((size_t)tl.sys * a.nx + line) * a.ng + (tl.r0 >> 5) + q) * a.nrhs + tl.n0;
-            const int ncol = min(NT, a.nrhs - tl.n0);
             if (warp_on) {
                 for (int c0 = 0; c0 < ncol; c0 += 16) {
                     float2 o[16];
 #pragma unroll
-                    for (int e = 0; e < 16; ++e)
-                        o[e] = on && to_r && c0 + e < ncol ? __ldcg(out + (size_t)(c0 + e) * N) : make_float2(0.f, 0.f);
-                    for (int u = 0; u < nterms; ++u) {
+                    for (int e = 0; e < 16; ++e) o[e] = old[e];
+                    if (c0 + 16 < ncol) fetch_old(c0 + 16);
+#pragma unroll
+                    for (int u = 0; u < 3; ++u) {
+                        if (u >= nterms) break;
                         const int sl = (tt + u) % SL;
-                        const uint32_t d = tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(sl * 2 * NT + c0);
+                        const uint32_t d = tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(sl * BS_SLOT_COLS + c0);
                         float re[16], im[16];
                         tc_ld16(d, re);
-                        tc_ld16(d + NT, im);
+                        tc_ld16(d + nt, im);
+                        if (nt <= 32) {   // Re = Ar Br - Ai Bi, Im = Ar Bi + Ai Br
+                            float t2[16];
+                            tc_ld16(d + 3 * nt, t2);
+#pragma unroll
+                            for (int e = 0; e < 16; ++e) re[e] -= t2[e];
+                            tc_ld16(d + 2 * nt, t2);
+#pragma unroll
+                            for (int e = 0; e < 16; ++e) im[e] += t2[e];
+                        }
 #pragma unroll
                         for (int e = 0; e < 16; ++e) {
                             const float sb = s_bscale[sl][c0 + e];
@@ -575,11 +696,11 @@ __global__ void __launch_bounds__(256) bcr_image_kernel(int n, int n_chunk, int 
     }
 }
 
-template <int NT, bool EVEN> cudaError_t launch_nt(const BsArgs &a, int grid, double flops, cudaStream_t st) {
-    const void *fn = (const void *)bcr_solve_kernel<NT, EVEN>;
+template <int NT> cudaError_t launch_nt(const BsArgs &a, int grid, double flops, cudaStream_t st) {
+    const void *fn = (const void *)bcr_solve_kernel<NT>;
     cudaError_t e = ensure_dyn_smem(fn, BsCfg<NT>::SMEM);
     if (e != cudaSuccess) return e;
-    HELM_TRACED_W(K_BCR_SOLVE, st, flops, (bcr_solve_kernel<NT, EVEN><<<grid, BS_THREADS, BsCfg<NT>::SMEM, st>>>(a)));
+    HELM_TRACED_W(K_BCR_SOLVE, st, flops, (bcr_solve_kernel<NT><<<grid, BS_THREADS, BsCfg<NT>::SMEM, st>>>(a)));
     return cudaGetLastError();
 }
 
@@ -599,7 +720,7 @@ cudaError_t launch_bcr_image(int n, const float2 *src, long long stride, bool tr
 }
 
 cudaError_t launch_bcr_solve(BsArgs a, const BsStep *steps, int n_steps, double flops, cudaStream_t st) {
-    if (n_steps > BS_MAX_PHASE) return cudaErrorInvalidValue;
+    if (n_steps > BS_MAX_PHASE || (a.nz & 1)) return cudaErrorInvalidValue;
     const BsLayout l = bs_layout(a.nz);
     a.nzr = l.nzr;
     a.n_chunk = l.n_chunk;
@@ -607,7 +728,6 @@ cudaError_t launch_bcr_solve(BsArgs a, const BsStep *steps, int n_steps, double 
     a.ng = l.ng;
     a.N = a.nx * a.nz;
     const int nt = a.nrhs <= 16 ? 16 : (a.nrhs <= 32 ? 32 : 64);
-    a.n_tiles = (a.nrhs + nt - 1) / nt;
     const int sms = device_sms();
     a.n_phase = n_steps;
     int tile = 0;
@@ -616,13 +736,19 @@ cudaError_t launch_bcr_solve(BsArgs a, const BsStep *steps, int n_steps, double 
         ph.tile0 = tile;
         ph.task0 = steps[p].task0;
         ph.tasks = steps[p].tasks;
-        // steps with few lines take lower tiles, so that more SMs share the blocks' stream
+        // steps with few lines take narrower and then lower tiles, so that more SMs share their
+        // products and the blocks' stream
         ph.mrows = 128;
-        auto tiles_of = [&](int rows) { return ph.tasks * a.ns * a.n_tiles * ((a.nz + rows - 1) / rows); };
-        while (ph.mrows > 32 && tiles_of(ph.mrows) < sms) ph.mrows /= 2;
-        ph.mt = (a.nz + ph.mrows - 1) / ph.mrows;
-        ph.done = 4 * ph.tasks * a.n_tiles * ph.mt;   // four epilogue warps count each tile
-        tile += tiles_of(ph.mrows);
+        ph.nt = steps[p].type == BS_BWD0 ? std::min(nt, BS_NT_BWD0) : nt;
+        auto tiles_of = [&]() {
+            ph.n_tiles = (a.nrhs + ph.nt - 1) / ph.nt;
+            ph.mt = (a.nz + ph.mrows - 1) / ph.mrows;
+            return ph.tasks * a.ns * ph.n_tiles * ph.mt;
+        };
+        while (ph.nt > 16 && tiles_of() < sms) ph.nt /= 2;
+        while (ph.mrows > 32 && tiles_of() < sms) ph.mrows /= 2;
+        tile += tiles_of();
+        ph.done = 4 * ph.tasks * ph.n_tiles * ph.mt;   // four epilogue warps count each tile
     }
     a.n_tile_total = tile;
     cudaError_t e = cudaMemsetAsync(a.ctl, 0, sizeof(unsigned) * bs_ctl_words(n_steps, a.ns), st);
@@ -633,10 +759,8 @@ cudaError_t launch_bcr_solve(BsArgs a, const BsStep *steps, int n_steps, double 
                                    a.nx, a.nz, a.ng, a.nrhs, n_cb, items, a.r, a.gr, a.skip, a.frozen)));
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     const int grid = std::min(sms, tile);
-    const bool even = (a.nz & 1) == 0;
-    if (nt == 16) return even ? launch_nt<16, true>(a, grid, flops, st) : launch_nt<16, false>(a, grid, flops, st);
-    if (nt == 32) return even ? launch_nt<32, true>(a, grid, flops, st) : launch_nt<32, false>(a, grid, flops, st);
-    return even ? launch_nt<64, true>(a, grid, flops, st) : launch_nt<64, false>(a, grid, flops, st);
+    if (nt == 16) return launch_nt<16>(a, grid, flops, st);
+    return nt == 32 ? launch_nt<32>(a, grid, flops, st) : launch_nt<64>(a, grid, flops, st);
 }
 
 }  // namespace helm

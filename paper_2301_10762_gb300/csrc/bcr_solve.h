@@ -28,10 +28,10 @@ enum { BS_FWD0 = 0, BS_FWD = 1, BS_LAST = 2, BS_BWD = 3, BS_BWD0 = 4 };
 constexpr int BS_MAX_PHASE = 64;
 
 struct BsStep {   // one dependent step of the solve: its tasks (the same for every system)
-    int task0, tasks;
+    int task0, tasks, type;
 };
 struct BsPhase {
-    int tile0, task0, tasks, mt, mrows, done;
+    int tile0, task0, tasks, nt, n_tiles, mt, mrows, done;   // nt x mrows: the step's tiles
 };
 struct BsArgs {
     int nx, nz, ns, nrhs, half;
@@ -46,7 +46,7 @@ struct BsArgs {
     const int *skip, *frozen;
     uint32_t tries;
     // set by launch_bcr_solve
-    int N, n_chunk, nzr, ng, n_tiles, n_phase, n_tile_total;
+    int N, n_chunk, nzr, ng, n_phase, n_tile_total;
     size_t mat_bytes;
     BsPhase ph[BS_MAX_PHASE];
 };

@@ -163,6 +163,31 @@ __device__ __forceinline__ bool mbar_wait_or_abort(uint64_t *bar, uint32_t parit
     }
     return false;
 }
+// The same for barriers that only this CTA arrives on (and its own bulk copies and tensor-core
+// commits complete): CTA scope, a non-suspending test first
+__device__ __forceinline__ bool mbar_test_cta(uint64_t *bar, uint32_t parity) {
+    uint32_t ok;
+    asm volatile(
+        "{\n .reg .pred p;\n mbarrier.test_wait.parity.acquire.cta.shared::cta.b64 p, [%1], %2;\n"
+        " selp.u32 %0, 1, 0, p;\n}\n"
+        : "=r"(ok)
+        : "r"(smem_u32(bar)), "r"(parity)
+        : "memory");
+    return ok != 0;
+}
+__device__ __forceinline__ bool mbar_wait_cta(uint64_t *bar, uint32_t parity, uint32_t max_tries, const int *abort_word) {
+    for (uint32_t t = 0; t < max_tries; ++t) {
+        if (mbar_test_cta(bar, parity) || mbar_try_wait(bar, parity)) return true;
+        if (*(const volatile int *)abort_word) return false;
+    }
+    return false;
+}
+// one lane of a converged warp, in the form that lets the compiler keep its operands uniform
+__device__ __forceinline__ bool elect_one() {
+    uint32_t p;
+    asm volatile("{\n .reg .pred q;\n elect.sync _|q, 0xffffffff;\n selp.u32 %0, 1, 0, q;\n}\n" : "=r"(p));
+    return p != 0;
+}
 // Abort protocol of the cluster kernels.  A CTA whose bounded wait gives up sets the abort word
 // (a __shared__ int at the same offset in every CTA) in every CTA of its cluster, so that the
 // others stop waiting and stop producing.  No CTA leaves before the final cluster barrier,
