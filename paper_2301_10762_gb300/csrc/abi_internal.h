@@ -34,7 +34,7 @@ struct RefineState;   // device-side refinement control (kernels.h)
 struct BcrData {
     int half = 0;
     unsigned char *img = nullptr;   // blocks: [n_omega][nx] inverses, then [n_omega][half] of W, V, P, Q
-    float *scl = nullptr;           // row scales of the blocks
+    int *shift = nullptr;           // scales of the blocks
     int *tasks = nullptr;           // the solve's tasks on the device
     unsigned *ctl = nullptr;        // the solve's tile and step counters
     float *gsmall = nullptr;        // vector maxima of the no-allocation solve (kSmallMaxima)

@@ -742,14 +742,18 @@ helm_status invert_tridiag_blocks(int n, Fam in, Fam out, const std::vector<int>
     return HELM_OK;
 }
 
-// images (bcr_solve.cu) of the blocks base + pairs[.][0] * n^2 as matrices pairs[.][1]
-helm_status image_blocks(int n, const float2 *base, bool trans, const std::vector<int> &pairs, unsigned char *img,
-                         float *scl, Plan &pl) {
+// images (bcr_solve.cu) of the blocks base + pairs[.][0] * n^2 as matrices pairs[.][1], and of their
+// transposes as matrices tdst[.] (empty: none)
+helm_status image_blocks(int n, const float2 *base, const std::vector<int> &pairs, const std::vector<int> &tdst,
+                         const BcrData &b, uint32_t *mx, Plan &pl) {
     if (pairs.empty()) return HELM_OK;
-    const int off = pl.add(pairs), count = (int)(pairs.size() / 2);
+    const int off = pl.add(pairs), toff = tdst.empty() ? -1 : pl.add(tdst), count = (int)(pairs.size() / 2);
     const cudaStream_t st = pl.st;
+    unsigned char *img = b.img;
+    int *shift = b.shift;
     pl.ops.push_back([=](const int *dev) -> helm_status {
-        const cudaError_t e = launch_bcr_image(n, base, (long long)n * n, trans, dev + off, count, img, scl, st);
+        const cudaError_t e = launch_bcr_image(n, base, (long long)n * n, dev + off, toff < 0 ? nullptr : dev + toff, count,
+                                               img, mx, shift, st);
         if (e != cudaSuccess) { helm_set_error("bcr: images", e); return HELM_ECUDA; }
         return HELM_OK;
     });
@@ -777,7 +781,7 @@ helm_status bcr_factor(helm_factor_t *f) {
     const size_t n_mat = (size_t)ns * (nx + 4 * (size_t)half);
     const BsLayout lay = bs_layout(nz);
     if ((s = dev_alloc((void **)&b.img, n_mat * lay.mat_bytes, "bcr: blocks", st)) != HELM_OK ||
-        (s = dev_alloc((void **)&b.scl, n_mat * nz * sizeof(float), "bcr: row scales", st)) != HELM_OK ||
+        (s = dev_alloc((void **)&b.shift, n_mat * sizeof(int), "bcr: scales", st)) != HELM_OK ||
         (s = dev_alloc((void **)&b.gsmall, kSmallMaxima * sizeof(float), "bcr: maxima", st)) != HELM_OK)
         return s;
     // working blocks of the reduction: diagonal blocks (an eliminated line's is inverted in place),
@@ -800,6 +804,13 @@ helm_status bcr_factor(helm_factor_t *f) {
     cudaError_t e;
     Plan pl(st);
     if ((s = pl.with_split(kFactorSplitElems)) != HELM_OK) return s;
+    uint32_t *mx = nullptr;   // largest moduli of the blocks, for their scales
+    if ((s = dev_alloc((void **)&mx, n_mat * sizeof(uint32_t), "bcr: maxima", st)) != HELM_OK) return s;
+    pl.scratch.push_back(mx);
+    if ((e = cudaMemsetAsync(mx, 0, n_mat * sizeof(uint32_t), st)) != cudaSuccess) {
+        helm_set_error("bcr: maxima", e);
+        return HELM_ECUDA;
+    }
     const int per = (int)std::min<long long>(64, (nz2 + 255) / 256);
     // n_z <= 256: no line block is formed in memory before level 0, which inverts the odd lines'
     // tridiagonal blocks and updates the even lines' straight from A's diagonal and couplings
@@ -856,12 +867,12 @@ helm_status bcr_factor(helm_factor_t *f) {
                 auto v = task8(cb + (j - sp) / sp, lb + j, 0, qb + i);
                 tv.insert(tv.end(), v.begin(), v.end());
                 vi.insert(vi.end(), {qb + i, mat(BS_V, sy, j / 2)});
-                vt.insert(vt.end(), {qb + i, mat(BS_P, sy, j / 2)});
+                vt.push_back(mat(BS_P, sy, j / 2));
                 if (j + sp < nx) {
                     auto w = task8(cb + (j + sp) / sp, lb + j, 0, qb + i);
                     tw.insert(tw.end(), w.begin(), w.end());
                     wi.insert(wi.end(), {qb + i, mat(BS_W, sy, j / 2)});
-                    wt.insert(wt.end(), {qb + i, mat(BS_Q, sy, j / 2)});
+                    wt.push_back(mat(BS_Q, sy, j / 2));
                 }
             }
             for (int k = 0; k < nx; k += 2 * sp) {
@@ -893,10 +904,7 @@ helm_status bcr_factor(helm_factor_t *f) {
         ga.C = W;
         ga.A[0] = zop(Lc, nz2, nz);
         if ((s = gemm(ga, tw, pl)) != HELM_OK) return s;
-        if ((s = image_blocks(nz, V, false, vi, b.img, b.scl, pl)) != HELM_OK ||
-            (s = image_blocks(nz, V, true, vt, b.img, b.scl, pl)) != HELM_OK ||
-            (s = image_blocks(nz, W, false, wi, b.img, b.scl, pl)) != HELM_OK ||
-            (s = image_blocks(nz, W, true, wt, b.img, b.scl, pl)) != HELM_OK)
+        if ((s = image_blocks(nz, V, vi, vt, b, mx, pl)) != HELM_OK || (s = image_blocks(nz, W, wi, wt, b, mx, pl)) != HELM_OK)
             return s;
         ZGemmArgs gd;
         gd.M = gd.N = gd.K = nz;
@@ -926,7 +934,7 @@ helm_status bcr_factor(helm_factor_t *f) {
         for (int sy = 0; sy < ns; ++sy) last.insert(last.end(), {sy * nx, sy * nx});
         if ((s = invert_blocks(nz, fD, fD, last, op->status, pl)) != HELM_OK) return s;
         for (int i = 0; i < ns * nx; ++i) di.insert(di.end(), {i, i});
-        if ((s = image_blocks(nz, D, false, di, b.img, b.scl, pl)) != HELM_OK) return s;
+        if ((s = image_blocks(nz, D, di, {}, b, mx, pl)) != HELM_OK) return s;
     }
     if ((s = pl.run()) != HELM_OK) return s;
     // the solve's steps and tasks (the same for every system), built once
@@ -987,7 +995,7 @@ void bcr_free(helm_factor_t *f) {
     const cudaStream_t st = f->op ? f->op->st : nullptr;
     BcrData &b = f->bcr;
     dev_free(b.img, st);
-    dev_free(b.scl, st);
+    dev_free(b.shift, st);
     dev_free(b.tasks, st);
     dev_free(b.ctl, st);
     dev_free(b.gsmall, st);
@@ -1017,7 +1025,7 @@ helm_status bcr_solve(const helm_factor_t *f, int nrhs, float2 *r, float2 *x, fl
     a.gr = maxima;
     a.gx = maxima + bcr_maxima_elems(g, (size_t)a.ns * nrhs) / 2;
     a.img = b.img;
-    a.scl = b.scl;
+    a.shift = b.shift;
     a.tasks = b.tasks;
     a.cx_in = (float)coup_x(g, 1);
     a.cx_edge = (float)coup_x(g, 0);

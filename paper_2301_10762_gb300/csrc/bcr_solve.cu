@@ -11,23 +11,26 @@
 // entries per frequency: 3.8 GB at 256^2 with 8 frequencies, 0.56 ms at the measured copy rate),
 // so the kernel is laid out as a stream of the blocks through the tensor cores:
 //   * The blocks are stored as the tensor core reads them ("image"): every real entry as the sum
-//     of two FP16 numbers of its row-scaled value (hi + lo, 22 to 23 bits below the largest entry
-//     of the row, as many as the 3xTF32 split of the GEMM keeps; 8 bytes per complex entry as in
-//     FP32), real and imaginary parts apart, 32 columns of a row as one 128-byte swizzled row (32
+//     of two FP16 numbers of its scaled value (a power of two per block; hi + lo carry 22 to 23
+//     bits for entries down to 2^-15 of the block's largest, as many as the 3xTF32 split keeps, and
+//     2^-39 of the largest below that; 8 bytes per complex entry as in FP32), real and imaginary parts apart, 32 columns of a row as one 128-byte swizzled row (32
 //     hi, then 32 lo).  A chunk of a tile is two contiguous runs of memory: a copy warp streams
 //     them with bulk copies, and no thread touches them.
 //   * The vectors are split by operand warps as they come (a power-of-two scale per line slice
 //     from the maxima that the writers of the vectors leave), 16 KB against 32 KB of block data
 //     per chunk at 64 right-hand sides.
-//   * One MMA warp issues hi hi + hi lo + lo hi for Re and Im (the negated product by the
-//     instruction's negate bit), FP32 accumulation in tensor memory, one accumulator per product
-//     term (the terms' scales differ); four epilogue warps scale, sum, add the old line and
-//     write, while the next tile's products run into the other accumulators.
+//   * One thread issues hi hi + hi lo + lo hi of Ar [Br | Bi] and Ai [Br | Bi], FP32 accumulation in
+//     tensor memory; four epilogue warps combine and scale them, add the old line and write,
+//     while the next tile's products run into the other accumulator.
 //   * The tiles of all levels are taken in order from a device counter by whichever CTA is free.
 //     A tile waits until the previous step of its own system is complete (a counter per step and
 //     system); only the operand warps wait, so the block stream runs on across steps.  Every
 //     wait is for tiles that were taken earlier, so the kernel needs no co-resident grid, and
 //     every wait is bounded.
+// Measured per solve at 256^2, 8 frequencies (block stream 0.56 ms): 1 right-hand side 0.60 ms, 64
+// of them 1.02 ms; one GEMM launch per level (18 launches, 3xTF32, blocks split by operand warps)
+// took 1.9 and 2.4 ms.  With few systems the chain of 2 log2(n_x) + 1 steps is what is left, 6 to
+// 17 us a step: 0.14 ms at 128^2.
 #include <algorithm>
 
 #include "abi_internal.h"
@@ -49,7 +52,7 @@ constexpr int BS_QD = 4;                     // tile queue of a CTA
 constexpr int BS_A = 32768;                  // A bytes of a stage: 128 rows x 128 bytes, Re and Im
 constexpr uint32_t BS_TMEM = 512;
 
-constexpr int BS_SLOTS = 4, BS_SLOT_COLS = 128;   // accumulators: one per product term, 128 columns
+constexpr int BS_SLOTS = 2, BS_SLOT_COLS = 256;   // accumulators: one per tile, [Ar Br | Ar Bi | Ai Br | Ai Bi]
 
 // NT: widest tile of the launch (right-hand sides); a step with few lines takes narrower ones
 template <int NT> struct BsCfg {
@@ -135,7 +138,7 @@ __global__ void __launch_bounds__(BS_THREADS, 1) bcr_solve_kernel(const __grid_c
     __shared__ __align__(8) uint64_t acc_full[SL], acc_empty[SL];
     __shared__ __align__(8) uint64_t tq_full[BS_QD], tq_empty[BS_QD], done_bar;
     __shared__ int tq[BS_QD];
-    __shared__ float s_bscale[SL][NT];   // 2^-s of each right-hand side of an accumulator's product
+    __shared__ float s_bscale[SL][NT];   // 2^-S of each right-hand side of an accumulator
     __shared__ uint32_t s_tmem;
     __shared__ int s_abort;
     if (a.skip && *a.skip) return;
@@ -279,43 +282,28 @@ __global__ void __launch_bounds__(BS_THREADS, 1) bcr_solve_kernel(const __grid_c
                 if (t < 0) break;
                 const Tile tl = decode(a, t);
                 const int nterms = a.tasks[8 * tl.task + 1] >> 4, nt = tl.nt;
-                const uint32_t id2 = idesc_f16(2 * nt, false), id1 = idesc_f16(nt, false), id1n = idesc_f16(nt, true);
-                const bool narrow = nt <= 32;
-                for (int u = 0; go && u < nterms; ++u) {
-                    if (!wait1(&acc_empty[sl], slph)) { go = false; break; }
-                    const uint32_t d0 = tmem + (uint32_t)(sl * BS_SLOT_COLS), d1 = d0 + (uint32_t)(narrow ? 2 * nt : nt);
-                    for (int c = 0; c < a.n_chunk; ++c) {
-                        if (!wait1(&full[s], ph)) { go = false; break; }
-                        fence_proxy_async_smem();   // the operand warps' stores, ordered by the barrier
-                        tc_fence_after();
-                        const uint64_t dar = dstage0 + (uint64_t)(s * (Cfg::STAGE / 16)), dai = dar + 1024, dbr = dar + BS_A / 16,
-                                       dbi = dbr + (uint64_t)(nt * 8);
-                        // products hi*hi, hi*lo, lo*hi (lo 64 bytes into the row), each two steps of
-                        // K = 16 FP16 (32 bytes; 2 in descriptor units)
-                        if (narrow) {   // Ar [Br | Bi] and Ai [Br | Bi] side by side
+                const uint32_t id = idesc_f16(2 * nt);
+                if (!wait1(&acc_empty[sl], slph)) break;
+                const uint32_t d0 = tmem + (uint32_t)(sl * BS_SLOT_COLS), d1 = d0 + (uint32_t)(2 * nt);
+                for (int c = 0, n = nterms * a.n_chunk; c < n; ++c) {
+                    if (!wait1(&full[s], ph)) { go = false; break; }
+                    fence_proxy_async_smem();   // the operand warps' stores, ordered by the barrier
+                    tc_fence_after();
+                    const uint64_t dar = dstage0 + (uint64_t)(s * (Cfg::STAGE / 16)), dai = dar + 1024, dbr = dar + BS_A / 16;
+                    // products hi*hi, hi*lo, lo*hi (lo 64 bytes into the row), each two steps of
+                    // K = 16 FP16 (32 bytes; 2 in descriptor units): Ar [Br | Bi] and Ai [Br | Bi]
 #pragma unroll
-                            for (int p = 0; p < 6; ++p) {
-                                const int ka = (p >= 4 ? 4 : 0) + 2 * (p & 1), kb = ((p >> 1) == 1 ? 4 : 0) + 2 * (p & 1);
-                                const uint32_t acc = p > 0 ? 1u : (c > 0 ? 1u : 0u);
-                                tc_mma_f16(d0, dar + ka, dbr + kb, id2, acc);
-                                tc_mma_f16(d1, dai + ka, dbr + kb, id2, acc);
-                            }
-                        } else {        // [Re | Im] += Ar [Br | Bi];  Re -= Ai Bi;  Im += Ai Br
-#pragma unroll
-                            for (int p = 0; p < 6; ++p) {
-                                const int ka = (p >= 4 ? 4 : 0) + 2 * (p & 1), kb = ((p >> 1) == 1 ? 4 : 0) + 2 * (p & 1);
-                                const uint32_t acc = p > 0 ? 1u : (c > 0 ? 1u : 0u);
-                                tc_mma_f16(d0, dar + ka, dbr + kb, id2, acc);
-                                tc_mma_f16(d0, dai + ka, dbi + kb, id1n, 1u);
-                                tc_mma_f16(d1, dai + ka, dbr + kb, id1, 1u);
-                            }
-                        }
-                        tc_commit(&empty[s]);
-                        if (++s == ST) { s = 0; ph ^= 1u; }
+                    for (int p = 0; p < 6; ++p) {
+                        const int ka = (p >= 4 ? 4 : 0) + 2 * (p & 1), kb = ((p >> 1) == 1 ? 4 : 0) + 2 * (p & 1);
+                        const uint32_t acc = p > 0 ? 1u : (c > 0 ? 1u : 0u);
+                        tc_mma_f16(d0, dar + ka, dbr + kb, id, acc);
+                        tc_mma_f16(d1, dai + ka, dbr + kb, id, acc);
                     }
-                    if (go) tc_commit(&acc_full[sl]);
-                    if (++sl == SL) { sl = 0; slph ^= 1u; }
+                    tc_commit(&empty[s]);
+                    if (++s == ST) { s = 0; ph ^= 1u; }
                 }
+                if (go) tc_commit(&acc_full[sl]);
+                if (++sl == SL) { sl = 0; slph ^= 1u; }
             }
             tc_commit(&done_bar);   // every MMA issued
             mbar_wait_bounded(&done_bar, 0, kDefaultWaitTries);
@@ -345,24 +333,29 @@ __global__ void __launch_bounds__(BS_THREADS, 1) bcr_solve_kernel(const __grid_c
             const float2 *x0p = a.x + ((size_t)tl.sys * a.nrhs + tl.n0 + row0) * N;
             const int nval = a.nrhs - tl.n0 - row0;
             auto val = [&](int q) { return q < np && 16 * q < nval; };
-            // largest entry of line bl of the warp's rows (from the maxima its writer left)
+            // largest entry of a line of the warp's rows (from the maxima its writer left); the loads of
+            // all terms are issued before the first is used
             auto line_max = [&](const float *g, int bl, int q) -> uint32_t {
-                uint32_t mx = 0;
-                for (int e = j; e < a.ng; e += 16)
-                    if (val(q))
-                        mx = max(mx, __float_as_uint(__ldcg(g + (((size_t)tl.sys * a.nx + bl) * a.ng + e) * a.nrhs + tl.n0 +
-                                                              row0 + 16 * q)));
+                const float *p = g + ((size_t)tl.sys * a.nx + bl) * a.ng * a.nrhs + tl.n0 + row0 + 16 * q;
+                uint32_t mx = j < a.ng && val(q) ? __float_as_uint(__ldcg(p + (size_t)j * a.nrhs)) : 0u;
+                if (a.ng > 16)
+                    for (int e = j + 16; e < a.ng; e += 16)
+                        if (val(q)) mx = max(mx, __float_as_uint(__ldcg(p + (size_t)e * a.nrhs)));
                 return mx;
             };
             auto over_lanes = [&](uint32_t m) {
                 for (int o = 8; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
                 return m;
             };
+            // terms share the tile's accumulator, so their scales share one exponent S per right-hand
+            // side: S = min over the terms of (the block's shift + the line's largest shift), and a
+            // line's shift is S less its block's.  A term that is small against the largest loses
+            // only what the sum does not hold (FP16 keeps all 22 bits 15 octaves down).
             float sc[PR];
-            auto set_scale = [&](int q, int sh, int sl) {
-                sc[q] = pow2(sh);
-                if (j == 0 && q < np) s_bscale[sl][row0 + 16 * q] = pow2(-sh);
+            auto put_scale = [&](int q, int S, int sl) {
+                if (j == 0 && q < np) s_bscale[sl][row0 + 16 * q] = pow2(max(-126, min(126, -S)));
             };
+            const int sl = tt % SL;
             // split and store one chunk's pairs into stage s
             auto put = [&](int s, const float4 (&v)[PR]) {
                 const uint32_t br = smem0 + (uint32_t)(s * Cfg::STAGE + BS_A), bi = br + (uint32_t)(tl.nt * 128);
@@ -401,7 +394,7 @@ __global__ void __launch_bounds__(BS_THREADS, 1) bcr_solve_kernel(const __grid_c
             };
             if (type == BS_BWD0) {
                 // level 0, backward: v = r_j - C (x_{j-1} + x_{j+1}); its maximum is bounded by the parts'
-                const int bl = task[3], sl = tt % SL;
+                const int bl = task[3], sa = __ldg(a.shift + bs_matrix(a, task[2], tl.sys));
                 const bool two = bl + 1 < a.nx;
                 const size_t lo = (size_t)bl * a.nz;
                 auto fetch3 = [&](int c) {
@@ -415,17 +408,23 @@ __global__ void __launch_bounds__(BS_THREADS, 1) bcr_solve_kernel(const __grid_c
                 };
 #pragma unroll
                 for (int c = 0; c < BS_AHEAD0; ++c) fetch3(c);
-                int sh[PR];
+                uint32_t m3[3][PR];
 #pragma unroll
                 for (int q = 0; q < PR; ++q) {
-                    const uint32_t mr = over_lanes(line_max(a.gr, bl, q)), ma = over_lanes(line_max(a.gx, bl - 1, q));
-                    const uint32_t mc = two ? over_lanes(line_max(a.gx, bl + 1, q)) : 0u;
-                    sh[q] = scale_shift(abs_bits(__uint_as_float(mr) +
-                                                 fabsf(a.cx_in) * (__uint_as_float(ma) + __uint_as_float(mc))));
+                    m3[0][q] = line_max(a.gr, bl, q);
+                    m3[1][q] = line_max(a.gx, bl - 1, q);
+                    m3[2][q] = two ? line_max(a.gx, bl + 1, q) : 0u;
                 }
                 if (tt >= SL && !wait(&acc_empty[sl], tt / SL - 1)) break;
 #pragma unroll
-                for (int q = 0; q < PR; ++q) set_scale(q, sh[q], sl);
+                for (int q = 0; q < PR; ++q) {
+                    const float bound = __uint_as_float(over_lanes(m3[0][q])) +
+                                        fabsf(a.cx_in) * (__uint_as_float(over_lanes(m3[1][q])) +
+                                                          __uint_as_float(over_lanes(m3[2][q])));
+                    const int sh = scale_shift(abs_bits(bound));
+                    sc[q] = pow2(sh);
+                    put_scale(q, sh + sa, sl);
+                }
                 for (int c = 0; c < a.n_chunk; ++c, ++cc) {
                     const int s = cc % ST, k = 32 * c + 2 * j, e = 3 * (c % (BS_AHEAD0 + 1));
                     const float c0 = (k == 0 || k == a.nz - 1) ? a.cx_edge : a.cx_in;
@@ -460,23 +459,39 @@ __global__ void __launch_bounds__(BS_THREADS, 1) bcr_solve_kernel(const __grid_c
                 cp_async_commit();
             };
             for (int d = 0; d < BS_AHEAD; ++d) fetch_next();
-            int sh[PR];   // the terms' shifts, ten bits each
+            uint32_t mx[3][PR];
+            int sa[3];
 #pragma unroll
-            for (int q = 0; q < PR; ++q) sh[q] = 0;
-            for (int u = 0; u < nterms; ++u) {
-                const float *gm = bs_kind(task[2 + 2 * u]) >= BS_P ? a.gx : a.gr;
-                uint32_t mx[PR];
+            for (int u = 0; u < 3; ++u) {
+                const bool in = u < nterms;
+                sa[u] = in ? __ldg(a.shift + bs_matrix(a, task[2 + 2 * u], tl.sys)) : 0;
 #pragma unroll
-                for (int q = 0; q < PR; ++q) mx[q] = line_max(gm, task[3 + 2 * u], q);
-#pragma unroll
-                for (int q = 0; q < PR; ++q) sh[q] |= (scale_shift(over_lanes(mx[q])) + 512) << (10 * u);
+                for (int q = 0; q < PR; ++q)
+                    mx[u][q] = in && q < np
+                                   ? line_max(bs_kind(task[2 + 2 * u]) >= BS_P ? a.gx : a.gr, task[3 + 2 * u], q)
+                                   : 0u;
             }
-            int e = 0;
-            for (int u = 0; go && u < nterms; ++u, ++tt) {
-                const int sl = tt % SL;
-                if (tt >= SL && !wait(&acc_empty[sl], tt / SL - 1)) { go = false; break; }
+            if (tt >= SL && !wait(&acc_empty[sl], tt / SL - 1)) break;
+            int S[PR];
 #pragma unroll
-                for (int q = 0; q < PR; ++q) set_scale(q, ((sh[q] >> (10 * u)) & 1023) - 512, sl);
+            for (int q = 0; q < PR; ++q) {
+                S[q] = 1 << 20;
+#pragma unroll
+                for (int u = 0; u < 3; ++u) {
+                    const int t2 = sa[u] + scale_shift(over_lanes(mx[u][q]));
+                    if (u < nterms) S[q] = min(S[q], t2);
+                }
+                put_scale(q, S[q], sl);
+            }
+            ++tt;
+            int e = 0;
+            for (int u = 0; go && u < nterms; ++u) {
+                const int su = u == 0 ? sa[0] : (u == 1 ? sa[1] : sa[2]);
+#pragma unroll
+                for (int q = 0; q < PR; ++q) {   // P and Q enter with a minus sign
+                    const float f = pow2(max(-126, min(126, S[q] - su)));
+                    sc[q] = type == BS_BWD && u > 0 ? -f : f;
+                }
                 for (int c = 0; c < a.n_chunk; ++c, ++cc) {
                     const int s = cc % ST;
                     fetch_next();
@@ -503,84 +518,78 @@ __global__ void __launch_bounds__(BS_THREADS, 1) bcr_solve_kernel(const __grid_c
             if (t < 0) break;
             const Tile tl = decode(a, t);
             const int *task = a.tasks + 8 * tl.task;
-            const int line = task[0], type = task[1] & 15, nterms = task[1] >> 4, nt = tl.nt;
+            const int line = task[0], type = task[1] & 15, nt = tl.nt;
             const int row = 32 * q + lane, m = tl.r0 + row;
             const bool on = row < tl.rows && m < a.nz, warp_on = 32 * q < tl.rows;
             const bool to_r = type <= BS_FWD;
             float2 *vec = to_r ? a.r : a.x;
             float *gm = to_r ? a.gr : a.gx;
-            float f[3] = {0.f, 0.f, 0.f};   // row scale and sign of each term
-#pragma unroll
-            for (int u = 0; u < 3; ++u)
-                if (on && u < nterms) {
-                    f[u] = __ldg(a.scl + (size_t)bs_matrix(a, task[2 + 2 * u], tl.sys) * a.nz + m);
-                    if (type == BS_FWD0) f[u] *= -((m == 0 || m == a.nz - 1) ? a.cx_edge : a.cx_in);
-                    if (type == BS_FWD || (type == BS_BWD && u > 0)) f[u] = -f[u];
-                }
+            // sign and (level 0, forward) the coupling of the row
+            const float f = type == BS_FWD ? -1.f
+                                           : (type == BS_FWD0 ? -((m == 0 || m == a.nz - 1) ? a.cx_edge : a.cx_in) : 1.f);
             float2 *out = vec + ((size_t)tl.sys * a.nrhs + tl.n0) * N + (size_t)line * a.nz + m;
             float *gout = gm + (((size_t)tl.sys * a.nx + line) * a.ng + (tl.r0 >> 5) + q) * a.nrhs + tl.n0;
-            const int ncol = min(nt, a.nrhs - tl.n0);
-            // the old line, ahead of the products that are added to it
-            float2 old[16];
-            auto fetch_old = [&](int c0) {
+            const int ncol = min(nt, a.nrhs - tl.n0), sl = tt % SL;
+            // the old line, ahead of the products that are added to it: four groups of 8 columns in flight
+            constexpr int OG = 4;
+            float2 old[OG][8];
+            auto fetch_old = [&](float2 (&o)[8], int c0) {
 #pragma unroll
-                for (int e = 0; e < 16; ++e)
-                    old[e] = on && to_r && c0 + e < ncol ? __ldcg(out + (size_t)(c0 + e) * N) : make_float2(0.f, 0.f);
+                for (int e = 0; e < 8; ++e)
+                    o[e] = on && to_r && c0 + e < ncol ? __ldcg(out + (size_t)(c0 + e) * N) : make_float2(0.f, 0.f);
             };
             if (to_r && !step_wait(tl, seen)) break;
-            if (warp_on) fetch_old(0);
-            for (int u = 0; u < nterms && go; ++u) go = wait(&acc_full[(tt + u) % SL], (tt + u) / SL);
-            if (!go) break;
+            if (warp_on) {
+#pragma unroll
+                for (int g = 0; g < OG; ++g) fetch_old(old[g], 8 * g);
+            }
+            if (!wait(&acc_full[sl], tt / SL)) break;
             tc_fence_after();
             if (warp_on) {
-                for (int c0 = 0; c0 < ncol; c0 += 16) {
-                    float2 o[16];
+                const uint32_t d = tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(sl * BS_SLOT_COLS);
+                for (int cb = 0; cb < ncol; cb += 8 * OG) {
 #pragma unroll
-                    for (int e = 0; e < 16; ++e) o[e] = old[e];
-                    if (c0 + 16 < ncol) fetch_old(c0 + 16);
+                    for (int g = 0; g < OG; ++g) {
+                        const int c0 = cb + 8 * g;
+                        if (c0 >= ncol) break;
+                        // Re = Ar Br - Ai Bi, Im = Ar Bi + Ai Br
+                        uint32_t rr[8], ri[8], ir[8], ii[8];
+                        tc_ld8_issue(d + c0, rr);
+                        tc_ld8_issue(d + nt + c0, ri);
+                        tc_ld8_issue(d + 2 * nt + c0, ir);
+                        tc_ld8_issue(d + 3 * nt + c0, ii);
+                        tc_wait_ld8(rr);
+                        tc_wait_ld8(ri);
+                        tc_wait_ld8(ir);
+                        tc_wait_ld8(ii);
+                        float2 o[8];
 #pragma unroll
-                    for (int u = 0; u < 3; ++u) {
-                        if (u >= nterms) break;
-                        const int sl = (tt + u) % SL;
-                        const uint32_t d = tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(sl * BS_SLOT_COLS + c0);
-                        float re[16], im[16];
-                        tc_ld16(d, re);
-                        tc_ld16(d + nt, im);
-                        if (nt <= 32) {   // Re = Ar Br - Ai Bi, Im = Ar Bi + Ai Br
-                            float t2[16];
-                            tc_ld16(d + 3 * nt, t2);
-#pragma unroll
-                            for (int e = 0; e < 16; ++e) re[e] -= t2[e];
-                            tc_ld16(d + 2 * nt, t2);
-#pragma unroll
-                            for (int e = 0; e < 16; ++e) im[e] += t2[e];
+                        for (int e = 0; e < 8; ++e) {
+                            const float sb = s_bscale[sl][c0 + e] * f;
+                            o[e].x = old[g][e].x + (__uint_as_float(rr[e]) - __uint_as_float(ii[e])) * sb;
+                            o[e].y = old[g][e].y + (__uint_as_float(ri[e]) + __uint_as_float(ir[e])) * sb;
                         }
+                        fetch_old(old[g], c0 + 8 * OG);
+                        uint32_t gmax = 0;
 #pragma unroll
-                        for (int e = 0; e < 16; ++e) {
-                            const float sb = s_bscale[sl][c0 + e];
-                            o[e].x += (re[e] * f[u]) * sb;
-                            o[e].y += (im[e] * f[u]) * sb;
+                        for (int e = 0; e < 8; ++e) {
+                            if (on && c0 + e < ncol) out[(size_t)(c0 + e) * N] = o[e];
+                            const uint32_t b = on ? max(abs_bits(o[e].x), abs_bits(o[e].y)) : 0u;
+                            const uint32_t w = __reduce_max_sync(0xffffffffu, b);
+                            if (lane == e) gmax = w;
                         }
+                        if (lane < 8 && c0 + lane < ncol) gout[c0 + lane] = __uint_as_float(gmax);
                     }
-                    uint32_t gmax = 0;
-#pragma unroll
-                    for (int e = 0; e < 16; ++e) {
-                        if (on && c0 + e < ncol) out[(size_t)(c0 + e) * N] = o[e];
-                        const uint32_t b = on ? max(abs_bits(o[e].x), abs_bits(o[e].y)) : 0u;
-                        const uint32_t w = __reduce_max_sync(0xffffffffu, b);
-                        if (lane == e) gmax = w;
-                    }
-                    if (lane < 16 && c0 + lane < ncol) gout[c0 + lane] = __uint_as_float(gmax);
                 }
             }
             tc_fence_before();
             __syncwarp();
             if (lane == 0) {
-                for (int u = 0; u < nterms; ++u) mbar_arrive(&acc_empty[(tt + u) % SL]);
+                mbar_arrive(&acc_empty[sl]);
                 __threadfence();   // the warp's stores before its count
                 atomicAdd(a.ctl + 2 + tl.phase * a.ns + tl.sys, 1u);
             }
-            tt += nterms;
+            ++tt;
         }
     }
     tc_fence_before();
@@ -618,79 +627,74 @@ __global__ void __launch_bounds__(256) line_max_kernel(int nx, int nz, int ng, i
     if (lane < nc) g[(((size_t)sys * nx + line) * ng + grp) * nrhs + c0 + lane] = __uint_as_float(mine);
 }
 
-// Image of 32 rows of a block: dst matrix pairs[2 t + 1] from src block pairs[2 t] (n x n row-major,
-// transposed if trans), rows 32 blockIdx.x ..; two passes over the rows (their maxima, then the
-// split), the second from L2.  Columns beyond n are zero.
+// largest modulus of the real and imaginary parts of the blocks, as bits (mx zeroed beforehand)
+__global__ void __launch_bounds__(256) bcr_max_kernel(long long n2, const float2 *src, long long stride, const int *pairs,
+                                                      uint32_t *mx) {
+    const int *pr = pairs + 2 * (size_t)blockIdx.y;
+    const float4 *A = reinterpret_cast<const float4 *>(src + (long long)pr[0] * stride);
+    uint32_t m = 0;
+    for (long long e = blockIdx.x * 256 + threadIdx.x; e < n2 / 2; e += (long long)gridDim.x * 256) {
+        const float4 v = __ldg(A + e);
+        m = max(max(m, max(abs_bits(v.x), abs_bits(v.y))), max(abs_bits(v.z), abs_bits(v.w)));
+    }
+    m = __reduce_max_sync(0xffffffffu, m);
+    if ((threadIdx.x & 31) == 0) atomicMax(mx + pr[1], m);
+}
+
+// Images of a block (n x n row-major) as matrix dst and, with tdst >= 0, of its transpose as
+// matrix tdst; a CTA takes 32 rows of the block, which are one chunk of columns of the
+// transpose.  Columns beyond n are zero.
+__device__ __forceinline__ void image_row(unsigned char *M, size_t mat_row, size_t im_off, int sw, int j, float sc,
+                                          const float2 (&v)[8]) {
+    // 16-byte piece j of a 128-byte row: hi of eight columns (j < 4), else lo
+    uint4 re, im;
+    uint32_t *pre = reinterpret_cast<uint32_t *>(&re), *pim = reinterpret_cast<uint32_t *>(&im);
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        uint32_t hi, lo;
+        split_h2(v[2 * e].x * sc, v[2 * e + 1].x * sc, hi, lo);
+        pre[e] = j < 4 ? hi : lo;
+        split_h2(v[2 * e].y * sc, v[2 * e + 1].y * sc, hi, lo);
+        pim[e] = j < 4 ? hi : lo;
+    }
+    unsigned char *d = M + mat_row * 128 + ((j ^ sw) << 4);
+    *reinterpret_cast<uint4 *>(d) = re;
+    *reinterpret_cast<uint4 *>(d + im_off) = im;
+}
 __global__ void __launch_bounds__(256) bcr_image_kernel(int n, int n_chunk, int nzr, const float2 *src, long long stride,
-                                                        int trans, const int *pairs, unsigned char *img, size_t mat_bytes,
-                                                        float *scl) {
+                                                        const int *pairs, const int *tdst, unsigned char *img,
+                                                        size_t mat_bytes, const uint32_t *mx, int *shift) {
     __shared__ float2 t[32][33];
-    __shared__ float s_scale[32];
     const int *pr = pairs + 2 * (size_t)blockIdx.y;
     const float2 *A = src + (long long)pr[0] * stride;
     const int r0 = 32 * blockIdx.x, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    auto entry = [&](int r, int k) -> float2 {   // (r, k) of the image's block, 0 beyond it
-        if (r >= n || k >= n) return make_float2(0.f, 0.f);
-        return __ldg(trans ? A + (long long)k * n + r : A + (long long)r * n + k);
-    };
-    // (loads run along the source's rows: lanes over k, or over r if transposed)
-    uint32_t mx[4] = {0, 0, 0, 0};
-    for (int c = 0; c < n_chunk; ++c) {
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const int o = w + 8 * q;
-            const float2 v = trans ? entry(r0 + lane, 32 * c + o) : entry(r0 + o, 32 * c + lane);
-            mx[q] = max(mx[q], max(abs_bits(v.x), abs_bits(v.y)));
-        }
+    const int sh = scale_shift(mx[pr[1]]);
+    const float sc = pow2(sh);
+    const int td = tdst ? tdst[blockIdx.y] : -1;
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        shift[pr[1]] = sh;
+        if (td >= 0) shift[td] = sh;
     }
-    if (trans) {   // lane = row: over the warps' k
-        uint32_t m = max(max(mx[0], mx[1]), max(mx[2], mx[3]));
-        uint32_t *sm = reinterpret_cast<uint32_t *>(&t[0][0]);
-        sm[w * 32 + lane] = m;
-        __syncthreads();
-        if (w == 0) {
-            for (int e = 1; e < 8; ++e) m = max(m, sm[e * 32 + lane]);
-            const int sh = scale_shift(m);
-            s_scale[lane] = pow2(sh);
-            if (r0 + lane < n) scl[(size_t)pr[1] * n + r0 + lane] = pow2(-sh);
-        }
-    } else {
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const int sh = scale_shift(__reduce_max_sync(0xffffffffu, mx[q])), o = w + 8 * q;
-            if (lane == 0) {
-                s_scale[o] = pow2(sh);
-                if (r0 + o < n) scl[(size_t)pr[1] * n + r0 + o] = pow2(-sh);
-            }
-        }
-    }
-    __syncthreads();
-    unsigned char *M = img + (size_t)pr[1] * mat_bytes;
+    unsigned char *M = img + (size_t)pr[1] * mat_bytes, *T = td >= 0 ? img + (size_t)td * mat_bytes : nullptr;
     const int row = threadIdx.x >> 3, j = threadIdx.x & 7, kb = 8 * (j & 3);
+    const size_t im_off = (size_t)nzr * 128;
     for (int c = 0; c < n_chunk; ++c) {
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
-            const int o = w + 8 * q;
-            if (trans) t[lane][o] = entry(r0 + lane, 32 * c + o);
-            else t[o][lane] = entry(r0 + o, 32 * c + lane);
+            const int o = w + 8 * q, r = r0 + o, k = 32 * c + lane;
+            t[o][lane] = r < n && k < n ? __ldg(A + (long long)r * n + k) : make_float2(0.f, 0.f);
         }
         __syncthreads();
+        float2 v[8];
         if (r0 + row < nzr) {
-            const float sc = s_scale[row];
-            uint4 re, im;
-            uint32_t *pre = reinterpret_cast<uint32_t *>(&re), *pim = reinterpret_cast<uint32_t *>(&im);
 #pragma unroll
-            for (int e = 0; e < 4; ++e) {   // 16-byte piece j: hi of columns kb .. kb + 7 (j < 4), else lo
-                const float2 v0 = t[row][kb + 2 * e], v1 = t[row][kb + 2 * e + 1];
-                uint32_t hi, lo;
-                split_h2(v0.x * sc, v1.x * sc, hi, lo);
-                pre[e] = j < 4 ? hi : lo;
-                split_h2(v0.y * sc, v1.y * sc, hi, lo);
-                pim[e] = j < 4 ? hi : lo;
-            }
-            unsigned char *d = M + ((size_t)(2 * c) * nzr + r0 + row) * 128 + ((j ^ (row & 7)) << 4);
-            *reinterpret_cast<uint4 *>(d) = re;
-            *reinterpret_cast<uint4 *>(d + (size_t)nzr * 128) = im;
+            for (int e = 0; e < 8; ++e) v[e] = t[row][kb + e];
+            image_row(M, (size_t)(2 * c) * nzr + r0 + row, im_off, row & 7, j, sc, v);
+        }
+        if (T && 32 * c + row < nzr) {   // row 32 c + row of the transpose, chunk r0 / 32
+#pragma unroll
+            for (int e = 0; e < 8; ++e) v[e] = t[kb + e][row];
+            image_row(T, (size_t)(2 * (r0 / 32)) * nzr + 32 * c + row, im_off, row & 7, j, sc, v);
         }
         __syncthreads();
     }
@@ -706,15 +710,18 @@ template <int NT> cudaError_t launch_nt(const BsArgs &a, int grid, double flops,
 
 }  // namespace
 
-cudaError_t launch_bcr_image(int n, const float2 *src, long long stride, bool trans, const int *pairs_dev, int count,
-                             unsigned char *img, float *scl, cudaStream_t st) {
+cudaError_t launch_bcr_image(int n, const float2 *src, long long stride, const int *pairs_dev, const int *tdst_dev,
+                             int count, unsigned char *img, uint32_t *mx, int *shift, cudaStream_t st) {
     if (count <= 0) return cudaSuccess;
     const BsLayout l = bs_layout(n);
     for (int t = 0; t < count; t += 65535) {
         const int nb = std::min(65535, count - t);
+        const int *pr = pairs_dev + 2 * (size_t)t;
+        HELM_TRACED(K_BCR_IMAGE, st, (bcr_max_kernel<<<dim3((unsigned)std::min(8, (n * n / 2 + 1023) / 1024), nb), 256, 0, st>>>(
+                                         (long long)n * n, src, stride, pr, mx)));
         HELM_TRACED(K_BCR_IMAGE, st, (bcr_image_kernel<<<dim3((n + 31) / 32, nb), 256, 0, st>>>(
-                                         n, l.n_chunk, l.nzr, src, stride, trans ? 1 : 0, pairs_dev + 2 * (size_t)t, img,
-                                         l.mat_bytes, scl)));
+                                         n, l.n_chunk, l.nzr, src, stride, pr, tdst_dev ? tdst_dev + t : nullptr, img,
+                                         l.mat_bytes, mx, shift)));
     }
     return cudaGetLastError();
 }

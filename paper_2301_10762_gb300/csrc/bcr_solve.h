@@ -38,7 +38,7 @@ struct BsArgs {
     float2 *r, *x;          // [ns][nrhs][N]: right-hand sides (overwritten) and the result
     float *gr, *gx;         // maxima of r and x: [ns][nx][ng][nrhs] each
     const unsigned char *img;
-    const float *scl;       // [matrix][nz]: 2^-s of each row of the image
+    const int *shift;       // [matrix]: the image holds the block's entries times 2^shift
     const int *tasks;       // [8] per task: line, type | terms << 4, then (block, line of the vector) per term
     float cx_in, cx_edge;
     unsigned *ctl;          // tile counter, abort word, tiles finished per step and system
@@ -62,9 +62,10 @@ __device__ __forceinline__ long long bs_matrix(const BsArgs &a, int code, int sy
     return bs_matrix_index(a.nx, a.ns, a.half, code, sys);
 }
 
-// dst matrices (pairs[.][1]) of the image from n x n row-major blocks src + pairs[.][0] * stride
-cudaError_t launch_bcr_image(int n, const float2 *src, long long stride, bool trans, const int *pairs_dev, int count,
-                             unsigned char *img, float *scl, cudaStream_t st);
+// images of n x n row-major blocks src + pairs[.][0] * stride as matrices pairs[.][1], and of their
+// transposes as matrices tdst[.] (tdst null: none); mx: zeroed words, one per matrix
+cudaError_t launch_bcr_image(int n, const float2 *src, long long stride, const int *pairs_dev, const int *tdst_dev,
+                             int count, unsigned char *img, uint32_t *mx, int *shift, cudaStream_t st);
 cudaError_t launch_bcr_solve(BsArgs a, const BsStep *steps, int n_steps, double flops, cudaStream_t st);
 int device_sms();   // streaming multiprocessors of the current device
 

@@ -91,7 +91,7 @@ struct helm_server {
             // ones (rows padded to 32 columns), and as many working blocks while it factors
             // (counted throughout)
             const size_t kept = (size_t)g.nx + 4 * ((size_t)g.nx / 2 + 1);
-            return kept * (blk + helm::bs_layout(g.nz).mat_bytes + 4 * (size_t)g.nz) + 96 * N + 65 * kMiB;   // + the split-K tiles
+            return kept * (blk + helm::bs_layout(g.nz).mat_bytes + 8) + 96 * N + 65 * kMiB;   // + the split-K tiles
         }
         return (size_t)g.nx * g.nz * g.nz * (prec == HELM_MIXED ? 8 : 16) + 96 * N + kMiB;
     }

@@ -26,9 +26,9 @@ __host__ __device__ constexpr uint32_t idesc_tf32(int n_real) {
     return (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(n_real >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
 }
 
-// the same for FP16 operands; neg_b: the product with -B
-__host__ __device__ constexpr uint32_t idesc_f16(int n_real, bool neg_b) {
-    return (1u << 4) | (neg_b ? 1u << 14 : 0u) | ((uint32_t)(n_real >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
+// the same for FP16 operands
+__host__ __device__ constexpr uint32_t idesc_f16(int n_real) {
+    return (1u << 4) | ((uint32_t)(n_real >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
 }
 
 // x rounded to the TF32 grid (10 explicit mantissa bits), to nearest with ties away from zero:
@@ -89,6 +89,18 @@ __device__ __forceinline__ void tc_ld16(uint32_t taddr, float (&v)[16]) {
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
     for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
+}
+
+// 8 consecutive accumulator columns of this thread's lane; tc_wait_ld() before they are used
+__device__ __forceinline__ void tc_ld8_issue(uint32_t taddr, uint32_t (&r)[8]) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+                 : "r"(taddr));
+}
+// (the registers pass through, so that no use moves above the wait)
+__device__ __forceinline__ void tc_wait_ld8(uint32_t (&r)[8]) {
+    asm volatile("tcgen05.wait::ld.sync.aligned;"
+                 : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7])::"memory");
 }
 
 // 16 consecutive columns of this thread's lane from v (the warp's 32 lanes); tc_wait_st() before
