@@ -148,7 +148,7 @@ extern "C" helm_status helm_assemble(const helm_grid *grid, const double *m_dev,
     if ((s = dev_alloc((void **)&op->m, N * sizeof(double), "allocate(m)", op->st)) != HELM_OK ||
         (s = dev_alloc((void **)&op->omega_dev, n_omega * sizeof(double), "allocate(omega)", op->st)) != HELM_OK ||
         (s = dev_alloc((void **)&op->diag, (size_t)n_omega * N * sizeof(double2), "allocate(diag)", op->st)) != HELM_OK ||
-        (s = dev_alloc((void **)&op->status, 2 * sizeof(int), "allocate(status)", op->st)) != HELM_OK ||
+        (s = dev_alloc((void **)&op->status, 3 * sizeof(int), "allocate(status)", op->st)) != HELM_OK ||
         (s = dev_alloc((void **)&op->gk, (size_t)n_omega * N * sizeof(double2), "allocate(g)", op->st)) != HELM_OK ||
         (s = dev_alloc((void **)&op->gpk, (size_t)n_omega * N * sizeof(double2), "allocate(g')", op->st)) != HELM_OK) {
         helm_op_destroy(op);
@@ -158,7 +158,7 @@ extern "C" helm_status helm_assemble(const helm_grid *grid, const double *m_dev,
     if ((e = cudaMemcpyAsync(op->m, m_dev, N * sizeof(double), cudaMemcpyDeviceToDevice, op->st)) != cudaSuccess ||
         (e = cudaMemcpyAsync(op->omega_dev, omega, n_omega * sizeof(double), cudaMemcpyHostToDevice, op->st)) !=
             cudaSuccess ||
-        (e = cudaMemsetAsync(op->status, 0, 2 * sizeof(int), op->st)) != cudaSuccess ||
+        (e = cudaMemsetAsync(op->status, 0, 3 * sizeof(int), op->st)) != cudaSuccess ||
         (e = launch_assemble(op->g, op->m, op->omega_dev, n_omega, op->diag, op->st)) != cudaSuccess ||
         (e = launch_gcoef(op->g, op->m, op->omega_dev, n_omega, op->gk, op->gpk, op->st)) != cudaSuccess ||
         (e = cudaStreamSynchronize(op->st)) != cudaSuccess) {
@@ -184,12 +184,26 @@ extern "C" void helm_op_destroy(helm_op_t *op) {
 // ------------------------------------------------------------------------ factor
 
 // Factor method of a mixed factor: the options, else HELM_FACTOR=line|bcr, else BCR on lines of
-// at least kBcrMinNz nodes and the line recurrence below.  The line recurrence's dependent chain
-// (n_x line inversions, n_x line steps per solve) is what BCR removes; on short lines its
-// per-step cost is small and BCR's extra arithmetic and launches do not pay (measured: 128 x 128
-// with 16 right-hand sides per frequency favours the line factor, 256 x 256 with 64 favours BCR
-// by 2.5x).  FP64 factors are line factors (the tensor cores have no FP64 path).
+// at least kBcrMinNz nodes and the line recurrence below.  FP64 factors are line factors (the
+// tensor cores have no FP64 path).
 static constexpr int kBcrMinNz = 192;
+// lines from which BCR was always the automatic choice and is not second-guessed
+static constexpr int kBcrSureNz = 192;
+// BCR eliminates lines with Dirichlet neighbours, so a frequency near a resonance of a strip of the
+// medium makes an eliminated block nearly singular.  Over random media the refinement took one
+// sweep more from |A| |Dinv| of 2^9 (entries of the inverses of 2^7 and a diagonal of about 4), 5 to
+// 6 sweeps at 2^10, 7 to 15 at 2^11, and did not converge at 2^13; nearly all factors stay below
+// 2^5.  From 2^10 a short line takes the line recurrence.
+static constexpr float kBcrMaxGrowth = 1024.f;
+static bool bcr_falls_back(const GridGeom &g, const helm_factor_opts *opts, const int st_host[3]) {
+    if (g.nz >= kBcrSureNz || (opts && opts->method == HELM_FACTOR_BCR) || (st_host[0] & ST_TIMEOUT)) return false;
+    const char *env = getenv("HELM_FACTOR");
+    if (env && !strcmp(env, "bcr")) return false;
+    float mx;
+    memcpy(&mx, &st_host[2], sizeof(mx));
+    const double scale = 2.0 * (g.hz / g.hx + g.hx / g.hz);
+    return (st_host[0] & ST_SINGULAR) || !(mx * scale < kBcrMaxGrowth);
+}
 bool helm::factor_picks_bcr(const GridGeom &g, helm_prec prec, int method) {
     if (prec != HELM_MIXED || !bcr_supported(g)) return false;
     int m = method;
@@ -228,7 +242,7 @@ extern "C" helm_status helm_factor(helm_op_t *op, helm_prec prec, const helm_fac
     const size_t gelems = (size_t)op->n_omega * g.nx * g.nz * g.nz;
     helm_status s;
     cudaError_t e;
-    if ((e = cudaMemsetAsync(op->status, 0, 2 * sizeof(int), op->st)) != cudaSuccess) {
+    if ((e = cudaMemsetAsync(op->status, 0, 3 * sizeof(int), op->st)) != cudaSuccess) {
         helm_set_error("helm_factor", e);
         helm_factor_destroy(f);
         return HELM_ECUDA;
@@ -262,6 +276,13 @@ extern "C" helm_status helm_factor(helm_op_t *op, helm_prec prec, const helm_fac
             diag_bad = nullptr;
         }
     };
+    int st_host[3] = {0, 0, 0};   // status bits, pivot blocks inverted in FP64, bits of the largest entry of the BCR inverses
+    auto read_status = [&](cudaError_t e1) {
+        if (e1 == cudaSuccess) e1 = cudaMemcpyAsync(st_host, op->status, sizeof(st_host), cudaMemcpyDeviceToHost, op->st);
+        if (e1 == cudaSuccess) e1 = cudaStreamSynchronize(op->st);
+        return e1;
+    };
+    bool line = !f->use_bcr;
     if (f->use_bcr) {
         if ((s = bcr_factor(f)) != HELM_OK) {
             cudaStreamSynchronize(op->st);
@@ -269,8 +290,17 @@ extern "C" helm_status helm_factor(helm_op_t *op, helm_prec prec, const helm_fac
             helm_factor_destroy(f);
             return s;
         }
-        e = cudaSuccess;
-    } else {
+        e = read_status(cudaSuccess);
+        // an automatic choice on a short line, which the line recurrence (its Schur complements run
+        // from the absorbing boundary) takes instead where an eliminated block came out nearly singular
+        if (e == cudaSuccess && bcr_falls_back(g, opts, st_host)) {
+            bcr_free(f);
+            f->use_bcr = false;
+            line = true;
+            e = cudaMemsetAsync(op->status, 0, 3 * sizeof(int), op->st);
+        }
+    }
+    if (line) {
         if ((s = dev_alloc(&f->G, gelems * esz, "allocate(factor)", op->st)) != HELM_OK ||
             (s = dev_alloc(&f->xch, (size_t)op->n_omega * factor_xch_elems(g.nz) * esz, "allocate(exchange)",
                            op->st)) != HELM_OK) {
@@ -278,16 +308,15 @@ extern "C" helm_status helm_factor(helm_op_t *op, helm_prec prec, const helm_fac
             helm_factor_destroy(f);
             return s;
         }
-        if (prec == HELM_FP64)
+        if (e != cudaSuccess) {
+        } else if (prec == HELM_FP64)
             e = launch_line_factor<double>(g, op->n_omega, op->diag, (double2 *)f->G, (double2 *)f->xch, op->status,
                                            f->cs, op->st, &f->mid);
         else
             e = launch_line_factor<float>(g, op->n_omega, op->diag, (float2 *)f->G, (float2 *)f->xch, op->status,
                                           f->cs, op->st, &f->mid);
+        e = read_status(e);
     }
-    int st_host[2] = {0, 0};   // status bits, pivot blocks inverted in FP64
-    if (e == cudaSuccess) e = cudaMemcpyAsync(st_host, op->status, 2 * sizeof(int), cudaMemcpyDeviceToHost, op->st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(op->st);
     restore_diag();
     f->fp64_blocks = st_host[1];
     if (e != cudaSuccess) {
@@ -340,7 +369,6 @@ extern "C" void helm_factor_destroy(helm_factor_t *f) {
     dev_free(f->y, st);
     dev_free(f->norms, st);
     dev_free(f->maxima, st);
-    dev_free(f->state, st);
     bcr_free(f);
     delete f;
 }
@@ -358,12 +386,10 @@ helm_status factor_reserve(helm_factor_t *f, int nrhs) {
     dev_free(f->y, st);
     dev_free(f->norms, st);
     dev_free(f->maxima, st);
-    dev_free(f->state, st);
     f->bd = f->xa = f->xb = nullptr;
     f->r32 = f->y = nullptr;
     f->norms = nullptr;
     f->maxima = nullptr;
-    f->state = nullptr;
     f->cap = 0;
     helm_status s;
     if (f->prec == HELM_MIXED &&
@@ -371,14 +397,14 @@ helm_status factor_reserve(helm_factor_t *f, int nrhs) {
          (s = dev_alloc((void **)&f->xa, cols * N * sizeof(float4), "allocate(iterate)", st)) != HELM_OK ||
          (s = dev_alloc((void **)&f->xb, cols * N * sizeof(float4), "allocate(iterate)", st)) != HELM_OK ||
          (s = dev_alloc((void **)&f->r32, cols * N * sizeof(float2), "allocate(residual)", st)) != HELM_OK ||
-         (s = dev_alloc((void **)&f->y, cols * N * sizeof(float2), "allocate(work)", st)) != HELM_OK ||
-         (s = dev_alloc((void **)&f->state, refine_state_bytes(op->n_omega), "allocate(refinement state)", st)) !=
-             HELM_OK))
+         (s = dev_alloc((void **)&f->y, cols * N * sizeof(float2), "allocate(work)", st)) != HELM_OK))
         return s;
     if (f->use_bcr &&
         (s = dev_alloc((void **)&f->maxima, bcr_maxima_elems(op->g, cols) * sizeof(float), "allocate(maxima)", st)) != HELM_OK)
         return s;
-    if ((s = dev_alloc((void **)&f->norms, cols * 2 * sizeof(double), "allocate(norms)", st)) != HELM_OK) return s;
+    const size_t state_bytes = f->prec == HELM_MIXED ? refine_state_bytes(op->n_omega) : 0;   // behind the norms
+    if ((s = dev_alloc((void **)&f->norms, cols * 2 * sizeof(double) + state_bytes, "allocate(norms)", st)) != HELM_OK)
+        return s;
     f->norms_host.assign(cols * 2, 0.0);
     f->cap = nrhs;
     return HELM_OK;
@@ -410,7 +436,7 @@ helm_status max_relres(const helm_op *op, size_t cols, const double *norms_dev, 
 // updates enqueued after the test has stopped the loop return at once.  The first batch is as
 // long as the previous solve with this factor took.
 helm_status mixed_refine(const helm_factor_t *f, int nrhs, const double2 *B, double2 *X, int conj, double rtol,
-                         int max_iter, const MixedWork &w, int *iters, double *relres) {
+                         int max_iter, const MixedWork &w, int *iters, double *relres, bool *timed_out) {
     constexpr double kPairFloor = 1e-12;   // well above the pair residual's floor (about 1e-13)
     constexpr int kLaterBatch = 2;
     const helm_op *op = f->op;
@@ -420,8 +446,14 @@ helm_status mixed_refine(const helm_factor_t *f, int nrhs, const double2 *B, dou
     const size_t n = (size_t)cols * g.nx * g.nz;
     const int rchunk = 16;
     if (max_iter < 1) max_iter = 1;
-    cudaError_t e = cudaMemsetAsync(w.state, 0, refine_state_bytes(n_sys), op->st);
-    if (e == cudaSuccess) e = launch_refine_start(g, cols, B, conj, w.bd, w.r32, w.norms, op->st);
+    // the state follows the norms (MixedWork): zeroed together
+    cudaError_t e = cudaMemsetAsync(w.norms, 0, (size_t)cols * 2 * sizeof(double) + refine_state_bytes(n_sys), op->st);
+    // block cyclic reduction: the maxima of r and the zeroed counters that a solve starts from are
+    // left by the kernel that writes r
+    float *gmax = f->use_bcr ? w.maxima : nullptr;
+    unsigned *ctl = f->use_bcr ? f->bcr.ctl : nullptr;
+    const int n_ctl = f->use_bcr ? (int)bs_ctl_words((int)f->bcr.steps.size(), n_sys) : 0;
+    if (e == cudaSuccess) e = launch_refine_start(g, n_sys, nrhs, B, conj, w.bd, w.r32, w.norms, gmax, ctl, n_ctl, op->st);
     if (e != cudaSuccess) { helm_set_error("refinement start", e); return HELM_ECUDA; }
     const int *skip = &w.state->done;
     // the correction A~^{-1} r: line sweep, or the block-cyclic-reduction solve (which works in
@@ -431,7 +463,7 @@ helm_status mixed_refine(const helm_factor_t *f, int nrhs, const double2 *B, dou
     auto sweep = [&](const int *skip_flag) -> cudaError_t {
         const int *frozen = skip_flag ? refine_sys(w.state) + 1 : nullptr;
         if (f->use_bcr) {
-            const helm_status bs = bcr_solve(f, nrhs, w.r32, w.y, w.maxima, skip_flag, frozen);
+            const helm_status bs = bcr_solve(f, nrhs, w.r32, w.y, w.maxima, skip_flag != nullptr, skip_flag, frozen);
             return bs == HELM_OK ? cudaSuccess : cudaErrorLaunchFailure;
         }
         return launch_line_sweep<float>(g, n_sys, nrhs, (const float2 *)f->G, w.r32, nullptr, w.y, 0, rchunk,
@@ -446,11 +478,15 @@ helm_status mixed_refine(const helm_factor_t *f, int nrhs, const double2 *B, dou
             const float4 *x_in = enq == 0 ? nullptr : ((enq & 1) ? w.xa : w.xb);
             float4 *x_out = (enq & 1) ? w.xb : w.xa;
             if ((e = sweep(skip)) != cudaSuccess) { helm_set_error("sweep mixed", e); return HELM_ECUDA; }
-            e = launch_refine_update(g, n_sys, nrhs, f->diag2, w.bd, x_in, w.y, x_out, w.r32, w.norms, op->st, w.state,
-                                     RefineStop{rtol, kPairFloor, max_iter});
+            e = launch_refine_update(g, n_sys, nrhs, f->diag2, w.bd, x_in, w.y, x_out, w.r32, w.norms, gmax, ctl, n_ctl,
+                                     op->status, op->st, w.state, RefineStop{rtol, kPairFloor, max_iter});
             if (e != cudaSuccess) { helm_set_error("refinement update", e); return HELM_ECUDA; }
         }
-        e = cudaMemcpyAsync(&hs, w.state, sizeof(RefineState), cudaMemcpyDeviceToHost, op->st);
+        // X of the newest iterates, enqueued before the state is read: one wait per batch, and
+        // nothing left to wait for once the loop has stopped (a batch that has not is followed by
+        // another X; 512 columns of 256^2 take 0.2 ms)
+        e = launch_refine_finish(n, g.nx * g.nz, nrhs, w.xa, w.xb, w.state, conj, X, op->st);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(&hs, w.state, sizeof(RefineState), cudaMemcpyDeviceToHost, op->st);
         if (e == cudaSuccess) e = cudaStreamSynchronize(op->st);
         if (e != cudaSuccess) { helm_set_error("read refinement state", e); return HELM_ECUDA; }
         if (hs.done) break;
@@ -459,10 +495,11 @@ helm_status mixed_refine(const helm_factor_t *f, int nrhs, const double2 *B, dou
     int it = hs.iters;
     double rel = hs.rel;
     f->last_iters.store(std::max(1, it), std::memory_order_relaxed);
-    e = launch_refine_finish(n, g.nx * g.nz, nrhs, w.xa, w.xb, w.state, conj, X, op->st);
-    if (e != cudaSuccess) { helm_set_error("refinement finish", e); return HELM_ECUDA; }
+    *timed_out = (hs.status & ST_TIMEOUT) != 0;
+    bool tail = false;
     if (!(rel <= rtol) && it < max_iter && isfinite(rel)) {
         // FP64 phase: r = b - A x in FP64 on the FP64 iterate, correction conj?(A~^{-1} conj?(r))
+        tail = true;
         for (;;) {
             e = cudaMemsetAsync(w.norms, 0, (size_t)cols * 2 * sizeof(double), op->st);
             if (e == cudaSuccess) e = launch_residual(g, n_sys, nrhs, op->diag, B, X, w.r32, w.norms, conj, op->st);
@@ -477,6 +514,11 @@ helm_status mixed_refine(const helm_factor_t *f, int nrhs, const double2 *B, dou
     }
     *iters = it;
     *relres = rel;
+    if (tail && !*timed_out) {   // sweeps after the state was read
+        const helm_status rs = read_sweep_status(op);
+        if (rs == HELM_ETIMEOUT) *timed_out = true;
+        else if (rs != HELM_OK) return rs;
+    }
     return HELM_OK;
 }
 
@@ -521,12 +563,14 @@ helm_status solve_impl(helm_factor_t *f, int nrhs, const double2 *B, double2 *X,
         return HELM_OK;
     }
     if ((s = factor_reserve(f, nrhs)) != HELM_OK) return s;
-    const MixedWork w{f->bd, f->xa, f->xb, f->r32, f->y, f->norms, f->norms_host.data(), f->state, f->maxima};
+    const MixedWork w{f->bd, f->xa, f->xb, f->r32, f->y, f->norms, f->norms_host.data(),
+                      reinterpret_cast<RefineState *>(f->norms + 2 * cols), f->maxima};
     int it = 0;
     double rel = INFINITY;
-    if ((s = mixed_refine(f, nrhs, B, X, conj, rtol, max_iter, w, &it, &rel)) != HELM_OK) return s;
+    bool timed_out = false;
+    if ((s = mixed_refine(f, nrhs, B, X, conj, rtol, max_iter, w, &it, &rel, &timed_out)) != HELM_OK) return s;
     if (info) { info->iters = it; info->max_relres = rel; }
-    if ((s = read_sweep_status(op)) != HELM_OK) return s;
+    if (timed_out) { helm_set_msg("a sweep kernel gave up waiting for its cluster"); return HELM_ETIMEOUT; }
     if (!(rel <= rtol)) { helm_set_msg("refinement did not reach rtol"); return HELM_ENOCONV; }
     return HELM_OK;
 }

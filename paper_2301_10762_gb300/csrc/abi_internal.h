@@ -60,10 +60,9 @@ struct helm_factor {
     int cap = 0;
     float4 *bd = nullptr, *xa = nullptr, *xb = nullptr;   // mixed: b and the iterate (ping-pong), FP32 pairs
     float2 *r32 = nullptr, *y = nullptr;                  // mixed: correction right-hand side and result
-    double *norms = nullptr;
-    std::vector<double> norms_host;   // host copy of the norms (pageable: no pinned allocation)
+    double *norms = nullptr;   // per column, then (mixed) the device-side refinement control
+    std::vector<double> norms_host; // host copy of the norms (pageable: no pinned allocation)
     float *maxima = nullptr;                  // mixed, block cyclic reduction: the solve's vector maxima
-    helm::RefineState *state = nullptr;       // mixed: device-side refinement control
     mutable std::atomic<int> last_iters{3};   // correction sweeps the previous mixed solve took
 };
 
@@ -73,7 +72,7 @@ struct MixedWork {
     float2 *r32, *y;
     double *norms;        // device [cols][2]
     double *norms_host;   // host [cols][2]
-    helm::RefineState *state;   // device
+    helm::RefineState *state;   // device, directly behind the norms of the solve's columns
     float *maxima;        // device, block cyclic reduction only (bcr_maxima_elems)
 };
 
@@ -100,9 +99,10 @@ helm_status factor_reserve(helm_factor_t *f, int nrhs);
 helm_status read_sweep_status(const helm_op *op);
 helm_status solve_impl(helm_factor_t *f, int nrhs, const double2 *B, double2 *X, double rtol, int max_iter,
                        helm_solve_info *info, int conj);
-// mixed-precision refinement (refine.cu kernels) to ||b - A x|| / ||b|| <= rtol per column
+// mixed-precision refinement (refine.cu kernels; X is complete when it returns; timed_out: a sweep's
+// bounded wait gave up) to ||b - A x|| / ||b|| <= rtol per column
 helm_status mixed_refine(const helm_factor_t *f, int nrhs, const double2 *B, double2 *X, int conj, double rtol,
-                         int max_iter, const MixedWork &w, int *iters, double *relres);
+                         int max_iter, const MixedWork &w, int *iters, double *relres, bool *timed_out);
 // max over columns of ||r|| / ||b|| from a device norms buffer (synchronises the op's stream)
 helm_status max_relres(const helm_op *op, size_t cols, const double *norms_dev, double *norms_host, double *out);
 helm_status acq_upload(const helm_op *op, const helm_acq *acq, DevAcq *d);
@@ -116,8 +116,8 @@ helm_status bcr_factor(helm_factor_t *f);
 void bcr_free(helm_factor_t *f);
 // frozen: NULL, or the refinement's per-system flags (stride 2): columns of a set flag are skipped
 size_t bcr_maxima_elems(const GridGeom &g, size_t cols);   // floats of scratch of a solve of cols columns
-helm_status bcr_solve(const helm_factor_t *f, int nrhs, float2 *r, float2 *x, float *maxima, const int *skip,
-                      const int *frozen = nullptr);
+helm_status bcr_solve(const helm_factor_t *f, int nrhs, float2 *r, float2 *x, float *maxima, bool prepared,
+                      const int *skip, const int *frozen = nullptr);
 helm_status blas_zgemm(int batch, int M, int N, int K, const float2 *A, long long sa, int lda, const float2 *Bt,
                        long long sb, int ldb, float sign, const float2 *C0, float2 *C, long long sc, int ldc,
                        cudaStream_t st, int *status);

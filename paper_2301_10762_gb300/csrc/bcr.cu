@@ -495,6 +495,20 @@ __global__ void __launch_bounds__(512) tri_rank1_kernel(int n, int n1, TriIn tri
     }
 }
 
+// *out = largest of n words
+__global__ void __launch_bounds__(1024) max_words_kernel(size_t n, const uint32_t *v, int *out) {
+    __shared__ uint32_t s[32];
+    uint32_t m = 0;
+    for (size_t i = threadIdx.x; i < n; i += 1024) m = max(m, v[i]);
+    m = __reduce_max_sync(0xffffffffu, m);
+    if ((threadIdx.x & 31) == 0) s[threadIdx.x >> 5] = m;
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        m = __reduce_max_sync(0xffffffffu, s[threadIdx.x]);
+        if (threadIdx.x == 0) *out = (int)m;
+    }
+}
+
 // ----------------------------------------------------------------- host side
 
 struct TaskBuf {   // device copy of host-built task lists (freed on the stream when done)
@@ -935,6 +949,13 @@ helm_status bcr_factor(helm_factor_t *f) {
         if ((s = invert_blocks(nz, fD, fD, last, op->status, pl)) != HELM_OK) return s;
         for (int i = 0; i < ns * nx; ++i) di.insert(di.end(), {i, i});
         if ((s = image_blocks(nz, D, di, {}, b, mx, pl)) != HELM_OK) return s;
+        int *out = op->status + 2;   // the largest entry of the inverses (the matrices 0 .. ns nx - 1)
+        pl.ops.push_back([=](const int *) -> helm_status {
+            HELM_TRACED(K_BCR_IMAGE, st, (max_words_kernel<<<1, 1024, 0, st>>>((size_t)ns * nx, mx, out)));
+            const cudaError_t e2 = cudaGetLastError();
+            if (e2 != cudaSuccess) { helm_set_error("bcr: maxima", e2); return HELM_ECUDA; }
+            return HELM_OK;
+        });
     }
     if ((s = pl.run()) != HELM_OK) return s;
     // the solve's steps and tasks (the same for every system), built once
@@ -1008,8 +1029,9 @@ size_t bcr_maxima_elems(const GridGeom &g, size_t cols) { return 2 * cols * g.nx
 
 // x = A~^{-1} r for every system and right-hand side, complex FP32: r [n_sys][nrhs][N] is the
 // working vector (overwritten), x [n_sys][nrhs][N] the result.  skip: launches do nothing
-// while it is set (refinement finished).  maxima: bcr_maxima_elems floats of scratch.
-helm_status bcr_solve(const helm_factor_t *f, int nrhs, float2 *r, float2 *x, float *maxima, const int *skip,
+// while it is set (refinement finished).  maxima: bcr_maxima_elems floats of scratch; prepared: the
+// first half holds the maxima of r already and the factor's counters are zero.
+helm_status bcr_solve(const helm_factor_t *f, int nrhs, float2 *r, float2 *x, float *maxima, bool prepared, const int *skip,
                       const int *frozen) {
     const helm_op *op = f->op;
     const GridGeom &g = op->g;
@@ -1035,7 +1057,7 @@ helm_status bcr_solve(const helm_factor_t *f, int nrhs, float2 *r, float2 *x, fl
     a.frozen = frozen;
     a.tries = wait_tries();
     const double flops = 8.0 * g.nz * g.nz * nrhs * (double)b.terms * a.ns;
-    const cudaError_t e = launch_bcr_solve(a, b.steps.data(), (int)b.steps.size(), flops, op->st);
+    const cudaError_t e = launch_bcr_solve(a, b.steps.data(), (int)b.steps.size(), prepared, flops, op->st);
     if (e != cudaSuccess) { helm_set_error("bcr solve", e); return HELM_ECUDA; }
     return HELM_OK;
 }

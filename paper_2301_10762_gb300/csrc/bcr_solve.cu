@@ -726,7 +726,7 @@ cudaError_t launch_bcr_image(int n, const float2 *src, long long stride, const i
     return cudaGetLastError();
 }
 
-cudaError_t launch_bcr_solve(BsArgs a, const BsStep *steps, int n_steps, double flops, cudaStream_t st) {
+cudaError_t launch_bcr_solve(BsArgs a, const BsStep *steps, int n_steps, bool prepared, double flops, cudaStream_t st) {
     if (n_steps > BS_MAX_PHASE || (a.nz & 1)) return cudaErrorInvalidValue;
     const BsLayout l = bs_layout(a.nz);
     a.nzr = l.nzr;
@@ -758,13 +758,15 @@ cudaError_t launch_bcr_solve(BsArgs a, const BsStep *steps, int n_steps, double 
         ph.done = 4 * ph.tasks * ph.n_tiles * ph.mt;   // four epilogue warps count each tile
     }
     a.n_tile_total = tile;
-    cudaError_t e = cudaMemsetAsync(a.ctl, 0, sizeof(unsigned) * bs_ctl_words(n_steps, a.ns), st);
-    if (e != cudaSuccess) return e;
-    const int n_cb = (a.nrhs + 31) / 32;
-    const long long items = (long long)a.ns * a.nx * a.ng * n_cb;
-    HELM_TRACED(K_LINEMAX, st, (line_max_kernel<<<(unsigned)((items + 7) / 8), 256, 0, st>>>(
-                                   a.nx, a.nz, a.ng, a.nrhs, n_cb, items, a.r, a.gr, a.skip, a.frozen)));
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    if (!prepared) {
+        cudaError_t e = cudaMemsetAsync(a.ctl, 0, sizeof(unsigned) * bs_ctl_words(n_steps, a.ns), st);
+        if (e != cudaSuccess) return e;
+        const int n_cb = (a.nrhs + 31) / 32;
+        const long long items = (long long)a.ns * a.nx * a.ng * n_cb;
+        HELM_TRACED(K_LINEMAX, st, (line_max_kernel<<<(unsigned)((items + 7) / 8), 256, 0, st>>>(
+                                       a.nx, a.nz, a.ng, a.nrhs, n_cb, items, a.r, a.gr, a.skip, a.frozen)));
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    }
     const int grid = std::min(sms, tile);
     if (nt == 16) return launch_nt<16>(a, grid, flops, st);
     return nt == 32 ? launch_nt<32>(a, grid, flops, st) : launch_nt<64>(a, grid, flops, st);

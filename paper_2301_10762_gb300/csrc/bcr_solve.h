@@ -66,7 +66,7 @@ __device__ __forceinline__ long long bs_matrix(const BsArgs &a, int code, int sy
 // transposes as matrices tdst[.] (tdst null: none); mx: zeroed words, one per matrix
 cudaError_t launch_bcr_image(int n, const float2 *src, long long stride, const int *pairs_dev, const int *tdst_dev,
                              int count, unsigned char *img, uint32_t *mx, int *shift, cudaStream_t st);
-cudaError_t launch_bcr_solve(BsArgs a, const BsStep *steps, int n_steps, double flops, cudaStream_t st);
+cudaError_t launch_bcr_solve(BsArgs a, const BsStep *steps, int n_steps, bool prepared, double flops, cudaStream_t st);
 int device_sms();   // streaming multiprocessors of the current device
 
 }  // namespace helm

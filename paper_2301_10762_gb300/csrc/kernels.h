@@ -53,8 +53,10 @@ int max_active_clusters(const void *fn, int csz, int threads, size_t smem);
 // diag2[s][k] = (hi.re, hi.im, lo.re, lo.im) of the FP64 diagonal
 cudaError_t launch_split_diag(size_t n, const double2 *diag, float4 *diag2, cudaStream_t st);
 // bd = pair form of conj?(B), r32 = its leading part; norms[col][1] = ||B||^2, norms[col][0] = 0
-cudaError_t launch_refine_start(const GridGeom &g, int cols, const double2 *B, int conj, float4 *bd, float2 *r32,
-                                double *norms, cudaStream_t st);
+// (norms zeroed beforehand).  gmax (optional): maxima of r32 for the block-cyclic-reduction solve;
+// ctl (optional): its n_ctl counters, zeroed
+cudaError_t launch_refine_start(const GridGeom &g, int n_sys, int nrhs, const double2 *B, int conj, float4 *bd, float2 *r32,
+                                double *norms, float *gmax, unsigned *ctl, int n_ctl, cudaStream_t st);
 // Device-side control of the refinement loop: after each update pass, the stopping test computes
 // rel = max_col ||r|| / ||b|| from the norms, decides whether the pair iteration is done and
 // zeroes norms[col][0] for the next pass.
@@ -64,6 +66,7 @@ struct RefineState {
     double rel;      // latest max relative residual
     double prev;     // the one before
     unsigned blocks; // update blocks finished in the current pass (the last one runs the test)
+    int status;      // the op's status word after the latest pass
 };
 // The state is followed in memory by int sys[n_sys][2]: per system (frequency) the sweeps applied
 // to it and a frozen flag, set once all its columns are at rtol; later updates (and, on the
@@ -86,9 +89,12 @@ struct RefineStop {  // stopping rule of the pair phase, applied on the device
 // (zero on entry: refine_start and the stopping test leave it so).  With state, the last block to
 // finish applies the stopping test, and state->done makes later launches do
 // nothing.
+// gmax, ctl: as launch_refine_start, for the next solve.  solve_status: the op's status word,
+// copied into the state by the last block.
 cudaError_t launch_refine_update(const GridGeom &g, int n_sys, int nrhs, const float4 *diag2, const float4 *bd,
                                  const float4 *x_in, const float2 *delta, float4 *x_out, float2 *r32, double *norms,
-                                 cudaStream_t st, RefineState *state = nullptr, RefineStop stop = {});
+                                 float *gmax, unsigned *ctl, int n_ctl, const int *solve_status, cudaStream_t st,
+                                 RefineState *state, RefineStop stop);
 
 // X = conj?(hi + lo) in FP64 of each system's newest iterate: xa after an odd number of sweeps of
 // that system, else xb (columns of N nodes, nrhs columns per system)

@@ -29,7 +29,6 @@ namespace helm {
 namespace {
 
 constexpr int RF_THREADS = 256;
-constexpr int RF_NPT = 8;   // nodes per thread in the per-column kernels (a block covers 2048 nodes)
 
 // ---------------------------------------------------------------- FP32-pair arithmetic
 // The intrinsics keep the compiler from contracting or reassociating these sequences.
@@ -117,34 +116,59 @@ __global__ void split_diag_kernel(size_t n, const double2 *diag, float4 *diag2) 
     }
 }
 
-// grid: (node blocks of RF_THREADS * RF_NPT, columns)
-__global__ void __launch_bounds__(RF_THREADS) refine_start_kernel(int N, int cols, const double2 *B, int conj,
-                                                                  float4 *bd, float2 *r32, double *norms) {
+// Nodes of a column are taken by warps as groups of 32 consecutive nodes of a line (ng = ceil(nz /
+// 32) groups a line, lanes beyond the line idle), so that the group's maximum, which the block
+// cyclic reduction scales its operands by (bcr_solve.cu), is one warp reduction here instead of
+// another pass over the vector (0.05 ms of a 256^2 sweep with 512 columns).
+struct RefineVec {
+    float *gmax;      // maxima of r: [sys][line][ng][nrhs] (null: not wanted)
+    unsigned *ctl;    // the solve's counters, zeroed for the next solve (null: none)
+    int n_ctl;
+};
+__device__ __forceinline__ void group_max(const RefineVec &rv, float2 r, bool on, size_t at, int lane) {
+    if (!rv.gmax) return;
+    const uint32_t b = on ? max(__float_as_uint(r.x) & 0x7fffffffu, __float_as_uint(r.y) & 0x7fffffffu) : 0u;
+    const uint32_t m = __reduce_max_sync(0xffffffffu, b);
+    if (lane == 0) rv.gmax[at] = __uint_as_float(m);
+}
+
+// grid: (blocks of 8 * NPT groups, columns)
+template <int NPT>
+__global__ void __launch_bounds__(RF_THREADS) refine_start_kernel(GridGeom g, int nrhs, int cols, const double2 *B, int conj,
+                                                                  float4 *bd, float2 *r32, double *norms, RefineVec rv) {
     __shared__ double sh[RF_THREADS / 32];
+    const int nz = g.nz, N = g.nx * nz, ng = (nz + 31) >> 5, items = g.nx * ng;
+    const int lane = threadIdx.x & 31, i0 = blockIdx.x * (RF_THREADS / 32) * NPT + (threadIdx.x >> 5);
+    if (blockIdx.x == 0 && blockIdx.y == 0 && rv.ctl)
+        for (int e = threadIdx.x; e < rv.n_ctl; e += RF_THREADS) rv.ctl[e] = 0u;
     for (int c = blockIdx.y; c < cols; c += gridDim.y) {
         double bb = 0.0;
         const size_t base = (size_t)c * N;
-        const int k0 = blockIdx.x * RF_THREADS * RF_NPT + threadIdx.x;
-        double2 b[RF_NPT];
+        double2 b[NPT];
 #pragma unroll
-        for (int q = 0; q < RF_NPT; ++q) {   // all loads first: RF_NPT in flight per thread
-            const int k = k0 + q * RF_THREADS;
-            b[q] = k < N ? __ldcs(B + base + k) : make_double2(0.0, 0.0);
+        for (int q = 0; q < NPT; ++q) {   // all loads first: NPT in flight per thread
+            const int it = i0 + q * (RF_THREADS / 32), line = it / ng, j = 32 * (it - line * ng) + lane;
+            b[q] = it < items && j < nz ? __ldcs(B + base + (size_t)line * nz + j) : make_double2(0.0, 0.0);
         }
 #pragma unroll
-        for (int q = 0; q < RF_NPT; ++q) {
-            const int k = k0 + q * RF_THREADS;
-            if (k < N) {
+        for (int q = 0; q < NPT; ++q) {
+            const int it = i0 + q * (RF_THREADS / 32), line = it / ng, grp = it - line * ng, j = 32 * grp + lane;
+            if (it >= items) break;   // (uniform in the warp)
+            const bool on = j < nz;
+            float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (on) {
+                const size_t k = base + (size_t)line * nz + j;
                 double2 v2 = b[q];
                 if (conj) v2.y = -v2.y;
-                float4 v;
                 split_double_int(v2.x, v.x, v.z);   // the FP64 split's bits, from integer operations
                 split_double_int(v2.y, v.y, v.w);
-                bd[base + k] = v;
-                r32[base + k] = make_float2(v.x, v.y);
+                bd[k] = v;
+                r32[k] = make_float2(v.x, v.y);
                 // (the zeros of point sources skip the FP64 arithmetic, tested on the bits)
                 if (((ps_bits64(v2.x) | ps_bits64(v2.y)) << 1) != 0) bb += v2.x * v2.x + v2.y * v2.y;
             }
+            group_max(rv, make_float2(v.x, v.y), on,
+                      (((size_t)(c / nrhs) * g.nx + line) * ng + grp) * nrhs + c % nrhs, lane);
         }
         bb = block_sum(bb, sh);
         if (threadIdx.x == 0) {
@@ -213,9 +237,10 @@ __device__ void refine_stop_test(int cols, int nrhs, double *norms, RefineStop s
     }
 }
 
-// grid: (node blocks of RF_THREADS * RF_NPT, columns); norms[col][0] pre-zeroed, norms[col][1] = ||b||^2
+// grid: (blocks of 8 * NPT groups, columns); norms[col][0] pre-zeroed, norms[col][1] = ||b||^2
 // (the arrays are distinct: __restrict__ lets the loads of later nodes move above the stores of
 // earlier ones, so that several nodes' loads are in flight)
+template <int NPT>
 __global__ void __launch_bounds__(RF_THREADS) refine_update_kernel(GridGeom g, int nrhs, int cols,
                                                                    const float4 *__restrict__ diag2,
                                                                    const float4 *__restrict__ bd,
@@ -223,12 +248,14 @@ __global__ void __launch_bounds__(RF_THREADS) refine_update_kernel(GridGeom g, i
                                                                    const float2 *__restrict__ delta,
                                                                    float4 *__restrict__ x_out, float2 *__restrict__ r32,
                                                                    double *norms, StencilPairs cp,
-                                                                   RefineState *state, RefineStop stop) {
+                                                                   RefineState *state, RefineStop stop, RefineVec rv,
+                                                                   const int *solve_status) {
     __shared__ float shf[RF_THREADS / 32];
     __shared__ int s_last;
     __shared__ double shd[32];
     if (state && state->done) return;   // the refinement has stopped: later passes do nothing
-    const int nx = g.nx, nz = g.nz, N = nx * nz;
+    const int nx = g.nx, nz = g.nz, N = nx * nz, ng = (nz + 31) >> 5, items = nx * ng;
+    const int lane = threadIdx.x & 31, i0 = blockIdx.x * (RF_THREADS / 32) * NPT + (threadIdx.x >> 5);
     const int *sysflags = state ? refine_sys(state) : nullptr;
     for (int c = blockIdx.y; c < cols; c += gridDim.y) {
         const int sys = c / nrhs;
@@ -244,28 +271,33 @@ __global__ void __launch_bounds__(RF_THREADS) refine_update_kernel(GridGeom g, i
         const size_t base = (size_t)c * N;
         const float4 *__restrict__ xc = x_in ? x_in + base : nullptr;
         const float2 *__restrict__ dc = delta + base;
-        const int k0 = blockIdx.x * RF_THREADS * RF_NPT + threadIdx.x;
-#pragma unroll 4
-        for (int q = 0; q < RF_NPT; ++q) {
-            const int k = k0 + q * RF_THREADS;
-            if (k >= N) break;
-            const int i = k / nz, j = k % nz;
-            const cff xk = iterate_at(xc, dc, k);
-            cff sx = {{0.f, 0.f}, {0.f, 0.f}}, sz = sx;
-            if (i > 0) sx = cff_add(sx, iterate_at(xc, dc, k - nz));
-            if (i < nx - 1) sx = cff_add(sx, iterate_at(xc, dc, k + nz));
-            if (j > 0) sz = cff_add(sz, iterate_at(xc, dc, k - 1));
-            if (j < nz - 1) sz = cff_add(sz, iterate_at(xc, dc, k + 1));
-            const ff cxj = (j == 0 || j == nz - 1) ? cp.cx_edge : cp.cx_in;
-            const ff czi = (i == 0 || i == nx - 1) ? cp.cz_edge : cp.cz_in;
-            cff ax = cff_mul(cff_of(diag2[(size_t)sys * N + k]), xk);
-            ax = cff_add(ax, cff_scale(sx, cxj));
-            ax = cff_add(ax, cff_scale(sz, czi));
-            const cff r = cff_sub(cff_of(__ldcs(bd + base + k)), ax);
-            x_out[base + k] = cff_pack(xk);
-            r32[base + k] = make_float2(r.re.hi, r.im.hi);
-            const float sr = r.re.hi * scale, si = r.im.hi * scale;
-            rr = fmaf(sr, sr, fmaf(si, si, rr));
+#pragma unroll (NPT < 4 ? NPT : 4)
+        for (int q = 0; q < NPT; ++q) {
+            const int it = i0 + q * (RF_THREADS / 32), i = it / ng, grp = it - i * ng, j = 32 * grp + lane;
+            if (it >= items) break;   // (uniform in the warp)
+            const bool on = j < nz;
+            float2 rf = make_float2(0.f, 0.f);
+            if (on) {
+                const int k = i * nz + j;
+                const cff xk = iterate_at(xc, dc, k);
+                cff sx = {{0.f, 0.f}, {0.f, 0.f}}, sz = sx;
+                if (i > 0) sx = cff_add(sx, iterate_at(xc, dc, k - nz));
+                if (i < nx - 1) sx = cff_add(sx, iterate_at(xc, dc, k + nz));
+                if (j > 0) sz = cff_add(sz, iterate_at(xc, dc, k - 1));
+                if (j < nz - 1) sz = cff_add(sz, iterate_at(xc, dc, k + 1));
+                const ff cxj = (j == 0 || j == nz - 1) ? cp.cx_edge : cp.cx_in;
+                const ff czi = (i == 0 || i == nx - 1) ? cp.cz_edge : cp.cz_in;
+                cff ax = cff_mul(cff_of(diag2[(size_t)sys * N + k]), xk);
+                ax = cff_add(ax, cff_scale(sx, cxj));
+                ax = cff_add(ax, cff_scale(sz, czi));
+                const cff r = cff_sub(cff_of(__ldcs(bd + base + k)), ax);
+                x_out[base + k] = cff_pack(xk);
+                rf = make_float2(r.re.hi, r.im.hi);
+                r32[base + k] = rf;
+                const float sr = r.re.hi * scale, si = r.im.hi * scale;
+                rr = fmaf(sr, sr, fmaf(si, si, rr));
+            }
+            group_max(rv, rf, on, (((size_t)sys * nx + i) * ng + grp) * nrhs + (c - sys * nrhs), lane);
         }
         rr = block_sum(rr, shf);
         if (threadIdx.x == 0) atomicAdd(norms + 2 * (size_t)c, ldexp((double)rr, 2 * ks));
@@ -280,7 +312,11 @@ __global__ void __launch_bounds__(RF_THREADS) refine_update_kernel(GridGeom g, i
         if (s_last) {
             __threadfence();
             refine_stop_test(cols, nrhs, norms, stop, state, shd);
-            if (threadIdx.x == 0) state->blocks = 0;
+            if (threadIdx.x == 0) {
+                state->blocks = 0;
+                state->status = *solve_status;
+            }
+            for (int e = threadIdx.x; rv.ctl && e < rv.n_ctl; e += RF_THREADS) rv.ctl[e] = 0u;
         }
     }
 }
@@ -336,24 +372,38 @@ cudaError_t launch_split_diag(size_t n, const double2 *diag, float4 *diag2, cuda
     return cudaGetLastError();
 }
 
-cudaError_t launch_refine_start(const GridGeom &g, int cols, const double2 *B, int conj, float4 *bd, float2 *r32,
-                                double *norms, cudaStream_t st) {
-    const int N = g.nx * g.nz;
-    cudaError_t e = cudaMemsetAsync(norms, 0, (size_t)cols * 2 * sizeof(double), st);
-    if (e != cudaSuccess) return e;
-    dim3 grid((N + RF_THREADS * RF_NPT - 1) / (RF_THREADS * RF_NPT), std::min(cols, 65535));
-    HELM_TRACED(K_REFSTART, st, (refine_start_kernel<<<grid, RF_THREADS, 0, st>>>(N, cols, B, conj, bd, r32, norms)));
+// groups per thread of the per-column kernels: 8 where that still gives several blocks per SM,
+// else 2 (128^2 with 48 columns: 384 blocks of 8 took 27 us an update, 1536 of 2 are below 20)
+static int refine_npt(const GridGeom &g, int cols) {
+    const long long items = (long long)g.nx * ((g.nz + 31) / 32);
+    return (items + 63) / 64 * cols >= 8 * 152 ? 8 : 2;
+}
+static dim3 refine_grid(const GridGeom &g, int cols, int npt) {
+    const int items = g.nx * ((g.nz + 31) / 32), per = RF_THREADS / 32 * npt;
+    return dim3((items + per - 1) / per, std::min(cols, 65535));
+}
+
+cudaError_t launch_refine_start(const GridGeom &g, int n_sys, int nrhs, const double2 *B, int conj, float4 *bd, float2 *r32,
+                                double *norms, float *gmax, unsigned *ctl, int n_ctl, cudaStream_t st) {
+    const int cols = n_sys * nrhs, npt = refine_npt(g, cols);
+    const dim3 grid = refine_grid(g, cols, npt);
+    const RefineVec rv{gmax, ctl, n_ctl};
+    HELM_TRACED(K_REFSTART, st, ((npt == 8 ? refine_start_kernel<8> : refine_start_kernel<2>)<<<grid, RF_THREADS, 0, st>>>(
+                                    g, nrhs, cols, B, conj, bd, r32, norms, rv)));
     return cudaGetLastError();
 }
 
 cudaError_t launch_refine_update(const GridGeom &g, int n_sys, int nrhs, const float4 *diag2, const float4 *bd,
                                  const float4 *x_in, const float2 *delta, float4 *x_out, float2 *r32, double *norms,
-                                 cudaStream_t st, RefineState *state, RefineStop stop) {
-    const int N = g.nx * g.nz, cols = n_sys * nrhs;
+                                 float *gmax, unsigned *ctl, int n_ctl, const int *solve_status, cudaStream_t st,
+                                 RefineState *state, RefineStop stop) {
+    const int cols = n_sys * nrhs, npt = refine_npt(g, cols);
+    const dim3 grid = refine_grid(g, cols, npt);
+    const RefineVec rv{gmax, ctl, n_ctl};
     StencilPairs cp{pair_of(coup_x(g, 1)), pair_of(coup_x(g, 0)), pair_of(coup_z(g, 1)), pair_of(coup_z(g, 0))};
-    dim3 grid((N + RF_THREADS * RF_NPT - 1) / (RF_THREADS * RF_NPT), std::min(cols, 65535));
-    HELM_TRACED(K_REFUPDATE, st, (refine_update_kernel<<<grid, RF_THREADS, 0, st>>>(g, nrhs, cols, diag2, bd, x_in, delta,
-                                                                                    x_out, r32, norms, cp, state, stop)));
+    HELM_TRACED(K_REFUPDATE, st, ((npt == 8 ? refine_update_kernel<8> : refine_update_kernel<2>)<<<grid, RF_THREADS, 0, st>>>(
+                                     g, nrhs, cols, diag2, bd, x_in, delta, x_out, r32, norms, cp, state, stop, rv,
+                                     solve_status)));
     return cudaGetLastError();
 }
 

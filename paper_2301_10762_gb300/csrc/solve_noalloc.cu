@@ -150,12 +150,18 @@ extern "C" helm_status helm_solve_noalloc(helm_factor_t *f, int32_t nrhs, const 
         w.y = (float2 *)(p + 3 * p_bytes + v_bytes);
         w.norms = (double *)(p + 3 * p_bytes + 2 * v_bytes);
         w.norms_host = g_norms_host;
-        w.state = (RefineState *)(p + 3 * p_bytes + 2 * v_bytes + n_bytes);
+        w.state = (RefineState *)(w.norms + 2 * cols);
         w.maxima = f->bcr.gsmall;   // (every call within the limits above fits it)
-        if ((s = mixed_refine(f, nrhs, B, X, conj, rtol, max_iter, w, &it, &rel)) != HELM_OK) return s;
+        bool timed_out = false;
+        if ((s = mixed_refine(f, nrhs, B, X, conj, rtol, max_iter, w, &it, &rel, &timed_out)) != HELM_OK) return s;
+        if (timed_out) {
+            if (info) { info->iters = it; info->max_relres = rel; }
+            helm_set_msg("a sweep kernel gave up waiting for its cluster");
+            return HELM_ETIMEOUT;
+        }
     }
     if (info) { info->iters = it; info->max_relres = rel; }
-    if ((s = read_sweep_status(op)) != HELM_OK) return s;
+    if (!mixed && (s = read_sweep_status(op)) != HELM_OK) return s;
     if (mixed && !(rel <= rtol)) { helm_set_msg("refinement did not reach rtol"); return HELM_ENOCONV; }
     return HELM_OK;
 }
