@@ -314,6 +314,75 @@ __device__ void polish_inverse16(const float2 *M, int ld, int kb, float2 *P, flo
     __syncthreads();
 }
 
+// 1 / x in FP64 to the last bit or two: the FP32 reciprocal and two Newton steps.  (The FP64 pipe
+// issues a warp instruction in 16 to 64 cycles here, so the division's thirty dependent ones cost
+// a pivot column more than the column itself.)  Outside FP32's comfortable range: __drcp_rn.
+__device__ __forceinline__ double fast_recip(double x) {
+    const float xf = (float)x;
+    if (!(xf > 1e-30f && xf < 1e30f)) return __drcp_rn(x);
+    double y = (double)__frcp_rn(xf);
+    y = fma(y, fma(-x, y, 1.0), y);
+    return fma(y, fma(-x, y, 1.0), y);
+}
+
+// FP64 inverse of the kb x kb block M (shared, row stride ld; the rest of the 16 x 16 tile taken as
+// the identity) into P (row stride NB) by the 256 threads of the CTA, thread (r, c) holding one
+// entry: Gauss-Jordan in place with partial pivoting, A (16 x 17) and B ping-pong, two barriers a
+// column.  Bounds: about 1100 cycles a column, half of them the FP64 pipe (8 instructions of every
+// warp at 2 lanes a cycle).  One warp holding the block in registers took 270 us a block (the
+// 128^2 factor 163 ms for three frequencies): half a lane a cycle, sixteen columns of eight
+// dependent instructions each per step.  False (CTA-wide) if a pivot was zero or not finite.
+__device__ bool cta_invert16(const double2 *M, int ld, int kb, double2 *P, double2 (*A)[NB + 1], double2 (*B)[NB + 1],
+                             int *s_piv) {
+    const int tid = threadIdx.x, r = tid >> 4, c = tid & 15, lane = tid & 31;
+    A[r][c] = (r < kb && c < kb) ? M[(size_t)r * ld + c] : make_double2(r == c ? 1.0 : 0.0, 0.0);
+    __syncthreads();
+    bool ok = true;
+    double2(*S)[NB + 1] = A, (*D)[NB + 1] = B;
+    for (int q = 0; q < NB; ++q) {
+        // every warp finds the pivot of column q by itself: largest modulus among rows q .. 15 (its
+        // FP32 bits with the row in the low four, as warp_invert16)
+        const double2 v = S[lane & 15][q];
+        const float vx = (float)v.x, vy = (float)v.y;
+        const bool cand = (lane & 15) >= q;
+        if (__any_sync(0xffffffffu, cand && !(isfinite(v.x) && isfinite(v.y)))) ok = false;
+        const float mag = fminf(vx * vx + vy * vy, 3.0e38f);
+        const unsigned key = cand ? ((__float_as_uint(mag) & ~0xFu) | (unsigned)(15 - (lane & 15))) : 0u;
+        const unsigned best = __reduce_max_sync(0xffffffffu, key);
+        const int p = 15 - (int)(best & 0xFu);
+        if ((best >> 4) == 0u || (best >> 23) >= 255u) ok = false;
+        if (tid == 0) s_piv[q] = p;
+        const double2 pv = S[p][q], pr = S[p][c];
+        const double rd = ok ? fast_recip(pv.x * pv.x + pv.y * pv.y) : 1.0;
+        const double2 inv = make_double2(pv.x * rd, -pv.y * rd);
+        const int src = r == q ? p : (r == p ? q : r);   // rows p and q change places
+        const double2 f = S[src][q];
+        double2 o;
+        if (r == q) {
+            o = c == q ? inv : cmul(pr, inv);
+        } else {
+            const double2 g = cmul(f, inv);   // column q: -f / pivot; elsewhere a - (f / pivot) pr
+            o = c == q ? make_double2(0.0, 0.0) : S[src][c];
+            cfms(o, g, c == q ? make_double2(1.0, 0.0) : pr);
+        }
+        D[r][c] = o;
+        __syncthreads();
+        double2(*t)[NB + 1] = S;
+        S = D;
+        D = t;
+    }
+    // the row exchanges q <-> p of the steps, undone as column exchanges in reverse order
+    int col = c;
+    for (int q = NB - 1; q >= 0; --q) {
+        const int p = s_piv[q];
+        col = col == q ? p : (col == p ? q : col);
+    }
+    // (column c of the result moves to `col`)
+    if (r < kb && col < kb) P[r * NB + col] = S[r][c];
+    __syncthreads();
+    return ok;
+}
+
 // max |I - M X| over the kb x kb block (M shared with row stride ld, X row stride NB), the rest
 // of the 16 x 16 tile taken as the identity; every thread of the 256-thread CTA returns it.
 template <typename T>
@@ -445,6 +514,9 @@ __global__ void __launch_bounds__(FAC_THREADS, 1) line_factor_smem_kernel(Factor
     __shared__ float s_nsred[FAC_THREADS / 32];
     // flagged pivot blocks: the FP32 entries and the FP64 inverse
     __shared__ __align__(16) double2 s_d64[kNS ? 2 : 1][kNS ? NB * NB : 1];
+    // FP64: work blocks of the pivot inversion
+    __shared__ __align__(16) double2 s_pa[kNS ? 1 : NB][NB + 1], s_pb[kNS ? 1 : NB][NB + 1];
+    __shared__ int s_piv[NB];
 
     V *Gs = a.G + (size_t)sys * nx * nz * nz;
     const double2 *dg = a.diag + (size_t)sys * nx * nz;
@@ -566,6 +638,10 @@ __global__ void __launch_bounds__(FAC_THREADS, 1) line_factor_smem_kernel(Factor
                         if (slot > 0 && kb == NB && bpc <= kSeedBlocks)
                             done = ns_invert16<T>(sW + (size_t)k0 * ldw + kc, ldw, s_seed[kl], recvP, s_nsM, s_nsX,
                                                   s_nsE, s_nsred);
+                    }
+                    if constexpr (!kNS) {
+                        if (!cta_invert16(sW + (size_t)k0 * ldw + kc, ldw, kb, recvP, s_pa, s_pb, s_piv) && tid == 0) s_bad = 1;
+                        done = true;
                     }
                     if (!done) {
                         if (tid < 32) {
@@ -756,10 +832,19 @@ int pick_cluster_size(int nz) {
 template <typename T>
 cudaError_t launch_line_factor(const GridGeom &g, int n_sys, const double2 *diag, cx_t<T> *G, cx_t<T> *xch,
                                int *status, int cs, cudaStream_t st, int *mid_out) {
-    const size_t smem_res = factor_smem_resident_bytes<T>(g.nz, cs);
-    const bool resident = smem_res <= 200 * 1024;
+    constexpr size_t kResidentMax = 216 * 1024;   // + up to 9 KB of static shared memory
     int teams = 1;
     cudaError_t e;
+    // a slab of eight CTAs that does not fit (FP64 from n_z = 200): one team of sixteen, one-sided,
+    // instead of the kernel with its panels in global memory (256^2, FP64: 990 ms)
+    if (cs == 8 && factor_smem_resident_bytes<T>(g.nz, cs) > kResidentMax &&
+        factor_smem_resident_bytes<T>(g.nz, 16) <= kResidentMax) {
+        const size_t s16 = factor_smem_resident_bytes<T>(g.nz, 16);
+        if ((e = ensure_dyn_smem((const void *)line_factor_smem_kernel<T>, s16)) != cudaSuccess) return e;
+        if (max_active_clusters((const void *)line_factor_smem_kernel<T>, 16, FAC_THREADS, s16) > 0) cs = 16;
+    }
+    const size_t smem_res = factor_smem_resident_bytes<T>(g.nz, cs);
+    const bool resident = smem_res <= kResidentMax;
     // HELM_FACTOR_TEAMS=1 forces the one-sided factorisation (for comparisons)
     const char *force = getenv("HELM_FACTOR_TEAMS");
     const bool allow_twisted = !(force && force[0] == '1');

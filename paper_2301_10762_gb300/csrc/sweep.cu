@@ -135,20 +135,22 @@ __device__ __forceinline__ int step_line(int s, int nx) { return s < nx ? s : 2 
 // (system, line, row tile, right-hand-side chunk).  b is the input in the working precision
 // (conjugated for the adjoint FP64 solve).  The CUDA-core sweep uses it; the tensor-path sweep
 // takes b_i into its own product instead.
-constexpr int PP_ROWS = 64;    // rows of G_i per CTA
 constexpr int PP_RHS = 16;     // right-hand sides per CTA
 constexpr int PP_KC = 32;      // K chunk
-// Register-blocked batched product: each thread computes 2 rows x 4 right-hand sides (64 rows
+// Register-blocked batched product: each thread computes RT rows x 4 right-hand sides (32 RT rows
 // x 16 right-hand sides per CTA of 128 threads), so every two shared loads of G feed eight
-// complex MACs.  A warp shares its right-hand sides (broadcast reads) and takes rows tr and
-// tr + 32, whose padded stride keeps the G reads free of bank conflicts.
-template <typename TG>
+// complex MACs at RT = 2.  A warp shares its right-hand sides (broadcast reads; a warp without any
+// skips the products) and takes rows tr, tr + 32, whose padded stride keeps the G reads free of
+// bank conflicts.  FP64 takes RT = 1: its pipe is the bound (2 lanes a cycle per SM), so more CTAs
+// count for more than reuse (64^2, 8 right-hand sides: 64 CTAs of RT = 2 took 78 us).
+template <typename TG, int RT>
 __global__ void __launch_bounds__(128) line_gb_prepass_kernel(GridGeom g, int nrhs, const cx_t<TG> *G,
                                                              const cx_t<TG> *B, cx_t<TG> *Y, int conj,
                                                              const int *skip, const int *frozen) {
     using V = cx_t<TG>;
     if (skip && *skip) return;
     const int nx = g.nx, nz = g.nz, N = nx * nz;
+    constexpr int PP_ROWS = 32 * RT;   // rows of G_i per CTA
     const int n_rt = (nz + PP_ROWS - 1) / PP_ROWS;
     const int n_ch = (nrhs + PP_RHS - 1) / PP_RHS;
     int bid = blockIdx.x;
@@ -166,9 +168,9 @@ __global__ void __launch_bounds__(128) line_gb_prepass_kernel(GridGeom g, int nr
     const int tr = tid & 31, tq = tid >> 5;    // rows tr, tr + 32; right-hand sides 4 tq .. 4 tq + 3
     const V *Bs = B + ((size_t)sys * nrhs + q0) * N + (size_t)i * nz;
     const V *Gi = G + ((size_t)sys * nx + i) * nz * nz + (size_t)r0 * nz;
-    V acc[2][4];
+    V acc[RT][4];
 #pragma unroll
-    for (int a2 = 0; a2 < 2; ++a2)
+    for (int a2 = 0; a2 < RT; ++a2)
 #pragma unroll
         for (int b2 = 0; b2 < 4; ++b2) acc[a2][b2] = mkc<TG>(TG(0), TG(0));
     for (int kc = 0; kc < nz; kc += PP_KC) {
@@ -186,21 +188,25 @@ __global__ void __launch_bounds__(128) line_gb_prepass_kernel(GridGeom g, int nr
             for (int j = lane; j < PP_KC; j += 32)
                 sg[r][j] = (r < nrows && j < kw) ? Gi[(size_t)r * nz + kc + j] : mkc<TG>(TG(0), TG(0));
         __syncthreads();
+        if (4 * tq < Rc) {
 #pragma unroll 4
-        for (int k = 0; k < PP_KC; ++k) {
-            const V g0 = sg[tr][k], g1 = sg[tr + 32][k];
+            for (int k = 0; k < PP_KC; ++k) {
+                V gk[RT];
 #pragma unroll
-            for (int b2 = 0; b2 < 4; ++b2) {
-                const V bb = sb[4 * tq + b2][k];
-                cfma(acc[0][b2], g0, bb);
-                cfma(acc[1][b2], g1, bb);
+                for (int a2 = 0; a2 < RT; ++a2) gk[a2] = sg[tr + 32 * a2][k];
+#pragma unroll
+                for (int b2 = 0; b2 < 4; ++b2) {
+                    const V bb = sb[4 * tq + b2][k];
+#pragma unroll
+                    for (int a2 = 0; a2 < RT; ++a2) cfma(acc[a2][b2], gk[a2], bb);
+                }
             }
         }
         __syncthreads();
     }
     V *Ys = Y + ((size_t)sys * nrhs + q0) * N + (size_t)i * nz + r0;
 #pragma unroll
-    for (int a2 = 0; a2 < 2; ++a2)
+    for (int a2 = 0; a2 < RT; ++a2)
 #pragma unroll
         for (int b2 = 0; b2 < 4; ++b2) {
             const int r = tr + 32 * a2, q = 4 * tq + b2;
@@ -848,6 +854,30 @@ cudaError_t launch_line_sweep(const GridGeom &g, int n_sys, int nrhs, const cx_t
     const int teams = (mid < g.nx - 1) ? 2 : 1;
     int cs = nz / 16;
     cs = cs < 1 ? 1 : (cs > 16 / teams ? 16 / teams : cs);
+    // FP64: the products, not the exchange, are the length of a step (2 lanes a cycle per SM: 8 us of
+    // a 10 us step at 64 rows x 8 right-hand sides on 4 CTAs).  CTAs per team and right-hand sides
+    // per cluster are taken for the least time of (waves of clusters) x (products of a step + about
+    // 3500 cycles of exchange), the line product's 2 multiply-adds of 2 lanes per entry.  64^2 with 8
+    // right-hand sides: 649 -> 278 us.
+    const bool fp64 = sizeof(TG) == 8;
+    int fp64_R = 0;
+    if (fp64 && nz >= 48) {   // (shorter lines are bound by the exchange: 40 x 37 ran 210 us as it was, 249 spread out)
+        double best = 0.0;
+        const int cs0 = cs;
+        for (int c = cs0; c <= 16 / teams; c = c < 8 && 2 * c > 8 ? 8 : 2 * c) {
+            const int csz = teams * c, rp = (nz + c - 1) / c;
+            for (int r = 1; r <= std::min(16, nrhs); ++r) {
+                if (rp * r > 128) break;   // (128 outputs per CTA measured best)
+                // (shared memory at the widest padding, in steps of 32 KB: few distinct queries)
+                const size_t need = 32 + vsz * (size_t)(nz + 8) * (5 * r + 2 * rp) + vsz * 2 * (size_t)r * rp;
+                const int act = std::max(1, max_active_clusters((const void *)line_sweep_kernel<TG, 0, 0, false>, csz, SW_THREADS,
+                                                                std::min(SW_SMEM_MAX, (need + 32767) / 32768 * 32768)));
+                const long waves = ((long)n_sys * ((nrhs + r - 1) / r) + act - 1) / act;
+                const double t = (double)waves * (2.0 * rp * r * nz + 3500.0);
+                if (fp64_R == 0 || t < best) { best = t; cs = c; fp64_R = r; }
+            }
+        }
+    }
     // tuning overrides: CTAs per team and right-hand sides per cluster
     const char *env_cs = getenv("HELM_SWEEP_CS"), *env_r = getenv("HELM_SWEEP_R");
     if (env_cs && atoi(env_cs) > 0) cs = std::min(atoi(env_cs), 16 / teams);
@@ -876,6 +906,7 @@ cudaError_t launch_line_sweep(const GridGeom &g, int n_sys, int nrhs, const cx_t
         int R = 1;
         while (R * 2 <= 16 && rpc * R * 2 <= 128) R *= 2;
         if (rchunk > 0 && R > rchunk) R = rchunk;
+        if (fp64 && fp64_R > 0) R = fp64_R;
         if (env_r && atoi(env_r) > 0) R = atoi(env_r);
         if (R > nrhs) R = nrhs;
         if (R < 1) R = 1;
@@ -935,8 +966,9 @@ cudaError_t launch_line_sweep(const GridGeom &g, int n_sys, int nrhs, const cx_t
             }
         }
         if (!mma) {   // CUDA-core sweep: Y_i = G_i b_i for all lines first
-            const long blocks = (long)n_sys * g.nx * ((nz + PP_ROWS - 1) / PP_ROWS) * ((nrhs + PP_RHS - 1) / PP_RHS);
-            HELM_TRACED(K_GBPRE, st, (line_gb_prepass_kernel<TG><<<(unsigned)blocks, 128, 0, st>>>(g, nrhs, G, B, Y, conj, skip, frozen)));
+            constexpr int RT = sizeof(TG) == 8 ? 1 : 2;
+            const long blocks = (long)n_sys * g.nx * ((nz + 32 * RT - 1) / (32 * RT)) * ((nrhs + PP_RHS - 1) / PP_RHS);
+            HELM_TRACED(K_GBPRE, st, (line_gb_prepass_kernel<TG, RT><<<(unsigned)blocks, 128, 0, st>>>(g, nrhs, G, B, Y, conj, skip, frozen)));
             e = cudaGetLastError();
             if (e != cudaSuccess) return e;
         }
