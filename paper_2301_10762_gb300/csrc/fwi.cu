@@ -339,50 +339,161 @@ __global__ void regR_kernel(GridGeom g, const double *v, double *out) {
 
 // ------------------------------------------------------ P2^{-1} by the 2D DCT-II
 // R = (nx-1)^2 L_nx (x) I + (nz-1)^2 I (x) L_nz with L_n the path-graph Laplacian,
-// which the orthonormal DCT-II C_n (C_n[a][j] = s_a cos(pi a (2j+1) / (2n))) diagonalises:
-// L_n = C_n^T diag(2 - 2 cos(pi a / n)) C_n.  Hence
-//   P2^{-1} r = (C_x (x) C_z)^T diag(1 / (alpha0 lam_ab + mu)) (C_x (x) C_z) r,
-// i.e. with r as the nx x nz matrix of the canonical order: C_x^T ((C_x r C_z^T) ./ L) C_z.
-__global__ void dct_matrix_kernel(int n, double *Cm, double *lam) {
-    const int e = blockIdx.x * blockDim.x + threadIdx.x;
-    if (e < n * n) {
-        const int a = e / n, j = e % n;
-        const double s = (a == 0) ? sqrt(1.0 / n) : sqrt(2.0 / n);
-        Cm[e] = s * cospi((double)a * (2 * j + 1) / (2.0 * n));
-    }
-    if (e < n) lam[e] = 2.0 - 2.0 * cospi((double)e / n);
+// which the orthonormal DCT-II C_n (C_n[a][j] = s_a cos(pi a (2j+1) / (2n)), s_0^2 = 1/n, else 2/n)
+// diagonalises: L_n = C_n^T diag(2 - 2 cos(pi a / n)) C_n.  Hence
+//   P2^{-1} r = (C_x (x) C_z)^T diag(1 / (alpha0 lam_ab + mu)) (C_x (x) C_z) r
+// in three passes: every line's transform along z; every column's transform along x, the division
+// (with all s_a^2) and the transform back; every line's transform back along z.  The products are
+// bound by the FP64 pipe (2 lanes a cycle per SM), so
+//   - C is not formed: its entries are n + 1 cosines cos(pi k / (2n)) up to sign, one table per
+//     direction, indexed by a (2j + 1) mod 4n (integer work, free beside FP64);
+//   - the symmetry C[a][n-1-j] = (-1)^a C[a][j] halves the multiply-adds: a line is folded into its
+//     even and odd parts first, or the even and odd sums are unfolded after;
+//   - a CTA per line (column) puts 128 of them on a 128^2 problem.
+// 128^2, one vector: 102 us a call with the matrices formed (2 launches) and four tiled products and
+// a scaling (5 launches), 2 n^3 multiply-adds each; three passes and the table now.
+__global__ void dct_table_kernel(int nx, int nz, double *tx, double *tz) {
+    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k <= nx) tx[k] = cospi((double)k / (2.0 * nx));
+    else if (k - nx - 1 <= nz) tz[k - nx - 1] = cospi((double)(k - nx - 1) / (2.0 * nz));
 }
 
-__global__ void p2_scale_kernel(int nx, int nz, const double *lx, const double *lz, double alpha0, double mu,
-                                double *T) {
-    const int e = blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= nx * nz) return;
-    const int a = e / nz, b = e % nz;
+constexpr int DCT_THREADS = 256;
+// +-T[.] = cos(pi idx / (2n)), 0 <= idx < 4n, times v
+__device__ __forceinline__ double cos_fma(const double *T, int n, int idx, double v, double acc) {
+    int k = idx > 2 * n ? 4 * n - idx : idx;
+    const bool neg = k > n;
+    k = neg ? 2 * n - k : k;
+    return fma(neg ? -v : v, T[k], acc);
+}
+// threads that share an output (adjacent lanes, a power of two)
+__device__ __forceinline__ int dct_parts(int outputs) {
+    int s = 1;
+    while (s < 8 && 2 * s * outputs <= 2 * DCT_THREADS) s *= 2;
+    return s;
+}
+// out(a, sum_j cos(pi a (2j+1) / (2n)) v_j) for every a, v folded: F[j] = v_j + v_{n-1-j} for even a,
+// F[h + j] = v_j - v_{n-1-j} for odd a, h = (n + 1) / 2 (the middle of an odd n once, and 0)
+template <typename Out> __device__ void dct_forward(const double *T, int n, const double *F, Out out) {
+    const int h = (n + 1) / 2, S = dct_parts(n), part = threadIdx.x % S;
+    const int rounds = (n * S + DCT_THREADS - 1) / DCT_THREADS;
+    for (int q = 0; q < rounds; ++q) {   // (uniform trip count: the shuffles need whole warps)
+        const int a = (q * DCT_THREADS + (int)threadIdx.x) / S;
+        double acc = 0.0, acc1 = 0.0;
+        if (a < n) {
+            const double *v = F + (a & 1) * h;
+            const int step = (int)((2ll * a * S) % (4 * n));
+            int idx = (int)(((long long)a * (2 * part + 1)) % (4 * n));
+            int j = part;
+            for (; j + S < h; j += 2 * S) {
+                acc = cos_fma(T, n, idx, v[j], acc);
+                idx += step;
+                if (idx >= 4 * n) idx -= 4 * n;
+                acc1 = cos_fma(T, n, idx, v[j + S], acc1);
+                idx += step;
+                if (idx >= 4 * n) idx -= 4 * n;
+            }
+            if (j < h) acc = cos_fma(T, n, idx, v[j], acc);
+            acc += acc1;
+        }
+        for (int o = 1; o < S; o *= 2) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+        if (a < n && part == 0) out(a, acc);
+    }
+}
+// out(j, sum_a cos(pi a (2j+1) / (2n)) t_a) for every j: the even and the odd a apart
+template <typename Out> __device__ void dct_backward(const double *T, int n, const double *t, Out out) {
+    const int h = (n + 1) / 2, S = dct_parts(h), part = threadIdx.x % S;
+    const int rounds = (h * S + DCT_THREADS - 1) / DCT_THREADS;
+    for (int q = 0; q < rounds; ++q) {
+        const int j = (q * DCT_THREADS + (int)threadIdx.x) / S;
+        double ev = 0.0, od = 0.0;
+        if (j < h) {
+            const int w = 2 * j + 1, step2 = (int)((2ll * w * S) % (4 * n));
+            int ie = (int)((2ll * part * w) % (4 * n)), io = (int)(((2ll * part + 1) * w) % (4 * n));
+            for (int a = 2 * part; a < n; a += 2 * S) {
+                ev = cos_fma(T, n, ie, t[a], ev);
+                ie += step2;
+                if (ie >= 4 * n) ie -= 4 * n;
+                if (a + 1 < n) od = cos_fma(T, n, io, t[a + 1], od);
+                io += step2;
+                if (io >= 4 * n) io -= 4 * n;
+            }
+        }
+        for (int o = 1; o < S; o *= 2) {
+            ev += __shfl_xor_sync(0xffffffffu, ev, o);
+            od += __shfl_xor_sync(0xffffffffu, od, o);
+        }
+        if (j < h && part == 0) {
+            out(j, ev + od);
+            if (n - 1 - j != j) out(n - 1 - j, ev - od);
+        }
+    }
+}
+// F of dct_forward from v_j = in[j * stride]
+__device__ __forceinline__ void dct_fold(int n, const double *in, size_t stride, double *F) {
+    const int h = (n + 1) / 2;
+    for (int j = threadIdx.x; j < h; j += DCT_THREADS) {
+        const double u = in[(size_t)j * stride];
+        const bool mid = n - 1 - j == j;
+        const double v = mid ? 0.0 : in[(size_t)(n - 1 - j) * stride];
+        F[j] = u + v;
+        F[h + j] = mid ? 0.0 : u - v;
+    }
+}
+// Scratch of a CTA: the table (n + 1) and two vectors of n + 1, in shared memory, or (big: lines of
+// more than DCT_SMEM_N nodes) the vectors in global memory at big + 2 (n + 1) * CTA and the table
+// where it is
+constexpr int DCT_SMEM_N = 6000;
+struct DctBuf {
+    const double *T;
+    double *u, *v;
+};
+__device__ __forceinline__ DctBuf dct_buf(int n, const double *table, double *big, double *smem) {
+    if (big) {
+        double *p = big + 2 * (size_t)(n + 1) * (blockIdx.x + (size_t)gridDim.x * blockIdx.y);
+        return DctBuf{table, p, p + n + 1};
+    }
+    for (int k = threadIdx.x; k <= n; k += DCT_THREADS) smem[k] = table[k];
+    return DctBuf{smem, smem + n + 1, smem + 2 * (n + 1)};
+}
+
+// z transforms of the lines (blockIdx.x) of the vectors (blockIdx.y): out = in C_z^T without s_b, or
+// (back) in C_z without s_b
+__global__ void __launch_bounds__(DCT_THREADS) dct_lines_kernel(int nx, int nz, const double *tz, int back, const double *in,
+                                                                double *out, double *big) {
+    extern __shared__ double dct_smem[];
+    const size_t off = ((size_t)blockIdx.y * nx + blockIdx.x) * nz;
+    const DctBuf b = dct_buf(nz, tz, big, dct_smem);
+    double *o = out + off;
+    if (back) {
+        for (int k = threadIdx.x; k < nz; k += DCT_THREADS) b.u[k] = in[off + k];
+        __syncthreads();
+        dct_backward(b.T, nz, b.u, [&](int j, double x) { o[j] = x; });
+    } else {
+        dct_fold(nz, in + off, 1, b.u);
+        __syncthreads();
+        dct_forward(b.T, nz, b.u, [&](int a, double x) { o[a] = x; });
+    }
+}
+
+// x transforms, the division and the transforms back of the columns (blockIdx.x), in place
+__global__ void __launch_bounds__(DCT_THREADS) dct_columns_kernel(int nx, int nz, const double *tx, const double *tz,
+                                                                  double alpha0, double mu, double *T1, double *big) {
+    extern __shared__ double dct_smem[];
+    double *col = T1 + (size_t)blockIdx.y * nx * nz + blockIdx.x;
+    const DctBuf b = dct_buf(nx, tx, big, dct_smem);
+    dct_fold(nx, col, nz, b.u);
+    __syncthreads();
+    const int e = blockIdx.x;
     const double sx = (double)(nx - 1) * (nx - 1), sz = (double)(nz - 1) * (nz - 1);
-    T[e] = T[e] / (alpha0 * (sx * lx[a] + sz * lz[b]) + mu);
-}
-
-// C[i][j] = sum_k A(i, k) B(k, j), A(i,k) = A[i*as0 + k*as1], B(k,j) = B[k*bs0 + j*bs1],
-// C row-major M x N.  DT x DT tiles in shared memory, FP64, k summed in ascending order.  The
-// small tiles give a 128 x 128 product 256 blocks, enough to occupy the FP64 units of every SM
-// (GB300's FP64 rate per SM is low).
-constexpr int DT = 8;
-__global__ void dgemm_strided_kernel(int M, int Nn, int K, const double *A, int as0, int as1, const double *B,
-                                     int bs0, int bs1, double *Cout) {
-    __shared__ double sA[DT][DT + 1], sB[DT][DT + 1];
-    const int tx = threadIdx.x % DT, ty = threadIdx.x / DT;
-    const int i = blockIdx.y * DT + ty, j = blockIdx.x * DT + tx;
-    double acc = 0.0;
-    for (int k0 = 0; k0 < K; k0 += DT) {
-        const int ka = k0 + tx, kb = k0 + ty;
-        sA[ty][tx] = (i < M && ka < K) ? A[(size_t)i * as0 + (size_t)ka * as1] : 0.0;
-        sB[ty][tx] = (kb < K && j < Nn) ? B[(size_t)kb * bs0 + (size_t)j * bs1] : 0.0;
-        __syncthreads();
-#pragma unroll
-        for (int t = 0; t < DT; ++t) acc = fma(sA[ty][t], sB[t][tx], acc);
-        __syncthreads();
-    }
-    if (i < M && j < Nn) Cout[(size_t)i * Nn + j] = acc;
+    const double lz = sz * (2.0 - 2.0 * cos_fma(tz, nz, 2 * e, 1.0, 0.0));
+    const double s2 = (e == 0 ? 1.0 : 2.0) / nz;
+    dct_forward(b.T, nx, b.u, [&](int a, double x) {
+        const double lx = sx * (2.0 - 2.0 * cos_fma(b.T, nx, 2 * a, 1.0, 0.0));
+        b.v[a] = x * (s2 * (a == 0 ? 1.0 : 2.0)) / (nx * (alpha0 * (lx + lz) + mu));
+    });
+    __syncthreads();
+    dct_backward(b.T, nx, b.v, [&](int j, double x) { col[(size_t)j * nz] = x; });
 }
 
 }  // namespace helm
@@ -477,45 +588,39 @@ struct Dotter {
     }
 };
 
-// P2^{-1} by the DCT (see dct_matrix_kernel)
+// P2^{-1} by the DCT (see dct_table_kernel), up to `batch` vectors at a time
 struct P2Solver {
-    int nx = 0, nz = 0;
+    int nx = 0, nz = 0, batch = 1;
     double alpha0 = 0, mu = 0;
-    double *Cx = nullptr, *Cz = nullptr, *lx = nullptr, *lz = nullptr, *T1 = nullptr, *T2 = nullptr;
-    helm_status init(Ws &ws, const GridGeom &g, double a0, double m0, cudaStream_t st) {
+    double *tx = nullptr, *tz = nullptr, *T1 = nullptr, *big_z = nullptr, *big_x = nullptr;
+    helm_status init(Ws &ws, const GridGeom &g, double a0, double m0, cudaStream_t st, int n_batch = 1) {
         nx = g.nx;
         nz = g.nz;
         alpha0 = a0;
         mu = m0;
+        batch = n_batch;
         helm_status s = HELM_OK;
-        Cx = ws.get<double>((size_t)nx * nx, &s);
-        Cz = ws.get<double>((size_t)nz * nz, &s);
-        lx = ws.get<double>(nx, &s);
-        lz = ws.get<double>(nz, &s);
-        T1 = ws.get<double>((size_t)nx * nz, &s);
-        T2 = ws.get<double>((size_t)nx * nz, &s);
+        tx = ws.get<double>((size_t)nx + nz + 2, &s);
+        T1 = ws.get<double>((size_t)nx * nz * batch, &s);
+        if (nz > DCT_SMEM_N) big_z = ws.get<double>(2 * ((size_t)nz + 1) * nx * batch, &s);
+        if (nx > DCT_SMEM_N) big_x = ws.get<double>(2 * ((size_t)nx + 1) * nz * batch, &s);
         if (s != HELM_OK) return s;
-        HELM_TRACED(K_DCTMAT, st, (dct_matrix_kernel<<<nblk((size_t)nx * nx), 256, 0, st>>>(nx, Cx, lx)));
-        HL();
-        HELM_TRACED(K_DCTMAT, st, (dct_matrix_kernel<<<nblk((size_t)nz * nz), 256, 0, st>>>(nz, Cz, lz)));
+        tz = tx + nx + 1;
+        if (smem(nz) > 48 * 1024) HK(ensure_dyn_smem((const void *)dct_lines_kernel, smem(nz)));
+        if (smem(nx) > 48 * 1024) HK(ensure_dyn_smem((const void *)dct_columns_kernel, smem(nx)));
+        HELM_TRACED(K_DCTMAT, st, (dct_table_kernel<<<nblk((size_t)nx + nz + 2, 32), 32, 0, st>>>(nx, nz, tx, tz)));
         HL();
         return HELM_OK;
     }
-    static void gemm(int M, int Nn, int K, const double *A, int as0, int as1, const double *B, int bs0, int bs1,
-                     double *C, cudaStream_t st) {
-        dim3 grid((Nn + DT - 1) / DT, (M + DT - 1) / DT);
-        HELM_TRACED(K_DGEMM, st, (dgemm_strided_kernel<<<grid, DT * DT, 0, st>>>(M, Nn, K, A, as0, as1, B, bs0, bs1, C)));
-    }
-    helm_status apply(const double *r, double *out, cudaStream_t st) {
-        // T1 = Cx r          (nx x nx)(nx x nz)
-        gemm(nx, nz, nx, Cx, nx, 1, r, nz, 1, T1, st);
-        // T2 = T1 Cz^T       (nx x nz)(nz x nz)^T
-        gemm(nx, nz, nz, T1, nz, 1, Cz, 1, nz, T2, st);
-        HELM_TRACED(K_P2SCALE, st, (p2_scale_kernel<<<nblk((size_t)nx * nz), 256, 0, st>>>(nx, nz, lx, lz, alpha0, mu, T2)));
-        // T1 = Cx^T T2
-        gemm(nx, nz, nx, Cx, 1, nx, T2, nz, 1, T1, st);
-        // out = T1 Cz
-        gemm(nx, nz, nz, T1, nz, 1, Cz, nz, 1, out, st);
+    static size_t smem(int n) { return n > DCT_SMEM_N ? 0 : 3 * ((size_t)n + 1) * sizeof(double); }
+    // out may be r
+    helm_status apply(const double *r, double *out, cudaStream_t st, int count = 1) {
+        HELM_TRACED(K_DGEMM, st, (dct_lines_kernel<<<dim3(nx, count), DCT_THREADS, smem(nz), st>>>(nx, nz, tz, 0, r, T1, big_z)));
+        HL();
+        HELM_TRACED(K_DGEMM, st, (dct_columns_kernel<<<dim3(nz, count), DCT_THREADS, smem(nx), st>>>(nx, nz, tx, tz, alpha0, mu,
+                                                                                                    T1, big_x)));
+        HL();
+        HELM_TRACED(K_DGEMM, st, (dct_lines_kernel<<<dim3(nx, count), DCT_THREADS, smem(nz), st>>>(nx, nz, tz, 1, T1, out, big_z)));
         HL();
         return HELM_OK;
     }
@@ -660,8 +765,10 @@ extern "C" helm_status helm_gamma_solve(const helm_grid *grid, double alpha0, do
     {
         Ws ws(st);
         P2Solver p2;
-        s = p2.init(ws, g, alpha0, mu, st);
-        for (int32_t c = 0; s == HELM_OK && c < ncol; ++c) s = p2.apply(R_dev + c * N, Z_dev + c * N, st);
+        const int batch = std::min<int32_t>(ncol, 16);
+        s = p2.init(ws, g, alpha0, mu, st, batch);
+        for (int32_t c = 0; s == HELM_OK && c < ncol; c += batch)
+            s = p2.apply(R_dev + c * N, Z_dev + c * N, st, std::min<int32_t>(batch, ncol - c));
         if (s == HELM_OK) {
             const cudaError_t e = cudaStreamSynchronize(st);
             if (e != cudaSuccess) { helm_set_error("helm_gamma_solve", e); s = HELM_ECUDA; }
