@@ -95,25 +95,23 @@ __global__ void bcr_form_kernel(GridGeom g, Coup cp, const double2 *diag, float2
 }
 
 // level 0 (couplings C = diag(cx)): kept line k (even) with eliminated neighbours k - 1, k + 1:
-//   D_k -= C Dinv_{k-1} C + C Dinv_{k+1} C,  L_k = -C Dinv_{k-1} C,  U_k = -C Dinv_{k+1} C
+//   D_k -= C Dinv_{k-1} C + C Dinv_{k+1} C
+// (its couplings, -C Dinv C of either neighbour, are written as images of the inverses)
 // implicit (diag != nullptr): D_k is not in memory yet and is taken from A's diagonal and the
 // line's vertical coupling (the tridiagonal line block) before the update
-__global__ void bcr_level0_kernel(GridGeom g, Coup cp, float2 *D, const float2 *Dinv, float2 *Lnew, float2 *Unew,
-                                  int half, const double2 *diag) {
+__global__ void bcr_level0_kernel(GridGeom g, Coup cp, float2 *D, const double2 *diag) {
     const int nz = g.nz, nx = g.nx, nz2 = nz * nz;
     const int k = 2 * blockIdx.y, s = blockIdx.z;
     const bool ha = k >= 1, hc = k + 1 < nx;
-    const float2 *Da = Dinv + ((size_t)s * nx + (ha ? k - 1 : 0)) * nz2;
-    const float2 *Dc = Dinv + ((size_t)s * nx + (hc ? k + 1 : 0)) * nz2;
+    const float2 *Da = D + ((size_t)s * nx + (ha ? k - 1 : 0)) * nz2;
+    const float2 *Dc = D + ((size_t)s * nx + (hc ? k + 1 : 0)) * nz2;
     float2 *Dk = D + ((size_t)s * nx + k) * nz2;
-    float2 *Lk = Lnew + ((size_t)s * half + k / 2) * nz2;
-    float2 *Uk = Unew + ((size_t)s * half + k / 2) * nz2;
     for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < nz2; e += gridDim.x * blockDim.x) {
         const int r = e / nz, c = e - r * nz;
         const float sc = cp.cx(r, nz) * cp.cx(c, nz);
-        float2 ta = make_float2(0.f, 0.f), tc = ta;
-        if (ha) { const float2 v = Da[e]; ta = make_float2(sc * v.x, sc * v.y); }
-        if (hc) { const float2 v = Dc[e]; tc = make_float2(sc * v.x, sc * v.y); }
+        float2 t = make_float2(0.f, 0.f);
+        if (ha) { const float2 v = Da[e]; t = make_float2(sc * v.x, sc * v.y); }
+        if (hc) { const float2 v = Dc[e]; t.x += sc * v.x; t.y += sc * v.y; }
         float2 d;
         if (diag) {
             const float cz = cp.cz(k, nx);
@@ -122,11 +120,7 @@ __global__ void bcr_level0_kernel(GridGeom g, Coup cp, float2 *D, const float2 *
         } else {
             d = Dk[e];
         }
-        d.x -= ta.x + tc.x;
-        d.y -= ta.y + tc.y;
-        Dk[e] = d;
-        if (k >= 2) Lk[e] = make_float2(-ta.x, -ta.y);
-        if (k + 2 < nx) Uk[e] = make_float2(-tc.x, -tc.y);
+        Dk[e] = make_float2(d.x - t.x, d.y - t.y);
     }
 }
 
@@ -756,19 +750,34 @@ helm_status invert_tridiag_blocks(int n, Fam in, Fam out, const std::vector<int>
     return HELM_OK;
 }
 
-// images (bcr_solve.cu) of the blocks base + pairs[.][0] * n^2 as matrices pairs[.][1], and of their
-// transposes as matrices tdst[.] (empty: none)
-helm_status image_blocks(int n, const float2 *base, const std::vector<int> &pairs, const std::vector<int> &tdst,
-                         const BcrData &b, uint32_t *mx, Plan &pl) {
+// images (bcr_solve.cu) of the inverses in slots pairs[.][0] of D as matrices pairs[.][1], and of
+// their level-0 couplings as matrices mdst[.] (empty: none)
+helm_status image_blocks(const GridGeom &g, const float2 *D, const std::vector<int> &pairs, const std::vector<int> &mdst,
+                         const BgArgs &ba, Plan &pl) {
     if (pairs.empty()) return HELM_OK;
-    const int off = pl.add(pairs), toff = tdst.empty() ? -1 : pl.add(tdst), count = (int)(pairs.size() / 2);
+    const int off = pl.add(pairs), moff = mdst.empty() ? -1 : pl.add(mdst), count = (int)(pairs.size() / 2);
     const cudaStream_t st = pl.st;
-    unsigned char *img = b.img;
-    int *shift = b.shift;
+    const Coup cp = coup_of(g);
+    const int n = g.nz;
     pl.ops.push_back([=](const int *dev) -> helm_status {
-        const cudaError_t e = launch_bcr_image(n, base, (long long)n * n, dev + off, toff < 0 ? nullptr : dev + toff, count,
-                                               img, mx, shift, st);
+        const cudaError_t e = launch_bcr_image(n, D, (long long)n * n, dev + off, moff < 0 ? nullptr : dev + moff, count,
+                                               cp.cx_in, cp.cx_edge, ba.im, st);
         if (e != cudaSuccess) { helm_set_error("bcr: images", e); return HELM_ECUDA; }
+        return HELM_OK;
+    });
+    return HELM_OK;
+}
+
+// products of images (bcr_gemm.cu), one launch
+helm_status image_gemm(const BgArgs &ba, const std::vector<int> &tasks, Plan &pl) {
+    if (tasks.empty()) return HELM_OK;
+    const int off = pl.add(tasks), n = (int)(tasks.size() / BG_TASK);
+    const cudaStream_t st = pl.st;
+    pl.ops.push_back([=](const int *dev) -> helm_status {
+        BgArgs a = ba;
+        a.tasks = dev + off;
+        const cudaError_t e = launch_bcr_gemm(a, n, st);
+        if (e != cudaSuccess) { helm_set_error("bcr: block products", e); return HELM_ECUDA; }
         return HELM_OK;
     });
     return HELM_OK;
@@ -790,41 +799,57 @@ helm_status bcr_factor(helm_factor_t *f) {
     BcrData &b = f->bcr;
     b.half = half;
     helm_status s;
-    const size_t blk = (size_t)nz2 * sizeof(float2);
-    // kept: the image of every line's inverse and of W, V, P, Q of the lines eliminated at levels >= 1
-    const size_t n_mat = (size_t)ns * (nx + 4 * (size_t)half);
+    // Images (bcr_solve.h), one family of matrices.  Kept: every line's inverse, and W, V, P, Q of
+    // the lines eliminated at levels >= 1.  Working: the couplings.  At level 0 both couplings
+    // through an odd line j are M_j = -C Dinv_j C (slot j / 2); above, U_k (to the next line of the
+    // spacing) and L_k = U_{k - sp}^T, ping-pong by level.
+    const size_t n_kept = (size_t)ns * (nx + 4 * (size_t)half);
+    const int m_stride = half, eighth = nx / 8 + 1;
+    const size_t m0 = n_kept, u0 = m0 + (size_t)ns * m_stride;
+    const size_t n_mat = u0 + 2 * (size_t)ns * (quart + eighth);
+    const int u_stride[2] = {quart, eighth};
+    auto u_base = [&](int buf, int which) {   // first matrix of U (which = 0) or L (1) of a buffer
+        return u0 + (size_t)ns * (buf == 0 ? which * quart : 2 * quart + which * eighth);
+    };
     const BsLayout lay = bs_layout(nz);
-    if ((s = dev_alloc((void **)&b.img, n_mat * lay.mat_bytes, "bcr: blocks", st)) != HELM_OK ||
+    if ((s = dev_alloc((void **)&b.img, n_kept * lay.mat_bytes, "bcr: blocks", st)) != HELM_OK ||
         (s = dev_alloc((void **)&b.shift, n_mat * sizeof(int), "bcr: scales", st)) != HELM_OK ||
         (s = dev_alloc((void **)&b.gsmall, kSmallMaxima * sizeof(float), "bcr: maxima", st)) != HELM_OK)
         return s;
-    // working blocks of the reduction: diagonal blocks (an eliminated line's is inverted in place),
-    // couplings L, U (ping-pong: line k of spacing sp at index k / sp), W and V of one level
-    float2 *D = nullptr, *LU[2][2] = {{nullptr, nullptr}, {nullptr, nullptr}}, *W = nullptr, *V = nullptr;
+    // working arrays: the working images and the diagonal blocks (an eliminated line's is inverted in
+    // place), FP32
+    float2 *D = nullptr;
+    BsImages im;
     struct Work {
-        float2 **p[7];
+        float2 **d;
+        BsImages *im;
         cudaStream_t st;
-        ~Work() { for (auto q : p) dev_free(*q, st); }
-    } work{{&D, &LU[0][0], &LU[0][1], &LU[1][0], &LU[1][1], &W, &V}, st};
-    if ((s = dev_alloc((void **)&D, (size_t)ns * nx * blk, "bcr: work", st)) != HELM_OK ||
-        (s = dev_alloc((void **)&LU[0][0], (size_t)ns * half * blk, "bcr: work", st)) != HELM_OK ||
-        (s = dev_alloc((void **)&LU[0][1], (size_t)ns * half * blk, "bcr: work", st)) != HELM_OK ||
-        (s = dev_alloc((void **)&LU[1][0], (size_t)ns * quart * blk, "bcr: work", st)) != HELM_OK ||
-        (s = dev_alloc((void **)&LU[1][1], (size_t)ns * quart * blk, "bcr: work", st)) != HELM_OK ||
-        (s = dev_alloc((void **)&W, (size_t)ns * quart * blk, "bcr: work", st)) != HELM_OK ||
-        (s = dev_alloc((void **)&V, (size_t)ns * quart * blk, "bcr: work", st)) != HELM_OK)
+        ~Work() {
+            dev_free(*d, st);
+            dev_free(im->work, st);
+            dev_free(im->mx, st);
+        }
+    } work{&D, &im, st};
+    im.kept = b.img;
+    im.n_kept = (int)n_kept;
+    im.shift = b.shift;
+    if ((s = dev_alloc((void **)&D, (size_t)ns * nx * nz2 * sizeof(float2), "bcr: work", st)) != HELM_OK ||
+        (s = dev_alloc((void **)&im.work, (n_mat - n_kept) * lay.mat_bytes, "bcr: work", st)) != HELM_OK ||
+        (s = dev_alloc((void **)&im.mx, n_mat * sizeof(uint32_t), "bcr: maxima", st)) != HELM_OK)
         return s;
-    const int lu_stride[2] = {half, quart};
     cudaError_t e;
-    Plan pl(st);
-    if ((s = pl.with_split(kFactorSplitElems)) != HELM_OK) return s;
-    uint32_t *mx = nullptr;   // largest moduli of the blocks, for their scales
-    if ((s = dev_alloc((void **)&mx, n_mat * sizeof(uint32_t), "bcr: maxima", st)) != HELM_OK) return s;
-    pl.scratch.push_back(mx);
-    if ((e = cudaMemsetAsync(mx, 0, n_mat * sizeof(uint32_t), st)) != cudaSuccess) {
+    if ((e = cudaMemsetAsync(im.mx, 0, n_mat * sizeof(uint32_t), st)) != cudaSuccess) {
         helm_set_error("bcr: maxima", e);
         return HELM_ECUDA;
     }
+    BgArgs ba{};
+    ba.nz = nz;
+    ba.im = im;
+    ba.D = D;
+    ba.status = op->status;
+    ba.tries = wait_tries();
+    Plan pl(st);
+    if ((s = pl.with_split(kFactorSplitElems)) != HELM_OK) return s;
     const int per = (int)std::min<long long>(64, (nz2 + 255) / 256);
     // n_z <= 256: no line block is formed in memory before level 0, which inverts the odd lines'
     // tridiagonal blocks and updates the even lines' straight from A's diagonal and couplings
@@ -850,108 +875,82 @@ helm_status bcr_factor(helm_factor_t *f) {
     }
     const Fam fD{D, nz2, nz};
     auto mat = [&](int kind, int sy, int slot) { return (int)bs_matrix_index(nx, ns, half, kind << 24 | slot, sy); };
-    int cur = 0, levels = 0;   // L, U of the current spacing in LU[cur]
+    int cur = 1, levels = 0;   // U, L of the spacing in buffer cur (from level 2 on)
     for (int sp = 1; sp < nx; sp *= 2, ++levels) {
-        std::vector<int> inv_pairs, tv, tw, td, tl, tu;
+        std::vector<int> inv_pairs, img_pairs, mdst;
         for (int sy = 0; sy < ns; ++sy)
-            for (int j = sp; j < nx; j += 2 * sp) inv_pairs.insert(inv_pairs.end(), {sy * nx + j, sy * nx + j});
+            for (int j = sp; j < nx; j += 2 * sp) {
+                inv_pairs.insert(inv_pairs.end(), {sy * nx + j, sy * nx + j});
+                img_pairs.insert(img_pairs.end(), {sy * nx + j, mat(BS_DINV, sy, j)});
+                if (sp == 1) mdst.push_back((int)m0 + sy * m_stride + j / 2);
+            }
         // level 0: the line blocks are still tridiagonal
         s = (sp == 1 && tri_level0) ? invert_tridiag_blocks(nz, fD, fD, inv_pairs, op->status, pl, tri)
                                     : invert_blocks(nz, fD, fD, inv_pairs, op->status, pl);
         if (s != HELM_OK) return s;
+        if ((s = image_blocks(g, D, img_pairs, mdst, ba, pl)) != HELM_OK) return s;
         if (sp == 1) {
-            float2 *D0 = D, *L1 = LU[0][0], *U1 = LU[0][1];
+            float2 *D0 = D;
             const Coup cp = coup_of(g);
             pl.ops.push_back([=](const int *) -> helm_status {
-                HELM_TRACED(K_BCR_L0, st, (bcr_level0_kernel<<<dim3(per, (nx + 1) / 2, ns), 256, 0, st>>>(
-                                              g, cp, D0, D0, L1, U1, half, tri_diag)));
+                HELM_TRACED(K_BCR_L0, st, (bcr_level0_kernel<<<dim3(per, (nx + 1) / 2, ns), 256, 0, st>>>(g, cp, D0, tri_diag)));
                 const cudaError_t e2 = cudaGetLastError();
                 if (e2 != cudaSuccess) { helm_set_error("bcr: level 0", e2); return HELM_ECUDA; }
                 return HELM_OK;
             });
-            continue;   // (level 0 writes LU[0], which stays current)
+            continue;
         }
-        const int nxt = cur ^ 1, cs = lu_stride[cur], nsd = lu_stride[nxt];
-        std::vector<int> vi, vt, wi, wt;   // images of V, P = V^T, W, Q = W^T
+        const int nxt = cur ^ 1;
+        // couplings of line k to its neighbours at distance sp
+        auto Uc = [&](int sy, int k) { return sp == 2 ? (int)m0 + sy * m_stride + k / 2 : (int)u_base(cur, 0) + sy * u_stride[cur] + k / sp; };
+        auto Lc = [&](int sy, int k) { return sp == 2 ? (int)m0 + sy * m_stride + k / 2 - 1 : (int)u_base(cur, 1) + sy * u_stride[cur] + k / sp; };
+        auto Un = [&](int sy, int k) { return (int)u_base(nxt, 0) + sy * u_stride[nxt] + k / (2 * sp); };
+        auto Ln = [&](int sy, int k) { return (int)u_base(nxt, 1) + sy * u_stride[nxt] + k / (2 * sp); };
+        std::vector<int> t1, t2, t3;   // V, P, W, Q; the new couplings and D -= L W^T; D -= U V^T
+        auto add = [](std::vector<int> &t, int flags, int ia, int ib, int out) { t.insert(t.end(), {flags, ia, ib, out}); };
         for (int sy = 0; sy < ns; ++sy) {
-            const int cb = sy * cs, nb = sy * nsd, lb = sy * nx, qb = sy * quart;
             for (int j = sp; j < nx; j += 2 * sp) {
-                const int i = (j - sp) / (2 * sp);
-                // V_j = U_{j-s} Dinv_j;  W_j = L_{j+s} Dinv_j
-                auto v = task8(cb + (j - sp) / sp, lb + j, 0, qb + i);
-                tv.insert(tv.end(), v.begin(), v.end());
-                vi.insert(vi.end(), {qb + i, mat(BS_V, sy, j / 2)});
-                vt.push_back(mat(BS_P, sy, j / 2));
+                const int di = mat(BS_DINV, sy, j), u = Uc(sy, j - sp);
+                add(t1, 0, u, di, mat(BS_V, sy, j / 2));    // V_j = U_{j-s} Dinv_j
+                add(t1, 0, di, u, mat(BS_P, sy, j / 2));    // P_j = V_j^T (Dinv_j is symmetric)
                 if (j + sp < nx) {
-                    auto w = task8(cb + (j + sp) / sp, lb + j, 0, qb + i);
-                    tw.insert(tw.end(), w.begin(), w.end());
-                    wi.insert(wi.end(), {qb + i, mat(BS_W, sy, j / 2)});
-                    wt.push_back(mat(BS_Q, sy, j / 2));
+                    const int l = Lc(sy, j + sp);
+                    add(t1, 0, l, di, mat(BS_W, sy, j / 2));   // W_j = L_{j+s} Dinv_j
+                    add(t1, 0, di, l, mat(BS_Q, sy, j / 2));
                 }
             }
             for (int k = 0; k < nx; k += 2 * sp) {
-                const bool ha = k >= sp, hc = k + sp < nx;
-                if (!ha && !hc) continue;
-                const int ck = cb + k / sp, nk = nb + k / (2 * sp), ia = qb + k / (2 * sp) - 1, ic = qb + k / (2 * sp);
-                // D_k -= L_k W_a^T + U_k V_c^T
-                auto d = task8(ha ? ck : -1, ha ? ia : 0, lb + k, lb + k, hc ? ck : -1, hc ? ic : 0);
-                td.insert(td.end(), d.begin(), d.end());
-                if (k >= 2 * sp) {   // L_k <- -L_k V_a^T
-                    auto l = task8(ck, ia, 0, nk);
-                    tl.insert(tl.end(), l.begin(), l.end());
-                }
-                if (k + 2 * sp < nx) {   // U_k <- -U_k W_c^T
-                    auto u = task8(ck, ic, 0, nk);
-                    tu.insert(tu.end(), u.begin(), u.end());
-                }
+                const int a = k - sp, c = k + sp;
+                if (a >= 0) add(t2, BG_FP32 | BG_NEG, Lc(sy, k), mat(BS_W, sy, a / 2), sy * nx + k);   // D_k -= L_k W_a^T
+                if (c < nx) add(t3, BG_FP32 | BG_NEG, Uc(sy, k), mat(BS_V, sy, c / 2), sy * nx + k);   // D_k -= U_k V_c^T
+                if (k >= 2 * sp) add(t2, BG_NEG, Lc(sy, k), mat(BS_V, sy, a / 2), Ln(sy, k));          // L_k <- -L_k V_a^T
+                if (k + 2 * sp < nx) add(t2, BG_NEG, Uc(sy, k), mat(BS_W, sy, c / 2), Un(sy, k));      // U_k <- -U_k W_c^T
             }
         }
-        float2 *Lc = LU[cur][0], *Uc = LU[cur][1], *Ln = LU[nxt][0], *Un = LU[nxt][1];
-        ZGemmArgs ga;
-        ga.M = ga.N = ga.K = nz;
-        ga.status = op->status;
-        ga.nterms = 1;
-        ga.B[0] = zop(D, nz2, nz);
-        ga.C = V; ga.c_stride = nz2; ga.ldc = nz;
-        ga.A[0] = zop(Uc, nz2, nz);
-        if ((s = gemm(ga, tv, pl)) != HELM_OK) return s;
-        ga.C = W;
-        ga.A[0] = zop(Lc, nz2, nz);
-        if ((s = gemm(ga, tw, pl)) != HELM_OK) return s;
-        if ((s = image_blocks(nz, V, vi, vt, b, mx, pl)) != HELM_OK || (s = image_blocks(nz, W, wi, wt, b, mx, pl)) != HELM_OK)
-            return s;
-        ZGemmArgs gd;
-        gd.M = gd.N = gd.K = nz;
-        gd.status = op->status;
-        gd.nterms = 2;
-        gd.A[0] = zop(Lc, nz2, nz); gd.B[0] = zop(W, nz2, nz); gd.sign[0] = -1.f;
-        gd.A[1] = zop(Uc, nz2, nz); gd.B[1] = zop(V, nz2, nz); gd.sign[1] = -1.f;
-        gd.C0 = zop(D, nz2, nz);
-        gd.C = D; gd.c_stride = nz2; gd.ldc = nz;
-        if ((s = gemm(gd, td, pl)) != HELM_OK) return s;
-        ZGemmArgs gl;
-        gl.M = gl.N = gl.K = nz;
-        gl.status = op->status;
-        gl.nterms = 1;
-        gl.sign[0] = -1.f;
-        gl.A[0] = zop(Lc, nz2, nz); gl.B[0] = zop(V, nz2, nz);
-        gl.C = Ln; gl.c_stride = nz2; gl.ldc = nz;
-        if ((s = gemm(gl, tl, pl)) != HELM_OK) return s;
-        gl.A[0] = zop(Uc, nz2, nz); gl.B[0] = zop(W, nz2, nz);
-        gl.C = Un;
-        if ((s = gemm(gl, tu, pl)) != HELM_OK) return s;
+        uint32_t *mxn = im.mx + u_base(nxt, 0);
+        const size_t mxb = 2 * (size_t)ns * u_stride[nxt] * sizeof(uint32_t);
+        if ((s = image_gemm(ba, t1, pl)) != HELM_OK) return s;
+        pl.ops.push_back([=](const int *) -> helm_status {   // (the buffer's maxima of two levels ago)
+            const cudaError_t e2 = cudaMemsetAsync(mxn, 0, mxb, st);
+            if (e2 != cudaSuccess) { helm_set_error("bcr: maxima", e2); return HELM_ECUDA; }
+            return HELM_OK;
+        });
+        if ((s = image_gemm(ba, t2, pl)) != HELM_OK || (s = image_gemm(ba, t3, pl)) != HELM_OK) return s;
         cur = nxt;
     }
-    // the last line left: line 0; then every line's inverse is in its slot of D
+    // the last line left: line 0
     {
-        std::vector<int> last, di;
-        for (int sy = 0; sy < ns; ++sy) last.insert(last.end(), {sy * nx, sy * nx});
+        std::vector<int> last, img_pairs;
+        for (int sy = 0; sy < ns; ++sy) {
+            last.insert(last.end(), {sy * nx, sy * nx});
+            img_pairs.insert(img_pairs.end(), {sy * nx, mat(BS_DINV, sy, 0)});
+        }
         if ((s = invert_blocks(nz, fD, fD, last, op->status, pl)) != HELM_OK) return s;
-        for (int i = 0; i < ns * nx; ++i) di.insert(di.end(), {i, i});
-        if ((s = image_blocks(nz, D, di, {}, b, mx, pl)) != HELM_OK) return s;
+        if ((s = image_blocks(g, D, img_pairs, {}, ba, pl)) != HELM_OK) return s;
         int *out = op->status + 2;   // the largest entry of the inverses (the matrices 0 .. ns nx - 1)
+        const uint32_t *mxd = im.mx;
         pl.ops.push_back([=](const int *) -> helm_status {
-            HELM_TRACED(K_BCR_IMAGE, st, (max_words_kernel<<<1, 1024, 0, st>>>((size_t)ns * nx, mx, out)));
+            HELM_TRACED(K_BCR_IMAGE, st, (max_words_kernel<<<1, 1024, 0, st>>>((size_t)ns * nx, mxd, out)));
             const cudaError_t e2 = cudaGetLastError();
             if (e2 != cudaSuccess) { helm_set_error("bcr: maxima", e2); return HELM_ECUDA; }
             return HELM_OK;

@@ -34,12 +34,11 @@
 #include <algorithm>
 
 #include "abi_internal.h"
+#include "bcr_image.cuh"
 #include "bcr_solve.h"
 #include "kernels.h"
 #include "tcgen05.cuh"
 #include "trace.h"
-
-#include <cuda_fp16.h>
 
 namespace helm {
 
@@ -68,35 +67,11 @@ template <int NT> struct BsCfg {
 constexpr int BS_AHEAD = 4, BS_AHEAD0 = 2;   // vector chunks in flight ahead of the one being split
 constexpr int BS_NT_BWD0 = 32;
 
-__device__ __forceinline__ void bulk_load(uint32_t dst, const void *src, uint32_t bytes, uint64_t *bar) {
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
-                 "l"(src), "r"(bytes), "r"(smem_u32(bar))
-                 : "memory");
-}
-__device__ __forceinline__ void mbar_arrive(uint64_t *bar) {
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
-}
 __device__ __forceinline__ unsigned ld_acquire(const unsigned *p) {
     unsigned v;
     asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
     return v;
 }
-__device__ __forceinline__ uint32_t abs_bits(float x) { return __float_as_uint(x) & 0x7fffffffu; }
-
-// shift s with max * 2^s in [2^14, 2^15) (FP16 range), from the bits of the maximum modulus; NaN
-// and infinite maxima get a finite scale and stay NaN or infinite in the split
-__device__ __forceinline__ int scale_shift(uint32_t max_bits) { return min(141 - (int)(max_bits >> 23), 100); }
-__device__ __forceinline__ float pow2(int s) { return __uint_as_float((uint32_t)(127 + s) << 23); }
-
-// (hi, lo) FP16 split of two scaled values, packed
-__device__ __forceinline__ void split_h2(float a, float b, uint32_t &hi, uint32_t &lo) {
-    const __half2 h = __floats2half2_rn(a, b);
-    const float2 f = __half22float2(h);
-    const __half2 l = __floats2half2_rn(a - f.x, b - f.y);
-    hi = *reinterpret_cast<const uint32_t *>(&h);
-    lo = *reinterpret_cast<const uint32_t *>(&l);
-}
-
 struct Tile {
     int phase, sys, task, n0, r0, rows, nt;
 };
@@ -196,7 +171,7 @@ __global__ void __launch_bounds__(BS_THREADS, 1) bcr_solve_kernel(const __grid_c
         if (!wait(&tq_full[i % BS_QD], i / BS_QD)) return -1;
         const int t = tq[i % BS_QD];
         __syncwarp();
-        if (lane == 0) mbar_arrive(&tq_empty[i % BS_QD]);
+        if (lane == 0) mbar_arrive_cta(&tq_empty[i % BS_QD]);
         return t;
     };
 
@@ -235,7 +210,7 @@ __global__ void __launch_bounds__(BS_THREADS, 1) bcr_solve_kernel(const __grid_c
                 }
                 if (!wait1(&tq_empty[i % BS_QD], (uint32_t)((i / BS_QD) & 1) ^ 1u)) break;
                 tq[i % BS_QD] = t;
-                mbar_arrive(&tq_full[i % BS_QD]);
+                mbar_arrive_cta(&tq_full[i % BS_QD]);
                 if (t < 0) break;
                 const Tile tl = decode(a, t);
                 const int *task = a.tasks + 8 * tl.task;
@@ -278,7 +253,7 @@ __global__ void __launch_bounds__(BS_THREADS, 1) bcr_solve_kernel(const __grid_c
             for (int i = 0; go; ++i) {
                 if (!wait1(&tq_full[i % BS_QD], (uint32_t)((i / BS_QD) & 1))) break;
                 const int t = tq[i % BS_QD];
-                mbar_arrive(&tq_empty[i % BS_QD]);
+                mbar_arrive_cta(&tq_empty[i % BS_QD]);
                 if (t < 0) break;
                 const Tile tl = decode(a, t);
                 const int nterms = a.tasks[8 * tl.task + 1] >> 4, nt = tl.nt;
@@ -353,7 +328,7 @@ __global__ void __launch_bounds__(BS_THREADS, 1) bcr_solve_kernel(const __grid_c
             // only what the sum does not hold (FP16 keeps all 22 bits 15 octaves down).
             float sc[PR];
             auto put_scale = [&](int q, int S, int sl) {
-                if (j == 0 && q < np) s_bscale[sl][row0 + 16 * q] = pow2(max(-126, min(126, -S)));
+                if (j == 0 && q < np) s_bscale[sl][row0 + 16 * q] = bs_pow2(max(-126, min(126, -S)));
             };
             const int sl = tt % SL;
             // split and store one chunk's pairs into stage s
@@ -366,10 +341,10 @@ __global__ void __launch_bounds__(BS_THREADS, 1) bcr_solve_kernel(const __grid_c
                         const int r = row0 + 16 * q;
                         const uint32_t in16 = (uint32_t)(j & 3) * 4;
                         const uint32_t oh = sw128(r, j >> 2) + in16, ol = sw128(r, 4 + (j >> 2)) + in16;
-                        split_h2(v[q].x * sc[q], v[q].z * sc[q], hi, lo);
+                        bs_split2(v[q].x * sc[q], v[q].z * sc[q], hi, lo);
                         asm volatile("st.shared.b32 [%0], %1;" ::"r"(br + oh), "r"(hi) : "memory");
                         asm volatile("st.shared.b32 [%0], %1;" ::"r"(br + ol), "r"(lo) : "memory");
-                        split_h2(v[q].y * sc[q], v[q].w * sc[q], hi, lo);
+                        bs_split2(v[q].y * sc[q], v[q].w * sc[q], hi, lo);
                         asm volatile("st.shared.b32 [%0], %1;" ::"r"(bi + oh), "r"(hi) : "memory");
                         asm volatile("st.shared.b32 [%0], %1;" ::"r"(bi + ol), "r"(lo) : "memory");
                     }
@@ -377,7 +352,7 @@ __global__ void __launch_bounds__(BS_THREADS, 1) bcr_solve_kernel(const __grid_c
                 // (the fence that makes these stores visible to the tensor core stands in the MMA
                 // warp: here it would also wait for every load the warp has in flight)
                 __syncwarp();
-                if (lane == 0) mbar_arrive(&full[s]);
+                if (lane == 0) mbar_arrive_cta(&full[s]);
             };
             // this lane's 16 bytes of row pair q in raw slot e
             auto raw = [&](int e, int q) { return raw0 + (uint32_t)((e * tl.nt + row0 + 16 * q) * 256 + 16 * j); };
@@ -421,8 +396,8 @@ __global__ void __launch_bounds__(BS_THREADS, 1) bcr_solve_kernel(const __grid_c
                     const float bound = __uint_as_float(over_lanes(m3[0][q])) +
                                         fabsf(a.cx_in) * (__uint_as_float(over_lanes(m3[1][q])) +
                                                           __uint_as_float(over_lanes(m3[2][q])));
-                    const int sh = scale_shift(abs_bits(bound));
-                    sc[q] = pow2(sh);
+                    const int sh = bs_scale_shift(bs_abs_bits(bound));
+                    sc[q] = bs_pow2(sh);
                     put_scale(q, sh + sa, sl);
                 }
                 for (int c = 0; c < a.n_chunk; ++c, ++cc) {
@@ -478,7 +453,7 @@ __global__ void __launch_bounds__(BS_THREADS, 1) bcr_solve_kernel(const __grid_c
                 S[q] = 1 << 20;
 #pragma unroll
                 for (int u = 0; u < 3; ++u) {
-                    const int t2 = sa[u] + scale_shift(over_lanes(mx[u][q]));
+                    const int t2 = sa[u] + bs_scale_shift(over_lanes(mx[u][q]));
                     if (u < nterms) S[q] = min(S[q], t2);
                 }
                 put_scale(q, S[q], sl);
@@ -489,7 +464,7 @@ __global__ void __launch_bounds__(BS_THREADS, 1) bcr_solve_kernel(const __grid_c
                 const int su = u == 0 ? sa[0] : (u == 1 ? sa[1] : sa[2]);
 #pragma unroll
                 for (int q = 0; q < PR; ++q) {   // P and Q enter with a minus sign
-                    const float f = pow2(max(-126, min(126, S[q] - su)));
+                    const float f = bs_pow2(max(-126, min(126, S[q] - su)));
                     sc[q] = type == BS_BWD && u > 0 ? -f : f;
                 }
                 for (int c = 0; c < a.n_chunk; ++c, ++cc) {
@@ -574,7 +549,7 @@ __global__ void __launch_bounds__(BS_THREADS, 1) bcr_solve_kernel(const __grid_c
 #pragma unroll
                         for (int e = 0; e < 8; ++e) {
                             if (on && c0 + e < ncol) out[(size_t)(c0 + e) * N] = o[e];
-                            const uint32_t b = on ? max(abs_bits(o[e].x), abs_bits(o[e].y)) : 0u;
+                            const uint32_t b = on ? max(bs_abs_bits(o[e].x), bs_abs_bits(o[e].y)) : 0u;
                             const uint32_t w = __reduce_max_sync(0xffffffffu, b);
                             if (lane == e) gmax = w;
                         }
@@ -585,7 +560,7 @@ __global__ void __launch_bounds__(BS_THREADS, 1) bcr_solve_kernel(const __grid_c
             tc_fence_before();
             __syncwarp();
             if (lane == 0) {
-                mbar_arrive(&acc_empty[sl]);
+                mbar_arrive_cta(&acc_empty[sl]);
                 __threadfence();   // the warp's stores before its count
                 atomicAdd(a.ctl + 2 + tl.phase * a.ns + tl.sys, 1u);
             }
@@ -620,7 +595,7 @@ __global__ void __launch_bounds__(256) line_max_kernel(int nx, int nz, int ng, i
             t[e] = k < nz && b + e < nc ? __ldg(p + (size_t)(b + e) * nx * nz) : make_float2(0.f, 0.f);
 #pragma unroll
         for (int e = 0; e < 8; ++e) {
-            const uint32_t w = __reduce_max_sync(0xffffffffu, max(abs_bits(t[e].x), abs_bits(t[e].y)));
+            const uint32_t w = __reduce_max_sync(0xffffffffu, max(bs_abs_bits(t[e].x), bs_abs_bits(t[e].y)));
             if (lane == b + e) mine = w;
         }
     }
@@ -635,66 +610,68 @@ __global__ void __launch_bounds__(256) bcr_max_kernel(long long n2, const float2
     uint32_t m = 0;
     for (long long e = blockIdx.x * 256 + threadIdx.x; e < n2 / 2; e += (long long)gridDim.x * 256) {
         const float4 v = __ldg(A + e);
-        m = max(max(m, max(abs_bits(v.x), abs_bits(v.y))), max(abs_bits(v.z), abs_bits(v.w)));
+        m = max(max(m, max(bs_abs_bits(v.x), bs_abs_bits(v.y))), max(bs_abs_bits(v.z), bs_abs_bits(v.w)));
     }
     m = __reduce_max_sync(0xffffffffu, m);
     if ((threadIdx.x & 31) == 0) atomicMax(mx + pr[1], m);
 }
 
-// Images of a block (n x n row-major) as matrix dst and, with tdst >= 0, of its transpose as
-// matrix tdst; a CTA takes 32 rows of the block, which are one chunk of columns of the
-// transpose.  Columns beyond n are zero.
-__device__ __forceinline__ void image_row(unsigned char *M, size_t mat_row, size_t im_off, int sw, int j, float sc,
-                                          const float2 (&v)[8]) {
-    // 16-byte piece j of a 128-byte row: hi of eight columns (j < 4), else lo
-    uint4 re, im;
-    uint32_t *pre = reinterpret_cast<uint32_t *>(&re), *pim = reinterpret_cast<uint32_t *>(&im);
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-        uint32_t hi, lo;
-        split_h2(v[2 * e].x * sc, v[2 * e + 1].x * sc, hi, lo);
-        pre[e] = j < 4 ? hi : lo;
-        split_h2(v[2 * e].y * sc, v[2 * e + 1].y * sc, hi, lo);
-        pim[e] = j < 4 ? hi : lo;
-    }
-    unsigned char *d = M + mat_row * 128 + ((j ^ sw) << 4);
-    *reinterpret_cast<uint4 *>(d) = re;
-    *reinterpret_cast<uint4 *>(d + im_off) = im;
-}
-__global__ void __launch_bounds__(256) bcr_image_kernel(int n, int n_chunk, int nzr, const float2 *src, long long stride,
-                                                        const int *pairs, const int *tdst, unsigned char *img,
-                                                        size_t mat_bytes, const uint32_t *mx, int *shift) {
+// Image of a block (n x n row-major) as matrix pairs[.][1]; with mdst, also of -C block C (C =
+// diag(cx), the coupling of a level-0 inverse) as matrix mdst[.].  A CTA takes 32 rows, a thread a
+// row and eight columns at a time; rows and columns beyond n are zero.
+__global__ void __launch_bounds__(128) bcr_image_kernel(int n, int n_chunk, int nzr, const float2 *src, long long stride,
+                                                        const int *pairs, const int *mdst, float cx_in, float cx_edge,
+                                                        BsImages im, size_t mat_bytes) {
     __shared__ float2 t[32][33];
     const int *pr = pairs + 2 * (size_t)blockIdx.y;
     const float2 *A = src + (long long)pr[0] * stride;
     const int r0 = 32 * blockIdx.x, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int sh = scale_shift(mx[pr[1]]);
-    const float sc = pow2(sh);
-    const int td = tdst ? tdst[blockIdx.y] : -1;
+    const uint32_t m0 = im.mx[pr[1]];
+    const int sh = bs_scale_shift(m0), md = mdst ? mdst[blockIdx.y] : -1;
+    const uint32_t m1 = bs_abs_bits(__uint_as_float(m0) * cx_in * cx_in);   // (the edge coupling is half the inner one)
+    const int shm = bs_scale_shift(m1);
+    const float sc = bs_pow2(sh), scm = bs_pow2(shm);
     if (blockIdx.x == 0 && threadIdx.x == 0) {
-        shift[pr[1]] = sh;
-        if (td >= 0) shift[td] = sh;
+        im.shift[pr[1]] = sh;
+        if (md >= 0) {
+            im.shift[md] = shm;
+            im.mx[md] = m1;
+        }
     }
-    unsigned char *M = img + (size_t)pr[1] * mat_bytes, *T = td >= 0 ? img + (size_t)td * mat_bytes : nullptr;
-    const int row = threadIdx.x >> 3, j = threadIdx.x & 7, kb = 8 * (j & 3);
-    const size_t im_off = (size_t)nzr * 128;
+    const int row = threadIdx.x >> 2, j = threadIdx.x & 3, r = r0 + row;
+    const float cr = (r == 0 || r == n - 1) ? cx_edge : cx_in;
+    auto put = [&](int mat, int c, float s, const float2 (&v)[8]) {
+        uint4 rh, rl, ih, il;
+        bs_split8(v, s, rh, rl, ih, il);
+        unsigned char *d = im.at(mat, mat_bytes) + ((size_t)(2 * c) * nzr + r) * 128;
+        *reinterpret_cast<uint4 *>(d + ((j ^ (r & 7)) << 4)) = rh;
+        *reinterpret_cast<uint4 *>(d + (((j + 4) ^ (r & 7)) << 4)) = rl;
+        d += (size_t)nzr * 128;
+        *reinterpret_cast<uint4 *>(d + ((j ^ (r & 7)) << 4)) = ih;
+        *reinterpret_cast<uint4 *>(d + (((j + 4) ^ (r & 7)) << 4)) = il;
+    };
     for (int c = 0; c < n_chunk; ++c) {
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const int o = w + 8 * q, r = r0 + o, k = 32 * c + lane;
-            t[o][lane] = r < n && k < n ? __ldg(A + (long long)r * n + k) : make_float2(0.f, 0.f);
+        for (int q = 0; q < 8; ++q) {
+            const int o = w + 4 * q, k = 32 * c + lane;
+            t[o][lane] = r0 + o < n && k < n ? __ldg(A + (long long)(r0 + o) * n + k) : make_float2(0.f, 0.f);
         }
         __syncthreads();
-        float2 v[8];
-        if (r0 + row < nzr) {
+        if (r < nzr) {
+            float2 v[8];
 #pragma unroll
-            for (int e = 0; e < 8; ++e) v[e] = t[row][kb + e];
-            image_row(M, (size_t)(2 * c) * nzr + r0 + row, im_off, row & 7, j, sc, v);
-        }
-        if (T && 32 * c + row < nzr) {   // row 32 c + row of the transpose, chunk r0 / 32
+            for (int e = 0; e < 8; ++e) v[e] = t[row][8 * j + e];
+            put(pr[1], c, sc, v);
+            if (md >= 0) {
 #pragma unroll
-            for (int e = 0; e < 8; ++e) v[e] = t[kb + e][row];
-            image_row(T, (size_t)(2 * (r0 / 32)) * nzr + 32 * c + row, im_off, row & 7, j, sc, v);
+                for (int e = 0; e < 8; ++e) {
+                    const int k = 32 * c + 8 * j + e;
+                    const float f = -cr * ((k == 0 || k == n - 1) ? cx_edge : cx_in);
+                    v[e].x *= f;
+                    v[e].y *= f;
+                }
+                put(md, c, scm, v);
+            }
         }
         __syncthreads();
     }
@@ -710,18 +687,18 @@ template <int NT> cudaError_t launch_nt(const BsArgs &a, int grid, double flops,
 
 }  // namespace
 
-cudaError_t launch_bcr_image(int n, const float2 *src, long long stride, const int *pairs_dev, const int *tdst_dev,
-                             int count, unsigned char *img, uint32_t *mx, int *shift, cudaStream_t st) {
+cudaError_t launch_bcr_image(int n, const float2 *src, long long stride, const int *pairs_dev, const int *mdst_dev,
+                             int count, float cx_in, float cx_edge, const BsImages &im, cudaStream_t st) {
     if (count <= 0) return cudaSuccess;
     const BsLayout l = bs_layout(n);
     for (int t = 0; t < count; t += 65535) {
         const int nb = std::min(65535, count - t);
         const int *pr = pairs_dev + 2 * (size_t)t;
         HELM_TRACED(K_BCR_IMAGE, st, (bcr_max_kernel<<<dim3((unsigned)std::min(8, (n * n / 2 + 1023) / 1024), nb), 256, 0, st>>>(
-                                         (long long)n * n, src, stride, pr, mx)));
-        HELM_TRACED(K_BCR_IMAGE, st, (bcr_image_kernel<<<dim3((n + 31) / 32, nb), 256, 0, st>>>(
-                                         n, l.n_chunk, l.nzr, src, stride, pr, tdst_dev ? tdst_dev + t : nullptr, img,
-                                         l.mat_bytes, mx, shift)));
+                                         (long long)n * n, src, stride, pr, im.mx)));
+        HELM_TRACED(K_BCR_IMAGE, st, (bcr_image_kernel<<<dim3((n + 31) / 32, nb), 128, 0, st>>>(
+                                         n, l.n_chunk, l.nzr, src, stride, pr, mdst_dev ? mdst_dev + t : nullptr, cx_in,
+                                         cx_edge, im, l.mat_bytes)));
     }
     return cudaGetLastError();
 }

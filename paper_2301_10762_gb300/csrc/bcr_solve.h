@@ -62,10 +62,37 @@ __device__ __forceinline__ long long bs_matrix(const BsArgs &a, int code, int sy
     return bs_matrix_index(a.nx, a.ns, a.half, code, sys);
 }
 
-// images of n x n row-major blocks src + pairs[.][0] * stride as matrices pairs[.][1], and of their
-// transposes as matrices tdst[.] (tdst null: none); mx: zeroed words, one per matrix
-cudaError_t launch_bcr_image(int n, const float2 *src, long long stride, const int *pairs_dev, const int *tdst_dev,
-                             int count, unsigned char *img, uint32_t *mx, int *shift, cudaStream_t st);
+// A family of images: matrices 0 .. n_kept - 1 stay with the factor, the others are its working blocks
+struct BsImages {
+    unsigned char *kept = nullptr, *work = nullptr;
+    int n_kept = 0;
+    int *shift = nullptr;      // [matrix]
+    uint32_t *mx = nullptr;    // [matrix]: bits of the largest modulus (or a bound); working array of the factor
+    __host__ __device__ unsigned char *at(int i, size_t mat_bytes) const {
+        return i < n_kept ? kept + (size_t)i * mat_bytes : work + (size_t)(i - n_kept) * mat_bytes;
+    }
+};
+// images of n x n row-major blocks src + pairs[.][0] * stride as matrices pairs[.][1], and of
+// -C block C (C = diag(cx)) as matrices mdst[.] (mdst null: none); im.mx zeroed beforehand
+cudaError_t launch_bcr_image(int n, const float2 *src, long long stride, const int *pairs_dev, const int *mdst_dev,
+                             int count, float cx_in, float cx_edge, const BsImages &im, cudaStream_t st);
+
+// Products of images (bcr_gemm.cu): tasks of BG_TASK ints (flags, matrix A, matrix B, output): the
+// image of +-A B^T as matrix `output`, or (BG_FP32) D block `output` += +-A B^T
+constexpr int BG_TASK = 4;
+enum { BG_NEG = 1, BG_FP32 = 2 };
+struct BgArgs {
+    int nz;
+    const int *tasks;
+    BsImages im;
+    float2 *D;               // [block][nz][nz]
+    int *status;
+    uint32_t tries;
+    // set by launch_bcr_gemm
+    int n_chunk, nzr, nt, n_tiles, log2_2k;
+    size_t mat_bytes;
+};
+cudaError_t launch_bcr_gemm(BgArgs a, int n_tasks, cudaStream_t st);
 cudaError_t launch_bcr_solve(BsArgs a, const BsStep *steps, int n_steps, bool prepared, double flops, cudaStream_t st);
 int device_sms();   // streaming multiprocessors of the current device
 

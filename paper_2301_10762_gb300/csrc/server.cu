@@ -87,11 +87,11 @@ struct helm_server {
         const size_t N = (size_t)g.nx * g.nz, blk = (size_t)g.nz * g.nz * 8;
         const helm::GridGeom geom{g.nx, g.nz, g.lx / (g.nx - 1), g.lz / (g.nz - 1), g.lumping};
         if (helm::factor_picks_bcr(geom, (helm_prec)prec, HELM_FACTOR_AUTO)) {
-            // block cyclic reduction: the inverses of every line and P, Q, W, V of the eliminated
-            // ones (rows padded to 32 columns), and as many working blocks while it factors
-            // (counted throughout)
-            const size_t kept = (size_t)g.nx + 4 * ((size_t)g.nx / 2 + 1);
-            return kept * (blk + helm::bs_layout(g.nz).mat_bytes + 8) + 96 * N + 65 * kMiB;   // + the split-K tiles
+            // block cyclic reduction: the images of every line's inverse and of P, Q, W, V of the
+            // eliminated ones, and while it factors (counted throughout) 1.25 n_x images of
+            // couplings and the FP32 diagonal blocks
+            const size_t kept = (size_t)g.nx + 4 * ((size_t)g.nx / 2 + 1), work = 5 * (size_t)g.nx / 4 + 5;
+            return (kept + work) * (helm::bs_layout(g.nz).mat_bytes + 8) + g.nx * blk + 96 * N + 65 * kMiB;   // + split-K tiles
         }
         return (size_t)g.nx * g.nz * g.nz * (prec == HELM_MIXED ? 8 : 16) + 96 * N + kMiB;
     }

@@ -26,9 +26,9 @@ __host__ __device__ constexpr uint32_t idesc_tf32(int n_real) {
     return (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(n_real >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
 }
 
-// the same for FP16 operands
-__host__ __device__ constexpr uint32_t idesc_f16(int n_real) {
-    return (1u << 4) | ((uint32_t)(n_real >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
+// the same for FP16 operands; neg_b: the product with -B
+__host__ __device__ constexpr uint32_t idesc_f16(int n_real, bool neg_b = false) {
+    return (1u << 4) | (neg_b ? 1u << 14 : 0u) | ((uint32_t)(n_real >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
 }
 
 // x rounded to the TF32 grid (10 explicit mantissa bits), to nearest with ties away from zero:

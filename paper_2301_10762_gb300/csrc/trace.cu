@@ -15,7 +15,7 @@ static const char *kNames[K_COUNT] = {
     "fill", "sub", "regR", "dct_table", "dct_pass", "line_gb_prepass", "split_diag", "refine_start", "refine_update",
     "refine_finish", "refine_accumulate", "field_grad", "g_coefficients", "hess_finish",
     "zgemm_tf32x3", "zinv_block", "bcr_form_blocks", "bcr_level0_update", "bcr_solve",
-    "zgemm_split_reduce", "bcr_image", "line_max",
+    "zgemm_split_reduce", "bcr_image", "line_max", "bcr_gemm",
 };
 
 namespace {
