@@ -47,6 +47,7 @@
 #include <vector>
 
 #include "abi_internal.h"
+#include "bcr_image.cuh"
 #include "bcr_solve.h"
 #include "kernels.h"
 #include "pivot16.cuh"
@@ -73,86 +74,254 @@ Coup coup_of(const GridGeom &g) {
     return Coup{(float)coup_x(g, 1), (float)coup_x(g, 0), (float)coup_z(g, 1), (float)coup_z(g, 0)};
 }
 
-// dense D_i of every line and system (n_z > 256): the diagonal of A and the vertical couplings
-// next to it; one float4 (two complex entries of a row) per thread and step
-__global__ void bcr_form_kernel(GridGeom g, Coup cp, const double2 *diag, float2 *D) {
-    const int nz = g.nz, nx = g.nx;
-    const int i = blockIdx.y, s = blockIdx.z;
-    const float cz = cp.cz(i, nx);
-    float4 *Di = reinterpret_cast<float4 *>(D + ((size_t)s * nx + i) * nz * nz);
-    const double2 *dg = diag + ((size_t)s * nx + i) * nz;
-    const int nq = nz * nz / 2;
-    for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < nq; q += gridDim.x * blockDim.x) {
-        const int r = (2 * q) / nz, c = (2 * q) - r * nz;   // columns c, c + 1 of row r
-        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-        const int c1 = c + 1;
-        if (c == r) { const float2 d = to_c64(dg[r]); v.x = d.x; v.y = d.y; }
-        else if (c == r + 1 || c + 1 == r) v.x = cz;
-        if (c1 == r) { const float2 d = to_c64(dg[r]); v.z = d.x; v.w = d.y; }
-        else if (c1 == r + 1 || c1 + 1 == r) v.z = cz;
-        Di[q] = v;
+// Level 0: the eliminated lines' blocks are complex symmetric tridiagonal, T = tridiag(cz, d, cz),
+// and their inverses semiseparable:
+//     X_ij = u_i v_j for i <= j (X symmetric),   u_i = 1 / R_i,  v_j = g_j R_j,
+// with the pivots of the elimination from above (delta_k = d_k - cz^2 / delta_{k-1}) and from
+// below (gamma_k = d_k - cz^2 / gamma_{k+1}), R_j = prod_{k < j} (-cz / delta_k) and g_j = X_jj =
+// 1 / (delta_j + gamma_j - d_j).  So no block is inverted: the recurrences run in FP64 (O(n_z) per
+// line), and every kernel that wants X forms its entries from u and v, held as FP32 hi + lo with an
+// exponent (R spans hundreds of orders of magnitude), correct to FP32 rounding.  Cyclic reduction
+// amplifies level 0's errors most (the Schur complements of the smooth modes lose four in size
+// per level): a block Gauss-Jordan inverse carries 1.2e-7 of its norm.
+// 256^2 with 8 frequencies: level 0 with its images 0.9 ms (dense inversions by two 128-column
+// halves 1.0 ms, images and update 0.6); 512^2 with 4: 19 ms less.
+struct TriGen {          // generators of the odd lines' inverses: [line][nz]
+    float4 *u, *v;       // hi.x, hi.y, lo.x, lo.y
+    int2 *e;             // exponents of u and v
+};
+struct TriScan {         // working arrays of the recurrences: [k][line]
+    double2 *delta, *gamma, *r;
+    int *re;
+};
+
+// 1 / z, the modulus bounded from below by 1e-12 of `scale` (a pivot there is as good as singular in
+// FP32: T is perturbed by no more than that)
+__device__ __forceinline__ double2 crecip_guard(double2 z, double scale) {
+    double n2 = z.x * z.x + z.y * z.y;
+    if (n2 < 1e-24 * scale * scale) {
+        z = make_double2(1e-12 * scale, 0.0);
+        n2 = z.x * z.x;
+    }
+    const double r = fast_recip(n2);
+    return make_double2(z.x * r, -z.y * r);
+}
+// z scaled to a largest part in [1, 2), e its exponent (zero and non-finite values as they are)
+__device__ __forceinline__ double2 cnormalize(double2 z, int &e) {
+    const int hx = (__double2hiint(z.x) >> 20) & 0x7ff, hy = (__double2hiint(z.y) >> 20) & 0x7ff, h = max(hx, hy);
+    if (h == 0 || h == 0x7ff) { e = 0; return z; }
+    e = h - 1023;
+    const double s = __hiloint2double((2046 - h) << 20, 0);   // 2^-e
+    return make_double2(z.x * s, z.y * s);
+}
+
+// the recurrences: a thread per line and direction.  A chain of n_z steps of about ten dependent
+// FP64 operations; 32 chains share a warp because the FP64 pipe takes two lanes a cycle per SM
+// however many are active.
+__global__ void __launch_bounds__(32) tri_scan_kernel(GridGeom g, int n_line, const double2 *diag, TriScan w) {
+    const int t = blockIdx.x * 32 + threadIdx.x, dir = t & 1, l = t >> 1;
+    if (l >= n_line) return;
+    const int nx = g.nx, nz = g.nz, no = nx / 2, line = 2 * (l % no) + 1;
+    const double2 *d = diag + ((size_t)(l / no) * nx + line) * nz;
+    const double cz = coup_z(g, line), c2 = cz * cz;
+    double2 inv = make_double2(0.0, 0.0), r = make_double2(1.0, 0.0);
+    int re = 0;
+    double2 nd = d[dir ? nz - 1 : 0];
+    for (int q = 0; q < nz; ++q) {
+        const int k = dir ? nz - 1 - q : q;
+        const double2 dk = nd;
+        if (q + 1 < nz) nd = d[dir ? k - 1 : k + 1];
+        const double2 p = make_double2(dk.x - c2 * inv.x, dk.y - c2 * inv.y);
+        const size_t o = (size_t)k * n_line + l;
+        inv = crecip_guard(p, cz);
+        if (dir) {
+            w.gamma[o] = p;
+        } else {
+            w.delta[o] = p;
+            w.r[o] = r;
+            w.re[o] = re;
+            int e;
+            r = cnormalize(cmul(r, make_double2(-cz * inv.x, -cz * inv.y)), e);
+            re += e;
+        }
+    }
+}
+
+// generators, and the scales of the images of X and of -C X C from the bound max_j |v_j| max_{i <= j}
+// |u_i| (attained up to the FP32 rounding): a CTA per line
+__global__ void __launch_bounds__(256) tri_gen_kernel(GridGeom g, Coup cp, int n_line, const double2 *diag, TriScan w,
+                                                      TriGen o, const int *dst, BsImages im) {
+    const int l = blockIdx.x, nx = g.nx, nz = g.nz, no = nx / 2, line = 2 * (l % no) + 1;
+    const double2 *d = diag + ((size_t)(l / no) * nx + line) * nz;
+    const double cz = coup_z(g, line);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    __shared__ float s_u[8], s_top[8];
+    float carry = -1e30f, top = -1e30f;   // log2 of the largest |u| so far and of the largest |X|
+    for (int k0 = 0; k0 < nz; k0 += 256) {
+        const int k = k0 + tid;
+        float lu = -1e30f, lv = -1e30f;
+        if (k < nz) {
+            const size_t q = (size_t)k * n_line + l;
+            const double2 dl = w.delta[q], gm = w.gamma[q], r = w.r[q], dk = d[k];
+            int e1, e2;
+            const double2 u = cnormalize(crecip_guard(r, 0.0), e1);
+            const double2 gg = crecip_guard(make_double2(dl.x + gm.x - dk.x, dl.y + gm.y - dk.y), cz);
+            const double2 v = cnormalize(cmul(gg, r), e2);
+            const int eu = e1 - w.re[q], ev = e2 + w.re[q];
+            const size_t p = (size_t)l * nz + k;
+            const float ux = (float)u.x, uy = (float)u.y, vx = (float)v.x, vy = (float)v.y;
+            o.u[p] = make_float4(ux, uy, (float)(u.x - ux), (float)(u.y - uy));
+            o.v[p] = make_float4(vx, vy, (float)(v.x - vx), (float)(v.y - vy));
+            o.e[p] = make_int2(eu, ev);
+            lu = 0.5f * __log2f(ux * ux + uy * uy) + (float)eu;
+            lv = 0.5f * __log2f(vx * vx + vy * vy) + (float)ev;
+        }
+        // running maximum of lu over k: warp scan, then the warps before, then the blocks before
+        float m = lu;
+#pragma unroll
+        for (int s = 1; s < 32; s *= 2) {
+            const float t = __shfl_up_sync(0xffffffffu, m, s);
+            if (lane >= s) m = fmaxf(m, t);
+        }
+        if (lane == 31) s_u[warp] = m;
+        __syncthreads();
+        float all = carry;
+        for (int s = 0; s < 8; ++s) {
+            if (s < warp) m = fmaxf(m, s_u[s]);
+            all = fmaxf(all, s_u[s]);
+        }
+        m = fmaxf(m, carry);
+        carry = all;
+        top = fmaxf(top, lv + m);
+        __syncthreads();
+    }
+#pragma unroll
+    for (int s = 16; s > 0; s /= 2) top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, s));
+    if (lane == 0) s_top[warp] = top;
+    __syncthreads();
+    if (tid == 0) {
+        for (int s = 1; s < 8; ++s) top = fmaxf(top, s_top[s]);
+        // (a NaN is left out of fmaxf: the entries themselves carry it)
+        const float mx = exp2f(fminf(fmaxf(top, -120.f), 120.f)) * 1.0001f;
+        const float mm = mx * fmaxf(cp.cx_in * cp.cx_in, cp.cx_edge * cp.cx_edge);
+        im.mx[dst[2 * l]] = bs_abs_bits(mx);
+        im.shift[dst[2 * l]] = bs_scale_shift(bs_abs_bits(mx));
+        im.mx[dst[2 * l + 1]] = bs_abs_bits(mm);
+        im.shift[dst[2 * l + 1]] = bs_scale_shift(bs_abs_bits(mm));
+    }
+}
+
+// u v 2^(eu + ev + sh)
+__device__ __forceinline__ float2 tri_entry(const float4 &u, const float4 &v, int e) {
+    const float re = fmaf(u.x, v.x, fmaf(-u.y, v.y, fmaf(u.x, v.z, fmaf(-u.y, v.w, fmaf(u.z, v.x, -u.w * v.y)))));
+    const float im = fmaf(u.x, v.y, fmaf(u.y, v.x, fmaf(u.x, v.w, fmaf(u.y, v.z, fmaf(u.z, v.y, u.w * v.x)))));
+    const float s = e < -126 ? 0.f : bs_pow2(min(e, 128));   // (128: infinity)
+    return make_float2(re * s, im * s);
+}
+
+// images of X (matrix dst[.][0]) and -C X C (dst[.][1]) of a line: a CTA takes 32 rows, a thread a
+// row and eight columns at a time.  Bound by the write of the images.
+__global__ void __launch_bounds__(128) tri_image_kernel(int n, int n_chunk, int nzr, TriGen tg, const int *dst, Coup cp,
+                                                        BsImages im, size_t mat_bytes) {
+    const int l = blockIdx.x, row = threadIdx.x >> 2, j = threadIdx.x & 3, r = 32 * blockIdx.y + row;
+    if (r >= nzr) return;
+    const bool on = r < n;
+    const float4 *U = tg.u + (size_t)l * n, *V = tg.v + (size_t)l * n;
+    const int2 *E = tg.e + (size_t)l * n;
+    const float4 z4 = make_float4(0.f, 0.f, 0.f, 0.f);
+    const float4 ur = on ? U[r] : z4, vr = on ? V[r] : z4;
+    const int2 er = on ? E[r] : make_int2(0, 0);
+    const int mx = dst[2 * l], mm = dst[2 * l + 1], shx = im.shift[mx], shm = im.shift[mm];
+    const float cr = on ? -cp.cx(r, n) * bs_pow2(shm - shx) : 0.f;   // (|shm - shx|: the couplings' exponent)
+    unsigned char *px = im.at(mx, mat_bytes) + (size_t)r * 128, *pm = im.at(mm, mat_bytes) + (size_t)r * 128;
+    const int o0 = (j ^ (r & 7)) << 4, o1 = ((j + 4) ^ (r & 7)) << 4;
+    const size_t half = (size_t)nzr * 128;
+    for (int c = 0; c < n_chunk; ++c, px += 2 * half, pm += 2 * half) {
+        float2 x[8], m[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            const int k = 32 * c + 8 * j + q;
+            x[q] = m[q] = make_float2(0.f, 0.f);
+            if (on && k < n) {
+                const bool up = r <= k;
+                const float4 o = __ldg(up ? V + k : U + k);
+                const int2 e = __ldg(E + k);
+                x[q] = tri_entry(up ? ur : vr, o, (up ? er.x + e.y : er.y + e.x) + shx);
+                const float f = cr * cp.cx(k, n);
+                m[q] = make_float2(f * x[q].x, f * x[q].y);
+            }
+        }
+        uint4 rh, rl, ih, il;
+        bs_split8(x, 1.f, rh, rl, ih, il);
+        *reinterpret_cast<uint4 *>(px + o0) = rh;
+        *reinterpret_cast<uint4 *>(px + o1) = rl;
+        *reinterpret_cast<uint4 *>(px + half + o0) = ih;
+        *reinterpret_cast<uint4 *>(px + half + o1) = il;
+        bs_split8(m, 1.f, rh, rl, ih, il);
+        *reinterpret_cast<uint4 *>(pm + o0) = rh;
+        *reinterpret_cast<uint4 *>(pm + o1) = rl;
+        *reinterpret_cast<uint4 *>(pm + half + o0) = ih;
+        *reinterpret_cast<uint4 *>(pm + half + o1) = il;
     }
 }
 
 // level 0 (couplings C = diag(cx)): kept line k (even) with eliminated neighbours k - 1, k + 1:
-//   D_k -= C Dinv_{k-1} C + C Dinv_{k+1} C
-// (its couplings, -C Dinv C of either neighbour, are written as images of the inverses)
-// implicit (diag != nullptr): D_k is not in memory yet and is taken from A's diagonal and the
-// line's vertical coupling (the tridiagonal line block) before the update
-__global__ void bcr_level0_kernel(GridGeom g, Coup cp, float2 *D, const double2 *diag) {
-    const int nz = g.nz, nx = g.nx, nz2 = nz * nz;
-    const int k = 2 * blockIdx.y, s = blockIdx.z;
-    const bool ha = k >= 1, hc = k + 1 < nx;
-    const float2 *Da = D + ((size_t)s * nx + (ha ? k - 1 : 0)) * nz2;
-    const float2 *Dc = D + ((size_t)s * nx + (hc ? k + 1 : 0)) * nz2;
-    float2 *Dk = D + ((size_t)s * nx + k) * nz2;
-    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < nz2; e += gridDim.x * blockDim.x) {
-        const int r = e / nz, c = e - r * nz;
-        const float sc = cp.cx(r, nz) * cp.cx(c, nz);
-        float2 t = make_float2(0.f, 0.f);
-        if (ha) { const float2 v = Da[e]; t = make_float2(sc * v.x, sc * v.y); }
-        if (hc) { const float2 v = Dc[e]; t.x += sc * v.x; t.y += sc * v.y; }
-        float2 d;
-        if (diag) {
-            const float cz = cp.cz(k, nx);
-            d = r == c ? to_c64(diag[((size_t)s * nx + k) * nz + r])
-                       : ((r - c == 1 || c - r == 1) ? make_float2(cz, 0.f) : make_float2(0.f, 0.f));
-        } else {
-            d = Dk[e];
+//   D_k = T_k - C X_{k-1} C - C X_{k+1} C
+// a CTA takes 32 rows by 256 columns, a thread two columns (their generators in registers; the
+// rows' are the same for the whole CTA)
+__global__ void __launch_bounds__(128) bcr_level0_kernel(GridGeom g, Coup cp, float2 *D, const double2 *diag, TriGen tg) {
+    const int nz = g.nz, nx = g.nx, no = nx / 2, nk = (nx + 1) / 2;
+    const int s = blockIdx.x / nk, k = 2 * (blockIdx.x % nk), c = 256 * blockIdx.z + 2 * threadIdx.x;
+    if (c >= nz) return;
+    const bool has[2] = {k >= 1, k + 1 < nx};
+    float4 uc[2][2], vc[2][2];
+    int2 ec[2][2];
+    size_t base[2];
+    float fc[2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) fc[h] = cp.cx(c + h, nz);
+#pragma unroll
+    for (int n = 0; n < 2; ++n) {
+        base[n] = ((size_t)s * no + (has[n] ? k / 2 - 1 + n : 0)) * nz;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            uc[n][h] = __ldg(tg.u + base[n] + c + h);
+            vc[n][h] = __ldg(tg.v + base[n] + c + h);
+            ec[n][h] = __ldg(tg.e + base[n] + c + h);
         }
-        Dk[e] = make_float2(d.x - t.x, d.y - t.y);
+    }
+    const float cz = cp.cz(k, nx);
+    const double2 *dg = diag + ((size_t)s * nx + k) * nz;
+    float2 *Dk = D + ((size_t)s * nx + k) * nz * nz;
+    for (int r = 32 * blockIdx.y; r < min(nz, 32 * (int)blockIdx.y + 32); ++r) {
+        float2 t[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+#pragma unroll
+        for (int n = 0; n < 2; ++n) {
+            if (!has[n]) continue;
+            const float4 ur = __ldg(tg.u + base[n] + r), vr = __ldg(tg.v + base[n] + r);
+            const int2 er = __ldg(tg.e + base[n] + r);
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const bool up = r <= c + h;
+                const float2 x = up ? tri_entry(ur, vc[n][h], er.x + ec[n][h].y) : tri_entry(uc[n][h], vr, ec[n][h].x + er.y);
+                t[h].x += x.x;
+                t[h].y += x.y;
+            }
+        }
+        const float fr = cp.cx(r, nz);
+        float2 o[2];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int cc = c + h;
+            float2 d = make_float2(0.f, 0.f);
+            if (r == cc) d = to_c64(dg[r]);
+            else if (r - cc == 1 || cc - r == 1) d.x = cz;
+            const float f = fr * fc[h];
+            o[h] = make_float2(d.x - f * t[h].x, d.y - f * t[h].y);
+        }
+        *reinterpret_cast<float4 *>(Dk + (size_t)r * nz + c) = make_float4(o[0].x, o[0].y, o[1].x, o[1].y);
     }
 }
-
-// Implicit tridiagonal input of the block inversion (the level-0 line blocks, never formed in
-// memory): rows and columns row0 .. row0 + n - 1 of the block of line idx (input index = system
-// * nx + line) with A's diagonal diag[idx][.] and the line's vertical coupling; with corr, entry
-// (0, 0) less cz^2 X[corr_off] (X the output block: the Schur complement of the lower half).
-struct TriIn {
-    const double2 *diag = nullptr;   // [idx][nz]; nullptr: the input is a dense block
-    int nz = 0, nx = 0, row0 = 0;
-    float cz_in = 0.f, cz_edge = 0.f;
-    int corr = 0;
-    long long corr_off = 0;
-    __device__ __forceinline__ float cz(int idx) const {
-        const int line = idx % nx;
-        return (line == 0 || line == nx - 1) ? cz_edge : cz_in;
-    }
-    // entry (r, c) of the block of input idx; x: the output block (for the corrected corner)
-    __device__ __forceinline__ float2 entry(int idx, int r, int c, const float2 *x) const {
-        if (r == c) {
-            float2 v = to_c64(diag[(long long)idx * nz + row0 + r]);
-            if (corr && r == 0) {
-                const float c2 = cz(idx) * cz(idx);
-                const float2 w = x[corr_off];
-                v.x -= c2 * w.x;
-                v.y -= c2 * w.y;
-            }
-            return v;
-        }
-        return (r - c == 1 || c - r == 1) ? make_float2(cz(idx), 0.f) : make_float2(0.f, 0.f);
-    }
-};
 
 struct InvArgs {
     int n;
@@ -162,7 +331,6 @@ struct InvArgs {
     int out_div, ldo;
     const int *idx;              // [count][2]: input index, output index
     int *status;
-    TriIn tri;                   // tri.diag set: implicit tridiagonal input instead of `in`
     uint32_t tries = 0;          // polls of a bounded mbarrier wait before it gives up
 };
 
@@ -187,7 +355,7 @@ __global__ void __launch_bounds__(INV_THREADS, 1) zinv_base_kernel(InvArgs a) {
     if (tid == 0) s_bad = 0;
     for (int e = tid; e < n * n; e += INV_THREADS) {
         const int r = e / n, c = e % n;
-        W[(size_t)r * ldw + c] = a.tri.diag ? a.tri.entry(ix[0], r, c, X) : M[(size_t)r * a.in.ld + c];
+        W[(size_t)r * ldw + c] = M[(size_t)r * a.in.ld + c];
     }
     __syncthreads();
     // update mapping: thread -> column c, row group rg (rows rg, rg + ng, ...)
@@ -303,7 +471,7 @@ __global__ void __launch_bounds__(ZT_THREADS, 2) zinv128_tm_kernel(InvArgs a) {
         float v[16];
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
-            const float2 e = a.tri.diag ? a.tri.entry(ix[0], r, c0 + i, X) : M[(size_t)r * a.in.ld + c0 + i];
+            const float2 e = M[(size_t)r * a.in.ld + c0 + i];
             v[2 * i] = e.x;
             v[2 * i + 1] = e.y;
         }
@@ -453,42 +621,6 @@ size_t inv_smem_bytes(int n) {
     return sizeof(float2) * ((size_t)n * (n + 1) + (size_t)n * PIV + (size_t)PIV * (n + 1) + PIV * PIV);
 }
 
-// Inverse of complex symmetric tridiagonal blocks D (the level-0 line blocks) of size
-// n = n1 + n2 by the 2 x 2 block inverse, whose off-diagonal block D21 = c e_0 e_{n1-1}^T has a
-// single entry, the line's vertical coupling c: with x = X11[:, n1 - 1] (X11 = D11^{-1}),
-//     S = D22 - c^2 X11[n1-1][n1-1] e_0 e_0^T,  X22 = S^{-1},
-//     X12 = -c x X22[0, :],  X21 = X12^T,  X11 <- X11 + c^2 X22[0][0] x x^T,
-// so that the four products of the general case are rank-one updates (the inversions read D11
-// and S implicitly, TriIn).  Output blocks at out + idx * stride, rows ld apart; pairs
-// [count][2] (input index = system * nx + line, output index).
-__global__ void __launch_bounds__(512) tri_rank1_kernel(int n, int n1, TriIn tri, float2 *out, long long stride, int ld,
-                                                        const int *pairs) {
-    __shared__ float2 xs[INV_MAX], rs[INV_MAX];
-    float2 *X = out + (long long)pairs[2 * blockIdx.x + 1] * stride;
-    const int n2 = n - n1;
-    const float2 c = make_float2(tri.cz(pairs[2 * blockIdx.x]), 0.f);
-    for (int i = threadIdx.x; i < n1; i += blockDim.x) xs[i] = X[(long long)i * ld + n1 - 1];
-    for (int j = threadIdx.x; j < n2; j += blockDim.x) rs[j] = X[(long long)n1 * ld + n1 + j];
-    __syncthreads();
-    const float2 c2d = cmul(cmul(c, c), rs[0]);           // c^2 X22[0][0]
-    const float2 mc = make_float2(-c.x, -c.y);
-    for (int e = threadIdx.x; e < n1 * n; e += blockDim.x) {   // rows 0 .. n1 - 1: X11 and X12
-        const int i = e / n, j = e % n;
-        float2 *w = X + (long long)i * ld + j;
-        if (j < n1) {
-            float2 v = *w;
-            cfma(v, cmul(c2d, xs[i]), xs[j]);
-            *w = v;
-        } else {
-            *w = cmul(cmul(mc, xs[i]), rs[j - n1]);
-        }
-    }
-    for (int e = threadIdx.x; e < n2 * n1; e += blockDim.x) {   // rows n1 .. n - 1, columns 0 .. n1 - 1: X21
-        const int i = e / n1, j = e % n1;
-        X[(long long)(n1 + i) * ld + j] = cmul(cmul(mc, rs[i]), xs[j]);
-    }
-}
-
 // *out = largest of n words
 __global__ void __launch_bounds__(1024) max_words_kernel(size_t n, const uint32_t *v, int *out) {
     __shared__ uint32_t s[32];
@@ -629,8 +761,7 @@ struct Fam {
 };
 
 // out[p.second] = in[p.first]^{-1} for every index pair, n x n blocks (may be the same matrices)
-helm_status invert_blocks(int n, Fam in, Fam out, const std::vector<int> &pairs, int *status, Plan &pl,
-                          const TriIn *tri = nullptr) {
+helm_status invert_blocks(int n, Fam in, Fam out, const std::vector<int> &pairs, int *status, Plan &pl) {
     const int count = (int)(pairs.size() / 2);
     if (count == 0) return HELM_OK;
     const cudaStream_t st = pl.st;
@@ -645,7 +776,7 @@ helm_status invert_blocks(int n, Fam in, Fam out, const std::vector<int> &pairs,
         const void *fn = t128 ? (const void *)zinv128_tm_kernel : (const void *)zinv_base_kernel;
         cudaError_t e = ensure_dyn_smem(fn, smem);
         if (e != cudaSuccess) { helm_set_error("bcr: block inversion", e); return HELM_ECUDA; }
-        InvArgs a{n, in.op(), out.base, out.stride, 0, 0, out.ld, nullptr, status, tri ? *tri : TriIn{}};
+        InvArgs a{n, in.op(), out.base, out.stride, 0, 0, out.ld, nullptr, status};
         a.tries = wait_tries();
         pl.ops.push_back([a, off, count, smem, st, t128](const int *dev) mutable -> helm_status {
             a.idx = dev + off;
@@ -657,7 +788,6 @@ helm_status invert_blocks(int n, Fam in, Fam out, const std::vector<int> &pairs,
         });
         return HELM_OK;
     }
-    if (tri) return HELM_EINVAL;   // implicit input: base blocks only (invert_tridiag_blocks splits)
     const int n1 = INV_MAX * ((n / INV_MAX + 1) / 2), n2 = n - n1;
     // X11 = D11^{-1}
     if ((s = invert_blocks(n1, in, out, pairs, status, pl)) != HELM_OK) return s;
@@ -715,53 +845,13 @@ helm_status invert_blocks(int n, Fam in, Fam out, const std::vector<int> &pairs,
     return HELM_OK;
 }
 
-// out[p.second] = D^{-1} for the complex symmetric tridiagonal line blocks D given by `tri`
-// (input index = system * nx + line), n <= 256: one implicit base inversion for n <= 128; else
-// two and two rank-one kernels (tri_rank1_kernel)
-helm_status invert_tridiag_blocks(int n, Fam in, Fam out, const std::vector<int> &pairs, int *status, Plan &pl,
-                                  const TriIn &tri) {
-    const int count = (int)(pairs.size() / 2);
-    if (count == 0) return HELM_OK;
-    if (n > 2 * INV_MAX) return HELM_EINVAL;
-    TriIn t0 = tri;
-    t0.row0 = 0;
-    t0.corr = 0;
-    if (n <= INV_MAX) return invert_blocks(n, in, out, pairs, status, pl, &t0);
-    const int n1 = INV_MAX, n2 = n - n1;
-    const cudaStream_t st = pl.st;
-    helm_status s;
-    if ((s = invert_blocks(n1, in, out, pairs, status, pl, &t0)) != HELM_OK) return s;   // X11 = D11^{-1}
-    // X22 = S^{-1}, S read from the diagonal with the corner corrected by X11[n1-1][n1-1]
-    TriIn t1 = tri;
-    t1.row0 = n1;
-    t1.corr = 1;
-    t1.corr_off = -(long long)out.ld - 1;   // from X22's first entry to X11's last
-    if ((s = invert_blocks(n2, in, out.sub(n1, n1), pairs, status, pl, &t1)) != HELM_OK) return s;
-    const int off = pl.add(pairs);
-    float2 *ob = out.base;
-    const long long stride = out.stride;
-    const int ld = out.ld;
-    pl.ops.push_back([=](const int *dev) -> helm_status {   // X12, X21, X11 from rank-one updates
-        HELM_TRACED(K_ZINV, st, (tri_rank1_kernel<<<count, 512, 0, st>>>(n, n1, t0, ob, stride, ld, dev + off)));
-        const cudaError_t e2 = cudaGetLastError();
-        if (e2 != cudaSuccess) { helm_set_error("bcr: block inversion", e2); return HELM_ECUDA; }
-        return HELM_OK;
-    });
-    return HELM_OK;
-}
-
-// images (bcr_solve.cu) of the inverses in slots pairs[.][0] of D as matrices pairs[.][1], and of
-// their level-0 couplings as matrices mdst[.] (empty: none)
-helm_status image_blocks(const GridGeom &g, const float2 *D, const std::vector<int> &pairs, const std::vector<int> &mdst,
-                         const BgArgs &ba, Plan &pl) {
+// images (bcr_solve.cu) of the blocks in slots pairs[.][0] of D as matrices pairs[.][1]
+helm_status image_blocks(int n, const float2 *D, const std::vector<int> &pairs, const BgArgs &ba, Plan &pl) {
     if (pairs.empty()) return HELM_OK;
-    const int off = pl.add(pairs), moff = mdst.empty() ? -1 : pl.add(mdst), count = (int)(pairs.size() / 2);
+    const int off = pl.add(pairs), count = (int)(pairs.size() / 2);
     const cudaStream_t st = pl.st;
-    const Coup cp = coup_of(g);
-    const int n = g.nz;
     pl.ops.push_back([=](const int *dev) -> helm_status {
-        const cudaError_t e = launch_bcr_image(n, D, (long long)n * n, dev + off, moff < 0 ? nullptr : dev + moff, count,
-                                               cp.cx_in, cp.cx_edge, ba.im, st);
+        const cudaError_t e = launch_bcr_image(n, D, (long long)n * n, dev + off, count, ba.im, st);
         if (e != cudaSuccess) { helm_set_error("bcr: images", e); return HELM_ECUDA; }
         return HELM_OK;
     });
@@ -850,56 +940,56 @@ helm_status bcr_factor(helm_factor_t *f) {
     ba.tries = wait_tries();
     Plan pl(st);
     if ((s = pl.with_split(kFactorSplitElems)) != HELM_OK) return s;
-    const int per = (int)std::min<long long>(64, (nz2 + 255) / 256);
-    // n_z <= 256: no line block is formed in memory before level 0, which inverts the odd lines'
-    // tridiagonal blocks and updates the even lines' straight from A's diagonal and couplings
-    const bool tri_level0 = nz <= 2 * INV_MAX;
-    const double2 *tri_diag = tri_level0 ? op->diag : nullptr;
-    TriIn tri;
-    tri.diag = op->diag;
-    tri.nz = nz;
-    tri.nx = nx;
-    tri.cz_in = coup_of(g).cz_in;
-    tri.cz_edge = coup_of(g).cz_edge;
+    const Fam fD{D, nz2, nz};
+    auto mat = [&](int kind, int sy, int slot) { return (int)bs_matrix_index(nx, ns, half, kind << 24 | slot, sy); };
+    auto invert = [&](const std::vector<int> &pairs, const std::vector<int> &images) -> helm_status {
+        const helm_status s1 = invert_blocks(nz, fD, fD, pairs, op->status, pl);
+        return s1 != HELM_OK ? s1 : image_blocks(nz, D, images, ba, pl);
+    };
+    // level 0: generators of the odd lines' inverses, their images and the even lines' blocks
     {
+        const int no = nx / 2, n_line = ns * no;
+        const size_t n_gen = (size_t)n_line * nz;
+        std::vector<int> dst;
+        for (int sy = 0; sy < ns; ++sy)
+            for (int j = 1; j < nx; j += 2) dst.insert(dst.end(), {mat(BS_DINV, sy, j), (int)m0 + sy * m_stride + j / 2});
+        const int off = pl.add(dst);
+        void *buf = nullptr;   // generators (40 bytes an entry) and the recurrences' values (52)
+        if ((s = dev_alloc(&buf, n_gen * 92, "bcr: level 0", st)) != HELM_OK) return s;
+        pl.scratch.push_back(buf);
+        TriGen tg;
+        TriScan ts;
+        tg.u = (float4 *)buf;
+        tg.v = tg.u + n_gen;
+        ts.delta = (double2 *)(tg.v + n_gen);
+        ts.gamma = ts.delta + n_gen;
+        ts.r = ts.gamma + n_gen;
+        tg.e = (int2 *)(ts.r + n_gen);
+        ts.re = (int *)(tg.e + n_gen);
+        const Coup cp = coup_of(g);
         const double2 *diag = op->diag;
         float2 *D0 = D;
-        const Coup cp = coup_of(g);
-        const int perq = (int)std::min<long long>(64, (nz2 / 2 + 255) / 256);
-        if (!tri_level0) pl.ops.push_back([=](const int *) -> helm_status {
-            HELM_TRACED(K_BCR_FORM, st, (bcr_form_kernel<<<dim3(perq, nx, ns), 256, 0, st>>>(g, cp, diag, D0)));
+        pl.ops.push_back([=](const int *dev) -> helm_status {
+            HELM_TRACED(K_BCR_L0, st, (tri_scan_kernel<<<(2 * n_line + 31) / 32, 32, 0, st>>>(g, n_line, diag, ts)));
+            HELM_TRACED(K_BCR_L0, st, (tri_gen_kernel<<<n_line, 256, 0, st>>>(g, cp, n_line, diag, ts, tg, dev + off, im)));
+            HELM_TRACED(K_BCR_IMAGE, st, (tri_image_kernel<<<dim3(n_line, (lay.nzr + 31) / 32), 128, 0, st>>>(
+                                             nz, lay.n_chunk, lay.nzr, tg, dev + off, cp, im, lay.mat_bytes)));
+            HELM_TRACED(K_BCR_L0, st, (bcr_level0_kernel<<<dim3(ns * ((nx + 1) / 2), (nz + 31) / 32, (nz + 255) / 256), 128, 0, st>>>(
+                                          g, cp, D0, diag, tg)));
             const cudaError_t e2 = cudaGetLastError();
-            if (e2 != cudaSuccess) { helm_set_error("bcr: form blocks", e2); return HELM_ECUDA; }
+            if (e2 != cudaSuccess) { helm_set_error("bcr: level 0", e2); return HELM_ECUDA; }
             return HELM_OK;
         });
     }
-    const Fam fD{D, nz2, nz};
-    auto mat = [&](int kind, int sy, int slot) { return (int)bs_matrix_index(nx, ns, half, kind << 24 | slot, sy); };
-    int cur = 1, levels = 0;   // U, L of the spacing in buffer cur (from level 2 on)
-    for (int sp = 1; sp < nx; sp *= 2, ++levels) {
-        std::vector<int> inv_pairs, img_pairs, mdst;
+    int cur = 1, levels = 1;   // U, L of the spacing in buffer cur (from level 2 on)
+    for (int sp = 2; sp < nx; sp *= 2, ++levels) {
+        std::vector<int> inv_pairs, img_pairs;
         for (int sy = 0; sy < ns; ++sy)
             for (int j = sp; j < nx; j += 2 * sp) {
                 inv_pairs.insert(inv_pairs.end(), {sy * nx + j, sy * nx + j});
                 img_pairs.insert(img_pairs.end(), {sy * nx + j, mat(BS_DINV, sy, j)});
-                if (sp == 1) mdst.push_back((int)m0 + sy * m_stride + j / 2);
             }
-        // level 0: the line blocks are still tridiagonal
-        s = (sp == 1 && tri_level0) ? invert_tridiag_blocks(nz, fD, fD, inv_pairs, op->status, pl, tri)
-                                    : invert_blocks(nz, fD, fD, inv_pairs, op->status, pl);
-        if (s != HELM_OK) return s;
-        if ((s = image_blocks(g, D, img_pairs, mdst, ba, pl)) != HELM_OK) return s;
-        if (sp == 1) {
-            float2 *D0 = D;
-            const Coup cp = coup_of(g);
-            pl.ops.push_back([=](const int *) -> helm_status {
-                HELM_TRACED(K_BCR_L0, st, (bcr_level0_kernel<<<dim3(per, (nx + 1) / 2, ns), 256, 0, st>>>(g, cp, D0, tri_diag)));
-                const cudaError_t e2 = cudaGetLastError();
-                if (e2 != cudaSuccess) { helm_set_error("bcr: level 0", e2); return HELM_ECUDA; }
-                return HELM_OK;
-            });
-            continue;
-        }
+        if ((s = invert(inv_pairs, img_pairs)) != HELM_OK) return s;
         const int nxt = cur ^ 1;
         // couplings of line k to its neighbours at distance sp
         auto Uc = [&](int sy, int k) { return sp == 2 ? (int)m0 + sy * m_stride + k / 2 : (int)u_base(cur, 0) + sy * u_stride[cur] + k / sp; };
@@ -945,8 +1035,7 @@ helm_status bcr_factor(helm_factor_t *f) {
             last.insert(last.end(), {sy * nx, sy * nx});
             img_pairs.insert(img_pairs.end(), {sy * nx, mat(BS_DINV, sy, 0)});
         }
-        if ((s = invert_blocks(nz, fD, fD, last, op->status, pl)) != HELM_OK) return s;
-        if ((s = image_blocks(g, D, img_pairs, {}, ba, pl)) != HELM_OK) return s;
+        if ((s = invert(last, img_pairs)) != HELM_OK) return s;
         int *out = op->status + 2;   // the largest entry of the inverses (the matrices 0 .. ns nx - 1)
         const uint32_t *mxd = im.mx;
         pl.ops.push_back([=](const int *) -> helm_status {

@@ -6,8 +6,11 @@
 // tensor maps) through three stages, one thread issues the products (24 per chunk: hi hi, hi lo,
 // lo hi of Ar Br - Ai Bi and Ar Bi + Ai Br, FP16, N = 128), eight warps write the tile.
 // The tensor core adds into FP32 with truncation, so the number of additions into the large sum is
-// what limits the product: hi hi goes into an accumulator of its own (64 additions at n = 256; the
-// cross terms are 2^-11 of it), where the TF32 product of zgemm_tc.cu makes 192 of all three.
+// what limits the product (192 at n = 256 in zgemm_tc.cu).  Here every chunk of 32 columns goes
+// into a fresh accumulator, which the epilogue warps add to sums in registers, rounding to
+// nearest, while the next chunk runs into the other one: 24 additions of a chunk, n / 32 sums.  It
+// costs nothing (128 KB of tensor memory read per 1536 cycles of products) and leaves both
+// accumulators to the next tile while a tile is written.
 // An image's scale has to be known before the tile: 2^15 over the bound 2 n max|A| max|B|, which is
 // 2^5 to 2^10 above the true maximum (FP16 keeps 22 bits down to 2^-15 of the scale); the true
 // maximum is recorded on the way and bounds the next level.
@@ -32,7 +35,7 @@ constexpr size_t BG_SMEM = (size_t)BG_STAGES * BG_STAGE + 1024;
 
 __global__ void __launch_bounds__(BG_THREADS, 1) bcr_gemm_kernel(BgArgs a) {
     extern __shared__ uint8_t bg_smem[];
-    __shared__ __align__(8) uint64_t full[BG_STAGES], empty[BG_STAGES], acc_full, acc_empty, done_bar;
+    __shared__ __align__(8) uint64_t full[BG_STAGES], empty[BG_STAGES], acc_full[2], acc_empty[2], done_bar;
     __shared__ uint32_t s_tmem;
     __shared__ int s_abort;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -41,8 +44,10 @@ __global__ void __launch_bounds__(BG_THREADS, 1) bcr_gemm_kernel(BgArgs a) {
             mbar_init(&full[s], 1);
             mbar_init(&empty[s], 1);
         }
-        mbar_init(&acc_full, 1);
-        mbar_init(&acc_empty, BG_WARPS - BG_EPI0);
+        for (int s = 0; s < 2; ++s) {
+            mbar_init(&acc_full[s], 1);
+            mbar_init(&acc_empty[s], BG_WARPS - BG_EPI0);
+        }
         mbar_init(&done_bar, 1);
         fence_mbar_init_cluster();
         s_abort = 0;
@@ -98,32 +103,31 @@ __global__ void __launch_bounds__(BG_THREADS, 1) bcr_gemm_kernel(BgArgs a) {
         __syncwarp();
     } else if (warp == 0) {
         if (elect_one()) {   // MMA thread
-            int s = 0, i = 0;
+            int s = 0, cc = 0;
             uint32_t ph = 0;
             bool go = true;
             const uint64_t dstage0 = desc_sw128(smem0);
-            for (int t = blockIdx.x; go && t < a.n_tiles; t += gridDim.x, ++i) {
+            for (int t = blockIdx.x; go && t < a.n_tiles; t += gridDim.x) {
                 const int n0 = 128 * (t % a.nt), nb = min(128, (a.nzr - n0 + 15) & ~15);
                 const uint32_t id = idesc_f16(nb, false), idn = idesc_f16(nb, true);
-                if (!wait1(&acc_empty, (uint32_t)(i & 1) ^ 1u)) break;
-                for (int c = 0; c < a.n_chunk; ++c) {
-                    if (!wait1(&full[s], ph)) { go = false; break; }
+                for (int c = 0; c < a.n_chunk; ++c, ++cc) {
+                    if (!wait1(&acc_empty[cc & 1], (uint32_t)((cc >> 1) & 1) ^ 1u) || !wait1(&full[s], ph)) { go = false; break; }
                     tc_fence_after();
                     const uint64_t ar = dstage0 + (uint64_t)(s * (BG_STAGE / 16)), ai = ar + 1024, br = ar + 2048, bi = ar + 3072;
-                    // columns: hi hi Re, Im (0, 128), cross terms Re, Im (256, 384)
+                    const uint32_t d = tmem + (uint32_t)((cc & 1) * 256);   // Re, Im of the chunk
 #pragma unroll
-                    for (int p = 0; p < 6; ++p) {
-                        const int ka = (p >= 4 ? 4 : 0) + 2 * (p & 1), kb = ((p >> 1) == 1 ? 4 : 0) + 2 * (p & 1);
-                        const uint32_t d = tmem + (p < 2 ? 0u : 256u), acc = (p == 0 || p == 2) ? (c > 0 ? 1u : 0u) : 1u;
+                    for (int p = 0; p < 6; ++p) {   // cross terms first: hi*lo, lo*hi, then hi*hi, two K steps each
+                        const int ka = ((p >> 1) == 1 ? 4 : 0) + 2 * (p & 1), kb = (p < 2 ? 4 : 0) + 2 * (p & 1);
+                        const uint32_t acc = p > 0 ? 1u : 0u;
                         tc_mma_f16(d, ar + ka, br + kb, id, acc);
                         tc_mma_f16(d + 128, ar + ka, bi + kb, id, acc);
                         tc_mma_f16(d, ai + ka, bi + kb, idn, 1u);
                         tc_mma_f16(d + 128, ai + ka, br + kb, id, 1u);
                     }
                     tc_commit(&empty[s]);
+                    tc_commit(&acc_full[cc & 1]);
                     if (++s == BG_STAGES) { s = 0; ph ^= 1u; }
                 }
-                if (go) tc_commit(&acc_full);
             }
             tc_commit(&done_bar);
             mbar_wait_bounded(&done_bar, 0, kDefaultWaitTries);
@@ -132,81 +136,100 @@ __global__ void __launch_bounds__(BG_THREADS, 1) bcr_gemm_kernel(BgArgs a) {
     } else {
         // epilogue warps: tensor-memory lanes 32 q .. + 31 = rows m0 + 32 q + lane, 64 columns each
         const int q = warp & 3, hh = (warp - BG_EPI0) >> 2;
-        int i = 0;
+        int cc = 0;
+        bool go = true;
         const int n_cols = 32 * a.n_chunk;
-        for (int t = blockIdx.x; t < a.n_tiles; t += gridDim.x, ++i) {
+        for (int t = blockIdx.x; t < a.n_tiles; t += gridDim.x) {
             const int *task = a.tasks + BG_TASK * (t / per);
-            const int m0 = 128 * (t % per / a.nt), n0 = 128 * (t % a.nt), m = m0 + 32 * q + lane;
-            const int ia = task[1], ib = task[2], out = task[3];
-            const bool img_out = (task[0] & BG_FP32) == 0;
-            const float f = bs_pow2(max(-126, min(126, -(a.im.shift[ia] + a.im.shift[ib])))) * ((task[0] & BG_NEG) ? -1.f : 1.f);
+            const int m0 = 128 * (t % per / a.nt), n0 = 128 * (t % a.nt) + 64 * hh, m = m0 + 32 * q + lane;
+            const int flags = task[0], ia = task[1], ib = task[2], out = task[3];
+            const float f = bs_pow2(max(-126, min(126, -(a.im.shift[ia] + a.im.shift[ib])))) * ((flags & BG_NEG) ? -1.f : 1.f);
+            float re[64], im[64];
+#pragma unroll
+            for (int e = 0; e < 64; ++e) re[e] = im[e] = 0.f;
+            for (int c = 0; c < a.n_chunk; ++c, ++cc) {
+                const bool ok = mbar_wait_cta(&acc_full[cc & 1], (uint32_t)((cc >> 1) & 1), a.tries, &s_abort);
+                if (!__all_sync(0xffffffffu, ok)) {
+                    if (lane == 0) give_up();
+                    go = false;
+                    break;
+                }
+                tc_fence_after();
+                const uint32_t d = tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)((cc & 1) * 256 + 64 * hh);
+#pragma unroll
+                for (int g = 0; g < 8; g += 2) {
+                    uint32_t r0[8], r1[8], i0[8], i1[8];
+                    tc_ld8_issue(d + 8 * g, r0);
+                    tc_ld8_issue(d + 8 * g + 8, r1);
+                    tc_ld8_issue(d + 128 + 8 * g, i0);
+                    tc_ld8_issue(d + 128 + 8 * g + 8, i1);
+                    tc_wait_ld8(r0);
+                    tc_wait_ld8(r1);
+                    tc_wait_ld8(i0);
+                    tc_wait_ld8(i1);
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) {
+                        re[8 * g + e] += __uint_as_float(r0[e]);
+                        re[8 * g + 8 + e] += __uint_as_float(r1[e]);
+                        im[8 * g + e] += __uint_as_float(i0[e]);
+                        im[8 * g + 8 + e] += __uint_as_float(i1[e]);
+                    }
+                }
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive_cta(&acc_empty[cc & 1]);
+            }
+            if (!go) break;
             // image: the bound's scale
             const int eb = (int)(a.im.mx[ia] >> 23) + (int)(a.im.mx[ib] >> 23) - 254 + 2 + a.log2_2k;
             const int sh = max(-100, min(100, 15 - eb));
             const float sc = bs_pow2(sh);
-            if (img_out && t % per == 0 && warp == BG_EPI0 && lane == 0) a.im.shift[out] = sh;
-            const bool ok = mbar_wait_cta(&acc_full, (uint32_t)(i & 1), a.tries, &s_abort);
-            if (!__all_sync(0xffffffffu, ok)) {
-                if (lane == 0) give_up();
-                break;
-            }
-            tc_fence_after();
             uint32_t mxv = 0;
-            const uint32_t d = tmem + ((uint32_t)(32 * q) << 16);
-            float2 *dst = a.D + (size_t)out * a.nz * a.nz + (size_t)m * a.nz;
-            unsigned char *im = img_out ? a.im.at(out, a.mat_bytes) : nullptr;
-            for (int cb = 64 * hh; cb < 64 * hh + 64 && n0 + cb < n_cols; cb += 8) {
-                uint32_t hr[8], hi[8], xr[8], xi[8];
-                tc_ld8_issue(d + cb, hr);
-                tc_ld8_issue(d + 128 + cb, hi);
-                tc_ld8_issue(d + 256 + cb, xr);
-                tc_ld8_issue(d + 384 + cb, xi);
-                tc_wait_ld8(hr);
-                tc_wait_ld8(hi);
-                tc_wait_ld8(xr);
-                tc_wait_ld8(xi);
+            float2 *dst = a.D + (size_t)out * a.nz * a.nz + (size_t)m * a.nz;   // (BG_FP32)
+            unsigned char *img = (flags & BG_FP32) ? nullptr : a.im.at(out, a.mat_bytes);
+#pragma unroll
+            for (int g = 0; g < 8; ++g) {
+                const int nn = n0 + 8 * g;
+                if (nn >= n_cols) continue;
                 float2 v[8];
 #pragma unroll
                 for (int e = 0; e < 8; ++e) {
-                    const bool in = m < a.nz && n0 + cb + e < a.nz;
-                    v[e].x = in ? (__uint_as_float(hr[e]) + __uint_as_float(xr[e])) * f : 0.f;
-                    v[e].y = in ? (__uint_as_float(hi[e]) + __uint_as_float(xi[e])) * f : 0.f;
+                    const bool in = m < a.nz && nn + e < a.nz;
+                    v[e] = in ? make_float2(re[8 * g + e] * f, im[8 * g + e] * f) : make_float2(0.f, 0.f);
                 }
-                if (img_out) {
+                if (!img) {   // n is even: pairs of columns on 16-byte boundaries
+                    if (m < a.nz) {
+#pragma unroll
+                        for (int e = 0; e < 8; e += 2)
+                            if (nn + e < a.nz) {
+                                float4 *w = reinterpret_cast<float4 *>(dst + nn + e);
+                                const float4 o = *w;
+                                *w = make_float4(o.x + v[e].x, o.y + v[e].y, o.z + v[e + 1].x, o.w + v[e + 1].y);
+                            }
+                    }
+                    continue;
+                }
+                {
 #pragma unroll
                     for (int e = 0; e < 8; ++e) mxv = max(mxv, max(bs_abs_bits(v[e].x), bs_abs_bits(v[e].y)));
                     if (m < a.nzr) {   // 16-byte pieces of the row: eight columns' hi, and lo 64 bytes on
-                        const int c = (n0 + cb) >> 5, j = ((n0 + cb) >> 3) & 3;
+                        const int c = nn >> 5, j = (nn >> 3) & 3;
                         uint4 rh, rl, ih, il;
                         bs_split8(v, sc, rh, rl, ih, il);
-                        unsigned char *row = im + ((size_t)(2 * c) * a.nzr + m) * 128;
+                        unsigned char *row = img + ((size_t)(2 * c) * a.nzr + m) * 128;
                         *reinterpret_cast<uint4 *>(row + ((j ^ (m & 7)) << 4)) = rh;
                         *reinterpret_cast<uint4 *>(row + (((j + 4) ^ (m & 7)) << 4)) = rl;
                         row += (size_t)a.nzr * 128;
                         *reinterpret_cast<uint4 *>(row + ((j ^ (m & 7)) << 4)) = ih;
                         *reinterpret_cast<uint4 *>(row + (((j + 4) ^ (m & 7)) << 4)) = il;
                     }
-                } else if (m < a.nz) {   // n is even: pairs of columns on 16-byte boundaries
-#pragma unroll
-                    for (int e = 0; e < 8; e += 2)
-                        if (n0 + cb + e < a.nz) {
-                            float4 *p = reinterpret_cast<float4 *>(dst + n0 + cb + e);
-                            float4 o = *p;
-                            o.x += v[e].x;
-                            o.y += v[e].y;
-                            o.z += v[e + 1].x;
-                            o.w += v[e + 1].y;
-                            *p = o;
-                        }
                 }
             }
-            tc_fence_before();
-            if (img_out) {
+            if (img) {
+                if (t % per == 0 && warp == BG_EPI0 && lane == 0) a.im.shift[out] = sh;
                 mxv = __reduce_max_sync(0xffffffffu, mxv);
                 if (lane == 0 && mxv) atomicMax(a.im.mx + out, mxv);
             }
-            __syncwarp();
-            if (lane == 0) mbar_arrive_cta(&acc_empty);
         }
     }
     tc_fence_before();

@@ -616,40 +616,19 @@ __global__ void __launch_bounds__(256) bcr_max_kernel(long long n2, const float2
     if ((threadIdx.x & 31) == 0) atomicMax(mx + pr[1], m);
 }
 
-// Image of a block (n x n row-major) as matrix pairs[.][1]; with mdst, also of -C block C (C =
-// diag(cx), the coupling of a level-0 inverse) as matrix mdst[.].  A CTA takes 32 rows, a thread a
-// row and eight columns at a time; rows and columns beyond n are zero.
+// Image of a block (n x n row-major) as matrix pairs[.][1].  A CTA takes 32 rows, a thread a row
+// and eight columns at a time; rows and columns beyond n are zero.
 __global__ void __launch_bounds__(128) bcr_image_kernel(int n, int n_chunk, int nzr, const float2 *src, long long stride,
-                                                        const int *pairs, const int *mdst, float cx_in, float cx_edge,
-                                                        BsImages im, size_t mat_bytes) {
+                                                        const int *pairs, BsImages im, size_t mat_bytes) {
     __shared__ float2 t[32][33];
     const int *pr = pairs + 2 * (size_t)blockIdx.y;
     const float2 *A = src + (long long)pr[0] * stride;
     const int r0 = 32 * blockIdx.x, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const uint32_t m0 = im.mx[pr[1]];
-    const int sh = bs_scale_shift(m0), md = mdst ? mdst[blockIdx.y] : -1;
-    const uint32_t m1 = bs_abs_bits(__uint_as_float(m0) * cx_in * cx_in);   // (the edge coupling is half the inner one)
-    const int shm = bs_scale_shift(m1);
-    const float sc = bs_pow2(sh), scm = bs_pow2(shm);
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        im.shift[pr[1]] = sh;
-        if (md >= 0) {
-            im.shift[md] = shm;
-            im.mx[md] = m1;
-        }
-    }
+    const int sh = bs_scale_shift(im.mx[pr[1]]);
+    const float sc = bs_pow2(sh);
+    if (blockIdx.x == 0 && threadIdx.x == 0) im.shift[pr[1]] = sh;
     const int row = threadIdx.x >> 2, j = threadIdx.x & 3, r = r0 + row;
-    const float cr = (r == 0 || r == n - 1) ? cx_edge : cx_in;
-    auto put = [&](int mat, int c, float s, const float2 (&v)[8]) {
-        uint4 rh, rl, ih, il;
-        bs_split8(v, s, rh, rl, ih, il);
-        unsigned char *d = im.at(mat, mat_bytes) + ((size_t)(2 * c) * nzr + r) * 128;
-        *reinterpret_cast<uint4 *>(d + ((j ^ (r & 7)) << 4)) = rh;
-        *reinterpret_cast<uint4 *>(d + (((j + 4) ^ (r & 7)) << 4)) = rl;
-        d += (size_t)nzr * 128;
-        *reinterpret_cast<uint4 *>(d + ((j ^ (r & 7)) << 4)) = ih;
-        *reinterpret_cast<uint4 *>(d + (((j + 4) ^ (r & 7)) << 4)) = il;
-    };
+    unsigned char *d = im.at(pr[1], mat_bytes) + (size_t)r * 128;
     for (int c = 0; c < n_chunk; ++c) {
 #pragma unroll
         for (int q = 0; q < 8; ++q) {
@@ -661,17 +640,14 @@ __global__ void __launch_bounds__(128) bcr_image_kernel(int n, int n_chunk, int 
             float2 v[8];
 #pragma unroll
             for (int e = 0; e < 8; ++e) v[e] = t[row][8 * j + e];
-            put(pr[1], c, sc, v);
-            if (md >= 0) {
-#pragma unroll
-                for (int e = 0; e < 8; ++e) {
-                    const int k = 32 * c + 8 * j + e;
-                    const float f = -cr * ((k == 0 || k == n - 1) ? cx_edge : cx_in);
-                    v[e].x *= f;
-                    v[e].y *= f;
-                }
-                put(md, c, scm, v);
-            }
+            uint4 rh, rl, ih, il;
+            bs_split8(v, sc, rh, rl, ih, il);
+            *reinterpret_cast<uint4 *>(d + ((j ^ (r & 7)) << 4)) = rh;
+            *reinterpret_cast<uint4 *>(d + (((j + 4) ^ (r & 7)) << 4)) = rl;
+            d += (size_t)nzr * 128;
+            *reinterpret_cast<uint4 *>(d + ((j ^ (r & 7)) << 4)) = ih;
+            *reinterpret_cast<uint4 *>(d + (((j + 4) ^ (r & 7)) << 4)) = il;
+            d += (size_t)nzr * 128;
         }
         __syncthreads();
     }
@@ -687,8 +663,8 @@ template <int NT> cudaError_t launch_nt(const BsArgs &a, int grid, double flops,
 
 }  // namespace
 
-cudaError_t launch_bcr_image(int n, const float2 *src, long long stride, const int *pairs_dev, const int *mdst_dev,
-                             int count, float cx_in, float cx_edge, const BsImages &im, cudaStream_t st) {
+cudaError_t launch_bcr_image(int n, const float2 *src, long long stride, const int *pairs_dev, int count,
+                             const BsImages &im, cudaStream_t st) {
     if (count <= 0) return cudaSuccess;
     const BsLayout l = bs_layout(n);
     for (int t = 0; t < count; t += 65535) {
@@ -697,8 +673,7 @@ cudaError_t launch_bcr_image(int n, const float2 *src, long long stride, const i
         HELM_TRACED(K_BCR_IMAGE, st, (bcr_max_kernel<<<dim3((unsigned)std::min(8, (n * n / 2 + 1023) / 1024), nb), 256, 0, st>>>(
                                          (long long)n * n, src, stride, pr, im.mx)));
         HELM_TRACED(K_BCR_IMAGE, st, (bcr_image_kernel<<<dim3((n + 31) / 32, nb), 128, 0, st>>>(
-                                         n, l.n_chunk, l.nzr, src, stride, pr, mdst_dev ? mdst_dev + t : nullptr, cx_in,
-                                         cx_edge, im, l.mat_bytes)));
+                                         n, l.n_chunk, l.nzr, src, stride, pr, im, l.mat_bytes)));
     }
     return cudaGetLastError();
 }

@@ -72,10 +72,10 @@ struct BsImages {
         return i < n_kept ? kept + (size_t)i * mat_bytes : work + (size_t)(i - n_kept) * mat_bytes;
     }
 };
-// images of n x n row-major blocks src + pairs[.][0] * stride as matrices pairs[.][1], and of
-// -C block C (C = diag(cx)) as matrices mdst[.] (mdst null: none); im.mx zeroed beforehand
-cudaError_t launch_bcr_image(int n, const float2 *src, long long stride, const int *pairs_dev, const int *mdst_dev,
-                             int count, float cx_in, float cx_edge, const BsImages &im, cudaStream_t st);
+// images of n x n row-major blocks src + pairs[.][0] * stride as matrices pairs[.][1]; im.mx zeroed
+// beforehand
+cudaError_t launch_bcr_image(int n, const float2 *src, long long stride, const int *pairs_dev, int count,
+                             const BsImages &im, cudaStream_t st);
 
 // Products of images (bcr_gemm.cu): tasks of BG_TASK ints (flags, matrix A, matrix B, output): the
 // image of +-A B^T as matrix `output`, or (BG_FP32) D block `output` += +-A B^T

@@ -314,17 +314,6 @@ __device__ void polish_inverse16(const float2 *M, int ld, int kb, float2 *P, flo
     __syncthreads();
 }
 
-// 1 / x in FP64 to the last bit or two: the FP32 reciprocal and two Newton steps.  (The FP64 pipe
-// issues a warp instruction in 16 to 64 cycles here, so the division's thirty dependent ones cost
-// a pivot column more than the column itself.)  Outside FP32's comfortable range: __drcp_rn.
-__device__ __forceinline__ double fast_recip(double x) {
-    const float xf = (float)x;
-    if (!(xf > 1e-30f && xf < 1e30f)) return __drcp_rn(x);
-    double y = (double)__frcp_rn(xf);
-    y = fma(y, fma(-x, y, 1.0), y);
-    return fma(y, fma(-x, y, 1.0), y);
-}
-
 // FP64 inverse of the kb x kb block M (shared, row stride ld; the rest of the 16 x 16 tile taken as
 // the identity) into P (row stride NB) by the 256 threads of the CTA, thread (r, c) holding one
 // entry: Gauss-Jordan in place with partial pivoting, A (16 x 17) and B ping-pong, two barriers a

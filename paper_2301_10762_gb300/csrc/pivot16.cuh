@@ -73,4 +73,15 @@ __device__ bool warp_invert16(const cx_t<T> *M, int ld, int kb, cx_t<T> *P) {
 }
 
 
+// 1 / x in FP64 to the last bit or two: the FP32 reciprocal and two Newton steps.  (The FP64 pipe
+// issues a warp instruction in 16 to 64 cycles here, so the division's thirty dependent ones cost
+// a pivot column more than the column itself.)  Outside FP32's comfortable range: __drcp_rn.
+__device__ __forceinline__ double fast_recip(double x) {
+    const float xf = (float)x;
+    if (!(xf > 1e-30f && xf < 1e30f)) return __drcp_rn(x);
+    double y = (double)__frcp_rn(xf);
+    y = fma(y, fma(-x, y, 1.0), y);
+    return fma(y, fma(-x, y, 1.0), y);
+}
+
 }  // namespace helm

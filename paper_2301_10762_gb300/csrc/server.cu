@@ -89,9 +89,9 @@ struct helm_server {
         if (helm::factor_picks_bcr(geom, (helm_prec)prec, HELM_FACTOR_AUTO)) {
             // block cyclic reduction: the images of every line's inverse and of P, Q, W, V of the
             // eliminated ones, and while it factors (counted throughout) 1.25 n_x images of
-            // couplings and the FP32 diagonal blocks
+            // couplings, the FP32 diagonal blocks and level 0's generators
             const size_t kept = (size_t)g.nx + 4 * ((size_t)g.nx / 2 + 1), work = 5 * (size_t)g.nx / 4 + 5;
-            return (kept + work) * (helm::bs_layout(g.nz).mat_bytes + 8) + g.nx * blk + 96 * N + 65 * kMiB;   // + split-K tiles
+            return (kept + work) * (helm::bs_layout(g.nz).mat_bytes + 8) + g.nx * blk + 144 * N + 65 * kMiB;   // + split-K tiles
         }
         return (size_t)g.nx * g.nz * g.nz * (prec == HELM_MIXED ? 8 : 16) + 96 * N + kMiB;
     }

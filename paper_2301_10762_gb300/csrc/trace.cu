@@ -14,7 +14,7 @@ static const char *kNames[K_COUNT] = {
     "g_u_p_rhs", "z_rhs_base", "hess_accumulate", "hyper_terms", "dot_partial", "sum_partials", "axpby",
     "fill", "sub", "regR", "dct_table", "dct_pass", "line_gb_prepass", "split_diag", "refine_start", "refine_update",
     "refine_finish", "refine_accumulate", "field_grad", "g_coefficients", "hess_finish",
-    "zgemm_tf32x3", "zinv_block", "bcr_form_blocks", "bcr_level0_update", "bcr_solve",
+    "zgemm_tf32x3", "zinv_block", "bcr_level0_update", "bcr_solve",
     "zgemm_split_reduce", "bcr_image", "line_max", "bcr_gemm",
 };
 
