@@ -58,7 +58,6 @@ namespace helm {
 
 namespace {
 
-constexpr int INV_THREADS = 512;
 constexpr int INV_MAX = 128;   // largest block inverted in one CTA's shared memory
 
 // ------------------------------------------------------------------- kernels
@@ -338,113 +337,89 @@ __device__ __forceinline__ long long op_off(int idx, int div, long long stride, 
     return div > 0 ? (long long)(idx / div) * stride_hi + (long long)(idx % div) * stride : (long long)idx * stride;
 }
 
-// X = M^{-1} of one n x n block (n <= 128) per CTA, in shared memory: block Gauss-Jordan over
-// 16-column blocks; the pivot block is inverted by one warp with partial pivoting, the other
-// rows get the rank-16 update from the staged old column panel U and R = P M[k rows, :].
-__global__ void __launch_bounds__(INV_THREADS, 1) zinv_base_kernel(InvArgs a) {
-    extern __shared__ __align__(16) unsigned char inv_smem[];
-    const int n = a.n, ldw = n + 1, tid = threadIdx.x;
-    float2 *W = reinterpret_cast<float2 *>(inv_smem);          // n x ldw
-    float2 *U = W + (size_t)n * ldw;                             // n x 16: old column panel
-    float2 *R = U + (size_t)n * PIV;                             // 16 x ldw: P times the pivot rows
-    float2 *P = R + (size_t)PIV * ldw;                           // 16 x 16: pivot-block inverse
-    __shared__ int s_bad;
-    const int *ix = a.idx + 2 * (size_t)blockIdx.x;
-    const float2 *M = a.in.base + op_off(ix[0], a.in.div, a.in.stride, a.in.stride_hi);
-    float2 *X = a.out + op_off(ix[1], a.out_div, a.out_stride, a.out_stride_hi);
-    if (tid == 0) s_bad = 0;
-    for (int e = tid; e < n * n; e += INV_THREADS) {
-        const int r = e / n, c = e % n;
-        W[(size_t)r * ldw + c] = M[(size_t)r * a.in.ld + c];
-    }
-    __syncthreads();
-    // update mapping: thread -> column c, row group rg (rows rg, rg + ng, ...)
-    const int ng = INV_THREADS / n, c = tid % n, rg = tid / n;
-    const int nb = (n + PIV - 1) / PIV;
-    for (int kb_i = 0; kb_i < nb; ++kb_i) {
-        const int k0 = kb_i * PIV, kb = min(PIV, n - k0);
-        for (int e = tid; e < n * PIV; e += INV_THREADS) {
-            const int r = e / PIV, u = e % PIV;
-            U[e] = u < kb ? W[(size_t)r * ldw + k0 + u] : make_float2(0.f, 0.f);
-        }
-        if (tid < 32) {
-            if (!warp_invert16<float>(W + (size_t)k0 * ldw + k0, ldw, kb, P) && tid == 0) s_bad = 1;
-        }
-        __syncthreads();
-        for (int e = tid; e < PIV * n; e += INV_THREADS) {
-            const int q = e / n, cc = e % n;
-            if (q < kb && (cc < k0 || cc >= k0 + kb)) {
-                float2 acc = make_float2(0.f, 0.f);
-                for (int u = 0; u < kb; ++u) cfma(acc, P[q * PIV + u], W[(size_t)(k0 + u) * ldw + cc]);
-                R[(size_t)q * ldw + cc] = acc;
-            }
-        }
-        __syncthreads();
-        if (rg < ng) {
-            const bool inblk = c >= k0 && c < k0 + kb;
-            float2 col[PIV];   // the R (or P) column this thread multiplies with
-#pragma unroll
-            for (int u = 0; u < PIV; ++u)
-                col[u] = u < kb ? (inblk ? P[u * PIV + (c - k0)] : R[(size_t)u * ldw + c]) : make_float2(0.f, 0.f);
-            for (int r = rg; r < n; r += ng) {
-                float2 *w = W + (size_t)r * ldw + c;
-                if (r >= k0 && r < k0 + kb) {
-                    *w = inblk ? P[(r - k0) * PIV + (c - k0)] : R[(size_t)(r - k0) * ldw + c];
-                    continue;
-                }
-                const float4 *ur = reinterpret_cast<const float4 *>(U + (size_t)r * PIV);
-                float2 p[4] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
-#pragma unroll
-                for (int h = 0; h < PIV / 2; ++h) {
-                    const float4 q = ur[h];
-                    cfma(p[(2 * h) & 3], make_float2(q.x, q.y), col[2 * h]);
-                    cfma(p[(2 * h + 1) & 3], make_float2(q.z, q.w), col[2 * h + 1]);
-                }
-                const float2 sum = make_float2((p[0].x + p[1].x) + (p[2].x + p[3].x), (p[0].y + p[1].y) + (p[2].y + p[3].y));
-                const float2 old = inblk ? make_float2(0.f, 0.f) : *w;
-                *w = make_float2(old.x - sum.x, old.y - sum.y);
-            }
-        }
-        __syncthreads();
-    }
-    for (int e = tid; e < n * n; e += INV_THREADS) {
-        const int r = e / n, cc = e % n;
-        X[(size_t)r * a.ldo + cc] = W[(size_t)r * ldw + cc];
-    }
-    if (tid == 0 && s_bad) atomicOr(a.status, ST_SINGULAR);
-}
-
-// X = M^{-1} of one 128 x 128 block per CTA with the block in tensor memory: lane r holds row r,
-// 256 FP32 columns (column 2c the real, 2c + 1 the imaginary part of entry c).  Each
-// Gauss-Jordan step (16 pivot columns K = k0 .. k0 + 15) is
-//     W <- W' + A' R'  (W' = W with the rows and columns K zeroed in tensor memory;
+// X = M^{-1} of one n x n block (n <= 128) per CTA by Gauss-Jordan in steps of 16 columns, partial
+// pivoting inside each 16 x 16 pivot block.  The block lives in registers: thread (r, h) of
+// 512 holds row r, columns 32 h .. + 31 (beyond n: the identity).  A step with the pivot columns
+// K = k0 .. k0 + 15 is
+//     W <- W' + A' R'  (W' = W with the rows and columns K zeroed;
 //                       A'[r][u] = -W[r][k0 + u] off the pivot rows, delta(r - k0, u) on them;
 //                       R' = P W[K, :] off the pivot columns, P on them, P = W[K, K]^{-1}),
-// one tcgen05 3xTF32 product of M = 128, N = 256 (R' expanded to real rows as in the GEMM),
-// K = 32, accumulated into W itself.  Shared memory holds only the product's operands, the
-// pivot rows and the 16 x 16 blocks (~103 KB), so that two CTAs share an SM and one's pivot
-// chain (one warp) overlaps the other's work.  Warp w owns tensor-memory lanes 32 (w mod 4) ..
-// + 31 and columns 128 (w / 4) .. + 127.
-constexpr int ZT_THREADS = 256;
-constexpr int ZT_WS = 129;   // pivot rows W[K, :] in shared memory: row stride (complex)
-constexpr int ZT_PS = 17;    // padded copy of P
-constexpr uint32_t ZT_A = 0, ZT_B = 32768, ZT_PK = 98304, ZT_P = ZT_PK + 2048, ZT_PPAD = ZT_P + 2048;
-size_t zinv128_tm_smem_bytes() { return (size_t)ZT_PPAD + sizeof(float2) * PIV * ZT_PS + 1024; }
+// one 3xTF32 product of M = 128, N = 2 n, K = 32 reals (R' expanded to real rows) into a fresh
+// accumulator in tensor memory, which the threads add to W: the tensor core truncates every sum,
+// and a step that accumulated into W itself lost up to an ulp of W twelve times over, which cost
+// the inverses of the upper levels a factor of 30 (3e-5 of their norm).
+// The chain of pivot blocks is what bounds it, so it runs ahead of the rest: warps 0 to 7 update the
+// next pivot block W[K1, K1] first and warp 0 inverts it while the other warps form R',
+// the tensor core multiplies and W is updated.
+constexpr int ZT_THREADS = 512;
+constexpr int ZT_WS = 129, ZT_PS = 17;   // row strides (complex) of the pivot rows and of the 16 x 16 blocks
+constexpr int ZT_TS = 65;                // row stride (complex) of half a block on its way in or out
+constexpr uint32_t ZT_A = 0, ZT_B = 32768, ZT_WK = 98304, ZT_P = ZT_WK + 8 * PIV * ZT_WS, ZT_BLK = ZT_P + 2 * 8 * PIV * PIV;
+constexpr size_t ZT_SMEM = ZT_BLK + 4 * 8 * PIV * ZT_PS + 1024;
 
-__global__ void __launch_bounds__(ZT_THREADS, 2) zinv128_tm_kernel(InvArgs a) {
+// 16 x 16 inverse in place by one warp: lane (r, h) holds row r, columns 8 h .. + 7 of M (shared, row
+// stride ZT_PS); P row stride 16.  Gauss-Jordan with partial pivoting without row swaps: at step
+// q the row p_q eliminates column q, whose slot then holds column p_q of the inverse.  Bounds: the
+// chain of a column (maximum, broadcast, reciprocal, update, about 200 cycles); the augmented form
+// [M | I] of warp_invert16 has twice the shuffles and products per lane.  False if a pivot was zero
+// or not finite.
+__device__ bool warp_invert16_inplace(const float2 *M, float2 *P) {
+    const int lane = threadIdx.x & 31, r = lane & 15, h = lane >> 4;
+    float2 a[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) a[j] = M[r * ZT_PS + 8 * h + j];
+    unsigned used = 0;
+    unsigned long long perm = 0;
+    int qinv = 0;
+    bool ok = true;
+#pragma unroll
+    for (int q = 0; q < 16; ++q) {
+        const int src = r + 16 * (q >> 3);
+        const float2 f = make_float2(__shfl_sync(0xffffffffu, a[q & 7].x, src), __shfl_sync(0xffffffffu, a[q & 7].y, src));
+        const float mag = f.x * f.x + f.y * f.y, rd = __frcp_rn(mag);
+        unsigned key = (__float_as_uint(fminf(mag, 3.0e38f)) & ~0xFu) | (unsigned)(15 - r);
+        if (!(isfinite(f.x) && isfinite(f.y))) key = 0xFFFFFFF0u | (unsigned)(15 - r);
+        if ((used >> r) & 1u) key = 0u;
+        const unsigned best = __reduce_max_sync(0xffffffffu, key);
+        const int p = 15 - (int)(best & 0xFu);
+        if ((best >> 4) == 0u || (best >> 23) >= 255u) ok = false;
+        used |= 1u << p;
+        perm |= (unsigned long long)p << (4 * q);
+        // (every lane's reciprocal, next to the maximum: off the chain)
+        const float2 inv = make_float2(__shfl_sync(0xffffffffu, f.x * rd, p), __shfl_sync(0xffffffffu, -f.y * rd, p));
+        const bool mine = r == p;
+        if (mine) qinv = q;
+        const float2 g = mine ? make_float2(-inv.x, -inv.y) : cmul(f, inv);
+        const int ps = p + 16 * h;
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            const float2 pj = make_float2(__shfl_sync(0xffffffffu, a[j].x, ps), __shfl_sync(0xffffffffu, a[j].y, ps));
+            float2 o = mine ? make_float2(0.f, 0.f) : a[j];
+            cfms(o, g, pj);
+            a[j] = o;
+        }
+        if (h == (q >> 3)) a[q & 7] = make_float2(-g.x, -g.y);
+    }
+#pragma unroll
+    for (int j = 0; j < 8; ++j) P[qinv * PIV + (int)((perm >> (4 * (8 * h + j))) & 15)] = a[j];
+    return ok;
+}
+
+__global__ void __launch_bounds__(ZT_THREADS, 1) zinv_kernel(InvArgs a) {
     extern __shared__ __align__(16) unsigned char zt_smem[];
     __shared__ __align__(8) uint64_t mma_bar;
     __shared__ uint32_t s_tmem;
     __shared__ int s_bad;
-    constexpr int n = 128;
+    const int n = a.n, nb = (n + PIV - 1) / PIV, np = nb * PIV;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int q = warp & 3, hh = warp >> 2, r = 32 * q + lane;
+    const int q = warp & 3, h = warp >> 2, r = 32 * q + lane, lr = lane & 15, lh = lane >> 4;
     const uint32_t base = (smem_u32(zt_smem) + 1023u) & ~1023u;
     unsigned char *gbase = zt_smem + (base - smem_u32(zt_smem));
-    float2 *Wk = reinterpret_cast<float2 *>(gbase + ZT_A);      // [16][ZT_WS], aliases the A tiles
-    float2 *Pk = reinterpret_cast<float2 *>(gbase + ZT_PK);     // [16][16]: the pivot block
-    float2 *P = reinterpret_cast<float2 *>(gbase + ZT_P);       // [16][16]: its inverse
-    float2 *Ps = reinterpret_cast<float2 *>(gbase + ZT_PPAD);   // [16][ZT_PS]: padded copy
+    float2 *Wk = reinterpret_cast<float2 *>(gbase + ZT_WK);      // [16][ZT_WS]: the pivot rows
+    float2 *Pb = reinterpret_cast<float2 *>(gbase + ZT_P);       // [2][16][16]: the pivot block's inverse, of even and odd steps
+    float2 *Nd = reinterpret_cast<float2 *>(gbase + ZT_BLK);     // [16][ZT_PS] each: W[K1, K1],
+    float2 *Un = Nd + PIV * ZT_PS, *Rn = Un + PIV * ZT_PS;       // W[K1, K] and R'[:, K1] of the next block,
+    float2 *Sn = Rn + PIV * ZT_PS;                               // and the next pivot block
     const uint32_t a_hi = base + ZT_A, a_lo = a_hi + 16384, b_hi = base + ZT_B, b_lo = b_hi + 32768;
     const int *ix = a.idx + 2 * (size_t)blockIdx.x;
     const float2 *M = a.in.base + op_off(ix[0], a.in.div, a.in.stride, a.in.stride_hi);
@@ -460,165 +435,211 @@ __global__ void __launch_bounds__(ZT_THREADS, 2) zinv128_tm_kernel(InvArgs a) {
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
+    // the block through shared memory, 64 columns at a time: whole rows of memory, a thread its own row
+    float2 *T = reinterpret_cast<float2 *>(gbase);
+    float2 w[32];
+#pragma unroll 1
+    for (int half = 0; half < 2; ++half) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const int rr = 8 * warp + i;
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                const int c = 64 * half + 32 * e + lane;
+                T[rr * ZT_TS + 32 * e + lane] =
+                    rr < n && c < n ? M[(size_t)rr * a.in.ld + c] : make_float2(rr == c ? 1.f : 0.f, 0.f);
+            }
+        }
+        __syncthreads();
+        if ((h >> 1) == half) {
+#pragma unroll
+            for (int i = 0; i < 32; ++i) w[i] = T[r * ZT_TS + 32 * (h & 1) + i];
+        }
+        __syncthreads();
+    }
+    // 16 columns of w by a warp-uniform half
+    auto copy16 = [&](float2 *dst, int half) {
+#pragma unroll
+        for (int u = 0; u < PIV; ++u) dst[lr * ZT_PS + u] = half ? w[16 + u] : w[u];
+    };
+    if (warp == 0 && lh == 0) copy16(Sn, 0);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t trow = s_tmem + ((uint32_t)(32 * q) << 16);   // this warp's lanes, column 0
-    // the block into tensor memory: lane r, columns 128 hh .. + 127
-#pragma unroll 1
-    for (int ch = 0; ch < 8; ++ch) {
-        const int col = 128 * hh + 16 * ch, c0 = col / 2;
-        float v[16];
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            const float2 e = M[(size_t)r * a.in.ld + c0 + i];
-            v[2 * i] = e.x;
-            v[2 * i + 1] = e.y;
-        }
-        tc_st16(trow + (uint32_t)col, v);
+    const uint32_t trow = s_tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(64 * h);   // this thread's lane and columns
+    if (warp == 0) {
+        if (!warp_invert16_inplace(Sn, Pb) && lane == 0) s_bad = 1;
     }
-    tc_wait_st();
-    constexpr uint32_t idesc = idesc_tf32(256);
+    const uint32_t idesc = idesc_tf32(2 * np);
     int phase = 0;
     bool aborted = false;
 #pragma unroll 1
-    for (int kb = 0; kb < n / PIV; ++kb) {
-        const int k0 = kb * PIV, qk = k0 >> 5, rk0 = k0 & 31;
-        const bool krow = q == qk && lane >= rk0 && lane < rk0 + PIV;   // this lane's row is a pivot row
-        tc_fence_before();
-        __syncthreads();   // the previous step's tensor-memory reads and shared-memory reads are done
-        tc_fence_after();
-        // (a) the column panel W[r][k0 + u], u = 8 hh .. 8 hh + 7 (kept for A'); the pivot block
-        float uf[16];
-        tc_ld16(trow + (uint32_t)(2 * k0 + 16 * hh), uf);
+    for (int kb = 0; kb < nb; ++kb) {
+        const int k0 = kb * PIV, bk = k0 >> 5, hf = kb & 1, k1 = k0 + PIV, bk1 = k1 >> 5, hf1 = hf ^ 1;
+        const bool krow = q == bk && lh == hf;           // this lane's row is a pivot row
+        const bool nrow = q == bk1 && lh == hf1;         // ... of the next step
+        // (a) the pivot rows; the column panel as A' and for the next pivot block; rows and columns
+        // K zeroed
+        if (nrow && h == bk1) copy16(Nd, hf1);
+        if (h == bk) {
+            if (nrow) copy16(Un, hf);
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                float4 v;
+                if (krow) {
+                    v = make_float4(lr == 2 * j ? 1.f : 0.f, 0.f, lr == 2 * j + 1 ? 1.f : 0.f, 0.f);
+                } else {
+                    const float2 u0 = hf ? w[16 + 2 * j] : w[2 * j], u1 = hf ? w[17 + 2 * j] : w[2 * j + 1];
+                    v = make_float4(-u0.x, -u0.y, -u1.x, -u1.y);
+                }
+                float4 hi, lo;
+                split4(v, 1.f, hi, lo);
+                st_shared_v4(a_hi + sw128(r, j), hi);
+                st_shared_v4(a_lo + sw128(r, j), lo);
+            }
+        }
         if (krow) {
 #pragma unroll
-            for (int i = 0; i < 8; ++i) Pk[(lane - rk0) * PIV + 8 * hh + i] = make_float2(uf[2 * i], uf[2 * i + 1]);
-        }
-        // (b) the pivot rows' quarter: rows K to shared memory, then W' (rows K and columns K
-        // zeroed) back; (c) the other quarters: columns K zeroed
-        if (q == qk) {
-#pragma unroll 1
-            for (int ch = 0; ch < 8; ++ch) {
-                const int col = 128 * hh + 16 * ch;
-                float v[16];
-                tc_ld16(trow + (uint32_t)col, v);
-                if (krow) {
-#pragma unroll
-                    for (int i = 0; i < 8; ++i) Wk[(lane - rk0) * ZT_WS + col / 2 + i] = make_float2(v[2 * i], v[2 * i + 1]);
-                }
-                const bool kcol = col >= 2 * k0 && col < 2 * k0 + 2 * PIV;
-                if (krow || kcol) {
-#pragma unroll
-                    for (int i = 0; i < 16; ++i) v[i] = 0.f;
-                }
-                tc_st16(trow + (uint32_t)col, v);
+            for (int i = 0; i < 32; ++i) {
+                Wk[lr * ZT_WS + 32 * h + i] = w[i];
+                w[i] = make_float2(0.f, 0.f);
             }
-        } else {
-            float z[16];
-#pragma unroll
-            for (int i = 0; i < 16; ++i) z[i] = 0.f;
-            tc_st16(trow + (uint32_t)(2 * k0 + 16 * hh), z);
         }
-        tc_wait_st();
-        __syncthreads();
-        // (d) the pivot block's inverse (one warp), and its padded copy
-        if (warp == 0) {
-            if (!warp_invert16<float>(Pk, PIV, PIV, P) && lane == 0) s_bad = 1;
+        if (h == bk) {
+#pragma unroll
+            for (int u = 0; u < PIV; ++u) {
+                if (hf) w[16 + u] = make_float2(0.f, 0.f);
+                else w[u] = make_float2(0.f, 0.f);
+            }
+        }
+        fence_proxy_async_smem();   // the A tiles, before the tensor core reads them
+        __syncthreads();   // (P of this step was written before the last barrier)
+        const float2 *P = Pb + hf * PIV * PIV;
+        // (b) the next pivot block: R'[:, K1], then W[K1, K1] - W[K1, K] R'[:, K1], and its inverse
+        if (kb + 1 < nb && warp < 8) {
+            const int i = tid >> 4, c = tid & 15;
+            float2 s0 = make_float2(0.f, 0.f), s1 = make_float2(0.f, 0.f);
+#pragma unroll
+            for (int u = 0; u < PIV; u += 2) {
+                cfma(s0, P[i * PIV + u], Wk[u * ZT_WS + k1 + c]);
+                cfma(s1, P[i * PIV + u + 1], Wk[(u + 1) * ZT_WS + k1 + c]);
+            }
+            Rn[i * ZT_PS + c] = make_float2(s0.x + s1.x, s0.y + s1.y);
+            asm volatile("bar.sync 1, 256;" ::: "memory");
+            s0 = Nd[i * ZT_PS + c];
+            s1 = make_float2(0.f, 0.f);
+#pragma unroll
+            for (int u = 0; u < PIV; u += 2) {
+                cfms(s0, Un[i * ZT_PS + u], Rn[u * ZT_PS + c]);
+                cfms(s1, Un[i * ZT_PS + u + 1], Rn[(u + 1) * ZT_PS + c]);
+            }
+            Sn[i * ZT_PS + c] = make_float2(s0.x + s1.x, s0.y + s1.y);
+            asm volatile("bar.sync 1, 256;" ::: "memory");
+            if (warp == 0 && !warp_invert16_inplace(Sn, Pb + hf1 * PIV * PIV) && lane == 0) s_bad = 1;
+        }
+        if (warp > 0) {
+            // (c) R' and the expanded B tiles: 32 columns c and u = 2j, 2j + 1 at a time; B row 2c = (Re,
+            // -Im), row 2c + 1 = (Im, Re) of R'[u][c], split into hi and lo
+#pragma unroll 1
+            for (int it = warp - 1; it < 32; it += 15) {
+                const int c = 32 * (it & 3) + lane, j = it >> 2;
+                if (c >= np) continue;
+                float2 x0, x1;
+                const float2 *p0 = P + 2 * j * PIV;
+                if (c >= k0 && c < k1) {
+                    x0 = p0[c - k0];
+                    x1 = p0[PIV + c - k0];
+                } else {
+                    x0 = x1 = make_float2(0.f, 0.f);
+#pragma unroll
+                    for (int v = 0; v < PIV; v += 2) {
+                        const float2 w0 = Wk[v * ZT_WS + c], w1 = Wk[(v + 1) * ZT_WS + c];
+                        const float4 a0 = *reinterpret_cast<const float4 *>(p0 + v);
+                        const float4 a1 = *reinterpret_cast<const float4 *>(p0 + PIV + v);
+                        cfma(x0, make_float2(a0.x, a0.y), w0);
+                        cfma(x1, make_float2(a1.x, a1.y), w0);
+                        cfma(x0, make_float2(a0.z, a0.w), w1);
+                        cfma(x1, make_float2(a1.z, a1.w), w1);
+                    }
+                }
+                // (lanes 4 apart start with different rows: eight distinct bank groups)
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {
+                    const bool im = ((lane >> 2) & 1) != e;
+                    float4 hi, lo;
+                    split4(im ? make_float4(x0.y, x0.x, x1.y, x1.x) : make_float4(x0.x, -x0.y, x1.x, -x1.y), 1.f, hi, lo);
+                    st_shared_v4(b_hi + sw128(2 * c + im, j), hi);
+                    st_shared_v4(b_lo + sw128(2 * c + im, j), lo);
+                }
+            }
+            fence_proxy_async_smem();   // the operand tiles, before the tensor core reads them
+            tc_fence_before();
+            asm volatile("bar.sync 2, 480;" ::: "memory");
+            // (d) A' R' into tensor memory, the cross terms first
+            if (warp == 15 && elect_one()) {
+                tc_fence_after();
+#pragma unroll
+                for (int p = 0; p < 3; ++p) {   // lo*hi, hi*lo, hi*hi
+                    const uint32_t aa = p == 0 ? a_lo : a_hi, bb = p == 1 ? b_lo : b_hi;
+#pragma unroll
+                    for (int kk = 0; kk < 4; ++kk)
+                        tc_mma(s_tmem, desc_sw128(aa + 32 * kk), desc_sw128(bb + 32 * kk), idesc, p + kk > 0 ? 1u : 0u);
+                }
+                tc_commit(&mma_bar);
+            }
             __syncwarp();
-            for (int e = lane; e < PIV * PIV; e += 32) Ps[(e >> 4) * ZT_PS + (e & 15)] = P[e];
         }
-        __syncthreads();
-        // (e) R' and the expanded B tiles: item (c, j), u = 2j, 2j + 1; B row 2c = (Re, -Im),
-        // row 2c + 1 = (Im, Re) of R'[u][c], split into hi and lo
-#pragma unroll 1
-        for (int it = tid; it < n * 8; it += ZT_THREADS) {
-            const int c = it >> 3, j = it & 7, u0 = 2 * j, u1 = u0 + 1;
-            float2 r0, r1;
-            if (c >= k0 && c < k0 + PIV) {
-                r0 = Ps[u0 * ZT_PS + (c - k0)];
-                r1 = Ps[u1 * ZT_PS + (c - k0)];
-            } else {
-                r0 = make_float2(0.f, 0.f);
-                r1 = r0;
-#pragma unroll
-                for (int v = 0; v < PIV; ++v) {
-                    const float2 w = Wk[v * ZT_WS + c];
-                    cfma(r0, Ps[u0 * ZT_PS + v], w);
-                    cfma(r1, Ps[u1 * ZT_PS + v], w);
-                }
-            }
-            float4 hi, lo;
-            split4(make_float4(r0.x, -r0.y, r1.x, -r1.y), 1.f, hi, lo);
-            st_shared_v4(b_hi + sw128(2 * c, j), hi);
-            st_shared_v4(b_lo + sw128(2 * c, j), lo);
-            split4(make_float4(r0.y, r0.x, r1.y, r1.x), 1.f, hi, lo);
-            st_shared_v4(b_hi + sw128(2 * c + 1, j), hi);
-            st_shared_v4(b_lo + sw128(2 * c + 1, j), lo);
-        }
-        __syncthreads();   // the pivot rows read: their storage becomes the A tiles
-        // (f) A' row r, chunks j = 4 hh .. 4 hh + 3 (u = 2j, 2j + 1 of this thread's panel part)
-#pragma unroll
-        for (int jj = 0; jj < 4; ++jj) {
-            const int j = 4 * hh + jj, u0 = 2 * j;
-            float4 v;
-            if (krow) {
-                v = make_float4(r - k0 == u0 ? 1.f : 0.f, 0.f, r - k0 == u0 + 1 ? 1.f : 0.f, 0.f);
-            } else {
-                v = make_float4(-uf[4 * jj], -uf[4 * jj + 1], -uf[4 * jj + 2], -uf[4 * jj + 3]);
-            }
-            float4 hi, lo;
-            split4(v, 1.f, hi, lo);
-            st_shared_v4(a_hi + sw128(r, j), hi);
-            st_shared_v4(a_lo + sw128(r, j), lo);
-        }
-        fence_proxy_async_smem();   // the operand tiles, before the tensor core reads them
-        tc_fence_before();
-        __syncthreads();
-        // (g) W' + A' R' into tensor memory
-        if (tid == 0) {
+        // (e) W += A' R'
+        const bool done = mbar_wait_bounded(&mma_bar, (uint32_t)phase, a.tries);
+        if (__all_sync(0xffffffffu, done)) {
             tc_fence_after();
 #pragma unroll
-            for (int p = 0; p < 3; ++p) {   // hi*hi, hi*lo, lo*hi
-                const uint32_t aa = p == 2 ? a_lo : a_hi, bb = p == 1 ? b_lo : b_hi;
+            for (int g = 0; g < 4; ++g) {
+                float v[16];
+                tc_ld16(trow + (uint32_t)(16 * g), v);
 #pragma unroll
-                for (int kk = 0; kk < 4; ++kk)
-                    tc_mma(s_tmem, desc_sw128(aa + 32 * kk), desc_sw128(bb + 32 * kk), idesc, 1u);
+                for (int e = 0; e < 8; ++e) {
+                    w[8 * g + e].x += v[2 * e];
+                    w[8 * g + e].y += v[2 * e + 1];
+                }
             }
-            tc_commit(&mma_bar);
         }
-        const bool done = mbar_wait_bounded(&mma_bar, (uint32_t)phase, a.tries);
+        tc_fence_before();
         if (__syncthreads_or(!done)) {   // uniform: every thread leaves the loop
             if (tid == 0) atomicOr(a.status, ST_TIMEOUT);
             aborted = true;
             break;
         }
-        phase ^= 1;
         tc_fence_after();
+        phase ^= 1;
     }
-    // the inverse out of tensor memory: lane r, columns 128 hh .. + 127
     if (!aborted) {
 #pragma unroll 1
-        for (int ch = 0; ch < 8; ++ch) {
-            const int col = 128 * hh + 16 * ch;
-            float v[16];
-            tc_ld16(trow + (uint32_t)col, v);
-            float4 *xr = reinterpret_cast<float4 *>(X + (size_t)r * a.ldo + col / 2);
+        for (int half = 0; half < 2; ++half) {
+            if ((h >> 1) == half) {
 #pragma unroll
-            for (int i = 0; i < 4; ++i) xr[i] = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
+                for (int i = 0; i < 32; ++i) T[r * ZT_TS + 32 * (h & 1) + i] = w[i];
+            }
+            __syncthreads();
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const int rr = 8 * warp + i;
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {
+                    const int c = 64 * half + 32 * e + lane;
+                    if (rr < n && c < n) X[(size_t)rr * a.ldo + c] = T[rr * ZT_TS + 32 * e + lane];
+                }
+            }
+            __syncthreads();
         }
     } else {
-        mbar_wait_bounded(&mma_bar, (uint32_t)phase, a.tries);   // an MMA that may still be in flight
+        mbar_wait_bounded(&mma_bar, (uint32_t)phase, kDefaultWaitTries);   // an MMA that may still be in flight
     }
     if (tid == 0 && s_bad) atomicOr(a.status, ST_SINGULAR);
     tc_fence_before();
     __syncthreads();
     if (warp == 0)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(s_tmem), "r"(256u) : "memory");
-}
-
-size_t inv_smem_bytes(int n) {
-    return sizeof(float2) * ((size_t)n * (n + 1) + (size_t)n * PIV + (size_t)PIV * (n + 1) + PIV * PIV);
 }
 
 // *out = largest of n words
@@ -768,20 +789,13 @@ helm_status invert_blocks(int n, Fam in, Fam out, const std::vector<int> &pairs,
     helm_status s;
     if (n <= INV_MAX) {
         const int off = pl.add(pairs);
-        // 128 x 128 blocks on 16-byte boundaries (two complex entries per access): the kernel
-        // with the block in tensor memory
-        const bool t128 = n == 128 && ((uintptr_t)in.base & 15) == 0 && ((uintptr_t)out.base & 15) == 0 &&
-                          (in.ld & 1) == 0 && (out.ld & 1) == 0 && (in.stride & 1) == 0 && (out.stride & 1) == 0;
-        const size_t smem = t128 ? zinv128_tm_smem_bytes() : inv_smem_bytes(n);
-        const void *fn = t128 ? (const void *)zinv128_tm_kernel : (const void *)zinv_base_kernel;
-        cudaError_t e = ensure_dyn_smem(fn, smem);
+        cudaError_t e = ensure_dyn_smem((const void *)zinv_kernel, ZT_SMEM);
         if (e != cudaSuccess) { helm_set_error("bcr: block inversion", e); return HELM_ECUDA; }
         InvArgs a{n, in.op(), out.base, out.stride, 0, 0, out.ld, nullptr, status};
         a.tries = wait_tries();
-        pl.ops.push_back([a, off, count, smem, st, t128](const int *dev) mutable -> helm_status {
+        pl.ops.push_back([a, off, count, st](const int *dev) mutable -> helm_status {
             a.idx = dev + off;
-            if (t128) HELM_TRACED(K_ZINV, st, (zinv128_tm_kernel<<<count, ZT_THREADS, smem, st>>>(a)));
-            else HELM_TRACED(K_ZINV, st, (zinv_base_kernel<<<count, INV_THREADS, smem, st>>>(a)));
+            HELM_TRACED(K_ZINV, st, (zinv_kernel<<<count, ZT_THREADS, ZT_SMEM, st>>>(a)));
             const cudaError_t e2 = cudaGetLastError();
             if (e2 != cudaSuccess) { helm_set_error("bcr: block inversion", e2); return HELM_ECUDA; }
             return HELM_OK;
