@@ -183,27 +183,27 @@ extern "C" void helm_op_destroy(helm_op_t *op) {
 
 // ------------------------------------------------------------------------ factor
 
-// Factor method of a mixed factor: the options, else HELM_FACTOR=line|bcr, else BCR on lines of
-// at least kBcrMinNz nodes and the line recurrence below.  FP64 factors are line factors (the
-// tensor cores have no FP64 path).
-static constexpr int kBcrMinNz = 192;
-// lines from which BCR was always the automatic choice and is not second-guessed
-static constexpr int kBcrSureNz = 192;
+// Factor method of a mixed factor: the options, else HELM_FACTOR=line|bcr, else BCR on lines of at
+// least kBcrLine nodes, and on shorter ones from kBcrShortLine nodes and as many lines on while its
+// blocks stay within kBcrShortBytes.  FP64 factors are line factors (the tensor cores have no FP64
+// path).
+static constexpr int kBcrLine = 192;
+// Both sides at one frequency, where the line factor is at its best (us, line / BCR): factor at
+// 64 x 64 860 / 650, 96 x 96 2450 / 910, 128 x 128 3700 / 1150; solve with 1 and 51 right-hand sides
+// at 64 x 64 220 / 290 and 410 / 470, at 80 x 80 400 / 400 and 560 / 590, at 96 x 96 460 / 400 and
+// 640 / 630, at 128 x 128 580 / 470 and 880 / 790; with eight frequencies and 51 right-hand sides at
+// 128 x 128 4500 / 1500.  Few lines favour the recurrence, whose chain is their number (48 x 96: solves
+// 280 / 320 and 370 / 510).
+static constexpr int kBcrShortLine = 96;
+// BCR holds about 3.5 (and 6 while it factors) times the line factor's bytes: a set of frequencies
+// whose blocks no longer are a small part of the device's memory stays with the smaller factor
+static constexpr size_t kBcrShortBytes = (size_t)16 << 30;
 // BCR eliminates lines with Dirichlet neighbours, so a frequency near a resonance of a strip of the
 // medium makes an eliminated block nearly singular.  Over random media the refinement took one
 // sweep more from |A| |Dinv| of 2^9 (entries of the inverses of 2^7 and a diagonal of about 4), 5 to
 // 6 sweeps at 2^10, 7 to 15 at 2^11, and did not converge at 2^13; nearly all factors stay below
 // 2^5.  From 2^10 a short line takes the line recurrence.
 static constexpr float kBcrMaxGrowth = 1024.f;
-static bool bcr_falls_back(const GridGeom &g, const helm_factor_opts *opts, const int st_host[3]) {
-    if (g.nz >= kBcrSureNz || (opts && opts->method == HELM_FACTOR_BCR) || (st_host[0] & ST_TIMEOUT)) return false;
-    const char *env = getenv("HELM_FACTOR");
-    if (env && !strcmp(env, "bcr")) return false;
-    float mx;
-    memcpy(&mx, &st_host[2], sizeof(mx));
-    const double scale = 2.0 * (g.hz / g.hx + g.hx / g.hz);
-    return (st_host[0] & ST_SINGULAR) || !(mx * scale < kBcrMaxGrowth);
-}
 bool helm::factor_picks_bcr(const GridGeom &g, helm_prec prec, int method) {
     if (prec != HELM_MIXED || !bcr_supported(g)) return false;
     int m = method;
@@ -211,12 +211,24 @@ bool helm::factor_picks_bcr(const GridGeom &g, helm_prec prec, int method) {
         const char *env = getenv("HELM_FACTOR");
         if (env && !strcmp(env, "line")) m = HELM_FACTOR_LINE;
         else if (env && !strcmp(env, "bcr")) m = HELM_FACTOR_BCR;
-        else m = g.nz >= kBcrMinNz ? HELM_FACTOR_BCR : HELM_FACTOR_LINE;
+        else m = g.nz >= kBcrLine ? HELM_FACTOR_BCR : HELM_FACTOR_LINE;
     }
     return m == HELM_FACTOR_BCR;
 }
-static bool pick_bcr(const helm_op *op, helm_prec prec, const helm_factor_opts *opts) {
-    return factor_picks_bcr(op->g, prec, opts ? opts->method : HELM_FACTOR_AUTO);
+// the automatic choice of BCR on a short line (taken back where it turns out badly)
+static bool picks_short_bcr(const helm_op *op, helm_prec prec, const helm_factor_opts *opts) {
+    const GridGeom &g = op->g;
+    const char *env = getenv("HELM_FACTOR");
+    if ((opts && opts->method != HELM_FACTOR_AUTO) || (env && (!strcmp(env, "line") || !strcmp(env, "bcr")))) return false;
+    return prec == HELM_MIXED && bcr_supported(g) && g.nz < kBcrLine && g.nz >= kBcrShortLine && g.nx >= kBcrShortLine &&
+           6 * sizeof(float2) * op->n_omega * g.nx * g.nz * g.nz <= kBcrShortBytes;
+}
+static bool bcr_falls_back(const GridGeom &g, const int st_host[3]) {
+    if (st_host[0] & ST_TIMEOUT) return false;
+    float mx;
+    memcpy(&mx, &st_host[2], sizeof(mx));
+    const double scale = 2.0 * (g.hz / g.hx + g.hx / g.hz);
+    return (st_host[0] & ST_SINGULAR) || !(mx * scale < kBcrMaxGrowth);
 }
 
 extern "C" helm_status helm_factor(helm_op_t *op, helm_prec prec, const helm_factor_opts *opts, helm_factor_t **out) {
@@ -235,7 +247,8 @@ extern "C" helm_status helm_factor(helm_op_t *op, helm_prec prec, const helm_fac
     if (!f) return HELM_ENOMEM;
     f->op = op;
     f->prec = prec;
-    f->use_bcr = pick_bcr(op, prec, opts);
+    const bool short_bcr = picks_short_bcr(op, prec, opts);
+    f->use_bcr = short_bcr || factor_picks_bcr(op->g, prec, opts ? opts->method : HELM_FACTOR_AUTO);
     const GridGeom &g = op->g;
     f->cs = pick_cluster_size(g.nz);
     const size_t esz = prec == HELM_FP64 ? sizeof(double2) : sizeof(float2);
@@ -284,16 +297,19 @@ extern "C" helm_status helm_factor(helm_op_t *op, helm_prec prec, const helm_fac
     };
     bool line = !f->use_bcr;
     if (f->use_bcr) {
-        if ((s = bcr_factor(f)) != HELM_OK) {
+        s = bcr_factor(f);
+        e = cudaSuccess;
+        if (s != HELM_OK && !(short_bcr && s == HELM_ENOMEM)) {
             cudaStreamSynchronize(op->st);
             restore_diag();
             helm_factor_destroy(f);
             return s;
         }
-        e = read_status(cudaSuccess);
+        if (s == HELM_OK) e = read_status(cudaSuccess);
         // an automatic choice on a short line, which the line recurrence (its Schur complements run
-        // from the absorbing boundary) takes instead where an eliminated block came out nearly singular
-        if (e == cudaSuccess && bcr_falls_back(g, opts, st_host)) {
+        // from the absorbing boundary, and it holds less) takes instead where an eliminated block
+        // came out nearly singular or the blocks did not fit
+        if (e == cudaSuccess && short_bcr && (s != HELM_OK || bcr_falls_back(g, st_host))) {
             bcr_free(f);
             f->use_bcr = false;
             line = true;
@@ -483,8 +499,8 @@ helm_status mixed_refine(const helm_factor_t *f, int nrhs, const double2 *B, dou
             if (e != cudaSuccess) { helm_set_error("refinement update", e); return HELM_ECUDA; }
         }
         // X of the newest iterates, enqueued before the state is read: one wait per batch, and
-        // nothing left to wait for once the loop has stopped (a batch that has not is followed by
-        // another X; 512 columns of 256^2 take 0.2 ms)
+        // nothing left to wait for once the loop has stopped (until then the kernel returns at once;
+        // 512 columns of 256^2 take 0.2 ms)
         e = launch_refine_finish(n, g.nx * g.nz, nrhs, w.xa, w.xb, w.state, conj, X, op->st);
         if (e == cudaSuccess) e = cudaMemcpyAsync(&hs, w.state, sizeof(RefineState), cudaMemcpyDeviceToHost, op->st);
         if (e == cudaSuccess) e = cudaStreamSynchronize(op->st);

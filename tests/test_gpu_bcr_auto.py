@@ -1,0 +1,42 @@
+"""The automatic choice of block cyclic reduction on lines of 96 to 191 nodes: taken on sizes (at
+least 96 lines, even nz, blocks within 16 GB), and taken back where an eliminated block is nearly
+singular: a slow disc of m = 36 in m = 1 on 96 x 96 has a mode trapped between the lines 32 and 64 at w
+= 5.548174513413695, and the inverse of the block of line 48 an entry of 5e3 (the limit is 2^10 / 4).
+|A^{-1}| |b| / |x| of the medium itself is below 1e2 for random b there and at w = 5, so a residual of
+1e-12 leaves an error below 1e-10; 1e-8 is the mixed path's bar."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import helmholtz as H
+
+hm = pytest.importorskip("paper_2301_10762_gb300.helm")
+
+pytestmark = pytest.mark.gpu
+
+AUTO = [(96, 96, 1, "bcr"), (130, 98, 2, "bcr"), (97, 190, 1, "bcr"), (95, 96, 1, "line"), (96, 94, 1, "line"),
+        (96, 97, 1, "line"), (40, 190, 1, "line"), (96, 96, 406, "line")]
+
+
+@pytest.mark.parametrize("nx,nz,n_omega,want", AUTO)
+def test_automatic_choice_on_sizes(nx, nz, n_omega, want):
+    m = np.full(nx * nz, 0.25)
+    op = hm.helm_assemble(nx, nz, 1.0, 1.0, torch.tensor(m, device="cuda"), np.linspace(5.0, 9.0, n_omega))
+    f = hm.helm_factor(op, hm.HELM_MIXED)
+    assert f.method == (hm.HELM_FACTOR_BCR if want == "bcr" else hm.HELM_FACTOR_LINE)
+
+
+@pytest.mark.parametrize("w,want", [(5.548174513413695, "line"), (5.0, "bcr")])
+def test_a_trapped_mode_takes_the_line_factor(w, want):
+    n = 96
+    x = np.linspace(0.0, 1.0, n)
+    X, Z = np.meshgrid(x, x, indexing="ij")
+    m = np.where((X - 48 / 95) ** 2 + (Z - 0.5) ** 2 < 0.25 ** 2, 36.0, 1.0).reshape(-1)
+    op = hm.helm_assemble(n, n, 1.0, 1.0, torch.tensor(m, device="cuda"), [w])
+    f = hm.helm_factor(op, hm.HELM_MIXED)
+    assert f.method == (hm.HELM_FACTOR_BCR if want == "bcr" else hm.HELM_FACTOR_LINE)
+    rng = np.random.default_rng(11)
+    B = rng.standard_normal((1, 5, n * n)) + 1j * rng.standard_normal((1, 5, n * n))
+    Y = hm.helm_solve(f, torch.tensor(B, device="cuda"), rtol=1e-12, max_iter=20)[0].cpu().numpy()
+    ref = H.Factor(H.helmholtz_matrix(H.Grid(n, n, 1.0, 1.0), m, w)).solve(B[0])
+    assert np.max(np.linalg.norm(Y[0] - ref, axis=1) / np.linalg.norm(ref, axis=1)) <= 1e-8
