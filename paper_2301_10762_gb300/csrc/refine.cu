@@ -333,6 +333,7 @@ __global__ void refine_accumulate_kernel(size_t n, const float2 *d, int conj, do
 
 __global__ void refine_finish_kernel(size_t n, int N, int nrhs, const float4 *xa, const float4 *xb,
                                      const RefineState *st, int conj, double2 *X) {
+    if (!st->done) return;   // (enqueued behind every batch of sweeps: the last one's counts)
     const int *sys = refine_sys(st);
     const size_t stride = (size_t)gridDim.x * blockDim.x;
     auto at = [&](size_t e) -> float4 {   // the newest iterate of this element's system
