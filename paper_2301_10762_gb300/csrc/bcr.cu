@@ -876,11 +876,13 @@ helm_status image_blocks(int n, const float2 *D, const std::vector<int> &pairs, 
 helm_status image_gemm(const BgArgs &ba, const std::vector<int> &tasks, Plan &pl) {
     if (tasks.empty()) return HELM_OK;
     const int off = pl.add(tasks), n = (int)(tasks.size() / BG_TASK);
+    int products = n;
+    for (int t = 0; t < n; ++t) products += (tasks[BG_TASK * t] & BG_TWO) != 0;
     const cudaStream_t st = pl.st;
     pl.ops.push_back([=](const int *dev) -> helm_status {
         BgArgs a = ba;
         a.tasks = dev + off;
-        const cudaError_t e = launch_bcr_gemm(a, n, st);
+        const cudaError_t e = launch_bcr_gemm(a, n, products, st);
         if (e != cudaSuccess) { helm_set_error("bcr: block products", e); return HELM_ECUDA; }
         return HELM_OK;
     });
@@ -1010,23 +1012,22 @@ helm_status bcr_factor(helm_factor_t *f) {
         auto Lc = [&](int sy, int k) { return sp == 2 ? (int)m0 + sy * m_stride + k / 2 - 1 : (int)u_base(cur, 1) + sy * u_stride[cur] + k / sp; };
         auto Un = [&](int sy, int k) { return (int)u_base(nxt, 0) + sy * u_stride[nxt] + k / (2 * sp); };
         auto Ln = [&](int sy, int k) { return (int)u_base(nxt, 1) + sy * u_stride[nxt] + k / (2 * sp); };
-        std::vector<int> t1, t2, t3;   // V, P, W, Q; the new couplings and D -= L W^T; D -= U V^T
-        auto add = [](std::vector<int> &t, int flags, int ia, int ib, int out) { t.insert(t.end(), {flags, ia, ib, out}); };
+        std::vector<int> t1, t2;   // V, W with their transposes P, Q; the new couplings and D -= L W^T + U V^T
+        auto add = [](std::vector<int> &t, int flags, int ia, int ib, int out, int ia2 = -1, int ib2 = -1) {
+            t.insert(t.end(), {flags, ia, ib, out, ia2, ib2});
+        };
         for (int sy = 0; sy < ns; ++sy) {
             for (int j = sp; j < nx; j += 2 * sp) {
                 const int di = mat(BS_DINV, sy, j), u = Uc(sy, j - sp);
-                add(t1, 0, u, di, mat(BS_V, sy, j / 2));    // V_j = U_{j-s} Dinv_j
-                add(t1, 0, di, u, mat(BS_P, sy, j / 2));    // P_j = V_j^T (Dinv_j is symmetric)
-                if (j + sp < nx) {
-                    const int l = Lc(sy, j + sp);
-                    add(t1, 0, l, di, mat(BS_W, sy, j / 2));   // W_j = L_{j+s} Dinv_j
-                    add(t1, 0, di, l, mat(BS_Q, sy, j / 2));
-                }
+                add(t1, BG_TR, u, di, mat(BS_V, sy, j / 2), mat(BS_P, sy, j / 2));   // V_j = U_{j-s} Dinv_j, P_j = V_j^T
+                if (j + sp < nx) add(t1, BG_TR, Lc(sy, j + sp), di, mat(BS_W, sy, j / 2), mat(BS_Q, sy, j / 2));   // W_j, Q_j
             }
             for (int k = 0; k < nx; k += 2 * sp) {
                 const int a = k - sp, c = k + sp;
-                if (a >= 0) add(t2, BG_FP32 | BG_NEG, Lc(sy, k), mat(BS_W, sy, a / 2), sy * nx + k);   // D_k -= L_k W_a^T
-                if (c < nx) add(t3, BG_FP32 | BG_NEG, Uc(sy, k), mat(BS_V, sy, c / 2), sy * nx + k);   // D_k -= U_k V_c^T
+                const int l = a >= 0 ? Lc(sy, k) : -1, w = a >= 0 ? mat(BS_W, sy, a / 2) : -1;   // D_k -= L_k W_a^T + U_k V_c^T
+                const int u = c < nx ? Uc(sy, k) : -1, v = c < nx ? mat(BS_V, sy, c / 2) : -1;
+                if (a >= 0) add(t2, BG_FP32 | BG_NEG | (c < nx ? BG_TWO : 0), l, w, sy * nx + k, u, v);
+                else if (c < nx) add(t2, BG_FP32 | BG_NEG, u, v, sy * nx + k);
                 if (k >= 2 * sp) add(t2, BG_NEG, Lc(sy, k), mat(BS_V, sy, a / 2), Ln(sy, k));          // L_k <- -L_k V_a^T
                 if (k + 2 * sp < nx) add(t2, BG_NEG, Uc(sy, k), mat(BS_W, sy, c / 2), Un(sy, k));      // U_k <- -U_k W_c^T
             }
@@ -1039,7 +1040,7 @@ helm_status bcr_factor(helm_factor_t *f) {
             if (e2 != cudaSuccess) { helm_set_error("bcr: maxima", e2); return HELM_ECUDA; }
             return HELM_OK;
         });
-        if ((s = image_gemm(ba, t2, pl)) != HELM_OK || (s = image_gemm(ba, t3, pl)) != HELM_OK) return s;
+        if ((s = image_gemm(ba, t2, pl)) != HELM_OK) return s;
         cur = nxt;
     }
     // the last line left: line 0

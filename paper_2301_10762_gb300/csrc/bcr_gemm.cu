@@ -1,5 +1,5 @@
 // Block products of the block-cyclic-reduction factor on images (bcr_solve.h) of the operands:
-//     C_t = +-A_t B_t^T        written as an image, or        D_t <- D_t - A_t B_t^T    (FP32)
+//     C_t = +-A_t B_t^T    written as an image, or    D_t <- D_t -+ (A_t B_t^T + A'_t B'_t^T)    (FP32)
 // for n x n blocks A_t, B_t.  The factor's couplings and their products with the inverses never
 // exist in FP32: the epilogue writes the next product's operands.  A CTA computes 128 x 128 tiles;
 // a copy thread streams the operands' chunks (64 KB for 32 columns of K, contiguous runs, no
@@ -30,12 +30,25 @@ namespace helm {
 namespace {
 
 constexpr int BG_WARPS = 10, BG_THREADS = 32 * BG_WARPS, BG_EPI0 = 2;   // MMA, copy, eight epilogue warps
-constexpr int BG_STAGE = 65536, BG_STAGES = 3;
-constexpr size_t BG_SMEM = (size_t)BG_STAGES * BG_STAGE + 1024;
+constexpr int BG_STAGE = 65536, BG_STAGES = 3, BG_QD = 4;
+constexpr int BG_OUT = 4096;   // staging of an epilogue warp: 32 rows of an image's chunk
+constexpr size_t BG_SMEM = (size_t)BG_STAGES * BG_STAGE + (BG_WARPS - BG_EPI0) * BG_OUT + 1024;
+
+__device__ __forceinline__ void red_add2(float2 *p, float x, float y) {
+    asm volatile("red.relaxed.gpu.global.add.v2.f32 [%0], {%1, %2};" ::"l"(p), "f"(x), "f"(y) : "memory");
+}
+
+struct BgTile {   // what the MMA thread and the epilogue need of a tile: read ahead by the copy thread
+    int flags, terms, out, shift;   // (image: its scale)
+    float f[2];                     // +-2^-(shift A + shift B) of the terms
+    int out_t, pad;                 // the transposed image's matrix, or -1
+};
 
 __global__ void __launch_bounds__(BG_THREADS, 1) bcr_gemm_kernel(BgArgs a) {
     extern __shared__ uint8_t bg_smem[];
     __shared__ __align__(8) uint64_t full[BG_STAGES], empty[BG_STAGES], acc_full[2], acc_empty[2], done_bar;
+    __shared__ __align__(8) uint64_t tq_full[BG_QD], tq_empty[BG_QD];
+    __shared__ BgTile tq[BG_QD];
     __shared__ uint32_t s_tmem;
     __shared__ int s_abort;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -47,6 +60,10 @@ __global__ void __launch_bounds__(BG_THREADS, 1) bcr_gemm_kernel(BgArgs a) {
         for (int s = 0; s < 2; ++s) {
             mbar_init(&acc_full[s], 1);
             mbar_init(&acc_empty[s], BG_WARPS - BG_EPI0);
+        }
+        for (int q = 0; q < BG_QD; ++q) {
+            mbar_init(&tq_full[q], 1);
+            mbar_init(&tq_empty[q], 1 + BG_WARPS - BG_EPI0);
         }
         mbar_init(&done_bar, 1);
         fence_mbar_init_cluster();
@@ -74,17 +91,38 @@ __global__ void __launch_bounds__(BG_THREADS, 1) bcr_gemm_kernel(BgArgs a) {
     };
     if (warp == 1) {
         if (elect_one()) {   // copy thread
-            int s = 0, issued = 0;
+            int s = 0, issued = 0, i = 0;
             uint32_t ph = 1;
             bool go = true;
             const size_t im_off = (size_t)a.nzr * 128;
-            for (int t = blockIdx.x; go && t < a.n_tiles; t += gridDim.x) {
-                const int *task = a.tasks + BG_TASK * (t / per);
+            for (int t = blockIdx.x; go && t < a.n_tiles; t += gridDim.x, ++i) {
+                int task[BG_TASK];
+#pragma unroll
+                for (int e = 0; e < BG_TASK; ++e) task[e] = __ldg(a.tasks + BG_TASK * (t / per) + e);
+                BgTile tl;
+                tl.flags = task[0];
+                tl.terms = (tl.flags & BG_TWO) ? 2 : 1;
+                tl.out_t = (tl.flags & BG_TR) ? task[4] : -1;
+                tl.out = task[3];
+                // image: the bound's scale
+                const int eb = (int)(a.im.mx[task[1]] >> 23) + (int)(a.im.mx[task[2]] >> 23) - 254 + 2 + a.log2_2k;
+                tl.shift = max(-100, min(100, 15 - eb));
+#pragma unroll
+                for (int u = 0; u < 2; ++u) {
+                    const int x = task[u < tl.terms ? 1 + 3 * u : 1], y = task[u < tl.terms ? 2 + 3 * u : 2];
+                    tl.f[u] = bs_pow2(max(-126, min(126, -(a.im.shift[x] + a.im.shift[y])))) * ((tl.flags & BG_NEG) ? -1.f : 1.f);
+                }
+                if (!wait1(&tq_empty[i % BG_QD], (uint32_t)((i / BG_QD) & 1) ^ 1u)) break;
+                tq[i % BG_QD] = tl;
+                mbar_arrive_cta(&tq_full[i % BG_QD]);
                 const int m0 = 128 * (t % per / a.nt), n0 = 128 * (t % a.nt);
                 const uint32_t ba = 128u * (uint32_t)min(128, a.nzr - m0), bb = 128u * (uint32_t)min(128, a.nzr - n0);
-                const unsigned char *pa = a.im.at(task[1], a.mat_bytes) + (size_t)m0 * 128;
-                const unsigned char *pb = a.im.at(task[2], a.mat_bytes) + (size_t)n0 * 128;
-                for (int c = 0; c < a.n_chunk; ++c, pa += 2 * im_off, pb += 2 * im_off) {
+                const unsigned char *pa = nullptr, *pb = nullptr;
+                for (int c = 0, n = a.n_chunk * tl.terms; c < n; ++c, pa += 2 * im_off, pb += 2 * im_off) {
+                    if (c % a.n_chunk == 0) {   // the next term
+                        pa = a.im.at(c == 0 ? task[1] : task[4], a.mat_bytes) + (size_t)m0 * 128;
+                        pb = a.im.at(c == 0 ? task[2] : task[5], a.mat_bytes) + (size_t)n0 * 128;
+                    }
                     if (!wait1(&empty[s], ph)) { go = false; break; }
                     const uint32_t dst = smem0 + (uint32_t)(s * BG_STAGE);
                     mbar_arrive_expect_tx(&full[s], 2 * (ba + bb));
@@ -103,14 +141,17 @@ __global__ void __launch_bounds__(BG_THREADS, 1) bcr_gemm_kernel(BgArgs a) {
         __syncwarp();
     } else if (warp == 0) {
         if (elect_one()) {   // MMA thread
-            int s = 0, cc = 0;
+            int s = 0, cc = 0, i = 0;
             uint32_t ph = 0;
             bool go = true;
             const uint64_t dstage0 = desc_sw128(smem0);
-            for (int t = blockIdx.x; go && t < a.n_tiles; t += gridDim.x) {
+            for (int t = blockIdx.x; go && t < a.n_tiles; t += gridDim.x, ++i) {
+                if (!wait1(&tq_full[i % BG_QD], (uint32_t)((i / BG_QD) & 1))) break;
+                const int terms = tq[i % BG_QD].terms;
+                mbar_arrive_cta(&tq_empty[i % BG_QD]);
                 const int n0 = 128 * (t % a.nt), nb = min(128, (a.nzr - n0 + 15) & ~15);
                 const uint32_t id = idesc_f16(nb, false), idn = idesc_f16(nb, true);
-                for (int c = 0; c < a.n_chunk; ++c, ++cc) {
+                for (int c = 0, n = a.n_chunk * terms; c < n; ++c, ++cc) {
                     if (!wait1(&acc_empty[cc & 1], (uint32_t)((cc >> 1) & 1) ^ 1u) || !wait1(&full[s], ph)) { go = false; break; }
                     tc_fence_after();
                     const uint64_t ar = dstage0 + (uint64_t)(s * (BG_STAGE / 16)), ai = ar + 1024, br = ar + 2048, bi = ar + 3072;
@@ -136,18 +177,37 @@ __global__ void __launch_bounds__(BG_THREADS, 1) bcr_gemm_kernel(BgArgs a) {
     } else {
         // epilogue warps: tensor-memory lanes 32 q .. + 31 = rows m0 + 32 q + lane, 64 columns each
         const int q = warp & 3, hh = (warp - BG_EPI0) >> 2;
-        int cc = 0;
+        int cc = 0, i = 0;
         bool go = true;
         const int n_cols = 32 * a.n_chunk;
-        for (int t = blockIdx.x; t < a.n_tiles; t += gridDim.x) {
-            const int *task = a.tasks + BG_TASK * (t / per);
+        unsigned char *stage = bg_smem + (smem0 - smem_u32(bg_smem)) + BG_STAGES * BG_STAGE + (warp - BG_EPI0) * BG_OUT;
+        auto stage_wait = [&]() {   // the copy out of the staging buffer has read it
+            if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+            __syncwarp();
+        };
+        auto stage_store = [&](unsigned char *dst, int bytes) {
+            fence_proxy_async_smem();
+            __syncwarp();
+            if (lane == 0)
+                asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;\n cp.async.bulk.commit_group;" ::"l"(dst),
+                             "r"(smem_u32(stage)), "r"(bytes)
+                             : "memory");
+        };
+        for (int t = blockIdx.x; t < a.n_tiles; t += gridDim.x, ++i) {
             const int m0 = 128 * (t % per / a.nt), n0 = 128 * (t % a.nt) + 64 * hh, m = m0 + 32 * q + lane;
-            const int flags = task[0], ia = task[1], ib = task[2], out = task[3];
-            const float f = bs_pow2(max(-126, min(126, -(a.im.shift[ia] + a.im.shift[ib])))) * ((flags & BG_NEG) ? -1.f : 1.f);
+            if (!__all_sync(0xffffffffu, mbar_wait_cta(&tq_full[i % BG_QD], (uint32_t)((i / BG_QD) & 1), a.tries, &s_abort))) {
+                if (lane == 0) give_up();
+                break;
+            }
+            const BgTile tl = tq[i % BG_QD];
+            __syncwarp();
+            if (lane == 0) mbar_arrive_cta(&tq_empty[i % BG_QD]);
+            const int flags = tl.flags, out = tl.out, sh = tl.shift;
             float re[64], im[64];
 #pragma unroll
             for (int e = 0; e < 64; ++e) re[e] = im[e] = 0.f;
-            for (int c = 0; c < a.n_chunk; ++c, ++cc) {
+            for (int c = 0; c < a.n_chunk * tl.terms; ++c, ++cc) {
+                const float f = c < a.n_chunk ? tl.f[0] : tl.f[1];
                 const bool ok = mbar_wait_cta(&acc_full[cc & 1], (uint32_t)((cc >> 1) & 1), a.tries, &s_abort);
                 if (!__all_sync(0xffffffffu, ok)) {
                     if (lane == 0) give_up();
@@ -169,10 +229,10 @@ __global__ void __launch_bounds__(BG_THREADS, 1) bcr_gemm_kernel(BgArgs a) {
                     tc_wait_ld8(i1);
 #pragma unroll
                     for (int e = 0; e < 8; ++e) {
-                        re[8 * g + e] += __uint_as_float(r0[e]);
-                        re[8 * g + 8 + e] += __uint_as_float(r1[e]);
-                        im[8 * g + e] += __uint_as_float(i0[e]);
-                        im[8 * g + 8 + e] += __uint_as_float(i1[e]);
+                        re[8 * g + e] = fmaf(f, __uint_as_float(r0[e]), re[8 * g + e]);
+                        re[8 * g + 8 + e] = fmaf(f, __uint_as_float(r1[e]), re[8 * g + 8 + e]);
+                        im[8 * g + e] = fmaf(f, __uint_as_float(i0[e]), im[8 * g + e]);
+                        im[8 * g + 8 + e] = fmaf(f, __uint_as_float(i1[e]), im[8 * g + 8 + e]);
                     }
                 }
                 tc_fence_before();
@@ -180,57 +240,71 @@ __global__ void __launch_bounds__(BG_THREADS, 1) bcr_gemm_kernel(BgArgs a) {
                 if (lane == 0) mbar_arrive_cta(&acc_empty[cc & 1]);
             }
             if (!go) break;
-            // image: the bound's scale
-            const int eb = (int)(a.im.mx[ia] >> 23) + (int)(a.im.mx[ib] >> 23) - 254 + 2 + a.log2_2k;
-            const int sh = max(-100, min(100, 15 - eb));
+            const int mb = m - lane;   // the warp's rows mb .. mb + 31
+            if (flags & BG_FP32) {
+                // the update is symmetric: entry (m, n) is added to D[n][m], 256 contiguous bytes of a
+                // column's 32 rows at a time, and without a load
+                float2 *dst = a.D + (size_t)out * a.nz * a.nz + m;
+                if (m < a.nz) {
+#pragma unroll
+                    for (int e = 0; e < 64; ++e)
+                        if (n0 + e < a.nz) red_add2(dst + (size_t)(n0 + e) * a.nz, re[e], im[e]);
+                }
+                continue;
+            }
             const float sc = bs_pow2(sh);
             uint32_t mxv = 0;
-            float2 *dst = a.D + (size_t)out * a.nz * a.nz + (size_t)m * a.nz;   // (BG_FP32)
-            unsigned char *img = (flags & BG_FP32) ? nullptr : a.im.at(out, a.mat_bytes);
+            unsigned char *img = a.im.at(out, a.mat_bytes), *img_t = tl.out_t >= 0 ? a.im.at(tl.out_t, a.mat_bytes) : nullptr;
+            const size_t half = (size_t)a.nzr * 128;
+            const int rows = min(32, a.nzr - mb);
 #pragma unroll
-            for (int g = 0; g < 8; ++g) {
-                const int nn = n0 + 8 * g;
+            for (int cb = 0; cb < 64; cb += 32) {
+                const int nn = n0 + cb, c = nn >> 5;
                 if (nn >= n_cols) continue;
-                float2 v[8];
 #pragma unroll
-                for (int e = 0; e < 8; ++e) {
-                    const bool in = m < a.nz && nn + e < a.nz;
-                    v[e] = in ? make_float2(re[8 * g + e] * f, im[8 * g + e] * f) : make_float2(0.f, 0.f);
-                }
-                if (!img) {   // n is even: pairs of columns on 16-byte boundaries
-                    if (m < a.nz) {
+                for (int p = 0; p < 2; ++p) {
+                    float *v = (p ? im : re) + cb;
 #pragma unroll
-                        for (int e = 0; e < 8; e += 2)
-                            if (nn + e < a.nz) {
-                                float4 *w = reinterpret_cast<float4 *>(dst + nn + e);
-                                const float4 o = *w;
-                                *w = make_float4(o.x + v[e].x, o.y + v[e].y, o.z + v[e + 1].x, o.w + v[e + 1].y);
-                            }
+                    for (int e = 0; e < 32; ++e) {
+                        if (m >= a.nz || nn + e >= a.nz) v[e] = 0.f;
+                        mxv = max(mxv, bs_abs_bits(v[e]));
+                        v[e] *= sc;
                     }
-                    continue;
-                }
-                {
+                    if (rows > 0) {   // rows of the image, in its layout: one contiguous piece of memory
+                        stage_wait();
 #pragma unroll
-                    for (int e = 0; e < 8; ++e) mxv = max(mxv, max(bs_abs_bits(v[e].x), bs_abs_bits(v[e].y)));
-                    if (m < a.nzr) {   // 16-byte pieces of the row: eight columns' hi, and lo 64 bytes on
-                        const int c = nn >> 5, j = (nn >> 3) & 3;
-                        uint4 rh, rl, ih, il;
-                        bs_split8(v, sc, rh, rl, ih, il);
-                        unsigned char *row = img + ((size_t)(2 * c) * a.nzr + m) * 128;
-                        *reinterpret_cast<uint4 *>(row + ((j ^ (m & 7)) << 4)) = rh;
-                        *reinterpret_cast<uint4 *>(row + (((j + 4) ^ (m & 7)) << 4)) = rl;
-                        row += (size_t)a.nzr * 128;
-                        *reinterpret_cast<uint4 *>(row + ((j ^ (m & 7)) << 4)) = ih;
-                        *reinterpret_cast<uint4 *>(row + (((j + 4) ^ (m & 7)) << 4)) = il;
+                        for (int j = 0; j < 4; ++j) {
+                            uint4 hi, lo;
+                            bs_split2(v[8 * j], v[8 * j + 1], hi.x, lo.x);
+                            bs_split2(v[8 * j + 2], v[8 * j + 3], hi.y, lo.y);
+                            bs_split2(v[8 * j + 4], v[8 * j + 5], hi.z, lo.z);
+                            bs_split2(v[8 * j + 6], v[8 * j + 7], hi.w, lo.w);
+                            *reinterpret_cast<uint4 *>(stage + lane * 128 + ((j ^ (lane & 7)) << 4)) = hi;
+                            *reinterpret_cast<uint4 *>(stage + lane * 128 + (((j + 4) ^ (lane & 7)) << 4)) = lo;
+                        }
+                        stage_store(img + (size_t)(2 * c + p) * half + (size_t)mb * 128, rows * 128);
+                    }
+                    if (img_t && mb < n_cols) {
+                        // the transpose: the warp's 32 rows are a chunk of row n; even lanes hold the hi
+                        // parts of two columns, odd lanes the lo parts, 128 bytes in all
+                        stage_wait();
+#pragma unroll
+                        for (int e = 0; e < 32; ++e) {
+                            const int o = (((lane >> 3) + 4 * (lane & 1)) ^ (e & 7)) * 16 + (lane & 6) * 2;
+                            *reinterpret_cast<uint32_t *>(stage + e * 128 + o) = bs_split_pair(v[e], lane);
+                        }
+                        stage_store(img_t + (size_t)(2 * (mb >> 5) + p) * half + (size_t)nn * 128, min(32, a.nzr - nn) * 128);
                     }
                 }
             }
-            if (img) {
-                if (t % per == 0 && warp == BG_EPI0 && lane == 0) a.im.shift[out] = sh;
-                mxv = __reduce_max_sync(0xffffffffu, mxv);
-                if (lane == 0 && mxv) atomicMax(a.im.mx + out, mxv);
+            if (t % per == 0 && warp == BG_EPI0 && lane == 0) {
+                a.im.shift[out] = sh;
+                if (img_t) a.im.shift[tl.out_t] = sh;
             }
+            mxv = __reduce_max_sync(0xffffffffu, mxv);
+            if (lane == 0 && mxv) atomicMax(a.im.mx + out, mxv);
         }
+        if (lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
     }
     tc_fence_before();
     __syncthreads();
@@ -240,7 +314,7 @@ __global__ void __launch_bounds__(BG_THREADS, 1) bcr_gemm_kernel(BgArgs a) {
 
 }  // namespace
 
-cudaError_t launch_bcr_gemm(BgArgs a, int n_tasks, cudaStream_t st) {
+cudaError_t launch_bcr_gemm(BgArgs a, int n_tasks, int n_products, cudaStream_t st) {
     if (n_tasks <= 0) return cudaSuccess;
     if (a.nz & 1) return cudaErrorInvalidValue;
     const BsLayout l = bs_layout(a.nz);
@@ -254,7 +328,7 @@ cudaError_t launch_bcr_gemm(BgArgs a, int n_tasks, cudaStream_t st) {
     cudaError_t e = ensure_dyn_smem((const void *)bcr_gemm_kernel, BG_SMEM);
     if (e != cudaSuccess) return e;
     const int grid = std::min(device_sms(), a.n_tiles);
-    HELM_TRACED_W(K_BCR_GEMM, st, 8.0 * a.nz * a.nz * (double)a.nz * n_tasks,
+    HELM_TRACED_W(K_BCR_GEMM, st, 8.0 * a.nz * a.nz * (double)a.nz * n_products,
                   (bcr_gemm_kernel<<<grid, BG_THREADS, BG_SMEM, st>>>(a)));
     return cudaGetLastError();
 }

@@ -31,6 +31,14 @@ __device__ __forceinline__ void bs_split2(float a, float b, uint32_t &hi, uint32
     hi = *reinterpret_cast<const uint32_t *>(&h);
     lo = *reinterpret_cast<const uint32_t *>(&l);
 }
+// hi parts of this lane's and the next lane's value (even lanes), lo parts of the lane before's and
+// this one's (odd lanes), packed; all lanes of the warp
+__device__ __forceinline__ uint32_t bs_split_pair(float x, int lane) {
+    const __half h = __float2half_rn(x), l = __float2half_rn(x - __half2float(h));
+    const uint32_t t = (uint32_t)__half_as_ushort(h) | (uint32_t)__half_as_ushort(l) << 16;
+    const uint32_t o = __shfl_xor_sync(0xffffffffu, t, 1);
+    return (lane & 1) ? ((o >> 16) | (t & 0xffff0000u)) : ((t & 0xffffu) | (o << 16));
+}
 // the 16-byte pieces (hi and lo, real and imaginary) of eight entries times sc
 __device__ __forceinline__ void bs_split8(const float2 (&v)[8], float sc, uint4 &rh, uint4 &rl, uint4 &ih, uint4 &il) {
     uint32_t *a = reinterpret_cast<uint32_t *>(&rh), *b = reinterpret_cast<uint32_t *>(&rl);

@@ -77,10 +77,12 @@ struct BsImages {
 cudaError_t launch_bcr_image(int n, const float2 *src, long long stride, const int *pairs_dev, int count,
                              const BsImages &im, cudaStream_t st);
 
-// Products of images (bcr_gemm.cu): tasks of BG_TASK ints (flags, matrix A, matrix B, output): the
-// image of +-A B^T as matrix `output`, or (BG_FP32) D block `output` += +-A B^T
-constexpr int BG_TASK = 4;
-enum { BG_NEG = 1, BG_FP32 = 2 };
+// Products of images (bcr_gemm.cu): tasks of BG_TASK ints (flags, matrix A, matrix B, output, and two
+// more): the image of +-A B^T as matrix `output` and, with BG_TR, of its transpose as the matrix in
+// the fifth place; or (BG_FP32) D block `output` += +-A B^T, with BG_TWO += +-(A B^T + A' B'^T), A'
+// and B' the fifth and sixth
+constexpr int BG_TASK = 6;
+enum { BG_NEG = 1, BG_FP32 = 2, BG_TWO = 4, BG_TR = 8 };
 struct BgArgs {
     int nz;
     const int *tasks;
@@ -92,7 +94,7 @@ struct BgArgs {
     int n_chunk, nzr, nt, n_tiles, log2_2k;
     size_t mat_bytes;
 };
-cudaError_t launch_bcr_gemm(BgArgs a, int n_tasks, cudaStream_t st);
+cudaError_t launch_bcr_gemm(BgArgs a, int n_tasks, int n_products, cudaStream_t st);
 cudaError_t launch_bcr_solve(BsArgs a, const BsStep *steps, int n_steps, bool prepared, double flops, cudaStream_t st);
 int device_sms();   // streaming multiprocessors of the current device
 
