@@ -184,8 +184,9 @@ extern "C" void helm_op_destroy(helm_op_t *op) {
 // ------------------------------------------------------------------------ factor
 
 // Factor method of a mixed factor: the options, else HELM_FACTOR=line|bcr, else BCR on lines of at
-// least kBcrLine nodes, and on shorter ones from kBcrShortLine nodes and as many lines on while its
-// blocks stay within kBcrShortBytes.  FP64 factors are line factors (the tensor cores have no FP64
+// least kBcrLine nodes, and on shorter or odd ones (an odd line gets one more, decoupled, node; only
+// the automatic choice takes it) from kBcrShortLine nodes and as many lines on while its blocks stay
+// within kBcrShortBytes.  FP64 factors are line factors (the tensor cores have no FP64
 // path).
 static constexpr int kBcrLine = 192;
 // Both sides at one frequency, where the line factor is at its best (us, line / BCR): factor at
@@ -202,7 +203,7 @@ static constexpr size_t kBcrShortBytes = (size_t)16 << 30;
 // medium makes an eliminated block nearly singular.  Over random media the refinement took one
 // sweep more from |A| |Dinv| of 2^9 (entries of the inverses of 2^7 and a diagonal of about 4), 5 to
 // 6 sweeps at 2^10, 7 to 15 at 2^11, and did not converge at 2^13; nearly all factors stay below
-// 2^5.  From 2^10 a short line takes the line recurrence.
+// 2^5.  From 2^10 a short or odd line takes the line recurrence.
 static constexpr float kBcrMaxGrowth = 1024.f;
 bool helm::factor_picks_bcr(const GridGeom &g, helm_prec prec, int method) {
     if (prec != HELM_MIXED || !bcr_supported(g)) return false;
@@ -215,12 +216,12 @@ bool helm::factor_picks_bcr(const GridGeom &g, helm_prec prec, int method) {
     }
     return m == HELM_FACTOR_BCR;
 }
-// the automatic choice of BCR on a short line (taken back where it turns out badly)
+// the automatic choice of BCR on a short or odd line (taken back where it turns out badly)
 static bool picks_short_bcr(const helm_op *op, helm_prec prec, const helm_factor_opts *opts) {
     const GridGeom &g = op->g;
     const char *env = getenv("HELM_FACTOR");
     if ((opts && opts->method != HELM_FACTOR_AUTO) || (env && (!strcmp(env, "line") || !strcmp(env, "bcr")))) return false;
-    return prec == HELM_MIXED && bcr_supported(g) && g.nz < kBcrLine && g.nz >= kBcrShortLine && g.nx >= kBcrShortLine &&
+    return prec == HELM_MIXED && (g.nz < kBcrLine || (g.nz & 1)) && g.nz >= kBcrShortLine && g.nx >= kBcrShortLine &&
            6 * sizeof(float2) * op->n_omega * g.nx * g.nz * g.nz <= kBcrShortBytes;
 }
 static bool bcr_falls_back(const GridGeom &g, const int st_host[3]) {
@@ -306,7 +307,7 @@ extern "C" helm_status helm_factor(helm_op_t *op, helm_prec prec, const helm_fac
             return s;
         }
         if (s == HELM_OK) e = read_status(cudaSuccess);
-        // an automatic choice on a short line, which the line recurrence (its Schur complements run
+        // an automatic choice on a short or odd line, which the line recurrence (its Schur complements run
         // from the absorbing boundary, and it holds less) takes instead where an eliminated block
         // came out nearly singular or the blocks did not fit
         if (e == cudaSuccess && short_bcr && (s != HELM_OK || bcr_falls_back(g, st_host))) {
@@ -412,8 +413,8 @@ helm_status factor_reserve(helm_factor_t *f, int nrhs) {
         ((s = dev_alloc((void **)&f->bd, cols * N * sizeof(float4), "allocate(rhs pairs)", st)) != HELM_OK ||
          (s = dev_alloc((void **)&f->xa, cols * N * sizeof(float4), "allocate(iterate)", st)) != HELM_OK ||
          (s = dev_alloc((void **)&f->xb, cols * N * sizeof(float4), "allocate(iterate)", st)) != HELM_OK ||
-         (s = dev_alloc((void **)&f->r32, cols * N * sizeof(float2), "allocate(residual)", st)) != HELM_OK ||
-         (s = dev_alloc((void **)&f->y, cols * N * sizeof(float2), "allocate(work)", st)) != HELM_OK))
+         (s = dev_alloc((void **)&f->r32, cols * op->g.nx * solve_line(f) * sizeof(float2), "allocate(residual)", st)) != HELM_OK ||
+         (s = dev_alloc((void **)&f->y, cols * op->g.nx * solve_line(f) * sizeof(float2), "allocate(work)", st)) != HELM_OK))
         return s;
     if (f->use_bcr &&
         (s = dev_alloc((void **)&f->maxima, bcr_maxima_elems(op->g, cols) * sizeof(float), "allocate(maxima)", st)) != HELM_OK)
@@ -466,10 +467,11 @@ helm_status mixed_refine(const helm_factor_t *f, int nrhs, const double2 *B, dou
     cudaError_t e = cudaMemsetAsync(w.norms, 0, (size_t)cols * 2 * sizeof(double) + refine_state_bytes(n_sys), op->st);
     // block cyclic reduction: the maxima of r and the zeroed counters that a solve starts from are
     // left by the kernel that writes r
+    const int ld = solve_line(f);   // line stride of r and y
     float *gmax = f->use_bcr ? w.maxima : nullptr;
     unsigned *ctl = f->use_bcr ? f->bcr.ctl : nullptr;
     const int n_ctl = f->use_bcr ? (int)bs_ctl_words((int)f->bcr.steps.size(), n_sys) : 0;
-    if (e == cudaSuccess) e = launch_refine_start(g, n_sys, nrhs, B, conj, w.bd, w.r32, w.norms, gmax, ctl, n_ctl, op->st);
+    if (e == cudaSuccess) e = launch_refine_start(g, n_sys, nrhs, B, conj, w.bd, w.r32, w.norms, ld, gmax, ctl, n_ctl, op->st);
     if (e != cudaSuccess) { helm_set_error("refinement start", e); return HELM_ECUDA; }
     const int *skip = &w.state->done;
     // the correction A~^{-1} r: line sweep, or the block-cyclic-reduction solve (which works in
@@ -494,7 +496,7 @@ helm_status mixed_refine(const helm_factor_t *f, int nrhs, const double2 *B, dou
             const float4 *x_in = enq == 0 ? nullptr : ((enq & 1) ? w.xa : w.xb);
             float4 *x_out = (enq & 1) ? w.xb : w.xa;
             if ((e = sweep(skip)) != cudaSuccess) { helm_set_error("sweep mixed", e); return HELM_ECUDA; }
-            e = launch_refine_update(g, n_sys, nrhs, f->diag2, w.bd, x_in, w.y, x_out, w.r32, w.norms, gmax, ctl, n_ctl,
+            e = launch_refine_update(g, n_sys, nrhs, f->diag2, w.bd, x_in, w.y, x_out, w.r32, w.norms, ld, gmax, ctl, n_ctl,
                                      op->status, op->st, w.state, RefineStop{rtol, kPairFloor, max_iter});
             if (e != cudaSuccess) { helm_set_error("refinement update", e); return HELM_ECUDA; }
         }
@@ -518,12 +520,12 @@ helm_status mixed_refine(const helm_factor_t *f, int nrhs, const double2 *B, dou
         tail = true;
         for (;;) {
             e = cudaMemsetAsync(w.norms, 0, (size_t)cols * 2 * sizeof(double), op->st);
-            if (e == cudaSuccess) e = launch_residual(g, n_sys, nrhs, op->diag, B, X, w.r32, w.norms, conj, op->st);
+            if (e == cudaSuccess) e = launch_residual(g, n_sys, nrhs, op->diag, B, X, w.r32, w.norms, conj, op->st, ld);
             if (e != cudaSuccess) { helm_set_error("residual", e); return HELM_ECUDA; }
             if ((s = max_relres(op, (size_t)cols, w.norms, w.norms_host, &rel)) != HELM_OK) return s;
             if (rel <= rtol || it >= max_iter || !isfinite(rel)) break;
             if ((e = sweep(nullptr)) != cudaSuccess) { helm_set_error("sweep mixed", e); return HELM_ECUDA; }
-            e = launch_refine_accumulate(n, w.y, conj, X, op->st);
+            e = launch_refine_accumulate(n, g.nz, ld, w.y, conj, X, op->st);
             if (e != cudaSuccess) { helm_set_error("refinement accumulate", e); return HELM_ECUDA; }
             ++it;
         }

@@ -109,6 +109,8 @@ helm_status acq_upload(const helm_op *op, const helm_acq *acq, DevAcq *d);
 // block cyclic reduction (bcr.cu)
 namespace helm {
 bool bcr_supported(const GridGeom &g);
+int bcr_line(const GridGeom &g);               // nodes of a line as BCR lays it out: an odd line has one more
+int solve_line(const helm_factor_t *f);        // line stride of the mixed solve's r32 and y
 // whether helm_factor builds a block-cyclic-reduction factor for this grid and precision
 // (method: a helm_factor_method; HELM_FACTOR_AUTO follows HELM_FACTOR and the line length)
 bool factor_picks_bcr(const GridGeom &g, helm_prec prec, int method);

@@ -268,10 +268,10 @@ __global__ void __launch_bounds__(128) tri_image_kernel(int n, int n_chunk, int 
 //   D_k = T_k - C X_{k-1} C - C X_{k+1} C
 // a CTA takes 32 rows by 256 columns, a thread two columns (their generators in registers; the
 // rows' are the same for the whole CTA)
-__global__ void __launch_bounds__(128) bcr_level0_kernel(GridGeom g, Coup cp, float2 *D, const double2 *diag, TriGen tg) {
+__global__ void __launch_bounds__(128) bcr_level0_kernel(GridGeom g, int np, Coup cp, float2 *D, const double2 *diag, TriGen tg) {
     const int nz = g.nz, nx = g.nx, no = nx / 2, nk = (nx + 1) / 2;
     const int s = blockIdx.x / nk, k = 2 * (blockIdx.x % nk), c = 256 * blockIdx.z + 2 * threadIdx.x;
-    if (c >= nz) return;
+    if (c >= np) return;
     const bool has[2] = {k >= 1, k + 1 < nx};
     float4 uc[2][2], vc[2][2];
     int2 ec[2][2];
@@ -284,15 +284,20 @@ __global__ void __launch_bounds__(128) bcr_level0_kernel(GridGeom g, Coup cp, fl
         base[n] = ((size_t)s * no + (has[n] ? k / 2 - 1 + n : 0)) * nz;
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
-            uc[n][h] = __ldg(tg.u + base[n] + c + h);
-            vc[n][h] = __ldg(tg.v + base[n] + c + h);
-            ec[n][h] = __ldg(tg.e + base[n] + c + h);
+            const int cc = min(c + h, nz - 1);
+            uc[n][h] = __ldg(tg.u + base[n] + cc);
+            vc[n][h] = __ldg(tg.v + base[n] + cc);
+            ec[n][h] = __ldg(tg.e + base[n] + cc);
         }
     }
     const float cz = cp.cz(k, nx);
     const double2 *dg = diag + ((size_t)s * nx + k) * nz;
-    float2 *Dk = D + ((size_t)s * nx + k) * nz * nz;
-    for (int r = 32 * blockIdx.y; r < min(nz, 32 * (int)blockIdx.y + 32); ++r) {
+    float2 *Dk = D + ((size_t)s * nx + k) * np * np;
+    for (int r = 32 * blockIdx.y; r < min(np, 32 * (int)blockIdx.y + 32); ++r) {
+        if (r >= nz) {   // an odd line's extra node: decoupled
+            *reinterpret_cast<float4 *>(Dk + (size_t)r * np + c) = make_float4(c == r ? 1.f : 0.f, 0.f, c + 1 == r ? 1.f : 0.f, 0.f);
+            continue;
+        }
         float2 t[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
 #pragma unroll
         for (int n = 0; n < 2; ++n) {
@@ -316,9 +321,9 @@ __global__ void __launch_bounds__(128) bcr_level0_kernel(GridGeom g, Coup cp, fl
             if (r == cc) d = to_c64(dg[r]);
             else if (r - cc == 1 || cc - r == 1) d.x = cz;
             const float f = fr * fc[h];
-            o[h] = make_float2(d.x - f * t[h].x, d.y - f * t[h].y);
+            o[h] = cc < nz ? make_float2(d.x - f * t[h].x, d.y - f * t[h].y) : make_float2(0.f, 0.f);
         }
-        *reinterpret_cast<float4 *>(Dk + (size_t)r * nz + c) = make_float4(o[0].x, o[0].y, o[1].x, o[1].y);
+        *reinterpret_cast<float4 *>(Dk + (size_t)r * np + c) = make_float4(o[0].x, o[0].y, o[1].x, o[1].y);
     }
 }
 
@@ -891,6 +896,10 @@ helm_status image_gemm(const BgArgs &ba, const std::vector<int> &tasks, Plan &pl
 
 }  // namespace
 
+int bcr_line(const GridGeom &g) { return g.nz + (g.nz & 1); }
+
+int solve_line(const helm_factor_t *f) { return f->use_bcr ? bcr_line(f->op->g) : f->op->g.nz; }
+
 bool bcr_supported(const GridGeom &g) { return (g.nz % 2) == 0 && g.nz >= 16 && g.nx >= 4; }
 
 // ------------------------------------------------------------------ factor
@@ -898,7 +907,8 @@ bool bcr_supported(const GridGeom &g) { return (g.nz % 2) == 0 && g.nz >= 16 && 
 helm_status bcr_factor(helm_factor_t *f) {
     helm_op *op = f->op;
     const GridGeom &g = op->g;
-    const int nx = g.nx, nz = g.nz, ns = op->n_omega;
+    // (an odd line has one more, decoupled, node here: pairs of entries on 16-byte boundaries)
+    const int nx = g.nx, nz = bcr_line(g), ns = op->n_omega;
     const long long nz2 = (long long)nz * nz;
     const int half = nx / 2 + 1, quart = nx / 4 + 1;
     const cudaStream_t st = op->st;
@@ -965,7 +975,7 @@ helm_status bcr_factor(helm_factor_t *f) {
     // level 0: generators of the odd lines' inverses, their images and the even lines' blocks
     {
         const int no = nx / 2, n_line = ns * no;
-        const size_t n_gen = (size_t)n_line * nz;
+        const size_t n_gen = (size_t)n_line * g.nz;
         std::vector<int> dst;
         for (int sy = 0; sy < ns; ++sy)
             for (int j = 1; j < nx; j += 2) dst.insert(dst.end(), {mat(BS_DINV, sy, j), (int)m0 + sy * m_stride + j / 2});
@@ -989,9 +999,9 @@ helm_status bcr_factor(helm_factor_t *f) {
             HELM_TRACED(K_BCR_L0, st, (tri_scan_kernel<<<(2 * n_line + 31) / 32, 32, 0, st>>>(g, n_line, diag, ts)));
             HELM_TRACED(K_BCR_L0, st, (tri_gen_kernel<<<n_line, 256, 0, st>>>(g, cp, n_line, diag, ts, tg, dev + off, im)));
             HELM_TRACED(K_BCR_IMAGE, st, (tri_image_kernel<<<dim3(n_line, (lay.nzr + 31) / 32), 128, 0, st>>>(
-                                             nz, lay.n_chunk, lay.nzr, tg, dev + off, cp, im, lay.mat_bytes)));
+                                             g.nz, lay.n_chunk, lay.nzr, tg, dev + off, cp, im, lay.mat_bytes)));
             HELM_TRACED(K_BCR_L0, st, (bcr_level0_kernel<<<dim3(ns * ((nx + 1) / 2), (nz + 31) / 32, (nz + 255) / 256), 128, 0, st>>>(
-                                          g, cp, D0, diag, tg)));
+                                          g, nz, cp, D0, diag, tg)));
             const cudaError_t e2 = cudaGetLastError();
             if (e2 != cudaSuccess) { helm_set_error("bcr: level 0", e2); return HELM_ECUDA; }
             return HELM_OK;
@@ -1141,7 +1151,8 @@ helm_status bcr_solve(const helm_factor_t *f, int nrhs, float2 *r, float2 *x, fl
     const BcrData &b = f->bcr;
     BsArgs a{};
     a.nx = g.nx;
-    a.nz = g.nz;
+    a.nz = bcr_line(g);
+    a.edge = g.nz - 1;
     a.ns = op->n_omega;
     a.nrhs = nrhs;
     a.half = b.half;

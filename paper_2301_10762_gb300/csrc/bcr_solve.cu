@@ -402,8 +402,8 @@ __global__ void __launch_bounds__(BS_THREADS, 1) bcr_solve_kernel(const __grid_c
                 }
                 for (int c = 0; c < a.n_chunk; ++c, ++cc) {
                     const int s = cc % ST, k = 32 * c + 2 * j, e = 3 * (c % (BS_AHEAD0 + 1));
-                    const float c0 = (k == 0 || k == a.nz - 1) ? a.cx_edge : a.cx_in;
-                    const float c1 = k + 1 == a.nz - 1 ? a.cx_edge : a.cx_in;
+                    const float c0 = (k == 0 || k == a.edge) ? a.cx_edge : a.cx_in;
+                    const float c1 = k + 1 == a.edge ? a.cx_edge : a.cx_in;
                     fetch3(c + BS_AHEAD0);
                     cp_async_wait<BS_AHEAD0>();
                     float4 v[PR];
@@ -501,7 +501,7 @@ __global__ void __launch_bounds__(BS_THREADS, 1) bcr_solve_kernel(const __grid_c
             float *gm = to_r ? a.gr : a.gx;
             // sign and (level 0, forward) the coupling of the row
             const float f = type == BS_FWD ? -1.f
-                                           : (type == BS_FWD0 ? -((m == 0 || m == a.nz - 1) ? a.cx_edge : a.cx_in) : 1.f);
+                                           : (type == BS_FWD0 ? -((m == 0 || m == a.edge) ? a.cx_edge : a.cx_in) : 1.f);
             float2 *out = vec + ((size_t)tl.sys * a.nrhs + tl.n0) * N + (size_t)line * a.nz + m;
             float *gout = gm + (((size_t)tl.sys * a.nx + line) * a.ng + (tl.r0 >> 5) + q) * a.nrhs + tl.n0;
             const int ncol = min(nt, a.nrhs - tl.n0), sl = tt % SL;

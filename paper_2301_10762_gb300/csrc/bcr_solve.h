@@ -35,7 +35,8 @@ struct BsPhase {
 };
 struct BsArgs {
     int nx, nz, ns, nrhs, half;
-    float2 *r, *x;          // [ns][nrhs][N]: right-hand sides (overwritten) and the result
+    int edge;               // last node of a line (nz - 1, or nz - 2 where nz counts a line's extra node)
+    float2 *r, *x;          // [ns][nrhs][nx * nz]: right-hand sides (overwritten) and the result
     float *gr, *gx;         // maxima of r and x: [ns][nx][ng][nrhs] each
     const unsigned char *img;
     const int *shift;       // [matrix]: the image holds the block's entries times 2^shift

@@ -37,7 +37,7 @@ cudaError_t launch_line_sweep(const GridGeom &g, int n_sys, int nrhs, const cx_t
                               const int *skip = nullptr, const int *frozen = nullptr);
 // FP64 residual B - A X (A^H X for conj), norms[col] += (||R||^2, ||B||^2); R32 = conj?(R) in FP32 if given
 cudaError_t launch_residual(const GridGeom &g, int n_sys, int nrhs, const double2 *diag, const double2 *B,
-                            const double2 *X, float2 *R32, double *norms, int conj, cudaStream_t st);
+                            const double2 *X, float2 *R32, double *norms, int conj, cudaStream_t st, int ld = 0);
 
 int pick_cluster_size(int nz);
 
@@ -56,7 +56,7 @@ cudaError_t launch_split_diag(size_t n, const double2 *diag, float4 *diag2, cuda
 // (norms zeroed beforehand).  gmax (optional): maxima of r32 for the block-cyclic-reduction solve;
 // ctl (optional): its n_ctl counters, zeroed
 cudaError_t launch_refine_start(const GridGeom &g, int n_sys, int nrhs, const double2 *B, int conj, float4 *bd, float2 *r32,
-                                double *norms, float *gmax, unsigned *ctl, int n_ctl, cudaStream_t st);
+                                double *norms, int ld, float *gmax, unsigned *ctl, int n_ctl, cudaStream_t st);
 // Device-side control of the refinement loop: after each update pass, the stopping test computes
 // rel = max_col ||r|| / ||b|| from the norms, decides whether the pair iteration is done and
 // zeroes norms[col][0] for the next pass.
@@ -93,7 +93,7 @@ struct RefineStop {  // stopping rule of the pair phase, applied on the device
 // copied into the state by the last block.
 cudaError_t launch_refine_update(const GridGeom &g, int n_sys, int nrhs, const float4 *diag2, const float4 *bd,
                                  const float4 *x_in, const float2 *delta, float4 *x_out, float2 *r32, double *norms,
-                                 float *gmax, unsigned *ctl, int n_ctl, const int *solve_status, cudaStream_t st,
+                                 int ld, float *gmax, unsigned *ctl, int n_ctl, const int *solve_status, cudaStream_t st,
                                  RefineState *state, RefineStop stop);
 
 // X = conj?(hi + lo) in FP64 of each system's newest iterate: xa after an odd number of sweeps of
@@ -101,7 +101,7 @@ cudaError_t launch_refine_update(const GridGeom &g, int n_sys, int nrhs, const f
 cudaError_t launch_refine_finish(size_t n, int N, int nrhs, const float4 *xa, const float4 *xb,
                                  const RefineState *state, int conj, double2 *X, cudaStream_t st);
 // X += conj?(delta) in FP64 (refinement tail with FP64 residuals)
-cudaError_t launch_refine_accumulate(size_t n, const float2 *delta, int conj, double2 *X, cudaStream_t st);
+cudaError_t launch_refine_accumulate(size_t n, int nz, int ld, const float2 *delta, int conj, double2 *X, cudaStream_t st);
 
 // ---- zgemm_tc.cu (batched complex GEMM on tcgen05, 3xTF32)
 // A family of complex FP32 matrices: matrix idx starts at base + (idx / div) * stride_hi +

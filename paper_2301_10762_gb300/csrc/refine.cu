@@ -124,6 +124,7 @@ struct RefineVec {
     float *gmax;      // maxima of r: [sys][line][ng][nrhs] (null: not wanted)
     unsigned *ctl;    // the solve's counters, zeroed for the next solve (null: none)
     int n_ctl;
+    int ld;           // line stride of r and of the correction: n_z, or one more (a zero) for odd lines
 };
 __device__ __forceinline__ void group_max(const RefineVec &rv, float2 r, bool on, size_t at, int lane) {
     if (!rv.gmax) return;
@@ -163,10 +164,11 @@ __global__ void __launch_bounds__(RF_THREADS) refine_start_kernel(GridGeom g, in
                 split_double_int(v2.x, v.x, v.z);   // the FP64 split's bits, from integer operations
                 split_double_int(v2.y, v.y, v.w);
                 bd[k] = v;
-                r32[k] = make_float2(v.x, v.y);
+                r32[((size_t)c * g.nx + line) * rv.ld + j] = make_float2(v.x, v.y);
                 // (the zeros of point sources skip the FP64 arithmetic, tested on the bits)
                 if (((ps_bits64(v2.x) | ps_bits64(v2.y)) << 1) != 0) bb += v2.x * v2.x + v2.y * v2.y;
             }
+            if (j == nz && rv.ld > nz) r32[((size_t)c * g.nx + line) * rv.ld + j] = make_float2(0.f, 0.f);
             group_max(rv, make_float2(v.x, v.y), on,
                       (((size_t)(c / nrhs) * g.nx + line) * ng + grp) * nrhs + c % nrhs, lane);
         }
@@ -183,9 +185,9 @@ struct StencilPairs {   // grid couplings as FP32 pairs: x (between lines), z (w
     ff cx_in, cx_edge, cz_in, cz_edge;
 };
 
-// x' = x + delta at node k (x absent: x' = delta)
-__device__ __forceinline__ cff iterate_at(const float4 *x, const float2 *d, size_t e) {
-    const float2 dv = d[e];
+// x' = x + delta at node e (of delta: ed; x absent: x' = delta)
+__device__ __forceinline__ cff iterate_at(const float4 *x, const float2 *d, size_t e, size_t ed) {
+    const float2 dv = d[ed];
     if (!x) return {{dv.x, 0.f}, {dv.y, 0.f}};
     const cff xv = cff_of(x[e]);
     return {ff_add1(xv.re, dv.x), ff_add1(xv.im, dv.y)};
@@ -270,7 +272,8 @@ __global__ void __launch_bounds__(RF_THREADS) refine_update_kernel(GridGeom g, i
         float rr = 0.f;
         const size_t base = (size_t)c * N;
         const float4 *__restrict__ xc = x_in ? x_in + base : nullptr;
-        const float2 *__restrict__ dc = delta + base;
+        const float2 *__restrict__ dc = delta + (size_t)c * nx * rv.ld;
+        float2 *__restrict__ rc = r32 + (size_t)c * nx * rv.ld;
 #pragma unroll (NPT < 4 ? NPT : 4)
         for (int q = 0; q < NPT; ++q) {
             const int it = i0 + q * (RF_THREADS / 32), i = it / ng, grp = it - i * ng, j = 32 * grp + lane;
@@ -278,13 +281,13 @@ __global__ void __launch_bounds__(RF_THREADS) refine_update_kernel(GridGeom g, i
             const bool on = j < nz;
             float2 rf = make_float2(0.f, 0.f);
             if (on) {
-                const int k = i * nz + j;
-                const cff xk = iterate_at(xc, dc, k);
+                const int k = i * nz + j, kd = i * rv.ld + j;
+                const cff xk = iterate_at(xc, dc, k, kd);
                 cff sx = {{0.f, 0.f}, {0.f, 0.f}}, sz = sx;
-                if (i > 0) sx = cff_add(sx, iterate_at(xc, dc, k - nz));
-                if (i < nx - 1) sx = cff_add(sx, iterate_at(xc, dc, k + nz));
-                if (j > 0) sz = cff_add(sz, iterate_at(xc, dc, k - 1));
-                if (j < nz - 1) sz = cff_add(sz, iterate_at(xc, dc, k + 1));
+                if (i > 0) sx = cff_add(sx, iterate_at(xc, dc, k - nz, kd - rv.ld));
+                if (i < nx - 1) sx = cff_add(sx, iterate_at(xc, dc, k + nz, kd + rv.ld));
+                if (j > 0) sz = cff_add(sz, iterate_at(xc, dc, k - 1, kd - 1));
+                if (j < nz - 1) sz = cff_add(sz, iterate_at(xc, dc, k + 1, kd + 1));
                 const ff cxj = (j == 0 || j == nz - 1) ? cp.cx_edge : cp.cx_in;
                 const ff czi = (i == 0 || i == nx - 1) ? cp.cz_edge : cp.cz_in;
                 cff ax = cff_mul(cff_of(diag2[(size_t)sys * N + k]), xk);
@@ -293,10 +296,11 @@ __global__ void __launch_bounds__(RF_THREADS) refine_update_kernel(GridGeom g, i
                 const cff r = cff_sub(cff_of(__ldcs(bd + base + k)), ax);
                 x_out[base + k] = cff_pack(xk);
                 rf = make_float2(r.re.hi, r.im.hi);
-                r32[base + k] = rf;
+                rc[kd] = rf;
                 const float sr = r.re.hi * scale, si = r.im.hi * scale;
                 rr = fmaf(sr, sr, fmaf(si, si, rr));
             }
+            if (j == nz && rv.ld > nz) rc[i * rv.ld + j] = make_float2(0.f, 0.f);
             group_max(rv, rf, on, (((size_t)sys * nx + i) * ng + grp) * nrhs + (c - sys * nrhs), lane);
         }
         rr = block_sum(rr, shf);
@@ -321,9 +325,9 @@ __global__ void __launch_bounds__(RF_THREADS) refine_update_kernel(GridGeom g, i
     }
 }
 
-__global__ void refine_accumulate_kernel(size_t n, const float2 *d, int conj, double2 *X) {
+__global__ void refine_accumulate_kernel(size_t n, int nz, int ld, const float2 *d, int conj, double2 *X) {
     for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < n; e += (size_t)gridDim.x * blockDim.x) {
-        const float2 v = d[e];
+        const float2 v = d[ld == nz ? e : e / nz * ld + e % nz];
         double2 x = X[e];
         x.x += (double)v.x;
         x.y += conj ? -(double)v.y : (double)v.y;
@@ -385,10 +389,10 @@ static dim3 refine_grid(const GridGeom &g, int cols, int npt) {
 }
 
 cudaError_t launch_refine_start(const GridGeom &g, int n_sys, int nrhs, const double2 *B, int conj, float4 *bd, float2 *r32,
-                                double *norms, float *gmax, unsigned *ctl, int n_ctl, cudaStream_t st) {
+                                double *norms, int ld, float *gmax, unsigned *ctl, int n_ctl, cudaStream_t st) {
     const int cols = n_sys * nrhs, npt = refine_npt(g, cols);
     const dim3 grid = refine_grid(g, cols, npt);
-    const RefineVec rv{gmax, ctl, n_ctl};
+    const RefineVec rv{gmax, ctl, n_ctl, ld};
     HELM_TRACED(K_REFSTART, st, ((npt == 8 ? refine_start_kernel<8> : refine_start_kernel<2>)<<<grid, RF_THREADS, 0, st>>>(
                                     g, nrhs, cols, B, conj, bd, r32, norms, rv)));
     return cudaGetLastError();
@@ -396,11 +400,11 @@ cudaError_t launch_refine_start(const GridGeom &g, int n_sys, int nrhs, const do
 
 cudaError_t launch_refine_update(const GridGeom &g, int n_sys, int nrhs, const float4 *diag2, const float4 *bd,
                                  const float4 *x_in, const float2 *delta, float4 *x_out, float2 *r32, double *norms,
-                                 float *gmax, unsigned *ctl, int n_ctl, const int *solve_status, cudaStream_t st,
+                                 int ld, float *gmax, unsigned *ctl, int n_ctl, const int *solve_status, cudaStream_t st,
                                  RefineState *state, RefineStop stop) {
     const int cols = n_sys * nrhs, npt = refine_npt(g, cols);
     const dim3 grid = refine_grid(g, cols, npt);
-    const RefineVec rv{gmax, ctl, n_ctl};
+    const RefineVec rv{gmax, ctl, n_ctl, ld};
     StencilPairs cp{pair_of(coup_x(g, 1)), pair_of(coup_x(g, 0)), pair_of(coup_z(g, 1)), pair_of(coup_z(g, 0))};
     HELM_TRACED(K_REFUPDATE, st, ((npt == 8 ? refine_update_kernel<8> : refine_update_kernel<2>)<<<grid, RF_THREADS, 0, st>>>(
                                      g, nrhs, cols, diag2, bd, x_in, delta, x_out, r32, norms, cp, state, stop, rv,
@@ -414,8 +418,8 @@ cudaError_t launch_refine_finish(size_t n, int N, int nrhs, const float4 *xa, co
     return cudaGetLastError();
 }
 
-cudaError_t launch_refine_accumulate(size_t n, const float2 *delta, int conj, double2 *X, cudaStream_t st) {
-    HELM_TRACED(K_REFACCUM, st, (refine_accumulate_kernel<<<flat_blocks(n), 256, 0, st>>>(n, delta, conj, X)));
+cudaError_t launch_refine_accumulate(size_t n, int nz, int ld, const float2 *delta, int conj, double2 *X, cudaStream_t st) {
+    HELM_TRACED(K_REFACCUM, st, (refine_accumulate_kernel<<<flat_blocks(n), 256, 0, st>>>(n, nz, ld, delta, conj, X)));
     return cudaGetLastError();
 }
 

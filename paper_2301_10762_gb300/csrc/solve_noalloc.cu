@@ -34,11 +34,14 @@ using namespace helm;
 namespace {
 
 constexpr size_t kScratchBytes = (size_t)32 << 20;   // 32 MiB per GPU
+// room for the extra node of an odd line in r32 and y of a block-cyclic-reduction factor (16 bytes a
+// line, from 97 nodes on: below 1/388 of the limit)
+constexpr size_t kPadBytes = (size_t)128 << 10;
 constexpr size_t kMaxCols = 16384;                    // columns (frequency x right-hand side) per call
 constexpr int kMaxDevices = 64;
 
 // the working memory of the no-allocation solve (device global memory, one per GPU)
-static __device__ __align__(256) unsigned char g_noalloc_scratch[kScratchBytes];
+static __device__ __align__(256) unsigned char g_noalloc_scratch[kScratchBytes + kPadBytes];
 
 std::mutex g_mu;
 void *g_dev_addr[kMaxDevices] = {};
@@ -102,6 +105,8 @@ extern "C" helm_status helm_solve_noalloc(helm_factor_t *f, int32_t nrhs, const 
     const bool mixed = f->prec == HELM_MIXED;
     const size_t p_bytes = mixed ? align256(cols * N * sizeof(float4)) : 0;   // bd, xa, xb
     const size_t v_bytes = mixed ? align256(cols * N * sizeof(float2)) : 0;   // r32, y
+    // as laid out: an odd line of a block-cyclic-reduction factor has one more node (kPadBytes)
+    const size_t vp_bytes = mixed ? align256(cols * g.nx * solve_line(f) * sizeof(float2)) : 0;
     const size_t n_bytes = align256(cols * 2 * sizeof(double));
     const size_t s_bytes = mixed ? align256(refine_state_bytes(n_sys)) : 0;
     if (cols > kMaxCols || 3 * p_bytes + 2 * v_bytes + n_bytes + s_bytes > kScratchBytes) {
@@ -147,8 +152,8 @@ extern "C" helm_status helm_solve_noalloc(helm_factor_t *f, int32_t nrhs, const 
         w.xa = (float4 *)(p + p_bytes);
         w.xb = (float4 *)(p + 2 * p_bytes);
         w.r32 = (float2 *)(p + 3 * p_bytes);
-        w.y = (float2 *)(p + 3 * p_bytes + v_bytes);
-        w.norms = (double *)(p + 3 * p_bytes + 2 * v_bytes);
+        w.y = (float2 *)(p + 3 * p_bytes + vp_bytes);
+        w.norms = (double *)(p + 3 * p_bytes + 2 * vp_bytes);
         w.norms_host = g_norms_host;
         w.state = (RefineState *)(w.norms + 2 * cols);
         w.maxima = f->bcr.gsmall;   // (every call within the limits above fits it)

@@ -1008,7 +1008,7 @@ template cudaError_t launch_line_sweep<float>(const GridGeom &, int, int, const 
 constexpr int RES_THREADS = 256;
 
 __global__ void __launch_bounds__(RES_THREADS) residual_kernel(GridGeom g, int nrhs, const double2 *diag,
-                                                               const double2 *B, const double2 *X, float2 *R32,
+                                                               const double2 *B, const double2 *X, float2 *R32, int ld,
                                                                double *norms, int conj, double cx_in, double cx_edge,
                                                                double cz_in, double cz_edge) {
     const int nx = g.nx, nz = g.nz, N = nx * nz;
@@ -1031,7 +1031,7 @@ __global__ void __launch_bounds__(RES_THREADS) residual_kernel(GridGeom g, int n
         if (j < nz - 1) { double2 v = x[k + 1]; ax.x += czi * v.x; ax.y += czi * v.y; }
         double2 b = B[col * N + k];
         double2 r = make_double2(b.x - ax.x, b.y - ax.y);
-        if (R32) R32[col * N + k] = make_float2((float)r.x, conj ? -(float)r.y : (float)r.y);
+        if (R32) R32[(col * nx + i) * ld + j] = make_float2((float)r.x, conj ? -(float)r.y : (float)r.y);
         rr = r.x * r.x + r.y * r.y;
         bb = b.x * b.x + b.y * b.y;
     }
@@ -1058,10 +1058,11 @@ __global__ void __launch_bounds__(RES_THREADS) residual_kernel(GridGeom g, int n
 }
 
 cudaError_t launch_residual(const GridGeom &g, int n_sys, int nrhs, const double2 *diag, const double2 *B,
-                            const double2 *X, float2 *R32, double *norms, int conj, cudaStream_t st) {
+                            const double2 *X, float2 *R32, double *norms, int conj, cudaStream_t st, int ld) {
     const int N = g.nx * g.nz;
+    if (ld == 0) ld = g.nz;
     dim3 grid((N + RES_THREADS - 1) / RES_THREADS, nrhs, n_sys);
-    HELM_TRACED(K_RESIDUAL, st, (residual_kernel<<<grid, RES_THREADS, 0, st>>>(g, nrhs, diag, B, X, R32, norms, conj, coup_x(g, 1), coup_x(g, 0), coup_z(g, 1), coup_z(g, 0))));
+    HELM_TRACED(K_RESIDUAL, st, (residual_kernel<<<grid, RES_THREADS, 0, st>>>(g, nrhs, diag, B, X, R32, ld, norms, conj, coup_x(g, 1), coup_x(g, 0), coup_z(g, 1), coup_z(g, 0))));
     return cudaGetLastError();
 }
 
