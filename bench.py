@@ -197,8 +197,12 @@ def kernel_cost(name, nx, nz, n_sys, nrhs):
 TF32_PER_BF16 = 1.1 / 2.25
 
 
-def tensor_peak(peaks, sustained=True):
+def tensor_peak(peaks, sustained=True, half=False):
+    """half: the FP16 rate (that of BF16); else TF32's"""
     key = "bf16_tflops_sustained" if sustained else "bf16_tflops"
+    if half:
+        return ((peaks[key], f"MEASURED_PEAKS.json {key} (of measured)") if key in peaks
+                else (1700.0 if sustained else 1900.0, "fallback BF16 (of fallback)"))
     if key in peaks:
         return peaks[key] * TF32_PER_BF16, f"MEASURED_PEAKS.json {key} x 1.1/2.25 (TF32/BF16 nominal; of measured)"
     return (1700.0 if sustained else 1900.0) * TF32_PER_BF16, "fallback BF16 x 1.1/2.25 (of fallback)"
@@ -250,12 +254,12 @@ def roofline(name, trace, breakdown, dims, peaks):
            "traffic": None}
     hbm = peaks.get("hbm_gbs")
     hbm_src = "MEASURED_PEAKS.json hbm_gbs (of measured)" if hbm else "fallback 6800 GB/s (of fallback)"
-    if name == "zgemm_tf32x3" and st.get("flops"):
-        # the tensor-core GEMM of the block-cyclic-reduction factor and solve: useful flops are
+    if name in ("zgemm_tf32x3", "bcr_solve", "bcr_gemm") and st.get("flops"):
+        # the tensor-core products of the block-cyclic-reduction factor and solve: useful flops are
         # 8 M N K per complex product term (the library counts them per launch); the tensor pipe
-        # issues three TF32 products per useful one (hi*hi + hi*lo + lo*hi)
+        # issues three products per useful one (hi*hi + hi*lo + lo*hi), of TF32 or FP16 operands
         useful = st["flops"] / (st["total_ms"] / 1e3) / 1e12
-        peak, src = tensor_peak(peaks, sustained=True)
+        peak, src = tensor_peak(peaks, sustained=True, half=name != "zgemm_tf32x3")
         out.update({"bound": "tensor", "achieved": useful, "peak": peak, "unit": "TFLOP/s", "frac": useful / peak,
                     "peak_source": src, "issued_tflops": 3 * useful, "issued_frac": 3 * useful / peak,
                     "algorithmic_flops_per_launch": st["flops"] / st["timed"]})

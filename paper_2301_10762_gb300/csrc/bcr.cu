@@ -292,7 +292,7 @@ __global__ void __launch_bounds__(128) bcr_level0_kernel(GridGeom g, int np, Cou
     }
     const float cz = cp.cz(k, nx);
     const double2 *dg = diag + ((size_t)s * nx + k) * nz;
-    float2 *Dk = D + ((size_t)s * nx + k) * np * np;
+    float2 *Dk = D + ((size_t)s * nk + k / 2) * np * np;   // (the odd lines' blocks are never formed)
     for (int r = 32 * blockIdx.y; r < min(np, 32 * (int)blockIdx.y + 32); ++r) {
         if (r >= nz) {   // an odd line's extra node: decoupled
             *reinterpret_cast<float4 *>(Dk + (size_t)r * np + c) = make_float4(c == r ? 1.f : 0.f, 0.f, c + 1 == r ? 1.f : 0.f, 0.f);
@@ -864,13 +864,13 @@ helm_status invert_blocks(int n, Fam in, Fam out, const std::vector<int> &pairs,
     return HELM_OK;
 }
 
-// images (bcr_solve.cu) of the blocks in slots pairs[.][0] of D as matrices pairs[.][1]
-helm_status image_blocks(int n, const float2 *D, const std::vector<int> &pairs, const BgArgs &ba, Plan &pl) {
+// images (bcr_solve.cu) of a part of the blocks in slots pairs[.][0] of D as matrices pairs[.][1]
+helm_status image_blocks(const BgArgs &ba, BsPart part, const std::vector<int> &pairs, Plan &pl) {
     if (pairs.empty()) return HELM_OK;
     const int off = pl.add(pairs), count = (int)(pairs.size() / 2);
     const cudaStream_t st = pl.st;
     pl.ops.push_back([=](const int *dev) -> helm_status {
-        const cudaError_t e = launch_bcr_image(n, D, (long long)n * n, dev + off, count, ba.im, st);
+        const cudaError_t e = launch_bcr_image(ba.nz, part, ba.D, (long long)ba.nz * ba.nz, dev + off, count, ba.im, st);
         if (e != cudaSuccess) { helm_set_error("bcr: images", e); return HELM_ECUDA; }
         return HELM_OK;
     });
@@ -894,6 +894,56 @@ helm_status image_gemm(const BgArgs &ba, const std::vector<int> &tasks, Plan &pl
     return HELM_OK;
 }
 
+// D[slots[t]] <- its inverse on and below the 128 x 128 blocks of the diagonal, for symmetric blocks:
+// the 2 x 2 block inverse with the products on images of the parts (invert_blocks has them as 3xTF32
+// GEMMs of FP32 blocks, with T^T and X21 as products of their own).  `node`: numbers the recursion.
+int invert_nodes(int n) {   // nodes of the recursion on n columns
+    if (n <= INV_MAX) return 0;
+    const int n1 = INV_MAX * ((n / INV_MAX + 1) / 2);
+    return 1 + invert_nodes(n1) + invert_nodes(n - n1);
+}
+helm_status invert_images(const BgArgs &ba, const std::vector<int> &slots, int r0, int n, int &node, Plan &pl) {
+    const int count = (int)slots.size(), nz = ba.nz;
+    if (n <= INV_MAX) {
+        std::vector<int> pairs;
+        for (int v : slots) pairs.insert(pairs.end(), {v, v});
+        const Fam d = Fam{ba.D, (long long)nz * nz, nz}.sub(r0, r0);
+        return invert_blocks(n, d, d, pairs, ba.status, pl);
+    }
+    const int id = ba.im.n_sub + 8 * node++, n1 = INV_MAX * ((n / INV_MAX + 1) / 2), n2 = n - n1, r1 = r0 + n1;
+    enum { D21, X11, T, X22, TT, X12 };
+    std::vector<int> pairs, tasks;
+    auto image = [&](int part, int pr, int pc, int m, int k) {
+        pairs.clear();
+        for (int t = 0; t < count; ++t) pairs.insert(pairs.end(), {slots[t], id + ba.im.sub * t + part});
+        return image_blocks(ba, BsPart{pr, pc, m, k}, pairs, pl);
+    };
+    // parts A (row ra, column ca) and B: m x n products of inner length k to row ro, column co
+    auto product = [&](int flags, int A, int ra, int ca, int B, int rb, int cb, int m, int nn, int k, int ro, int co, int out,
+                       int out_t) {
+        BgArgs a = ba;
+        a.m = m; a.n = nn; a.k = k;
+        a.ra = ra; a.ca = ca; a.rb = rb; a.cb = cb; a.ro = ro; a.co = co;
+        tasks.clear();
+        for (int t = 0; t < count; ++t) {
+            const int v = id + ba.im.sub * t;
+            tasks.insert(tasks.end(), {flags, v + A, v + B, (flags & BG_FP32) ? slots[t] : v + out, v + out_t, slots[t]});
+        }
+        return image_gemm(a, tasks, pl);
+    };
+    helm_status s;
+    if ((s = invert_images(ba, slots, r0, n1, node, pl)) != HELM_OK ||
+        (s = image(D21, r1, r0, n2, n1)) != HELM_OK || (s = image(X11, r0, r0, n1, n1)) != HELM_OK ||
+        // T = X11 D21^T with T^T, D22 -= D21 T
+        (s = product(BG_TR, X11, r0, r0, D21, r1, r0, n1, n2, n1, r0, r1, T, TT)) != HELM_OK ||
+        (s = product(BG_NEG | BG_FP32, D21, r1, r0, TT, r1, r0, n2, n2, n1, r1, r1, 0, 0)) != HELM_OK ||
+        (s = invert_images(ba, slots, r1, n2, node, pl)) != HELM_OK || (s = image(X22, r1, r1, n2, n2)) != HELM_OK ||
+        // X12 = -T X22 (its transpose X21 to memory), X11 -= T X21
+        (s = product(BG_NEG | BG_STORE, T, r0, r1, X22, r1, r1, n1, n2, n2, r0, r1, X12, 0)) != HELM_OK)
+        return s;
+    return product(BG_NEG | BG_FP32, T, r0, r1, X12, r0, r1, n1, n1, n2, r0, r0, 0, 0);
+}
+
 }  // namespace
 
 int bcr_line(const GridGeom &g) { return g.nz + (g.nz & 1); }
@@ -910,7 +960,7 @@ helm_status bcr_factor(helm_factor_t *f) {
     // (an odd line has one more, decoupled, node here: pairs of entries on 16-byte boundaries)
     const int nx = g.nx, nz = bcr_line(g), ns = op->n_omega;
     const long long nz2 = (long long)nz * nz;
-    const int half = nx / 2 + 1, quart = nx / 4 + 1;
+    const int half = nx / 2 + 1, quart = nx / 4 + 1, nk = (nx + 1) / 2;
     const cudaStream_t st = op->st;
     BcrData &b = f->bcr;
     b.half = half;
@@ -922,7 +972,10 @@ helm_status bcr_factor(helm_factor_t *f) {
     const size_t n_kept = (size_t)ns * (nx + 4 * (size_t)half);
     const int m_stride = half, eighth = nx / 8 + 1;
     const size_t m0 = n_kept, u0 = m0 + (size_t)ns * m_stride;
-    const size_t n_mat = u0 + 2 * (size_t)ns * (quart + eighth);
+    const size_t n_sub = u0 + 2 * (size_t)ns * (quart + eighth);   // parts of a level's blocks (BsImages)
+    const int sub = 8 * std::max(1, invert_nodes(nz));
+    const size_t n_mat = n_sub + (nz > INV_MAX ? (size_t)sub * ns * quart : 0);
+    const size_t n_img = n_sub + (nz > INV_MAX ? 2 * (size_t)ns * quart : 0);
     const int u_stride[2] = {quart, eighth};
     auto u_base = [&](int buf, int which) {   // first matrix of U (which = 0) or L (1) of a buffer
         return u0 + (size_t)ns * (buf == 0 ? which * quart : 2 * quart + which * eighth);
@@ -932,27 +985,31 @@ helm_status bcr_factor(helm_factor_t *f) {
         (s = dev_alloc((void **)&b.shift, n_mat * sizeof(int), "bcr: scales", st)) != HELM_OK ||
         (s = dev_alloc((void **)&b.gsmall, kSmallMaxima * sizeof(float), "bcr: maxima", st)) != HELM_OK)
         return s;
-    // working arrays: the working images and the diagonal blocks (an eliminated line's is inverted in
-    // place), FP32
-    float2 *D = nullptr;
-    BsImages im;
+    // working arrays: the diagonal blocks of the even lines (FP32, an eliminated line's is inverted in
+    // place), the working images, level 0's generators (40 bytes an entry) and recurrences (52), the
+    // maxima; one allocation, whose size is the same in every factor of a grid (several of different
+    // sizes next to the kept blocks left the pool remapping memory: 2.5 ms a factor at 256^2)
+    const size_t n_gen = (size_t)ns * (nx / 2) * g.nz;
+    auto up = [](size_t v) { return (v + 1023) & ~(size_t)1023; };
+    const size_t d_bytes = up((size_t)ns * nk * nz2 * sizeof(float2)), w_bytes = up((n_img - n_kept) * lay.mat_bytes);
+    unsigned char *work = nullptr;
     struct Work {
-        float2 **d;
-        BsImages *im;
+        unsigned char **p;
         cudaStream_t st;
-        ~Work() {
-            dev_free(*d, st);
-            dev_free(im->work, st);
-            dev_free(im->mx, st);
-        }
-    } work{&D, &im, st};
+        ~Work() { dev_free(*p, st); }
+    } work_owner{&work, st};
+    if ((s = dev_alloc((void **)&work, d_bytes + w_bytes + up(n_gen * 92) + n_mat * sizeof(uint32_t), "bcr: work", st)) != HELM_OK)
+        return s;
+    float2 *D = reinterpret_cast<float2 *>(work);
+    BsImages im;
     im.kept = b.img;
+    im.work = work + d_bytes;
+    im.mx = reinterpret_cast<uint32_t *>(work + d_bytes + w_bytes + up(n_gen * 92));
     im.n_kept = (int)n_kept;
     im.shift = b.shift;
-    if ((s = dev_alloc((void **)&D, (size_t)ns * nx * nz2 * sizeof(float2), "bcr: work", st)) != HELM_OK ||
-        (s = dev_alloc((void **)&im.work, (n_mat - n_kept) * lay.mat_bytes, "bcr: work", st)) != HELM_OK ||
-        (s = dev_alloc((void **)&im.mx, n_mat * sizeof(uint32_t), "bcr: maxima", st)) != HELM_OK)
-        return s;
+    im.n_sub = (int)n_sub;
+    im.sub = sub;
+    im.sub0 = (int)(n_sub - n_kept);
     cudaError_t e;
     if ((e = cudaMemsetAsync(im.mx, 0, n_mat * sizeof(uint32_t), st)) != cudaSuccess) {
         helm_set_error("bcr: maxima", e);
@@ -965,27 +1022,35 @@ helm_status bcr_factor(helm_factor_t *f) {
     ba.status = op->status;
     ba.tries = wait_tries();
     Plan pl(st);
-    if ((s = pl.with_split(kFactorSplitElems)) != HELM_OK) return s;
-    const Fam fD{D, nz2, nz};
     auto mat = [&](int kind, int sy, int slot) { return (int)bs_matrix_index(nx, ns, half, kind << 24 | slot, sy); };
-    auto invert = [&](const std::vector<int> &pairs, const std::vector<int> &images) -> helm_status {
-        const helm_status s1 = invert_blocks(nz, fD, fD, pairs, op->status, pl);
-        return s1 != HELM_OK ? s1 : image_blocks(nz, D, images, ba, pl);
+    auto dblk = [&](int sy, int k) { return sy * nk + k / 2; };   // D block of an even line
+    // inverses of the blocks pairs[.][0] of D as matrices pairs[.][1]
+    auto invert = [&](const std::vector<int> &pairs) -> helm_status {
+        std::vector<int> slots;
+        for (size_t t = 0; t < pairs.size(); t += 2) slots.push_back(pairs[t]);
+        if (nz > INV_MAX) {
+            uint32_t *mxs = im.mx + n_sub;
+            const size_t bytes = (size_t)sub * ns * quart * sizeof(uint32_t);
+            pl.ops.push_back([=](const int *) -> helm_status {   // (the level before's maxima)
+                const cudaError_t e2 = cudaMemsetAsync(mxs, 0, bytes, st);
+                if (e2 != cudaSuccess) { helm_set_error("bcr: maxima", e2); return HELM_ECUDA; }
+                return HELM_OK;
+            });
+        }
+        int node = 0;
+        const helm_status s1 = invert_images(ba, slots, 0, nz, node, pl);
+        return s1 != HELM_OK ? s1 : image_blocks(ba, BsPart{0, 0, nz, nz}, pairs, pl);
     };
     // level 0: generators of the odd lines' inverses, their images and the even lines' blocks
     {
         const int no = nx / 2, n_line = ns * no;
-        const size_t n_gen = (size_t)n_line * g.nz;
         std::vector<int> dst;
         for (int sy = 0; sy < ns; ++sy)
             for (int j = 1; j < nx; j += 2) dst.insert(dst.end(), {mat(BS_DINV, sy, j), (int)m0 + sy * m_stride + j / 2});
         const int off = pl.add(dst);
-        void *buf = nullptr;   // generators (40 bytes an entry) and the recurrences' values (52)
-        if ((s = dev_alloc(&buf, n_gen * 92, "bcr: level 0", st)) != HELM_OK) return s;
-        pl.scratch.push_back(buf);
         TriGen tg;
         TriScan ts;
-        tg.u = (float4 *)buf;
+        tg.u = reinterpret_cast<float4 *>(work + d_bytes + w_bytes);
         tg.v = tg.u + n_gen;
         ts.delta = (double2 *)(tg.v + n_gen);
         ts.gamma = ts.delta + n_gen;
@@ -1009,13 +1074,10 @@ helm_status bcr_factor(helm_factor_t *f) {
     }
     int cur = 1, levels = 1;   // U, L of the spacing in buffer cur (from level 2 on)
     for (int sp = 2; sp < nx; sp *= 2, ++levels) {
-        std::vector<int> inv_pairs, img_pairs;
+        std::vector<int> inv;
         for (int sy = 0; sy < ns; ++sy)
-            for (int j = sp; j < nx; j += 2 * sp) {
-                inv_pairs.insert(inv_pairs.end(), {sy * nx + j, sy * nx + j});
-                img_pairs.insert(img_pairs.end(), {sy * nx + j, mat(BS_DINV, sy, j)});
-            }
-        if ((s = invert(inv_pairs, img_pairs)) != HELM_OK) return s;
+            for (int j = sp; j < nx; j += 2 * sp) inv.insert(inv.end(), {dblk(sy, j), mat(BS_DINV, sy, j)});
+        if ((s = invert(inv)) != HELM_OK) return s;
         const int nxt = cur ^ 1;
         // couplings of line k to its neighbours at distance sp
         auto Uc = [&](int sy, int k) { return sp == 2 ? (int)m0 + sy * m_stride + k / 2 : (int)u_base(cur, 0) + sy * u_stride[cur] + k / sp; };
@@ -1036,8 +1098,8 @@ helm_status bcr_factor(helm_factor_t *f) {
                 const int a = k - sp, c = k + sp;
                 const int l = a >= 0 ? Lc(sy, k) : -1, w = a >= 0 ? mat(BS_W, sy, a / 2) : -1;   // D_k -= L_k W_a^T + U_k V_c^T
                 const int u = c < nx ? Uc(sy, k) : -1, v = c < nx ? mat(BS_V, sy, c / 2) : -1;
-                if (a >= 0) add(t2, BG_FP32 | BG_NEG | (c < nx ? BG_TWO : 0), l, w, sy * nx + k, u, v);
-                else if (c < nx) add(t2, BG_FP32 | BG_NEG, u, v, sy * nx + k);
+                if (a >= 0) add(t2, BG_FP32 | BG_NEG | (c < nx ? BG_TWO : 0), l, w, dblk(sy, k), u, v);
+                else if (c < nx) add(t2, BG_FP32 | BG_NEG, u, v, dblk(sy, k));
                 if (k >= 2 * sp) add(t2, BG_NEG, Lc(sy, k), mat(BS_V, sy, a / 2), Ln(sy, k));          // L_k <- -L_k V_a^T
                 if (k + 2 * sp < nx) add(t2, BG_NEG, Uc(sy, k), mat(BS_W, sy, c / 2), Un(sy, k));      // U_k <- -U_k W_c^T
             }
@@ -1055,12 +1117,9 @@ helm_status bcr_factor(helm_factor_t *f) {
     }
     // the last line left: line 0
     {
-        std::vector<int> last, img_pairs;
-        for (int sy = 0; sy < ns; ++sy) {
-            last.insert(last.end(), {sy * nx, sy * nx});
-            img_pairs.insert(img_pairs.end(), {sy * nx, mat(BS_DINV, sy, 0)});
-        }
-        if ((s = invert(last, img_pairs)) != HELM_OK) return s;
+        std::vector<int> last;
+        for (int sy = 0; sy < ns; ++sy) last.insert(last.end(), {dblk(sy, 0), mat(BS_DINV, sy, 0)});
+        if ((s = invert(last)) != HELM_OK) return s;
         int *out = op->status + 2;   // the largest entry of the inverses (the matrices 0 .. ns nx - 1)
         const uint32_t *mxd = im.mx;
         pl.ops.push_back([=](const int *) -> helm_status {

@@ -41,7 +41,7 @@ __device__ __forceinline__ void red_add2(float2 *p, float x, float y) {
 struct BgTile {   // what the MMA thread and the epilogue need of a tile: read ahead by the copy thread
     int flags, terms, out, shift;   // (image: its scale)
     float f[2];                     // +-2^-(shift A + shift B) of the terms
-    int out_t, pad;                 // the transposed image's matrix, or -1
+    int out_t, blk;                 // the transposed image's matrix, or -1; the D block
 };
 
 __global__ void __launch_bounds__(BG_THREADS, 1) bcr_gemm_kernel(BgArgs a) {
@@ -79,7 +79,7 @@ __global__ void __launch_bounds__(BG_THREADS, 1) bcr_gemm_kernel(BgArgs a) {
     tc_fence_after();
     const uint32_t tmem = s_tmem;
     const uint32_t smem0 = (smem_u32(bg_smem) + 1023u) & ~1023u;
-    const int per = a.nt * a.nt;   // tiles of a task
+    const int per = a.mt * a.nt, mr = (a.m + 7) & ~7, nr = (a.n + 7) & ~7;   // tiles of a task; rows of its operands
     auto give_up = [&]() {
         atomicOr(a.status, ST_TIMEOUT);
         s_abort = 1;
@@ -103,6 +103,7 @@ __global__ void __launch_bounds__(BG_THREADS, 1) bcr_gemm_kernel(BgArgs a) {
                 tl.flags = task[0];
                 tl.terms = (tl.flags & BG_TWO) ? 2 : 1;
                 tl.out_t = (tl.flags & BG_TR) ? task[4] : -1;
+                tl.blk = (tl.flags & BG_STORE) ? task[5] : task[3];
                 tl.out = task[3];
                 // image: the bound's scale
                 const int eb = (int)(a.im.mx[task[1]] >> 23) + (int)(a.im.mx[task[2]] >> 23) - 254 + 2 + a.log2_2k;
@@ -116,12 +117,12 @@ __global__ void __launch_bounds__(BG_THREADS, 1) bcr_gemm_kernel(BgArgs a) {
                 tq[i % BG_QD] = tl;
                 mbar_arrive_cta(&tq_full[i % BG_QD]);
                 const int m0 = 128 * (t % per / a.nt), n0 = 128 * (t % a.nt);
-                const uint32_t ba = 128u * (uint32_t)min(128, a.nzr - m0), bb = 128u * (uint32_t)min(128, a.nzr - n0);
+                const uint32_t ba = 128u * (uint32_t)min(128, mr - m0), bb = 128u * (uint32_t)min(128, nr - n0);
                 const unsigned char *pa = nullptr, *pb = nullptr;
                 for (int c = 0, n = a.n_chunk * tl.terms; c < n; ++c, pa += 2 * im_off, pb += 2 * im_off) {
                     if (c % a.n_chunk == 0) {   // the next term
-                        pa = a.im.at(c == 0 ? task[1] : task[4], a.mat_bytes) + (size_t)m0 * 128;
-                        pb = a.im.at(c == 0 ? task[2] : task[5], a.mat_bytes) + (size_t)n0 * 128;
+                        pa = a.im.at(c == 0 ? task[1] : task[4], a.mat_bytes) + (size_t)(a.ca >> 5) * 2 * im_off + (size_t)(a.ra + m0) * 128;
+                        pb = a.im.at(c == 0 ? task[2] : task[5], a.mat_bytes) + (size_t)(a.cb >> 5) * 2 * im_off + (size_t)(a.rb + n0) * 128;
                     }
                     if (!wait1(&empty[s], ph)) { go = false; break; }
                     const uint32_t dst = smem0 + (uint32_t)(s * BG_STAGE);
@@ -149,7 +150,7 @@ __global__ void __launch_bounds__(BG_THREADS, 1) bcr_gemm_kernel(BgArgs a) {
                 if (!wait1(&tq_full[i % BG_QD], (uint32_t)((i / BG_QD) & 1))) break;
                 const int terms = tq[i % BG_QD].terms;
                 mbar_arrive_cta(&tq_empty[i % BG_QD]);
-                const int n0 = 128 * (t % a.nt), nb = min(128, (a.nzr - n0 + 15) & ~15);
+                const int n0 = 128 * (t % a.nt), nb = min(128, (nr - n0 + 15) & ~15);
                 const uint32_t id = idesc_f16(nb, false), idn = idesc_f16(nb, true);
                 for (int c = 0, n = a.n_chunk * terms; c < n; ++c, ++cc) {
                     if (!wait1(&acc_empty[cc & 1], (uint32_t)((cc >> 1) & 1) ^ 1u) || !wait1(&full[s], ph)) { go = false; break; }
@@ -179,7 +180,7 @@ __global__ void __launch_bounds__(BG_THREADS, 1) bcr_gemm_kernel(BgArgs a) {
         const int q = warp & 3, hh = (warp - BG_EPI0) >> 2;
         int cc = 0, i = 0;
         bool go = true;
-        const int n_cols = 32 * a.n_chunk;
+        const int n_cols = (a.n + 31) & ~31, m_cols = (a.m + 31) & ~31;
         unsigned char *stage = bg_smem + (smem0 - smem_u32(bg_smem)) + BG_STAGES * BG_STAGE + (warp - BG_EPI0) * BG_OUT;
         auto stage_wait = [&]() {   // the copy out of the staging buffer has read it
             if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
@@ -241,32 +242,35 @@ __global__ void __launch_bounds__(BG_THREADS, 1) bcr_gemm_kernel(BgArgs a) {
             }
             if (!go) break;
             const int mb = m - lane;   // the warp's rows mb .. mb + 31
-            if (flags & BG_FP32) {
+            if (flags & (BG_FP32 | BG_STORE)) {
                 // the update is symmetric: entry (m, n) is added to D[n][m], 256 contiguous bytes of a
                 // column's 32 rows at a time, and without a load
-                float2 *dst = a.D + (size_t)out * a.nz * a.nz + m;
-                if (m < a.nz) {
+                float2 *dst = a.D + ((size_t)tl.blk * a.nz + a.co + n0) * a.nz + a.ro + m;
+                if (m < a.m) {
 #pragma unroll
                     for (int e = 0; e < 64; ++e)
-                        if (n0 + e < a.nz) red_add2(dst + (size_t)(n0 + e) * a.nz, re[e], im[e]);
+                        if (n0 + e < a.n) {
+                            if (flags & BG_STORE) dst[(size_t)e * a.nz] = make_float2(re[e], im[e]);
+                            else red_add2(dst + (size_t)e * a.nz, re[e], im[e]);
+                        }
                 }
-                continue;
+                if (!(flags & BG_STORE)) continue;
             }
             const float sc = bs_pow2(sh);
             uint32_t mxv = 0;
             unsigned char *img = a.im.at(out, a.mat_bytes), *img_t = tl.out_t >= 0 ? a.im.at(tl.out_t, a.mat_bytes) : nullptr;
             const size_t half = (size_t)a.nzr * 128;
-            const int rows = min(32, a.nzr - mb);
+            const int rows = min(32, mr - mb);
 #pragma unroll
             for (int cb = 0; cb < 64; cb += 32) {
-                const int nn = n0 + cb, c = nn >> 5;
+                const int nn = n0 + cb, c = (a.co + nn) >> 5;
                 if (nn >= n_cols) continue;
 #pragma unroll
                 for (int p = 0; p < 2; ++p) {
                     float *v = (p ? im : re) + cb;
 #pragma unroll
                     for (int e = 0; e < 32; ++e) {
-                        if (m >= a.nz || nn + e >= a.nz) v[e] = 0.f;
+                        if (m >= a.m || nn + e >= a.n) v[e] = 0.f;
                         mxv = max(mxv, bs_abs_bits(v[e]));
                         v[e] *= sc;
                     }
@@ -282,9 +286,9 @@ __global__ void __launch_bounds__(BG_THREADS, 1) bcr_gemm_kernel(BgArgs a) {
                             *reinterpret_cast<uint4 *>(stage + lane * 128 + ((j ^ (lane & 7)) << 4)) = hi;
                             *reinterpret_cast<uint4 *>(stage + lane * 128 + (((j + 4) ^ (lane & 7)) << 4)) = lo;
                         }
-                        stage_store(img + (size_t)(2 * c + p) * half + (size_t)mb * 128, rows * 128);
+                        stage_store(img + (size_t)(2 * c + p) * half + (size_t)(a.ro + mb) * 128, rows * 128);
                     }
-                    if (img_t && mb < n_cols) {
+                    if (img_t && mb < m_cols) {
                         // the transpose: the warp's 32 rows are a chunk of row n; even lanes hold the hi
                         // parts of two columns, odd lanes the lo parts, 128 bytes in all
                         stage_wait();
@@ -293,7 +297,7 @@ __global__ void __launch_bounds__(BG_THREADS, 1) bcr_gemm_kernel(BgArgs a) {
                             const int o = (((lane >> 3) + 4 * (lane & 1)) ^ (e & 7)) * 16 + (lane & 6) * 2;
                             *reinterpret_cast<uint32_t *>(stage + e * 128 + o) = bs_split_pair(v[e], lane);
                         }
-                        stage_store(img_t + (size_t)(2 * (mb >> 5) + p) * half + (size_t)nn * 128, min(32, a.nzr - nn) * 128);
+                        stage_store(img_t + (size_t)(2 * ((a.ro + mb) >> 5) + p) * half + (size_t)(a.co + nn) * 128, min(32, nr - nn) * 128);
                     }
                 }
             }
@@ -302,7 +306,10 @@ __global__ void __launch_bounds__(BG_THREADS, 1) bcr_gemm_kernel(BgArgs a) {
                 if (img_t) a.im.shift[tl.out_t] = sh;
             }
             mxv = __reduce_max_sync(0xffffffffu, mxv);
-            if (lane == 0 && mxv) atomicMax(a.im.mx + out, mxv);
+            if (lane == 0 && mxv) {
+                atomicMax(a.im.mx + out, mxv);
+                if (img_t) atomicMax(a.im.mx + tl.out_t, mxv);
+            }
         }
         if (lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
     }
@@ -318,17 +325,19 @@ cudaError_t launch_bcr_gemm(BgArgs a, int n_tasks, int n_products, cudaStream_t 
     if (n_tasks <= 0) return cudaSuccess;
     if (a.nz & 1) return cudaErrorInvalidValue;
     const BsLayout l = bs_layout(a.nz);
-    a.n_chunk = l.n_chunk;
+    if (a.k == 0) a.m = a.n = a.k = a.nz;
+    a.n_chunk = (a.k + 31) / 32;
     a.nzr = l.nzr;
     a.mat_bytes = l.mat_bytes;
-    a.nt = (a.nz + 127) / 128;
-    a.n_tiles = n_tasks * a.nt * a.nt;
+    a.mt = (a.m + 127) / 128;
+    a.nt = (a.n + 127) / 128;
+    a.n_tiles = n_tasks * a.mt * a.nt;
     a.log2_2k = 1;
-    while ((1 << a.log2_2k) < 2 * a.nz) ++a.log2_2k;
+    while ((1 << a.log2_2k) < 2 * a.k) ++a.log2_2k;
     cudaError_t e = ensure_dyn_smem((const void *)bcr_gemm_kernel, BG_SMEM);
     if (e != cudaSuccess) return e;
     const int grid = std::min(device_sms(), a.n_tiles);
-    HELM_TRACED_W(K_BCR_GEMM, st, 8.0 * a.nz * a.nz * (double)a.nz * n_products,
+    HELM_TRACED_W(K_BCR_GEMM, st, 8.0 * a.m * a.n * (double)a.k * n_products,
                   (bcr_gemm_kernel<<<grid, BG_THREADS, BG_SMEM, st>>>(a)));
     return cudaGetLastError();
 }

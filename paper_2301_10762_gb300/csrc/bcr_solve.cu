@@ -602,38 +602,51 @@ __global__ void __launch_bounds__(256) line_max_kernel(int nx, int nz, int ng, i
     if (lane < nc) g[(((size_t)sys * nx + line) * ng + grp) * nrhs + c0 + lane] = __uint_as_float(mine);
 }
 
-// largest modulus of the real and imaginary parts of the blocks, as bits (mx zeroed beforehand)
-__global__ void __launch_bounds__(256) bcr_max_kernel(long long n2, const float2 *src, long long stride, const int *pairs,
+// largest modulus of the real and imaginary parts of a part of the blocks, as bits (mx zeroed
+// beforehand): a CTA takes 32 rows, up to the end of their 128 x 128 block on the diagonal
+__global__ void __launch_bounds__(256) bcr_max_kernel(int n, BsPart pt, const float2 *src, long long stride, const int *pairs,
                                                       uint32_t *mx) {
     const int *pr = pairs + 2 * (size_t)blockIdx.y;
-    const float4 *A = reinterpret_cast<const float4 *>(src + (long long)pr[0] * stride);
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, r0 = pt.r0 + 32 * blockIdx.x;
+    const int end = min(pt.c0 + pt.n, (r0 | 127) + 1);
     uint32_t m = 0;
-    for (long long e = blockIdx.x * 256 + threadIdx.x; e < n2 / 2; e += (long long)gridDim.x * 256) {
-        const float4 v = __ldg(A + e);
-        m = max(max(m, max(bs_abs_bits(v.x), bs_abs_bits(v.y))), max(bs_abs_bits(v.z), bs_abs_bits(v.w)));
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const int r = r0 + w + 8 * q;
+        if (r >= pt.r0 + pt.m) continue;
+        const float4 *A = reinterpret_cast<const float4 *>(src + (long long)pr[0] * stride + (long long)r * n + pt.c0);
+        for (int e = lane; e < (end - pt.c0) / 2; e += 32) {
+            const float4 v = __ldg(A + e);
+            m = max(max(m, max(bs_abs_bits(v.x), bs_abs_bits(v.y))), max(bs_abs_bits(v.z), bs_abs_bits(v.w)));
+        }
     }
     m = __reduce_max_sync(0xffffffffu, m);
-    if ((threadIdx.x & 31) == 0) atomicMax(mx + pr[1], m);
+    if (lane == 0 && m) atomicMax(mx + pr[1], m);
 }
 
-// Image of a block (n x n row-major) as matrix pairs[.][1].  A CTA takes 32 rows, a thread a row
-// and eight columns at a time; rows and columns beyond n are zero.
-__global__ void __launch_bounds__(128) bcr_image_kernel(int n, int n_chunk, int nzr, const float2 *src, long long stride,
+// Image of a part of a symmetric block (n x n row-major) as matrix pairs[.][1].  A CTA takes 32 rows, a
+// thread a row and eight columns at a time; rows and columns beyond n are zero.
+__global__ void __launch_bounds__(128) bcr_image_kernel(int n, BsPart pt, int nzr, const float2 *src, long long stride,
                                                         const int *pairs, BsImages im, size_t mat_bytes) {
     __shared__ float2 t[32][33];
     const int *pr = pairs + 2 * (size_t)blockIdx.y;
     const float2 *A = src + (long long)pr[0] * stride;
-    const int r0 = 32 * blockIdx.x, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int r0 = pt.r0 + 32 * blockIdx.x, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int sh = bs_scale_shift(im.mx[pr[1]]);
     const float sc = bs_pow2(sh);
     if (blockIdx.x == 0 && threadIdx.x == 0) im.shift[pr[1]] = sh;
     const int row = threadIdx.x >> 2, j = threadIdx.x & 3, r = r0 + row;
-    unsigned char *d = im.at(pr[1], mat_bytes) + (size_t)r * 128;
-    for (int c = 0; c < n_chunk; ++c) {
+    const size_t half = (size_t)nzr * 128;
+    unsigned char *d = im.at(pr[1], mat_bytes) + (size_t)(pt.c0 >> 5) * 2 * half + (size_t)r * 128;
+    for (int c = 0; c < (pt.n + 31) / 32; ++c) {
+        const int k0 = pt.c0 + 32 * c;
+        const bool up = (r0 >> 7) < (k0 >> 7);   // above the diagonal: the mirror image's rows
 #pragma unroll
         for (int q = 0; q < 8; ++q) {
-            const int o = w + 4 * q, k = 32 * c + lane;
-            t[o][lane] = r0 + o < n && k < n ? __ldg(A + (long long)(r0 + o) * n + k) : make_float2(0.f, 0.f);
+            const int o = w + 4 * q, rr = (up ? k0 : r0) + o, k = (up ? r0 : k0) + lane;
+            const float2 v = rr < n && k < n ? __ldg(A + (long long)rr * n + k) : make_float2(0.f, 0.f);
+            if (up) t[lane][o] = v;
+            else t[o][lane] = v;
         }
         __syncthreads();
         if (r < nzr) {
@@ -644,10 +657,10 @@ __global__ void __launch_bounds__(128) bcr_image_kernel(int n, int n_chunk, int 
             bs_split8(v, sc, rh, rl, ih, il);
             *reinterpret_cast<uint4 *>(d + ((j ^ (r & 7)) << 4)) = rh;
             *reinterpret_cast<uint4 *>(d + (((j + 4) ^ (r & 7)) << 4)) = rl;
-            d += (size_t)nzr * 128;
+            d += half;
             *reinterpret_cast<uint4 *>(d + ((j ^ (r & 7)) << 4)) = ih;
             *reinterpret_cast<uint4 *>(d + (((j + 4) ^ (r & 7)) << 4)) = il;
-            d += (size_t)nzr * 128;
+            d += half;
         }
         __syncthreads();
     }
@@ -663,17 +676,16 @@ template <int NT> cudaError_t launch_nt(const BsArgs &a, int grid, double flops,
 
 }  // namespace
 
-cudaError_t launch_bcr_image(int n, const float2 *src, long long stride, const int *pairs_dev, int count,
+cudaError_t launch_bcr_image(int n, BsPart part, const float2 *src, long long stride, const int *pairs_dev, int count,
                              const BsImages &im, cudaStream_t st) {
     if (count <= 0) return cudaSuccess;
     const BsLayout l = bs_layout(n);
+    const unsigned rows = (part.m + 31) / 32;
     for (int t = 0; t < count; t += 65535) {
-        const int nb = std::min(65535, count - t);
+        const dim3 grid(rows, std::min(65535, count - t));
         const int *pr = pairs_dev + 2 * (size_t)t;
-        HELM_TRACED(K_BCR_IMAGE, st, (bcr_max_kernel<<<dim3((unsigned)std::min(8, (n * n / 2 + 1023) / 1024), nb), 256, 0, st>>>(
-                                         (long long)n * n, src, stride, pr, im.mx)));
-        HELM_TRACED(K_BCR_IMAGE, st, (bcr_image_kernel<<<dim3((n + 31) / 32, nb), 128, 0, st>>>(
-                                         n, l.n_chunk, l.nzr, src, stride, pr, im, l.mat_bytes)));
+        HELM_TRACED(K_BCR_IMAGE, st, (bcr_max_kernel<<<grid, 256, 0, st>>>(n, part, src, stride, pr, im.mx)));
+        HELM_TRACED(K_BCR_IMAGE, st, (bcr_image_kernel<<<grid, 128, 0, st>>>(n, part, l.nzr, src, stride, pr, im, l.mat_bytes)));
     }
     return cudaGetLastError();
 }

@@ -69,21 +69,32 @@ struct BsImages {
     int n_kept = 0;
     int *shift = nullptr;      // [matrix]
     uint32_t *mx = nullptr;    // [matrix]: bits of the largest modulus (or a bound); working array of the factor
+    // from n_sub on: parts of a block that is being inverted, eight matrices (scales) to a node of its
+    // recursion and `sub` to a block, whose parts fill two images from number sub0 (of the working
+    // ones) on: the first four of a node one, the others the other
+    int n_sub = 0x7fffffff, sub = 8, sub0 = 0;
     __host__ __device__ unsigned char *at(int i, size_t mat_bytes) const {
-        return i < n_kept ? kept + (size_t)i * mat_bytes : work + (size_t)(i - n_kept) * mat_bytes;
+        if (i < n_kept) return kept + (size_t)i * mat_bytes;
+        const int j = i - n_sub;
+        return work + (size_t)(j < 0 ? i - n_kept : sub0 + 2 * (j / sub) + ((j >> 2) & 1)) * mat_bytes;
     }
 };
-// images of n x n row-major blocks src + pairs[.][0] * stride as matrices pairs[.][1]; im.mx zeroed
-// beforehand
-cudaError_t launch_bcr_image(int n, const float2 *src, long long stride, const int *pairs_dev, int count,
+struct BsPart {   // rows r0 .. + m and columns c0 .. + n of a block (r0 and c0 multiples of 128)
+    int r0, c0, m, n;
+};
+// images of the part of n x n row-major symmetric blocks src + pairs[.][0] * stride as that part of the
+// matrices pairs[.][1]; 128 x 128 blocks above the diagonal are taken from below it (and need not be
+// in memory); im.mx zeroed beforehand
+cudaError_t launch_bcr_image(int n, BsPart part, const float2 *src, long long stride, const int *pairs_dev, int count,
                              const BsImages &im, cudaStream_t st);
 
 // Products of images (bcr_gemm.cu): tasks of BG_TASK ints (flags, matrix A, matrix B, output, and two
 // more): the image of +-A B^T as matrix `output` and, with BG_TR, of its transpose as the matrix in
 // the fifth place; or (BG_FP32) D block `output` += +-A B^T, with BG_TWO += +-(A B^T + A' B'^T), A'
-// and B' the fifth and sixth
+// and B' the fifth and sixth; BG_STORE: an image whose transpose is stored to D block in the sixth place.
+// The updates (BG_FP32) are symmetric.
 constexpr int BG_TASK = 6;
-enum { BG_NEG = 1, BG_FP32 = 2, BG_TWO = 4, BG_TR = 8 };
+enum { BG_NEG = 1, BG_FP32 = 2, BG_TWO = 4, BG_TR = 8, BG_STORE = 16 };
 struct BgArgs {
     int nz;
     const int *tasks;
@@ -91,8 +102,11 @@ struct BgArgs {
     float2 *D;               // [block][nz][nz]
     int *status;
     uint32_t tries;
+    // the products of a launch: m x n of inner length k, from row ra and column ca of A, row rb and
+    // column cb of B, to row ro and column co (k = 0: whole blocks)
+    int m, n, k, ra, ca, rb, cb, ro, co;
     // set by launch_bcr_gemm
-    int n_chunk, nzr, nt, n_tiles, log2_2k;
+    int n_chunk, nzr, mt, nt, n_tiles, log2_2k;
     size_t mat_bytes;
 };
 cudaError_t launch_bcr_gemm(BgArgs a, int n_tasks, int n_products, cudaStream_t st);

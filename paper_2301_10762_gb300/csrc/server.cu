@@ -83,20 +83,25 @@ struct helm_server {
     std::vector<std::thread> workers;
 
     // device bytes as admission counts them (see helm_server.h)
+    static bool picks_bcr(const helm_grid &g, int prec) {
+        const helm::GridGeom geom{g.nx, g.nz, g.lx / (g.nx - 1), g.lz / (g.nz - 1), g.lumping};
+        return helm::factor_picks_bcr(geom, (helm_prec)prec, HELM_FACTOR_AUTO);
+    }
     size_t factor_bytes(const helm_grid &g, int prec) const {
         const size_t N = (size_t)g.nx * g.nz, blk = (size_t)g.nz * g.nz * 8;
-        const helm::GridGeom geom{g.nx, g.nz, g.lx / (g.nx - 1), g.lz / (g.nz - 1), g.lumping};
-        if (helm::factor_picks_bcr(geom, (helm_prec)prec, HELM_FACTOR_AUTO)) {
+        if (picks_bcr(g, prec)) {
             // block cyclic reduction: the images of every line's inverse and of P, Q, W, V of the
-            // eliminated ones, and while it factors (counted throughout) 1.25 n_x images of
-            // couplings, the FP32 diagonal blocks and level 0's generators
-            const size_t kept = (size_t)g.nx + 4 * ((size_t)g.nx / 2 + 1), work = 5 * (size_t)g.nx / 4 + 5;
-            return (kept + work) * (helm::bs_layout(g.nz).mat_bytes + 8) + g.nx * blk + 144 * N + 65 * kMiB;   // + split-K tiles
+            // eliminated ones, and while it factors (counted throughout) 1.75 n_x images of
+            // couplings and of parts of the blocks that are inverted, the FP32 blocks of every other
+            // line and level 0's generators
+            const size_t kept = (size_t)g.nx + 4 * ((size_t)g.nx / 2 + 1), work = 7 * (size_t)g.nx / 4 + 7;
+            return (kept + work) * (helm::bs_layout(g.nz).mat_bytes + 8) + (g.nx + 1) / 2 * blk + 144 * N + kMiB;
         }
         return (size_t)g.nx * g.nz * g.nz * (prec == HELM_MIXED ? 8 : 16) + 96 * N + kMiB;
     }
     size_t scratch_bytes(const helm_grid &g, int prec, int nrhs) const {   // refinement scratch in the factor
-        return prec == HELM_MIXED ? (size_t)g.nx * (64 * g.nz + 8 * helm::bs_layout(g.nz).ng) * nrhs + (size_t)nrhs * 16
+        const size_t maxima = picks_bcr(g, prec) ? 8 * (size_t)helm::bs_layout(g.nz).ng : 0;
+        return prec == HELM_MIXED ? (size_t)g.nx * (64 * (size_t)g.nz + maxima) * nrhs + (size_t)nrhs * 16
                                   : (size_t)nrhs * 16;
     }
     size_t staging_bytes(const helm_grid &g, int nrhs) const {   // device B and X of a batch
@@ -276,9 +281,8 @@ void helm_server::run_batch(const Model &md, std::vector<Pending> &batch, Slot *
         const double om = r0.omega;
         if ((status = helm_assemble(&md.grid, md.m_dev, &om, 1, sl->st, &sl->op)) != HELM_OK) goto out;
         // (the method that factor_bytes counted: a short line's automatic choice is the larger factor)
-        const helm::GridGeom geom{md.grid.nx, md.grid.nz, md.grid.lx / (md.grid.nx - 1), md.grid.lz / (md.grid.nz - 1), md.grid.lumping};
         helm_factor_opts fo{};
-        fo.method = helm::factor_picks_bcr(geom, (helm_prec)r0.prec, HELM_FACTOR_AUTO) ? HELM_FACTOR_BCR : HELM_FACTOR_LINE;
+        fo.method = picks_bcr(md.grid, r0.prec) ? HELM_FACTOR_BCR : HELM_FACTOR_LINE;
         if ((status = helm_factor(sl->op, (helm_prec)r0.prec, &fo, &sl->f)) != HELM_OK) goto out;
     }
     if ((status = dev_alloc((void **)&Bd, rhs * N * sizeof(helm_c128), "server: allocate(B)", sl->st)) != HELM_OK ||
