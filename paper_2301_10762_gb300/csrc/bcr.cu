@@ -1061,7 +1061,7 @@ helm_status bcr_factor(helm_factor_t *f) {
         const double2 *diag = op->diag;
         float2 *D0 = D;
         pl.ops.push_back([=](const int *dev) -> helm_status {
-            HELM_TRACED(K_BCR_L0, st, (tri_scan_kernel<<<(2 * n_line + 31) / 32, 32, 0, st>>>(g, n_line, diag, ts)));
+            HELM_TRACED(K_BCR_L0, st, (tri_scan_kernel<<<(2 * n_line + 32 - 1) / 32, 32, 0, st>>>(g, n_line, diag, ts)));
             HELM_TRACED(K_BCR_L0, st, (tri_gen_kernel<<<n_line, 256, 0, st>>>(g, cp, n_line, diag, ts, tg, dev + off, im)));
             HELM_TRACED(K_BCR_IMAGE, st, (tri_image_kernel<<<dim3(n_line, (lay.nzr + 31) / 32), 128, 0, st>>>(
                                              g.nz, lay.n_chunk, lay.nzr, tg, dev + off, cp, im, lay.mat_bytes)));

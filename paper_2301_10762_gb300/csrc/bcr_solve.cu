@@ -72,6 +72,9 @@ __device__ __forceinline__ unsigned ld_acquire(const unsigned *p) {
     asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
     return v;
 }
+struct BsQ {   // a queue entry: the tile, its task and the shifts of the task's blocks, read ahead by the copy thread
+    int t, task[8], sa[3];
+};
 struct Tile {
     int phase, sys, task, n0, r0, rows, nt;
 };
@@ -112,7 +115,7 @@ __global__ void __launch_bounds__(BS_THREADS, 1) bcr_solve_kernel(const __grid_c
     __shared__ __align__(8) uint64_t full[ST], empty[ST];   // a stage written (the copy warp's bytes and the operand warps), read by its MMAs
     __shared__ __align__(8) uint64_t acc_full[SL], acc_empty[SL];
     __shared__ __align__(8) uint64_t tq_full[BS_QD], tq_empty[BS_QD], done_bar;
-    __shared__ int tq[BS_QD];
+    __shared__ BsQ tq[BS_QD];
     __shared__ float s_bscale[SL][NT];   // 2^-S of each right-hand side of an accumulator
     __shared__ uint32_t s_tmem;
     __shared__ int s_abort;
@@ -167,12 +170,12 @@ __global__ void __launch_bounds__(BS_THREADS, 1) bcr_solve_kernel(const __grid_c
         return false;
     };
     // next tile of the queue (i-th): its number, or -1 at the end or after a give-up
-    auto next_tile = [&](int i) -> int {
+    auto next_tile = [&](int i, BsQ &e) -> int {
         if (!wait(&tq_full[i % BS_QD], i / BS_QD)) return -1;
-        const int t = tq[i % BS_QD];
+        e = tq[i % BS_QD];
         __syncwarp();
         if (lane == 0) mbar_arrive_cta(&tq_empty[i % BS_QD]);
-        return t;
+        return e.t;
     };
 
     // the step before tile tl's of the same system is complete (seen: the last one found complete)
@@ -201,24 +204,57 @@ __global__ void __launch_bounds__(BS_THREADS, 1) bcr_solve_kernel(const __grid_c
             int cs = 0, issued = 0;
             uint32_t cph = 1;   // parity of the stage's previous release (the first round passes at once)
             bool go = true;
-            for (int i = 0; go; ++i) {
-                int t;
-                for (;;) {   // the tiles of a converged system are passed over
-                    t = (int)atomicAdd(a.ctl, 1u);
-                    if (t >= a.n_tile_total) { t = -1; break; }
-                    if (!a.frozen || !a.frozen[2 * decode(a, t).sys]) break;
+            // the next tile: its ticket, its task and its blocks' shifts, one access after the other and two
+            // chunks of the present tile apart (together they take 2 to 3 us)
+            BsQ ne;
+            Tile ntl{};
+            int4 a0, a1;
+            int part = 0, frozen = 0;
+            auto advance = [&]() {
+                if (part == 0) {
+                    ne.t = (int)atomicAdd(a.ctl, 1u);
+                } else if (part == 1) {
+                    if (ne.t >= a.n_tile_total) ne.t = -1;
+                    if (ne.t >= 0) {
+                        ntl = decode(a, ne.t);
+                        a0 = __ldg(reinterpret_cast<const int4 *>(a.tasks + 8 * ntl.task));
+                        a1 = __ldg(reinterpret_cast<const int4 *>(a.tasks + 8 * ntl.task) + 1);
+                        frozen = a.frozen ? a.frozen[2 * ntl.sys] : 0;
+                    }
+                } else if (ne.t >= 0) {
+                    ne.task[0] = a0.x; ne.task[1] = a0.y; ne.task[2] = a0.z; ne.task[3] = a0.w;
+                    ne.task[4] = a1.x; ne.task[5] = a1.y; ne.task[6] = a1.z; ne.task[7] = a1.w;
+#pragma unroll
+                    for (int u = 0; u < 3; ++u)
+                        ne.sa[u] = u < (ne.task[1] >> 4) ? __ldg(a.shift + bs_matrix(a, ne.task[2 + 2 * u], ntl.sys)) : 0;
                 }
+                ++part;
+            };
+            for (int i = 0; go; ++i) {
+                for (;;) {   // the tiles of a converged system are passed over
+                    while (part < 3) advance();
+                    if (ne.t < 0 || !frozen) break;
+                    part = 0;
+                }
+                const BsQ e = ne;
+                const Tile tl = ntl;
+                const int *task = e.task;
+                part = 0;
                 if (!wait1(&tq_empty[i % BS_QD], (uint32_t)((i / BS_QD) & 1) ^ 1u)) break;
-                tq[i % BS_QD] = t;
+                tq[i % BS_QD] = e;
                 mbar_arrive_cta(&tq_full[i % BS_QD]);
-                if (t < 0) break;
-                const Tile tl = decode(a, t);
-                const int *task = a.tasks + 8 * tl.task;
+                if (e.t < 0) break;
                 const int nterms = task[1] >> 4;
+                // taking a ticket early keeps the stream of blocks going (256^2, 8 frequencies, 8 columns: 657 -> 614 us), but
+                // binds a tile of the next step to this SM while others may be idle (the chain of a 128^2
+                // system 117 -> 129 us): only in steps of four tiles an SM and more
+                const BsPhase &ph = a.ph[tl.phase];
+                const bool ahead = (long long)ph.tasks * a.ns * ph.n_tiles * ph.mt >= 4ll * gridDim.x;
                 const uint32_t bytes = (uint32_t)tl.rows * 128u;
                 const size_t im_off = (size_t)a.nzr * 128;
                 for (int u = 0; go && u < nterms; ++u) {
-                    const unsigned char *src = a.img + (size_t)bs_matrix(a, task[2 + 2 * u], tl.sys) * a.mat_bytes +
+                    const int code = u == 0 ? task[2] : (u == 1 ? task[4] : task[6]);
+                    const unsigned char *src = a.img + (size_t)bs_matrix(a, code, tl.sys) * a.mat_bytes +
                                                (size_t)tl.r0 * 128;
                     for (int c = 0; c < a.n_chunk; ++c, src += 2 * im_off) {
                         if (!wait1(&empty[cs], cph)) { go = false; break; }
@@ -228,6 +264,7 @@ __global__ void __launch_bounds__(BS_THREADS, 1) bcr_solve_kernel(const __grid_c
                         bulk_load(dst + 16384, src + im_off, bytes, &full[cs]);
                         ++issued;
                         if (++cs == ST) { cs = 0; cph ^= 1u; }
+                        if (ahead && part < 3 && (issued & 1)) advance();
                     }
                 }
             }
@@ -252,11 +289,10 @@ __global__ void __launch_bounds__(BS_THREADS, 1) bcr_solve_kernel(const __grid_c
             const uint64_t dstage0 = desc_sw128(smem0);
             for (int i = 0; go; ++i) {
                 if (!wait1(&tq_full[i % BS_QD], (uint32_t)((i / BS_QD) & 1))) break;
-                const int t = tq[i % BS_QD];
+                const int t = tq[i % BS_QD].t, nterms = tq[i % BS_QD].task[1] >> 4;
                 mbar_arrive_cta(&tq_empty[i % BS_QD]);
                 if (t < 0) break;
-                const Tile tl = decode(a, t);
-                const int nterms = a.tasks[8 * tl.task + 1] >> 4, nt = tl.nt;
+                const int nt = decode(a, t).nt;
                 const uint32_t id = idesc_f16(2 * nt);
                 if (!wait1(&acc_empty[sl], slph)) break;
                 const uint32_t d0 = tmem + (uint32_t)(sl * BS_SLOT_COLS), d1 = d0 + (uint32_t)(2 * nt);
@@ -297,10 +333,11 @@ __global__ void __launch_bounds__(BS_THREADS, 1) bcr_solve_kernel(const __grid_c
         int cc = 0, tt = 0, seen = -1;
         bool go = true;
         for (int i = 0; go; ++i) {
-            const int t = next_tile(i);
+            BsQ entry;
+            const int t = next_tile(i, entry);
             if (t < 0) break;
             const Tile tl = decode(a, t);
-            const int *task = a.tasks + 8 * tl.task;
+            const int *task = entry.task;
             const int type = task[1] & 15, nterms = task[1] >> 4, np = tl.nt / 16;
             if (!step_wait(tl, seen)) break;
             const int row0 = 8 * (ow >> 2) + (ow & 3) + 4 * h;   // row of pair q: row0 + 16 q
@@ -369,7 +406,7 @@ __global__ void __launch_bounds__(BS_THREADS, 1) bcr_solve_kernel(const __grid_c
             };
             if (type == BS_BWD0) {
                 // level 0, backward: v = r_j - C (x_{j-1} + x_{j+1}); its maximum is bounded by the parts'
-                const int bl = task[3], sa = __ldg(a.shift + bs_matrix(a, task[2], tl.sys));
+                const int bl = task[3], sa = entry.sa[0];
                 const bool two = bl + 1 < a.nx;
                 const size_t lo = (size_t)bl * a.nz;
                 auto fetch3 = [&](int c) {
@@ -426,7 +463,11 @@ __global__ void __launch_bounds__(BS_THREADS, 1) bcr_solve_kernel(const __grid_c
             const float2 *fv = r0p;
             auto fetch_next = [&]() {
                 if (fu < nterms) {
-                    if (fc == 0) fv = (bs_kind(task[2 + 2 * fu]) >= BS_P ? x0p : r0p) + (size_t)task[3 + 2 * fu] * a.nz;
+                    if (fc == 0) {
+                        const int code = fu == 0 ? task[2] : (fu == 1 ? task[4] : task[6]);
+                        const int line = fu == 0 ? task[3] : (fu == 1 ? task[5] : task[7]);
+                        fv = (bs_kind(code) >= BS_P ? x0p : r0p) + (size_t)line * a.nz;
+                    }
                     fetch(fe, fv, fc, true);
                     if (++fc == a.n_chunk) { fc = 0; ++fu; }
                     if (++fe == BS_AHEAD + 1) fe = 0;
@@ -435,11 +476,10 @@ __global__ void __launch_bounds__(BS_THREADS, 1) bcr_solve_kernel(const __grid_c
             };
             for (int d = 0; d < BS_AHEAD; ++d) fetch_next();
             uint32_t mx[3][PR];
-            int sa[3];
+            const int *sa = entry.sa;
 #pragma unroll
             for (int u = 0; u < 3; ++u) {
                 const bool in = u < nterms;
-                sa[u] = in ? __ldg(a.shift + bs_matrix(a, task[2 + 2 * u], tl.sys)) : 0;
 #pragma unroll
                 for (int q = 0; q < PR; ++q)
                     mx[u][q] = in && q < np
@@ -489,10 +529,11 @@ __global__ void __launch_bounds__(BS_THREADS, 1) bcr_solve_kernel(const __grid_c
         int tt = 0, seen = -1;
         bool go = true;
         for (int i = 0; go; ++i) {
-            const int t = next_tile(i);
+            BsQ entry;
+            const int t = next_tile(i, entry);
             if (t < 0) break;
             const Tile tl = decode(a, t);
-            const int *task = a.tasks + 8 * tl.task;
+            const int *task = entry.task;
             const int line = task[0], type = task[1] & 15, nt = tl.nt;
             const int row = 32 * q + lane, m = tl.r0 + row;
             const bool on = row < tl.rows && m < a.nz, warp_on = 32 * q < tl.rows;
