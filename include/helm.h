@@ -135,12 +135,13 @@ void helm_op_destroy(helm_op_t *op);
  * level by level (log2(nx) levels), so that each level is a batch of independent dense block
  * inversions and block products over all lines and frequencies, run on the tensor cores
  * (operands as the sum of two FP16 numbers with a common scale, or with the 3xTF32 split; FP32
- * accumulation).  Its storage is about 3.5 nx nz^2 complex FP32 entries per frequency (6 while it
+ * accumulation).  Its storage is about 3 nx nz^2 entries of 8 bytes per frequency (5.3 while it
  * factors).  HELM_FACTOR_AUTO (unless the environment sets HELM_FACTOR=line or =bcr): BCR for
- * HELM_MIXED on lines of nz >= 192 nodes (where the line recurrence's chain of nx dependent line
- * inversions dominates), and from nz = 96 on where there are at least 96 lines and its blocks stay
- * within 16 GB, unless one of them comes out nearly singular (a resonance of a strip of the
- * medium) or the memory is not there; else the line recurrence. */
+ * HELM_MIXED on lines of an even nz >= 192 nodes (where the line recurrence's chain of nx dependent
+ * line inversions dominates), and from nz = 96 on, odd nz included (laid out with one decoupled node
+ * more), where there are at least 96 lines and its blocks stay within 16 GB, unless one of them comes
+ * out nearly singular (a resonance of a strip of the medium) or the memory is not there; else the
+ * line recurrence. */
 typedef enum { HELM_FACTOR_AUTO = 0, HELM_FACTOR_LINE = 1, HELM_FACTOR_BCR = 2 } helm_factor_method;
 typedef struct {
     int32_t method;       /* helm_factor_method */

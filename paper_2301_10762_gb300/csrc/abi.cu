@@ -196,7 +196,7 @@ static constexpr int kBcrLine = 192;
 // 128 x 128 4500 / 1500.  Few lines favour the recurrence, whose chain is their number (48 x 96: solves
 // 280 / 320 and 370 / 510).
 static constexpr int kBcrShortLine = 96;
-// BCR holds about 3.5 (and 6 while it factors) times the line factor's bytes: a set of frequencies
+// BCR holds about 3 (and 5.3 while it factors; 6 counted) times the line factor's bytes: a set of frequencies
 // whose blocks no longer are a small part of the device's memory stays with the smaller factor
 static constexpr size_t kBcrShortBytes = (size_t)16 << 30;
 // BCR eliminates lines with Dirichlet neighbours, so a frequency near a resonance of a strip of the

@@ -12,8 +12,8 @@
 //         L_k <- -L_k Dinv_a L_a      (coupling to k - 2s)
 //         U_k <- -U_k Dinv_c U_c      (coupling to k + 2s)
 // until one line is left (line 0, whose inverse ends the factor).  Every level is a batch of
-// independent dense block products and inversions over all lines and frequencies, which the
-// tensor-core GEMM (zgemm_tc.cu) and the batched block inversion below run; the depth of the
+// independent dense block products and inversions over all lines and frequencies, which
+// bcr_gemm.cu and the batched block inversion below run; the depth of the
 // dependent chain is log2(n_x) levels instead of n_x lines.  By symmetry L_k = U_a^T and
 // U_k = L_c^T, so every product is a GEMM of row-major operands:
 //     W_a = L_k Dinv_a (= (Dinv_a U_a)^T),   V_c = U_k Dinv_c (= (Dinv_c L_c)^T),
@@ -28,15 +28,21 @@
 //     last line:         x_0 = Dinv_0 b_0
 //     backward, level l: x_j = Dinv_j b_j - P_j x_{j-s} - Q_j x_{j+s}
 //     backward, level 0: x_j = Dinv_j (b_j - C (x_{j-1} + x_{j+1})).
-// Everything is complex FP32 (3xTF32 tensor products): the factor is the preconditioner of
-// the FP64-residual refinement of the mixed path, exactly as the line factor is.
+// The factor is the preconditioner of the FP64-residual refinement of the mixed path, exactly as the
+// line factor is.  Blocks that are factored further (D) are complex FP32; couplings, their products
+// and the inverses exist only as images (bcr_solve.h: every real entry the sum of two FP16 numbers,
+// 22 bits), which the products (bcr_gemm.cu) read and write.  Residuals after 1, 2, 3 sweeps at 128^2:
+// 1.5e-5, 6.4e-10, 1.5e-13 (with FP32 blocks, 3xTF32 products and truncating sums throughout: 5.7e-9
+// after 2 and 1.4e-12 after 3; the line factor 6e-11 and 1.4e-13).  What decides it is the sums: the
+// tensor core truncates, so long ones go through registers (bcr_gemm.cu, zinv_kernel).
 //
-// Dense inversion of a batch of n x n blocks: n <= 128 in shared memory, one CTA per block
-// (block Gauss-Jordan over 16-column blocks, partial pivoting inside each pivot block, as in
-// the line factor); larger n by the 2 x 2 block inverse of a symmetric matrix
+// Level 0 inverts no block (TriGen below).  Above it, a batch of dense inversions: n <= 128 one CTA per
+// block (zinv_kernel); larger n by the 2 x 2 block inverse of a symmetric matrix
 //     [[D11, D21^T], [D21, D22]]^{-1}:  X11 = D11^{-1}, T = X11 D21^T, S = D22 - D21 T,
 //     X22 = S^{-1}, X12 = -T X22, X21 = X12^T, X11 <- X11 - T X21,
-// with the products on the tensor cores and the two half-size inverses recursive.
+// with the products on the tensor cores and the two half-size inverses recursive (invert_images).
+// Time at 256^2 with 8 frequencies, of a 6.9 ms factor: level 0 0.9 ms, inversions 1.8, their parts'
+// products and images 1.4, the levels' products 2.3, images of the inverses 0.4.
 #include <math.h>
 #include <stdlib.h>
 
@@ -83,7 +89,7 @@ Coup coup_of(const GridGeom &g) {
 // exponent (R spans hundreds of orders of magnitude), correct to FP32 rounding.  Cyclic reduction
 // amplifies level 0's errors most (the Schur complements of the smooth modes lose four in size
 // per level): a block Gauss-Jordan inverse carries 1.2e-7 of its norm.
-// 256^2 with 8 frequencies: level 0 with its images 0.9 ms (dense inversions by two 128-column
+// 256^2 with 8 frequencies: level 0 with its images 0.9 ms, a quarter of it the recurrences (dense inversions by two 128-column
 // halves 1.0 ms, images and update 0.6); 512^2 with 4: 19 ms less.
 struct TriGen {          // generators of the odd lines' inverses: [line][nz]
     float4 *u, *v;       // hi.x, hi.y, lo.x, lo.y

@@ -7,14 +7,14 @@
 //     last line           x_0 = Dinv_0 r_0
 //     level l, backward   x_j = Dinv_j r_j - P_j x_{j-s} - Q_j x_{j+s}             j = s mod 2s
 //     level 0, backward   x_j = Dinv_j (r_j - C (x_{j-1} + x_{j+1}))               j odd
-// The blocks are read once per solve and nothing else comes close in bytes (3.5 n_x n_z^2 complex
-// entries per frequency: 3.8 GB at 256^2 with 8 frequencies, 0.56 ms at the measured copy rate),
-// so the kernel is laid out as a stream of the blocks through the tensor cores:
+// The blocks are read once per solve (the odd lines' inverses twice) and nothing else comes close in
+// bytes (3.5 n_x n_z^2 complex entries of 8 bytes per frequency: 3.8 GB at 256^2 with 8 frequencies,
+// 0.56 ms at the measured copy rate), so the kernel is laid out as a stream of the blocks through the tensor cores:
 //   * The blocks are stored as the tensor core reads them ("image"): every real entry as the sum
 //     of two FP16 numbers of its scaled value (a power of two per block; hi + lo carry 22 to 23
 //     bits for entries down to 2^-15 of the block's largest, as many as the 3xTF32 split keeps, and
-//     2^-39 of the largest below that; 8 bytes per complex entry as in FP32), real and imaginary parts apart, 32 columns of a row as one 128-byte swizzled row (32
-//     hi, then 32 lo).  A chunk of a tile is two contiguous runs of memory: a copy warp streams
+//     2^-39 of the largest below that; 8 bytes per complex entry as in FP32), real and imaginary
+//     parts apart, 32 columns of a row as one 128-byte swizzled row (32 hi, then 32 lo).  A chunk of a tile is two contiguous runs of memory: a copy warp streams
 //     them with bulk copies, and no thread touches them.
 //   * The vectors are split by operand warps as they come (a power-of-two scale per line slice
 //     from the maxima that the writers of the vectors leave), 16 KB against 32 KB of block data
@@ -27,10 +27,10 @@
 //     system); only the operand warps wait, so the block stream runs on across steps.  Every
 //     wait is for tiles that were taken earlier, so the kernel needs no co-resident grid, and
 //     every wait is bounded.
-// Measured per solve at 256^2, 8 frequencies (block stream 0.56 ms): 1 right-hand side 0.60 ms, 64
-// of them 1.02 ms; one GEMM launch per level (18 launches, 3xTF32, blocks split by operand warps)
-// took 1.9 and 2.4 ms.  With few systems the chain of 2 log2(n_x) + 1 steps is what is left, 6 to
-// 17 us a step: 0.14 ms at 128^2.
+// Measured per solve at 256^2, 8 frequencies (block stream 0.56 ms): 1 right-hand side 0.61 ms, 64
+// of them 1.12 ms (vectors and products restart at every tile); one GEMM launch per level (18
+// launches, 3xTF32, blocks split by operand warps) took 1.9 and 2.4 ms.  With few systems the chain
+// of 2 log2(n_x) + 1 steps is what is left, 6 to 17 us a step: 0.12 ms at 128^2.
 #include <algorithm>
 
 #include "abi_internal.h"

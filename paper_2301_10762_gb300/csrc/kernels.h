@@ -89,7 +89,8 @@ struct RefineStop {  // stopping rule of the pair phase, applied on the device
 // (zero on entry: refine_start and the stopping test leave it so).  With state, the last block to
 // finish applies the stopping test, and state->done makes later launches do
 // nothing.
-// gmax, ctl: as launch_refine_start, for the next solve.  solve_status: the op's status word,
+// ld: line stride of delta and r32 (n_z, or one more where odd lines have a decoupled node, which is
+// written as zero).  gmax, ctl: as launch_refine_start, for the next solve.  solve_status: the op's status word,
 // copied into the state by the last block.
 cudaError_t launch_refine_update(const GridGeom &g, int n_sys, int nrhs, const float4 *diag2, const float4 *bd,
                                  const float4 *x_in, const float2 *delta, float4 *x_out, float2 *r32, double *norms,

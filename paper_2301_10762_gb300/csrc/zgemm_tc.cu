@@ -2,9 +2,9 @@
 // tensor memory), with the 3xTF32 split that keeps the products near FP32 accuracy:
 //     C_t = C0_t + sum_u s_u A_{t,u} Bt_{t,u}^T      (t: task, u <= 3 terms, s_u = +-1)
 // A (M x K) and Bt (N x K) are row-major complex matrices (interleaved re, im); C and C0 are
-// row-major or column-major.  This is the dense contraction of the block-cyclic-reduction
-// factor and solve (block products of the line blocks; all right-hand sides of a system as
-// the N dimension of the solve's products).
+// row-major or column-major.  This is the library's product of FP32 blocks: helm_zgemm_batched,
+// and the products of helm_zinv_batched above n = 128 (the block-cyclic-reduction factor and solve
+// have theirs on FP16 pairs, bcr_gemm.cu and bcr_solve.cu).
 //
 // Complex products as real ones: with A taken as the real M x 2K matrix of its interleaved
 // entries, and each complex row b of Bt expanded into the two real rows
