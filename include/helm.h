@@ -141,7 +141,8 @@ void helm_op_destroy(helm_op_t *op);
  * line inversions dominates), and from nz = 96 on, odd nz included (laid out with one decoupled node
  * more), where there are at least 96 lines and its blocks stay within 16 GB, unless one of them comes
  * out nearly singular (a resonance of a strip of the medium) or the memory is not there; else the
- * line recurrence. */
+ * line recurrence.  A factor chosen on that second count becomes the line factor where a solve does
+ * not converge with it, and the solve is repeated (helm_solve_noalloc allocates nothing and does not). */
 typedef enum { HELM_FACTOR_AUTO = 0, HELM_FACTOR_LINE = 1, HELM_FACTOR_BCR = 2 } helm_factor_method;
 typedef struct {
     int32_t method;       /* helm_factor_method */

@@ -48,6 +48,7 @@ constexpr size_t kSmallMaxima = (size_t)1 << 16;
 struct helm_factor {
     helm_op *op = nullptr;
     bool use_bcr = false;  // mixed: block-cyclic-reduction factor on the tensor cores
+    bool auto_bcr = false; // ... chosen where the line factor would do (taken back if a refinement fails)
     BcrData bcr;
     helm_prec prec = HELM_FP64;
     int cs = 1;
@@ -110,6 +111,7 @@ helm_status acq_upload(const helm_op *op, const helm_acq *acq, DevAcq *d);
 namespace helm {
 bool bcr_supported(const GridGeom &g);
 int bcr_line(const GridGeom &g);               // nodes of a line as BCR lays it out: an odd line has one more
+bool factor_retry_line(helm_factor_t *f);
 int solve_line(const helm_factor_t *f);        // line stride of the mixed solve's r32 and y
 // whether helm_factor builds a block-cyclic-reduction factor for this grid and precision
 // (method: a helm_factor_method; HELM_FACTOR_AUTO follows HELM_FACTOR and the line length)

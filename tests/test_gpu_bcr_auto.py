@@ -1,7 +1,7 @@
 """The automatic choice of block cyclic reduction on lines of 96 to 191 nodes and on odd lines (which
 get a decoupled node): taken on sizes (at least 96 lines, blocks within 16 GB), and taken back where an eliminated block is nearly
 singular: a slow disc of m = 36 in m = 1 on 96 x 96 has a mode trapped between the lines 32 and 64 at w
-= 5.548174513413695, and the inverse of the block of line 48 an entry of 5e3 (the limit is 2^10 / 4).
+= 5.548174513413695, and the inverse of the block of line 48 an entry of 5e3 (the limit is 2^9 / 4).
 |A^{-1}| |b| / |x| of the medium itself is below 1e2 for random b there and at w = 5, so a residual of
 1e-12 leaves an error below 1e-10; 1e-8 is the mixed path's bar."""
 import numpy as np
@@ -68,3 +68,29 @@ def test_odd_lines_match_oracle(nx, nz, n_omega, nrhs):
         for q in range(n_omega):
             ref = getattr(fo[q], how)(B[q, :n])
             assert np.max(np.linalg.norm(X[q] - ref, axis=1) / np.linalg.norm(ref, axis=1)) <= 1e-8
+
+
+def test_a_solve_that_does_not_converge_is_repeated_with_the_line_factor():
+    """One sweep leaves 1e-5 with either factor: HELM_ENOCONV as ever, but an automatic factor has become
+    the line factor by then, and the next call uses it; an explicit one stays."""
+    nx, nz = 97, 99
+    rng = np.random.default_rng(7)
+    m = (1.0 / (1.0 + 0.5 * rng.uniform(0, 1, (nx, nz))) ** 2).reshape(-1)
+    op = hm.helm_assemble(nx, nz, 1.0, 1.0, torch.tensor(m, device="cuda"), [6.0])
+    B = rng.standard_normal((1, 4, nx * nz)) + 1j * rng.standard_normal((1, 4, nx * nz))
+    Bd = torch.tensor(B, device="cuda")
+    f = hm.helm_factor(op, hm.HELM_MIXED)
+    assert f.method == hm.HELM_FACTOR_BCR
+    with pytest.raises(hm.HelmError):
+        hm.helm_solve(f, Bd, rtol=1e-12, max_iter=1)
+    assert f.method == hm.HELM_FACTOR_LINE
+    Y = hm.helm_solve(f, Bd, rtol=1e-12, max_iter=20)[0].cpu().numpy()
+    ref = H.Factor(H.helmholtz_matrix(H.Grid(nx, nz, 1.0, 1.0), m, 6.0)).solve(B[0])
+    assert np.max(np.linalg.norm(Y[0] - ref, axis=1) / np.linalg.norm(ref, axis=1)) <= 1e-8
+    m2 = np.full(24 * 32, 0.5)
+    op2 = hm.helm_assemble(24, 32, 1.0, 1.0, torch.tensor(m2, device="cuda"), [6.0])
+    f2 = hm.helm_factor(op2, hm.HELM_MIXED, method=hm.HELM_FACTOR_BCR)
+    B2 = torch.tensor(rng.standard_normal((1, 2, 24 * 32)) + 0j, device="cuda")
+    with pytest.raises(hm.HelmError):
+        hm.helm_solve(f2, B2, rtol=1e-12, max_iter=1)
+    assert f2.method == hm.HELM_FACTOR_BCR
