@@ -818,29 +818,49 @@ int pick_cluster_size(int nz) {
     return p >= 8 ? 8 : (p >= 4 ? 4 : (p >= 2 ? 2 : 1));
 }
 
+// dynamic shared memory that the slab-resident kernel can take: what a block may opt in to less the
+// kernel's static arrays (sm_103a: 227 KB less 9 KB in FP64, and less 23 KB in complex FP32, whose
+// Newton-Schulz blocks and seeds are static); 0 where the device does not say
+template <typename T> static size_t factor_resident_max() {
+    int dev = 0, optin = 0;
+    cudaFuncAttributes fa;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess ||
+        cudaFuncGetAttributes(&fa, (const void *)line_factor_smem_kernel<T>) != cudaSuccess) {
+        cudaGetLastError();
+        return 0;
+    }
+    return (size_t)optin > fa.sharedSizeBytes ? (size_t)optin - fa.sharedSizeBytes : 0;
+}
+
 template <typename T>
 cudaError_t launch_line_factor(const GridGeom &g, int n_sys, const double2 *diag, cx_t<T> *G, cx_t<T> *xch,
                                int *status, int cs, cudaStream_t st, int *mid_out) {
-    constexpr size_t kResidentMax = 216 * 1024;   // + up to 9 KB of static shared memory
     int teams = 1;
     cudaError_t e;
-    // a slab of eight CTAs that does not fit (FP64 from n_z = 200): one team of sixteen, one-sided,
-    // instead of the kernel with its panels in global memory (256^2, FP64: 990 ms)
-    if (cs == 8 && factor_smem_resident_bytes<T>(g.nz, cs) > kResidentMax &&
-        factor_smem_resident_bytes<T>(g.nz, 16) <= kResidentMax) {
-        const size_t s16 = factor_smem_resident_bytes<T>(g.nz, 16);
-        if ((e = ensure_dyn_smem((const void *)line_factor_smem_kernel<T>, s16)) != cudaSuccess) return e;
-        if (max_active_clusters((const void *)line_factor_smem_kernel<T>, 16, FAC_THREADS, s16) > 0) cs = 16;
+    const size_t resident_max = factor_resident_max<T>();
+    // a slab that fits and that the device takes
+    auto fits = [&](int c) {
+        const size_t b = factor_smem_resident_bytes<T>(g.nz, c);
+        if (b > resident_max) return false;
+        if (ensure_dyn_smem((const void *)line_factor_smem_kernel<T>, b) == cudaSuccess) return true;
+        cudaGetLastError();
+        return false;
+    };
+    bool resident = fits(cs);
+    // a slab of eight CTAs that does not fit (FP64 from n_z = 200, complex FP32 from 308): one team of
+    // sixteen, one-sided, instead of the kernel with its panels in global memory (64 lines, two
+    // frequencies: FP64 n_z = 240 215 -> 94 ms, FP32 n_z = 320 81 -> 32, n_z = 384 113 -> 46)
+    if (!resident && cs == 8 && fits(16) &&
+        max_active_clusters((const void *)line_factor_smem_kernel<T>, 16, FAC_THREADS,
+                            factor_smem_resident_bytes<T>(g.nz, 16)) > 0) {
+        cs = 16;
+        resident = true;
     }
     const size_t smem_res = factor_smem_resident_bytes<T>(g.nz, cs);
-    const bool resident = smem_res <= kResidentMax;
     // HELM_FACTOR_TEAMS=1 forces the one-sided factorisation (for comparisons)
     const char *force = getenv("HELM_FACTOR_TEAMS");
     const bool allow_twisted = !(force && force[0] == '1');
-    if (resident) {
-        e = ensure_dyn_smem((const void *)line_factor_smem_kernel<T>, smem_res);
-        if (e != cudaSuccess) return e;
-    }
     if (resident && allow_twisted) {
         // two teams (twisted) when a cluster of 2 cs CTAs can be scheduled
         if (2 * cs <= 16) {
