@@ -21,6 +21,7 @@
 #include <stdlib.h>
 #include "kernels.h"
 #include "mma_tf32.cuh"
+#include "sweep_shape.h"
 #include "trace.h"
 
 namespace helm {
@@ -854,29 +855,18 @@ cudaError_t launch_line_sweep(const GridGeom &g, int n_sys, int nrhs, const cx_t
     const int teams = (mid < g.nx - 1) ? 2 : 1;
     int cs = nz / 16;
     cs = cs < 1 ? 1 : (cs > 16 / teams ? 16 / teams : cs);
-    // FP64: the products, not the exchange, are the length of a step (2 lanes a cycle per SM: 8 us of
-    // a 10 us step at 64 rows x 8 right-hand sides on 4 CTAs).  CTAs per team and right-hand sides
-    // per cluster are taken for the least time of (waves of clusters) x (products of a step + about
-    // 3500 cycles of exchange), the line product's 2 multiply-adds of 2 lanes per entry.  64^2 with 8
-    // right-hand sides: 649 -> 278 us.
     const bool fp64 = sizeof(TG) == 8;
     int fp64_R = 0;
-    if (fp64 && nz >= 48) {   // (shorter lines are bound by the exchange: 40 x 37 ran 210 us as it was, 249 spread out)
-        double best = 0.0;
-        const int cs0 = cs;
-        for (int c = cs0; c <= 16 / teams; c = c < 8 && 2 * c > 8 ? 8 : 2 * c) {
-            const int csz = teams * c, rp = (nz + c - 1) / c;
-            for (int r = 1; r <= std::min(16, nrhs); ++r) {
-                if (rp * r > 128) break;   // (128 outputs per CTA measured best)
-                // (shared memory at the widest padding, in steps of 32 KB: few distinct queries)
-                const size_t need = 32 + vsz * (size_t)(nz + 8) * (5 * r + 2 * rp) + vsz * 2 * (size_t)r * rp;
-                const int act = std::max(1, max_active_clusters((const void *)line_sweep_kernel<TG, 0, 0, false>, csz, SW_THREADS,
-                                                                std::min(SW_SMEM_MAX, (need + 32767) / 32768 * 32768)));
-                const long waves = ((long)n_sys * ((nrhs + r - 1) / r) + act - 1) / act;
-                const double t = (double)waves * (2.0 * rp * r * nz + 3500.0);
-                if (fp64_R == 0 || t < best) { best = t; cs = c; fp64_R = r; }
-            }
-        }
+    if (fp64) {
+        const SweepShape sh = sweep_shape_fp64(nz, teams, n_sys, nrhs, cs, [&](int c, int r) {
+            // (shared memory at the widest padding, in steps of 32 KB: few distinct queries)
+            const int rp = (nz + c - 1) / c;
+            const size_t need = 32 + vsz * (size_t)(nz + 8) * (5 * r + 2 * rp) + vsz * 2 * (size_t)r * rp;
+            return max_active_clusters((const void *)line_sweep_kernel<TG, 0, 0, false>, teams * c, SW_THREADS,
+                                       std::min(SW_SMEM_MAX, (need + 32767) / 32768 * 32768));
+        });
+        cs = sh.cs;
+        fp64_R = sh.R;
     }
     // tuning overrides: CTAs per team and right-hand sides per cluster
     const char *env_cs = getenv("HELM_SWEEP_CS"), *env_r = getenv("HELM_SWEEP_R");
@@ -889,6 +879,7 @@ cudaError_t launch_line_sweep(const GridGeom &g, int n_sys, int nrhs, const cx_t
     const int force_mma = (env_mma && *env_mma) ? (atoi(env_mma) > 0 ? 1 : 0) : -1;
     cudaError_t e;
     for (;;) {
+        cs = sweep_filled_ctas(nz, cs);
         const int rpc = (nz + cs - 1) / cs;
         // threads per output (K split): as many as fit the CTA's 256 threads twice over
         auto tpo_of = [&](int R) {

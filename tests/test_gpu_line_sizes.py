@@ -36,3 +36,15 @@ def test_mixed_line_factor_around_the_slabs_shared_memory(nx, nz, method):
     assert f.method == hm.HELM_FACTOR_LINE
     X = hm.helm_solve(f, torch.tensor(B, device="cuda"), rtol=1e-12, max_iter=20)[0]
     assert _error(X, ref) <= 1e-8
+
+
+@pytest.mark.parametrize("nx,nz,nrhs,teams", [(8, 48, 5, 2), (8, 49, 5, 2), (7, 50, 1, 2), (9, 57, 3, 2), (6, 99, 2, 2), (5, 49, 3, 1),
+                                              (6, 100, 3, 1), (5, 113, 1, 1)])
+def test_fp64_sweep_teams_without_idle_ctas(nx, nz, nrhs, teams, monkeypatch):
+    """Line lengths that a doubled number of CTAs does not divide into filled ones (49 on 8 CTAs: seven
+    rows each, the eighth none; 100 on 16: the last without rows).  FP64 bar 1e-9."""
+    if teams == 1:
+        monkeypatch.setenv("HELM_FACTOR_TEAMS", "1")
+    op, B, ref = _case(nx, nz, 1, nrhs)
+    f = hm.helm_factor(op, hm.HELM_FP64)
+    assert _error(hm.helm_solve(f, torch.tensor(B, device="cuda"))[0], ref) <= 1e-9
