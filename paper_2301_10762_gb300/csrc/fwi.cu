@@ -343,29 +343,31 @@ __global__ void regR_kernel(GridGeom g, const double *v, double *out) {
 // diagonalises: L_n = C_n^T diag(2 - 2 cos(pi a / n)) C_n.  Hence
 //   P2^{-1} r = (C_x (x) C_z)^T diag(1 / (alpha0 lam_ab + mu)) (C_x (x) C_z) r
 // in three passes: every line's transform along z; every column's transform along x, the division
-// (with all s_a^2) and the transform back; every line's transform back along z.  The products are
-// bound by the FP64 pipe (2 lanes a cycle per SM), so
-//   - C is not formed: its entries are n + 1 cosines cos(pi k / (2n)) up to sign, one table per
-//     direction, indexed by a (2j + 1) mod 4n (integer work, free beside FP64);
+// (with all s_a^2) and the transform back; every line's transform back along z.  From about 200 nodes a
+// line on the passes are bound by the multiply-adds in the FP64 pipe (2 lanes a cycle per SM; 2 n^3 of them on
+// an n x n grid, 0.46 of the 0.54 ms of kernels at 512^2), below by launches and latency, so
+//   - C is not formed: its entries are 2n + 1 cosines cos(pi k / (2n)), one table per direction,
+//     indexed by a (2j + 1) mod 4n (integer work beside FP64).  The sign is in the table: selected on
+//     the operand instead, it doubled the time of every sum (512^2: 1272 us a call against 589);
 //   - the symmetry C[a][n-1-j] = (-1)^a C[a][j] halves the multiply-adds: a line is folded into its
 //     even and odd parts first, or the even and odd sums are unfolded after;
 //   - a CTA per line (column) puts 128 of them on a 128^2 problem.
-// 128^2, one vector: 102 us a call with the matrices formed (2 launches) and four tiled products and
-// a scaling (5 launches), 2 n^3 multiply-adds each; three passes and the table now.
+// One vector, us a call: with the matrices formed (2 launches), four tiled products and a scaling (5
+// launches) 84 at 64^2, 101 at 128^2, 113 at 160^2, 196 at 256^2, 1072 at 512^2; three passes and
+// the table 57, 64, 83, 123, 589 (64 to 512, square and not, odd and even: the least gain is 1.36, just
+// above a line per SM).
+__device__ __forceinline__ double dct_entry(int n, int k) {
+    return k <= n ? cospi((double)k / (2.0 * n)) : -cospi((double)(2 * n - k) / (2.0 * n));
+}
 __global__ void dct_table_kernel(int nx, int nz, double *tx, double *tz) {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k <= nx) tx[k] = cospi((double)k / (2.0 * nx));
-    else if (k - nx - 1 <= nz) tz[k - nx - 1] = cospi((double)(k - nx - 1) / (2.0 * nz));
+    const int k = blockIdx.x * blockDim.x + threadIdx.x, kz = k - 2 * nx - 1;
+    if (kz < 0) tx[k] = dct_entry(nx, k);
+    else if (kz <= 2 * nz) tz[kz] = dct_entry(nz, kz);
 }
 
 constexpr int DCT_THREADS = 256;
-// +-T[.] = cos(pi idx / (2n)), 0 <= idx < 4n, times v
-__device__ __forceinline__ double cos_fma(const double *T, int n, int idx, double v, double acc) {
-    int k = idx > 2 * n ? 4 * n - idx : idx;
-    const bool neg = k > n;
-    k = neg ? 2 * n - k : k;
-    return fma(neg ? -v : v, T[k], acc);
-}
+// cos(pi idx / (2n)), 0 <= idx < 4n
+__device__ __forceinline__ double dct_cos(const double *T, int n, int idx) { return T[min(idx, 4 * n - idx)]; }
 // threads that share an output (adjacent lanes, a power of two)
 __device__ __forceinline__ int dct_parts(int outputs) {
     int s = 1;
@@ -386,14 +388,14 @@ template <typename Out> __device__ void dct_forward(const double *T, int n, cons
             int idx = (int)(((long long)a * (2 * part + 1)) % (4 * n));
             int j = part;
             for (; j + S < h; j += 2 * S) {
-                acc = cos_fma(T, n, idx, v[j], acc);
+                acc = fma(dct_cos(T, n, idx), v[j], acc);
                 idx += step;
                 if (idx >= 4 * n) idx -= 4 * n;
-                acc1 = cos_fma(T, n, idx, v[j + S], acc1);
+                acc1 = fma(dct_cos(T, n, idx), v[j + S], acc1);
                 idx += step;
                 if (idx >= 4 * n) idx -= 4 * n;
             }
-            if (j < h) acc = cos_fma(T, n, idx, v[j], acc);
+            if (j < h) acc = fma(dct_cos(T, n, idx), v[j], acc);
             acc += acc1;
         }
         for (int o = 1; o < S; o *= 2) acc += __shfl_xor_sync(0xffffffffu, acc, o);
@@ -411,10 +413,10 @@ template <typename Out> __device__ void dct_backward(const double *T, int n, con
             const int w = 2 * j + 1, step2 = (int)((2ll * w * S) % (4 * n));
             int ie = (int)((2ll * part * w) % (4 * n)), io = (int)(((2ll * part + 1) * w) % (4 * n));
             for (int a = 2 * part; a < n; a += 2 * S) {
-                ev = cos_fma(T, n, ie, t[a], ev);
+                ev = fma(dct_cos(T, n, ie), t[a], ev);
                 ie += step2;
                 if (ie >= 4 * n) ie -= 4 * n;
-                if (a + 1 < n) od = cos_fma(T, n, io, t[a + 1], od);
+                if (a + 1 < n) od = fma(dct_cos(T, n, io), t[a + 1], od);
                 io += step2;
                 if (io >= 4 * n) io -= 4 * n;
             }
@@ -440,21 +442,20 @@ __device__ __forceinline__ void dct_fold(int n, const double *in, size_t stride,
         F[h + j] = mid ? 0.0 : u - v;
     }
 }
-// Scratch of a CTA: the table (n + 1) and two vectors of n + 1, in shared memory, or (big: lines of
-// more than DCT_SMEM_N nodes) the vectors in global memory at big + 2 (n + 1) * CTA and the table
+// Scratch of a CTA: the table (2n + 1) and `vectors` vectors of n + 1, in shared memory, or (big: lines
+// of more than DCT_SMEM_N nodes) the vectors in global memory at big + vectors (n + 1) * CTA and the table
 // where it is
 constexpr int DCT_SMEM_N = 6000;
+constexpr int DCT_LINE_VECS = 1, DCT_COL_VECS = 2;
+__host__ __device__ inline size_t dct_vec_elems(int n, int vectors) { return (size_t)vectors * (n + 1); }
 struct DctBuf {
     const double *T;
-    double *u, *v;
+    double *u;
 };
-__device__ __forceinline__ DctBuf dct_buf(int n, const double *table, double *big, double *smem) {
-    if (big) {
-        double *p = big + 2 * (size_t)(n + 1) * (blockIdx.x + (size_t)gridDim.x * blockIdx.y);
-        return DctBuf{table, p, p + n + 1};
-    }
-    for (int k = threadIdx.x; k <= n; k += DCT_THREADS) smem[k] = table[k];
-    return DctBuf{smem, smem + n + 1, smem + 2 * (n + 1)};
+__device__ __forceinline__ DctBuf dct_buf(int n, int vectors, const double *table, double *big, double *smem) {
+    if (big) return DctBuf{table, big + dct_vec_elems(n, vectors) * (blockIdx.x + (size_t)gridDim.x * blockIdx.y)};
+    for (int k = threadIdx.x; k <= 2 * n; k += DCT_THREADS) smem[k] = table[k];
+    return DctBuf{smem, smem + 2 * n + 1};
 }
 
 // z transforms of the lines (blockIdx.x) of the vectors (blockIdx.y): out = in C_z^T without s_b, or
@@ -463,7 +464,7 @@ __global__ void __launch_bounds__(DCT_THREADS) dct_lines_kernel(int nx, int nz, 
                                                                 double *out, double *big) {
     extern __shared__ double dct_smem[];
     const size_t off = ((size_t)blockIdx.y * nx + blockIdx.x) * nz;
-    const DctBuf b = dct_buf(nz, tz, big, dct_smem);
+    const DctBuf b = dct_buf(nz, DCT_LINE_VECS, tz, big, dct_smem);
     double *o = out + off;
     if (back) {
         for (int k = threadIdx.x; k < nz; k += DCT_THREADS) b.u[k] = in[off + k];
@@ -481,19 +482,23 @@ __global__ void __launch_bounds__(DCT_THREADS) dct_columns_kernel(int nx, int nz
                                                                   double alpha0, double mu, double *T1, double *big) {
     extern __shared__ double dct_smem[];
     double *col = T1 + (size_t)blockIdx.y * nx * nz + blockIdx.x;
-    const DctBuf b = dct_buf(nx, tx, big, dct_smem);
+    const DctBuf b = dct_buf(nx, DCT_COL_VECS, tx, big, dct_smem);
+    double *t = b.u + nx + 1;
     dct_fold(nx, col, nz, b.u);
     __syncthreads();
+    dct_forward(b.T, nx, b.u, [&](int a, double x) { t[a] = x; });
+    __syncthreads();
+    // (once per output with all threads: in dct_forward's lanes it cost the FP64 pipe as much as the sums)
     const int e = blockIdx.x;
     const double sx = (double)(nx - 1) * (nx - 1), sz = (double)(nz - 1) * (nz - 1);
-    const double lz = sz * (2.0 - 2.0 * cos_fma(tz, nz, 2 * e, 1.0, 0.0));
+    const double lz = sz * (2.0 - 2.0 * dct_cos(tz, nz, 2 * e));
     const double s2 = (e == 0 ? 1.0 : 2.0) / nz;
-    dct_forward(b.T, nx, b.u, [&](int a, double x) {
-        const double lx = sx * (2.0 - 2.0 * cos_fma(b.T, nx, 2 * a, 1.0, 0.0));
-        b.v[a] = x * (s2 * (a == 0 ? 1.0 : 2.0)) / (nx * (alpha0 * (lx + lz) + mu));
-    });
+    for (int a = threadIdx.x; a < nx; a += DCT_THREADS) {
+        const double lx = sx * (2.0 - 2.0 * dct_cos(b.T, nx, 2 * a));
+        t[a] = t[a] * (s2 * (a == 0 ? 1.0 : 2.0)) / (nx * (alpha0 * (lx + lz) + mu));
+    }
     __syncthreads();
-    dct_backward(b.T, nx, b.v, [&](int j, double x) { col[(size_t)j * nz] = x; });
+    dct_backward(b.T, nx, t, [&](int j, double x) { col[(size_t)j * nz] = x; });
 }
 
 }  // namespace helm
@@ -600,27 +605,35 @@ struct P2Solver {
         mu = m0;
         batch = n_batch;
         helm_status s = HELM_OK;
-        tx = ws.get<double>((size_t)nx + nz + 2, &s);
+        tx = ws.get<double>(2 * ((size_t)nx + nz) + 2, &s);
         T1 = ws.get<double>((size_t)nx * nz * batch, &s);
-        if (nz > DCT_SMEM_N) big_z = ws.get<double>(2 * ((size_t)nz + 1) * nx * batch, &s);
-        if (nx > DCT_SMEM_N) big_x = ws.get<double>(2 * ((size_t)nx + 1) * nz * batch, &s);
+        if (nz > DCT_SMEM_N) big_z = ws.get<double>(dct_vec_elems(nz, DCT_LINE_VECS) * nx * batch, &s);
+        if (nx > DCT_SMEM_N) big_x = ws.get<double>(dct_vec_elems(nx, DCT_COL_VECS) * nz * batch, &s);
         if (s != HELM_OK) return s;
-        tz = tx + nx + 1;
-        if (smem(nz) > 48 * 1024) HK(ensure_dyn_smem((const void *)dct_lines_kernel, smem(nz)));
-        if (smem(nx) > 48 * 1024) HK(ensure_dyn_smem((const void *)dct_columns_kernel, smem(nx)));
-        HELM_TRACED(K_DCTMAT, st, (dct_table_kernel<<<nblk((size_t)nx + nz + 2, 32), 32, 0, st>>>(nx, nz, tx, tz)));
+        tz = tx + 2 * nx + 1;
+        if (smem(nz, DCT_LINE_VECS) > 48 * 1024) HK(ensure_dyn_smem((const void *)dct_lines_kernel, smem(nz, DCT_LINE_VECS)));
+        if (smem(nx, DCT_COL_VECS) > 48 * 1024) HK(ensure_dyn_smem((const void *)dct_columns_kernel, smem(nx, DCT_COL_VECS)));
+        HELM_TRACED(K_DCTMAT, st, (dct_table_kernel<<<nblk(2 * ((size_t)nx + nz) + 2, 32), 32, 0, st>>>(nx, nz, tx, tz)));
         HL();
         return HELM_OK;
     }
-    static size_t smem(int n) { return n > DCT_SMEM_N ? 0 : 3 * ((size_t)n + 1) * sizeof(double); }
+    static size_t smem(int n, int vectors) {
+        return n > DCT_SMEM_N ? 0 : (2 * (size_t)n + 1 + dct_vec_elems(n, vectors)) * sizeof(double);
+    }
+    // vectors at a time: 16 while their scratch stays within 64 MB (one vector's is 1 to 4 N values)
+    static int max_batch(const GridGeom &g) {
+        const size_t v = sizeof(double) * ((size_t)g.nx * g.nz + (g.nz > DCT_SMEM_N ? dct_vec_elems(g.nz, DCT_LINE_VECS) * g.nx : 0) +
+                                           (g.nx > DCT_SMEM_N ? dct_vec_elems(g.nx, DCT_COL_VECS) * g.nz : 0));
+        return (int)std::max<size_t>(1, std::min<size_t>(16, ((size_t)64 << 20) / v));
+    }
     // out may be r
     helm_status apply(const double *r, double *out, cudaStream_t st, int count = 1) {
-        HELM_TRACED(K_DGEMM, st, (dct_lines_kernel<<<dim3(nx, count), DCT_THREADS, smem(nz), st>>>(nx, nz, tz, 0, r, T1, big_z)));
+        HELM_TRACED(K_DGEMM, st, (dct_lines_kernel<<<dim3(nx, count), DCT_THREADS, smem(nz, DCT_LINE_VECS), st>>>(nx, nz, tz, 0, r, T1, big_z)));
         HL();
-        HELM_TRACED(K_DGEMM, st, (dct_columns_kernel<<<dim3(nz, count), DCT_THREADS, smem(nx), st>>>(nx, nz, tx, tz, alpha0, mu,
+        HELM_TRACED(K_DGEMM, st, (dct_columns_kernel<<<dim3(nz, count), DCT_THREADS, smem(nx, DCT_COL_VECS), st>>>(nx, nz, tx, tz, alpha0, mu,
                                                                                                     T1, big_x)));
         HL();
-        HELM_TRACED(K_DGEMM, st, (dct_lines_kernel<<<dim3(nx, count), DCT_THREADS, smem(nz), st>>>(nx, nz, tz, 1, T1, out, big_z)));
+        HELM_TRACED(K_DGEMM, st, (dct_lines_kernel<<<dim3(nx, count), DCT_THREADS, smem(nz, DCT_LINE_VECS), st>>>(nx, nz, tz, 1, T1, out, big_z)));
         HL();
         return HELM_OK;
     }
@@ -765,7 +778,7 @@ extern "C" helm_status helm_gamma_solve(const helm_grid *grid, double alpha0, do
     {
         Ws ws(st);
         P2Solver p2;
-        const int batch = std::min<int32_t>(ncol, 16);
+        const int batch = std::min<int32_t>(ncol, P2Solver::max_batch(g));
         s = p2.init(ws, g, alpha0, mu, st, batch);
         for (int32_t c = 0; s == HELM_OK && c < ncol; c += batch)
             s = p2.apply(R_dev + c * N, Z_dev + c * N, st, std::min<int32_t>(batch, ncol - c));
