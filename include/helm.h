@@ -141,8 +141,10 @@ void helm_op_destroy(helm_op_t *op);
  * line inversions dominates), and from nz = 96 on, odd nz included (laid out with one decoupled node
  * more), where there are at least 96 lines and its blocks stay within 16 GB, unless one of them comes
  * out nearly singular (a resonance of a strip of the medium) or the memory is not there; else the
- * line recurrence.  A factor chosen on that second count becomes the line factor where a solve does
- * not converge with it, and the solve is repeated (helm_solve_noalloc allocates nothing and does not). */
+ * line recurrence.  The first solve that does not converge on a factor chosen on that second count is
+ * repeated on the line factor, unless rtol is below 1e-15 or B is not finite; if that converges the factor
+ * stays the line factor, else the next solve is on the BCR factor again and not repeated
+ * (helm_solve_noalloc allocates nothing and repeats nothing). */
 typedef enum { HELM_FACTOR_AUTO = 0, HELM_FACTOR_LINE = 1, HELM_FACTOR_BCR = 2 } helm_factor_method;
 typedef struct {
     int32_t method;       /* helm_factor_method */
@@ -193,7 +195,7 @@ void helm_set_wait_tries(int64_t tries);
 uint32_t helm_fault_mask(void);
 
 /* helm_factor_get_method -- the method a factor was built with (HELM_FACTOR_LINE or
- * HELM_FACTOR_BCR); -1 for NULL. */
+ * HELM_FACTOR_BCR), or, where a solve was repeated on the other one, that of the last solve; -1 for NULL. */
 int32_t helm_factor_get_method(const helm_factor_t *f);
 
 /* helm_factor_fp64_blocks -- HELM_MIXED: number of 16 x 16 pivot blocks of the factor that

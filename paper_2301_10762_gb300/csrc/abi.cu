@@ -206,6 +206,8 @@ static constexpr size_t kBcrShortBytes = (size_t)16 << 30;
 // 2600; the medians are 10 to 70.  From 2^9 a short or odd line takes the line recurrence.  A solve on
 // an automatic factor that does not converge all the same is repeated with the line factor.
 static constexpr float kBcrMaxGrowth = 512.f;
+// residuals in FP64 end at a few ulp of |A| |x| / |b| (1e-14 and more where |x| / |b| is some tens)
+static constexpr double kTightestRtol = 1e-15;
 bool helm::factor_picks_bcr(const GridGeom &g, helm_prec prec, int method) {
     if (prec != HELM_MIXED || !bcr_supported(g)) return false;
     int m = method;
@@ -253,8 +255,8 @@ static helm_status line_factor(helm_factor_t *f, cudaError_t &e) {
     return HELM_OK;
 }
 
-// An automatic BCR factor on which a refinement did not converge becomes the line factor (which the
-// automatic choice would else have been): false if that fails too.
+// The line factor (which the automatic choice would else have been) beside an automatic BCR factor on
+// which a refinement did not converge, and in its place; once per factor.  False if it cannot be had.
 bool helm::factor_retry_line(helm_factor_t *f) {
     helm_op *op = f->op;
     if (!f->auto_bcr) return false;
@@ -272,11 +274,21 @@ bool helm::factor_retry_line(helm_factor_t *f) {
         f->G = f->xch = nullptr;
         return false;
     }
-    bcr_free(f);
     f->use_bcr = false;
+    f->line_stand_in = true;
     f->fp64_blocks = st_host[1];
     f->last_iters.store(3, std::memory_order_relaxed);
     return true;
+}
+
+void helm::factor_back_to_bcr(helm_factor_t *f) {
+    if (!f->line_stand_in) return;
+    f->line_stand_in = false;
+    dev_free(f->G, f->op->st);
+    dev_free(f->xch, f->op->st);
+    f->G = f->xch = nullptr;
+    f->use_bcr = true;
+    f->fp64_blocks = 0;
 }
 
 extern "C" helm_status helm_factor(helm_op_t *op, helm_prec prec, const helm_factor_opts *opts, helm_factor_t **out) {
@@ -576,6 +588,16 @@ helm_status mixed_refine(const helm_factor_t *f, int nrhs, const double2 *B, dou
     return HELM_OK;
 }
 
+// whether every column of a mixed solve's right-hand sides has a finite norm (synchronises the op's stream)
+static helm_status finite_rhs(const helm_op *op, size_t cols, const double *norms_dev, double *norms_host, bool *out) {
+    cudaError_t e = cudaMemcpyAsync(norms_host, norms_dev, cols * 2 * sizeof(double), cudaMemcpyDeviceToHost, op->st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(op->st);
+    if (e != cudaSuccess) { helm_set_error("read right-hand side norms", e); return HELM_ECUDA; }
+    *out = true;
+    for (size_t c = 0; c < cols; ++c) *out = *out && isfinite(norms_host[2 * c + 1]);
+    return HELM_OK;
+}
+
 helm_status read_sweep_status(const helm_op *op) {
     int st_host = 0;
     cudaError_t e = cudaMemcpyAsync(&st_host, op->status, sizeof(int), cudaMemcpyDeviceToHost, op->st);
@@ -616,6 +638,7 @@ helm_status solve_impl(helm_factor_t *f, int nrhs, const double2 *B, double2 *X,
         }
         return HELM_OK;
     }
+    factor_back_to_bcr(f);
     if ((s = factor_reserve(f, nrhs)) != HELM_OK) return s;
     const MixedWork w{f->bd, f->xa, f->xb, f->r32, f->y, f->norms, f->norms_host.data(),
                       reinterpret_cast<RefineState *>(f->norms + 2 * cols), f->maxima};
@@ -623,9 +646,19 @@ helm_status solve_impl(helm_factor_t *f, int nrhs, const double2 *B, double2 *X,
     double rel = INFINITY;
     bool timed_out = false;
     if ((s = mixed_refine(f, nrhs, B, X, conj, rtol, max_iter, w, &it, &rel, &timed_out)) != HELM_OK) return s;
-    if (!timed_out && isfinite(rel) && !(rel <= rtol) && factor_retry_line(f) &&
-        (s = mixed_refine(f, nrhs, B, X, conj, rtol, max_iter, w, &it, &rel, &timed_out)) != HELM_OK)
-        return s;
+    // Not converged on an automatic BCR factor: once per factor, the solve is repeated on the line factor,
+    // which converges in the sweeps that it would have taken had it been chosen.  It stays if it does
+    // (the BCR factor was at fault); else the limits were the caller's, and the next solve is on the BCR
+    // factor again.  No factor meets an rtol below kTightestRtol or a right-hand side that is not finite.
+    bool repeat = !timed_out && !(rel <= rtol) && rtol >= kTightestRtol && f->auto_bcr;
+    if (repeat && !isfinite(rel) && (s = finite_rhs(op, cols, w.norms, w.norms_host, &repeat)) != HELM_OK) return s;
+    if (repeat && factor_retry_line(f)) {
+        if ((s = mixed_refine(f, nrhs, B, X, conj, rtol, max_iter, w, &it, &rel, &timed_out)) != HELM_OK) return s;
+        if (!timed_out && rel <= rtol) {
+            bcr_free(f);
+            f->line_stand_in = false;
+        }
+    }
     if (info) { info->iters = it; info->max_relres = rel; }
     if (timed_out) { helm_set_msg("a sweep kernel gave up waiting for its cluster"); return HELM_ETIMEOUT; }
     if (!(rel <= rtol)) { helm_set_msg("refinement did not reach rtol"); return HELM_ENOCONV; }

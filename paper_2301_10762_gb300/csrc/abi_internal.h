@@ -48,7 +48,8 @@ constexpr size_t kSmallMaxima = (size_t)1 << 16;
 struct helm_factor {
     helm_op *op = nullptr;
     bool use_bcr = false;  // mixed: block-cyclic-reduction factor on the tensor cores
-    bool auto_bcr = false; // ... chosen where the line factor would do (taken back if a refinement fails)
+    bool auto_bcr = false; // ... chosen where the line factor would do: an unconverged solve is repeated on that
+    bool line_stand_in = false;   // G, next to the BCR blocks, was built for such a repeat, which did not converge either
     BcrData bcr;
     helm_prec prec = HELM_FP64;
     int cs = 1;
@@ -112,6 +113,7 @@ namespace helm {
 bool bcr_supported(const GridGeom &g);
 int bcr_line(const GridGeom &g);               // nodes of a line as BCR lays it out: an odd line has one more
 bool factor_retry_line(helm_factor_t *f);
+void factor_back_to_bcr(helm_factor_t *f);     // ends a stand-in of the line factor (called as a solve begins)
 int solve_line(const helm_factor_t *f);        // line stride of the mixed solve's r32 and y
 // whether helm_factor builds a block-cyclic-reduction factor for this grid and precision
 // (method: a helm_factor_method; HELM_FACTOR_AUTO follows HELM_FACTOR and the line length)

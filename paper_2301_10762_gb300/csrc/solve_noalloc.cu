@@ -105,8 +105,6 @@ extern "C" helm_status helm_solve_noalloc(helm_factor_t *f, int32_t nrhs, const 
     const bool mixed = f->prec == HELM_MIXED;
     const size_t p_bytes = mixed ? align256(cols * N * sizeof(float4)) : 0;   // bd, xa, xb
     const size_t v_bytes = mixed ? align256(cols * N * sizeof(float2)) : 0;   // r32, y
-    // as laid out: an odd line of a block-cyclic-reduction factor has one more node (kPadBytes)
-    const size_t vp_bytes = mixed ? align256(cols * g.nx * solve_line(f) * sizeof(float2)) : 0;
     const size_t n_bytes = align256(cols * 2 * sizeof(double));
     const size_t s_bytes = mixed ? align256(refine_state_bytes(n_sys)) : 0;
     if (cols > kMaxCols || 3 * p_bytes + 2 * v_bytes + n_bytes + s_bytes > kScratchBytes) {
@@ -123,6 +121,9 @@ extern "C" helm_status helm_solve_noalloc(helm_factor_t *f, int32_t nrhs, const 
     void *base = nullptr;
     helm_status s = scratch_address(op->dev, &base);
     if (s != HELM_OK) return s;
+    if (mixed) factor_back_to_bcr(f);
+    // as laid out: an odd line of a block-cyclic-reduction factor has one more node (kPadBytes)
+    const size_t vp_bytes = mixed ? align256(cols * g.nx * solve_line(f) * sizeof(float2)) : 0;
     unsigned char *p = (unsigned char *)base;
     const double2 *B = (const double2 *)B_dev;
     double2 *X = (double2 *)X_dev;
