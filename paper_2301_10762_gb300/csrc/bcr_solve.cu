@@ -362,10 +362,12 @@ __global__ void __launch_bounds__(BS_THREADS, 1) bcr_solve_kernel(const __grid_c
             // terms share the tile's accumulator, so their scales share one exponent S per right-hand
             // side: S = min over the terms of (the block's shift + the line's largest shift), and a
             // line's shift is S less its block's.  A term that is small against the largest loses
-            // only what the sum does not hold (FP16 keeps all 22 bits 15 octaves down).
+            // only what the sum does not hold (FP16 keeps all 22 bits 15 octaves down).  S ends at 126,
+            // whose 2^-S is the smallest normal number: small lines times blocks of small entries
+            // (far from square cells) keep fewer bits there instead of a wrong scale.
             float sc[PR];
             auto put_scale = [&](int q, int S, int sl) {
-                if (j == 0 && q < np) s_bscale[sl][row0 + 16 * q] = bs_pow2(max(-126, min(126, -S)));
+                if (j == 0 && q < np) s_bscale[sl][row0 + 16 * q] = bs_pow2(max(-126, -S));
             };
             const int sl = tt % SL;
             // split and store one chunk's pairs into stage s
@@ -433,7 +435,7 @@ __global__ void __launch_bounds__(BS_THREADS, 1) bcr_solve_kernel(const __grid_c
                     const float bound = __uint_as_float(over_lanes(m3[0][q])) +
                                         fabsf(a.cx_in) * (__uint_as_float(over_lanes(m3[1][q])) +
                                                           __uint_as_float(over_lanes(m3[2][q])));
-                    const int sh = bs_scale_shift(bs_abs_bits(bound));
+                    const int sh = min(bs_scale_shift(bs_abs_bits(bound)), 126 - sa);
                     sc[q] = bs_pow2(sh);
                     put_scale(q, sh + sa, sl);
                 }
@@ -490,7 +492,7 @@ __global__ void __launch_bounds__(BS_THREADS, 1) bcr_solve_kernel(const __grid_c
             int S[PR];
 #pragma unroll
             for (int q = 0; q < PR; ++q) {
-                S[q] = 1 << 20;
+                S[q] = 126;
 #pragma unroll
                 for (int u = 0; u < 3; ++u) {
                     const int t2 = sa[u] + bs_scale_shift(over_lanes(mx[u][q]));
