@@ -139,8 +139,9 @@ void helm_op_destroy(helm_op_t *op);
  * factors).  HELM_FACTOR_AUTO (unless the environment sets HELM_FACTOR=line or =bcr): BCR for
  * HELM_MIXED on lines of an even nz >= 192 nodes (where the line recurrence's chain of nx dependent
  * line inversions dominates), and from nz = 96 on, odd nz included (laid out with one decoupled node
- * more), where there are at least 96 lines and its blocks stay within 16 GB, unless one of them comes
- * out nearly singular (a resonance of a strip of the medium) or the memory is not there; else the
+ * more), where there are at least 96 lines and its blocks (counted at 48 n_omega nx nz^2 bytes) stay
+ * within 1 GB, or within 16 GB and an eighth of the device memory that is available, unless one of them
+ * comes out nearly singular (a resonance of a strip of the medium) or the memory is not there; else the
  * line recurrence.  The first solve that does not converge on a factor chosen on that second count is
  * repeated on the line factor, unless rtol is below 1e-15 or B is not finite; if that converges the factor
  * stays the line factor, else the next solve is on the BCR factor again and not repeated

@@ -14,6 +14,7 @@
 #include "helm.h"
 #include "kernels.h"
 #include "abi_internal.h"
+#include "factor_choice.h"
 
 using namespace helm;
 
@@ -196,9 +197,6 @@ static constexpr int kBcrLine = 192;
 // 128 x 128 4500 / 1500.  Few lines favour the recurrence, whose chain is their number (48 x 96: solves
 // 280 / 320 and 370 / 510).
 static constexpr int kBcrShortLine = 96;
-// BCR holds about 3 (and 5.3 while it factors; 6 counted) times the line factor's bytes: a set of frequencies
-// whose blocks no longer are a small part of the device's memory stays with the smaller factor
-static constexpr size_t kBcrShortBytes = (size_t)16 << 30;
 // BCR eliminates lines with Dirichlet neighbours, so a frequency near a resonance of a strip of the
 // medium makes an eliminated block nearly singular.  Over 2100 random media (residual 1e-12, the line
 // factor's 3 to 4 sweeps) the refinement took a sweep more from |A| |Dinv| of about 2^8 (entries of the
@@ -219,13 +217,28 @@ bool helm::factor_picks_bcr(const GridGeom &g, helm_prec prec, int method) {
     }
     return m == HELM_FACTOR_BCR;
 }
+// device memory that a caller could still allocate: free, or held unused by the pool of this library's
+// (and the caller's) stream-ordered allocations
+static size_t device_available() {
+    size_t free_b = 0, total = 0;
+    if (cudaMemGetInfo(&free_b, &total) != cudaSuccess) { cudaGetLastError(); return 0; }
+    int dev = 0;
+    cudaMemPool_t pool;
+    uint64_t reserved = 0, used = 0;
+    if (cudaGetDevice(&dev) == cudaSuccess && cudaDeviceGetDefaultMemPool(&pool, dev) == cudaSuccess &&
+        cudaMemPoolGetAttribute(pool, cudaMemPoolAttrReservedMemCurrent, &reserved) == cudaSuccess &&
+        cudaMemPoolGetAttribute(pool, cudaMemPoolAttrUsedMemCurrent, &used) == cudaSuccess && reserved > used)
+        free_b += (size_t)(reserved - used);
+    cudaGetLastError();
+    return free_b;
+}
 // the automatic choice of BCR on a short or odd line (taken back where it turns out badly)
 static bool picks_short_bcr(const helm_op *op, helm_prec prec, const helm_factor_opts *opts) {
     const GridGeom &g = op->g;
     const char *env = getenv("HELM_FACTOR");
     if ((opts && opts->method != HELM_FACTOR_AUTO) || (env && (!strcmp(env, "line") || !strcmp(env, "bcr")))) return false;
     return prec == HELM_MIXED && (g.nz < kBcrLine || (g.nz & 1)) && g.nz >= kBcrShortLine && g.nx >= kBcrShortLine &&
-           6 * sizeof(float2) * op->n_omega * g.nx * g.nz * g.nz <= kBcrShortBytes;
+           short_bcr_fits(short_bcr_bytes(op->n_omega, g.nx, g.nz), device_available);
 }
 static bool bcr_falls_back(const GridGeom &g, const int st_host[3]) {
     if (st_host[0] & ST_TIMEOUT) return false;

@@ -9,7 +9,7 @@ ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
 
 @pytest.mark.skipif(shutil.which("g++") is None, reason="no host C++ compiler")
-@pytest.mark.parametrize("name", ["sweep_shape"])
+@pytest.mark.parametrize("name", ["sweep_shape", "factor_choice"])
 def test_rule(name, tmp_path):
     exe = str(tmp_path / name)
     src = os.path.join(ROOT, "tests", "cpp", name + "_check.cpp")
