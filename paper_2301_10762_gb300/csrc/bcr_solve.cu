@@ -269,14 +269,13 @@ __global__ void __launch_bounds__(BS_THREADS, 1) bcr_solve_kernel(const __grid_c
                 }
             }
             // no copy may land after the CTA has left.  (A stage's barrier completes with the operand
-            // warps' arrivals too, which an abort may leave out: then a fixed time is waited)
-            const int s0 = *(volatile int *)&s_abort;
-            if (s0) {
-                abort_drain();
-            } else {
-                for (int c = max(0, issued - ST); c < issued; ++c)
-                    mbar_wait_bounded(&full[c % ST], (uint32_t)((c / ST) & 1), kDefaultWaitTries);
-            }
+            // warps' arrivals too, which an abort may leave out, also one that comes while this waits:
+            // then a fixed time is waited)
+            for (int c = max(0, issued - ST); c < issued; ++c)
+                if (!mbar_wait_cta(&full[c % ST], (uint32_t)((c / ST) & 1), kDefaultWaitTries, &s_abort)) {
+                    abort_drain();
+                    break;
+                }
         }
         __syncwarp();
     } else if (warp == 0) {
