@@ -37,7 +37,7 @@ helm_status helm_zgemm_batched(int32_t batch, int32_t M, int32_t N, int32_t K, c
 
 /* helm_zinv_batched -- X_t = A_t^{-1} for t < batch, complex FP32, n x n complex symmetric
  * matrices (A = A^T, the line blocks of the Helmholtz operator and their Schur complements).
- * n <= 128: block Gauss-Jordan in one CTA's shared memory over 16-column blocks, each 16 x 16
+ * n <= 128: block Gauss-Jordan in one CTA (the block in registers) over 16-column blocks, each 16 x 16
  * pivot block inverted by one warp with partial pivoting; n > 128: the 2 x 2 block inverse of a
  * symmetric matrix with 128-multiple leading blocks, its products on the tensor cores
  * (helm_zgemm_batched) and its two half-size inverses recursive.  A and X row-major with row

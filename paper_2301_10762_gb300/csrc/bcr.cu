@@ -90,7 +90,7 @@ Coup coup_of(const GridGeom &g) {
 // amplifies level 0's errors most (the Schur complements of the smooth modes lose four in size
 // per level): a block Gauss-Jordan inverse carries 1.2e-7 of its norm.
 // 256^2 with 8 frequencies: level 0 with its images 0.9 ms, a quarter of it the recurrences (dense inversions by two 128-column
-// halves 1.0 ms, images and update 0.6); 512^2 with 4: 19 ms less.
+// halves 1.0 ms, images and update 0.6); 512^2 with 8: 19 ms less.
 struct TriGen {          // generators of the odd lines' inverses: [line][nz]
     float4 *u, *v;       // hi.x, hi.y, lo.x, lo.y
     int2 *e;             // exponents of u and v
@@ -335,20 +335,15 @@ __global__ void __launch_bounds__(128) bcr_level0_kernel(GridGeom g, int np, Cou
 
 struct InvArgs {
     int n;
-    ZOperand in;                 // row-major, ld = in.ld
-    float2 *out;                 // row-major, ld = ldo
-    long long out_stride, out_stride_hi;
-    int out_div, ldo;
-    const int *idx;              // [count][2]: input index, output index
+    float2 *X;                   // blocks, row-major
+    long long stride;
+    int ld;
+    const int *idx;              // [count]: block
     int *status;
     uint32_t tries = 0;          // polls of a bounded mbarrier wait before it gives up
 };
 
-__device__ __forceinline__ long long op_off(int idx, int div, long long stride, long long stride_hi) {
-    return div > 0 ? (long long)(idx / div) * stride_hi + (long long)(idx % div) * stride : (long long)idx * stride;
-}
-
-// X = M^{-1} of one n x n block (n <= 128) per CTA by Gauss-Jordan in steps of 16 columns, partial
+// X <- X^{-1} of one n x n block (n <= 128) per CTA by Gauss-Jordan in steps of 16 columns, partial
 // pivoting inside each 16 x 16 pivot block.  The block lives in registers: thread (r, h) of
 // 512 holds row r, columns 32 h .. + 31 (beyond n: the identity).  A step with the pivot columns
 // K = k0 .. k0 + 15 is
@@ -432,9 +427,7 @@ __global__ void __launch_bounds__(ZT_THREADS, 1) zinv_kernel(InvArgs a) {
     float2 *Un = Nd + PIV * ZT_PS, *Rn = Un + PIV * ZT_PS;       // W[K1, K] and R'[:, K1] of the next block,
     float2 *Sn = Rn + PIV * ZT_PS;                               // and the next pivot block
     const uint32_t a_hi = base + ZT_A, a_lo = a_hi + 16384, b_hi = base + ZT_B, b_lo = b_hi + 32768;
-    const int *ix = a.idx + 2 * (size_t)blockIdx.x;
-    const float2 *M = a.in.base + op_off(ix[0], a.in.div, a.in.stride, a.in.stride_hi);
-    float2 *X = a.out + op_off(ix[1], a.out_div, a.out_stride, a.out_stride_hi);
+    float2 *X = a.X + a.idx[blockIdx.x] * a.stride;
     if (tid == 0) {
         s_bad = 0;
         mbar_init(&mma_bar, 1);
@@ -458,7 +451,7 @@ __global__ void __launch_bounds__(ZT_THREADS, 1) zinv_kernel(InvArgs a) {
             for (int e = 0; e < 2; ++e) {
                 const int c = 64 * half + 32 * e + lane;
                 T[rr * ZT_TS + 32 * e + lane] =
-                    rr < n && c < n ? M[(size_t)rr * a.in.ld + c] : make_float2(rr == c ? 1.f : 0.f, 0.f);
+                    rr < n && c < n ? X[(size_t)rr * a.ld + c] : make_float2(rr == c ? 1.f : 0.f, 0.f);
             }
         }
         __syncthreads();
@@ -638,7 +631,7 @@ __global__ void __launch_bounds__(ZT_THREADS, 1) zinv_kernel(InvArgs a) {
 #pragma unroll
                 for (int e = 0; e < 2; ++e) {
                     const int c = 64 * half + 32 * e + lane;
-                    if (rr < n && c < n) X[(size_t)rr * a.ldo + c] = T[rr * ZT_TS + 32 * e + lane];
+                    if (rr < n && c < n) X[(size_t)rr * a.ld + c] = T[rr * ZT_TS + 32 * e + lane];
                 }
             }
             __syncthreads();
@@ -684,13 +677,13 @@ helm_status upload_ints(const std::vector<int> &h, TaskBuf &b, cudaStream_t st) 
     return HELM_OK;
 }
 
+// partial tiles of the split-K products of helm_zgemm_batched and helm_zinv_batched: 64 MB (8 products of
+// 256 x 256 split 16 ways)
+constexpr size_t kSplitElems = (size_t)8 << 20;
+
 // A recorded sequence of launches: every task list goes into one host array, uploaded with a
 // single copy before the launches are enqueued (a copy from pageable host memory waits for the
 // stream, so one copy per launch would serialise the host with the GPU at every launch).
-// partial tiles of split-K GEMM launches: 64 MB for a factorisation (its deep levels: 8 tasks of
-// 256 x 256 split 16 ways)
-constexpr size_t kFactorSplitElems = (size_t)8 << 20;
-
 struct Plan {
     cudaStream_t st;
     std::vector<int> ints;
@@ -724,52 +717,24 @@ struct Plan {
     }
 };
 
-ZOperand zop(const float2 *base, long long stride, int ld, int div = 0, long long stride_hi = 0) {
+ZOperand zop(const float2 *base, long long stride, int ld) {
     ZOperand o;
     o.base = base;
     o.stride = stride;
     o.ld = ld;
-    o.div = div;
-    o.stride_hi = stride_hi;
     return o;
-}
-
-std::vector<int> task8(int a0, int b0, int c0, int c, int a1 = -1, int b1 = -1, int a2 = -1, int b2 = -1) {
-    return {a0, a1, a2, b0, b1, b2, c0, c};
-}
-
-// product terms of a task list (a term is present when its A index is not negative)
-long long count_terms(const int *tasks, size_t n_tasks, int nterms) {
-    long long t = 0;
-    for (size_t i = 0; i < n_tasks; ++i)
-        for (int u = 0; u < nterms; ++u) t += tasks[8 * i + u] >= 0;
-    return t;
-}
-
-// family counts of a launch's operands from its (host) task list, where not given
-void count_families(ZGemmArgs &a, const std::vector<int> &tasks) {
-    for (int u = 0; u < a.nterms; ++u) {
-        int ma = -1, mb = -1;
-        for (size_t t = 0; t < tasks.size(); t += 8)
-            if (tasks[t + u] >= 0) {
-                ma = std::max(ma, tasks[t + u]);
-                mb = std::max(mb, tasks[t + 3 + u]);
-            }
-        auto set = [](ZOperand &o, int mx) {
-            if (o.count == 0 && mx >= 0) o.count = o.div > 0 ? mx / o.div + 1 : mx + 1;
-        };
-        set(a.A[u], ma);
-        set(a.B[u], mb);
-    }
 }
 
 helm_status gemm(const ZGemmArgs &a0, const std::vector<int> &tasks, Plan &pl) {
     if (tasks.empty()) return HELM_OK;
-    const int off = pl.add(tasks), n = (int)(tasks.size() / 8);
+    const int off = pl.add(tasks), n = (int)(tasks.size() / 4);
     ZGemmArgs a = a0;
-    count_families(a, tasks);
+    for (int t = 0; t < n; ++t) {
+        a.A.count = std::max<long long>(a.A.count, tasks[4 * t] + 1);
+        a.B.count = std::max<long long>(a.B.count, tasks[4 * t + 1] + 1);
+    }
     a.tries = wait_tries();
-    a.flops = 8.0 * a.M * a.N * a.K * (double)count_terms(tasks.data(), (size_t)n, a.nterms);
+    a.flops = 8.0 * a.M * a.N * a.K * n;
     a.part = pl.split;
     a.part_cap = pl.split_cap;
     const cudaStream_t st = pl.st;
@@ -792,17 +757,17 @@ struct Fam {
     ZOperand op() const { return zop(base, stride, ld); }
 };
 
-// out[p.second] = in[p.first]^{-1} for every index pair, n x n blocks (may be the same matrices)
-helm_status invert_blocks(int n, Fam in, Fam out, const std::vector<int> &pairs, int *status, Plan &pl) {
-    const int count = (int)(pairs.size() / 2);
+// X[i] <- X[i]^{-1} for every block i of the list, n x n, symmetric above INV_MAX columns
+helm_status invert_blocks(int n, Fam X, const std::vector<int> &blocks, int *status, Plan &pl) {
+    const int count = (int)blocks.size();
     if (count == 0) return HELM_OK;
     const cudaStream_t st = pl.st;
     helm_status s;
     if (n <= INV_MAX) {
-        const int off = pl.add(pairs);
+        const int off = pl.add(blocks);
         cudaError_t e = ensure_dyn_smem((const void *)zinv_kernel, ZT_SMEM);
         if (e != cudaSuccess) { helm_set_error("bcr: block inversion", e); return HELM_ECUDA; }
-        InvArgs a{n, in.op(), out.base, out.stride, 0, 0, out.ld, nullptr, status};
+        InvArgs a{n, X.base, X.stride, X.ld, nullptr, status};
         a.tries = wait_tries();
         pl.ops.push_back([a, off, count, st](const int *dev) mutable -> helm_status {
             a.idx = dev + off;
@@ -815,7 +780,7 @@ helm_status invert_blocks(int n, Fam in, Fam out, const std::vector<int> &pairs,
     }
     const int n1 = INV_MAX * ((n / INV_MAX + 1) / 2), n2 = n - n1;
     // X11 = D11^{-1}
-    if ((s = invert_blocks(n1, in, out, pairs, status, pl)) != HELM_OK) return s;
+    if ((s = invert_blocks(n1, X, blocks, status, pl)) != HELM_OK) return s;
     // scratch T (n1 x n2) and Tt = T^T (n2 x n1) per block: allocated now (stream-ordered, usable
     // by the launches enqueued later), released on the stream after the last launch that reads it
     float2 *T = nullptr, *Tt = nullptr;
@@ -829,25 +794,19 @@ helm_status invert_blocks(int n, Fam in, Fam out, const std::vector<int> &pairs,
     // (released by the plan after its last launch)
     pl.scratch.push_back(T);
     pl.scratch.push_back(Tt);
-    const Fam X11 = out.sub(0, 0), X12 = out.sub(0, n1), X21 = out.sub(n1, 0), X22 = out.sub(n1, n1);
-    const Fam D21 = in.sub(n1, 0), D22 = in.sub(n1, n1);
+    const Fam X11 = X.sub(0, 0), X12 = X.sub(0, n1), X21 = X.sub(n1, 0), X22 = X.sub(n1, n1);
     const Fam FT{T, ts, n2}, FTt{Tt, ts, n1};
     std::vector<int> tk;
-    auto run = [&](int M, int N, int K, Fam A, Fam B, const Fam *C0, Fam C, float sign, int which_a, int which_b,
-                   int which_c0, int which_c) -> helm_status {
-        // which_*: 0 the input index, 1 the output index, 2 the block's position in the batch
+    auto run = [&](int M, int N, int K, Fam A, Fam B, const Fam *C0, Fam C, float sign) -> helm_status {
+        // matrices of X by the block, of T and its transpose by the position in the batch
+        auto id = [&](const Fam &f, int t) { return f.base == T || f.base == Tt ? t : blocks[t]; };
         tk.clear();
-        for (int t = 0; t < count; ++t) {
-            const int id[3] = {pairs[2 * t], pairs[2 * t + 1], t};
-            auto v = task8(id[which_a], id[which_b], C0 ? id[which_c0] : 0, id[which_c]);
-            tk.insert(tk.end(), v.begin(), v.end());
-        }
+        for (int t = 0; t < count; ++t) tk.insert(tk.end(), {id(A, t), id(B, t), C0 ? id(*C0, t) : 0, id(C, t)});
         ZGemmArgs g;
         g.M = M; g.N = N; g.K = K;
-        g.nterms = 1;
-        g.A[0] = A.op();
-        g.B[0] = B.op();
-        g.sign[0] = sign;
+        g.A = A.op();
+        g.B = B.op();
+        g.sign = sign;
         if (C0) g.C0 = C0->op();
         g.C = C.base;
         g.c_stride = C.stride;
@@ -855,19 +814,17 @@ helm_status invert_blocks(int n, Fam in, Fam out, const std::vector<int> &pairs,
         g.status = status;
         return gemm(g, tk, pl);
     };
+    // (X21 and X22 hold D21 and D22 until they are written)
     // T = X11 D12 = X11 D21^T;  Tt = D21 X11 (= T^T, X11 symmetric)
-    if ((s = run(n1, n2, n1, X11, D21, nullptr, FT, 1.f, 1, 0, 0, 2)) != HELM_OK) return s;
-    if ((s = run(n2, n1, n1, D21, X11, nullptr, FTt, 1.f, 0, 1, 0, 2)) != HELM_OK) return s;
-    // S = D22 - D21 T  -> X22, then X22 = S^{-1} in place
-    if ((s = run(n2, n2, n1, D21, FTt, &D22, X22, -1.f, 0, 2, 0, 1)) != HELM_OK) return s;
-    std::vector<int> self(pairs.size());
-    for (int t = 0; t < count; ++t) self[2 * t] = self[2 * t + 1] = pairs[2 * t + 1];
-    if ((s = invert_blocks(n2, X22, X22, self, status, pl)) != HELM_OK) return s;
+    if ((s = run(n1, n2, n1, X11, X21, nullptr, FT, 1.f)) != HELM_OK) return s;
+    if ((s = run(n2, n1, n1, X21, X11, nullptr, FTt, 1.f)) != HELM_OK) return s;
+    // X22 = S = D22 - D21 T, then its inverse
+    if ((s = run(n2, n2, n1, X21, FTt, &X22, X22, -1.f)) != HELM_OK) return s;
+    if ((s = invert_blocks(n2, X22, blocks, status, pl)) != HELM_OK) return s;
     // X12 = -T X22;  X21 = -X22 T^T;  X11 <- X11 - T X21
-    if ((s = run(n1, n2, n2, FT, X22, nullptr, X12, -1.f, 2, 1, 0, 1)) != HELM_OK) return s;
-    if ((s = run(n2, n1, n2, X22, FT, nullptr, X21, -1.f, 1, 2, 0, 1)) != HELM_OK) return s;
-    if ((s = run(n1, n1, n2, FT, X12, &X11, X11, -1.f, 2, 1, 1, 1)) != HELM_OK) return s;
-    return HELM_OK;
+    if ((s = run(n1, n2, n2, FT, X22, nullptr, X12, -1.f)) != HELM_OK) return s;
+    if ((s = run(n2, n1, n2, X22, FT, nullptr, X21, -1.f)) != HELM_OK) return s;
+    return run(n1, n1, n2, FT, X12, &X11, X11, -1.f);
 }
 
 // images (bcr_solve.cu) of a part of the blocks in slots pairs[.][0] of D as matrices pairs[.][1]
@@ -911,10 +868,7 @@ int invert_nodes(int n) {   // nodes of the recursion on n columns
 helm_status invert_images(const BgArgs &ba, const std::vector<int> &slots, int r0, int n, int &node, Plan &pl) {
     const int count = (int)slots.size(), nz = ba.nz;
     if (n <= INV_MAX) {
-        std::vector<int> pairs;
-        for (int v : slots) pairs.insert(pairs.end(), {v, v});
-        const Fam d = Fam{ba.D, (long long)nz * nz, nz}.sub(r0, r0);
-        return invert_blocks(n, d, d, pairs, ba.status, pl);
+        return invert_blocks(n, Fam{ba.D, (long long)nz * nz, nz}.sub(r0, r0), slots, ba.status, pl);
     }
     const int id = ba.im.n_sub + 8 * node++, n1 = INV_MAX * ((n / INV_MAX + 1) / 2), n2 = n - n1, r1 = r0 + n1;
     enum { D21, X11, T, X22, TT, X12 };
@@ -1248,28 +1202,24 @@ helm_status blas_zgemm(int batch, int M, int N, int K, const float2 *A, long lon
                        cudaStream_t st, int *status) {
     ZGemmArgs a;
     a.M = M; a.N = N; a.K = K;
-    a.nterms = 1;
-    a.A[0] = zop(A, sa, lda);
-    a.B[0] = zop(Bt, sb, ldb);
-    a.sign[0] = sign;
+    a.A = zop(A, sa, lda);
+    a.B = zop(Bt, sb, ldb);
+    a.sign = sign;
     if (C0) a.C0 = zop(C0, sc, ldc);
     a.C = C; a.c_stride = sc; a.ldc = ldc;
     a.status = status;
     std::vector<int> tasks;
-    for (int t = 0; t < batch; ++t) {
-        auto v = task8(t, t, t, t);
-        tasks.insert(tasks.end(), v.begin(), v.end());
-    }
+    for (int t = 0; t < batch; ++t) tasks.insert(tasks.end(), {t, t, t, t});
     Plan pl(st);
-    helm_status s = pl.with_split(kFactorSplitElems);
+    helm_status s = pl.with_split(kSplitElems);
     if (s == HELM_OK) s = gemm(a, tasks, pl);
     return s == HELM_OK ? pl.run() : s;
 }
 
 helm_status blas_zinv(int batch, int n, const float2 *A, long long sa, int lda, float2 *X, long long sx, int ldx,
                       cudaStream_t st, int *status) {
-    std::vector<int> pairs;
-    for (int t = 0; t < batch; ++t) pairs.insert(pairs.end(), {t, t});
+    std::vector<int> blocks(batch);
+    for (int t = 0; t < batch; ++t) blocks[t] = t;
     if (A != X) {   // copy into X first: the recursion works in place on the output blocks
         // blocks stacked without gaps on both sides are one 2D copy of batch * n rows
         const bool stacked = sa == (long long)n * lda && sx == (long long)n * ldx;
@@ -1284,8 +1234,8 @@ helm_status blas_zinv(int batch, int n, const float2 *A, long long sa, int lda, 
     }
     const Fam f{X, sx, ldx};
     Plan pl(st);
-    helm_status s = pl.with_split(kFactorSplitElems);
-    if (s == HELM_OK) s = invert_blocks(n, f, f, pairs, status, pl);
+    helm_status s = pl.with_split(kSplitElems);
+    if (s == HELM_OK) s = invert_blocks(n, f, blocks, status, pl);
     return s == HELM_OK ? pl.run() : s;
 }
 

@@ -105,35 +105,28 @@ cudaError_t launch_refine_finish(size_t n, int N, int nrhs, const float4 *xa, co
 cudaError_t launch_refine_accumulate(size_t n, int nz, int ld, const float2 *delta, int conj, double2 *X, cudaStream_t st);
 
 // ---- zgemm_tc.cu (batched complex GEMM on tcgen05, 3xTF32)
-// A family of complex FP32 matrices: matrix idx starts at base + (idx / div) * stride_hi +
-// (idx % div) * stride (div <= 0: base + idx * stride); rows are ld elements apart.
+// A family of complex FP32 matrices: matrix idx starts at base + idx * stride; rows are ld elements
+// apart.
 struct ZOperand {
     const float2 *base = nullptr;
-    long long stride = 0, stride_hi = 0;
-    int div = 0;
+    long long stride = 0;
     int ld = 0;
-    // matrices of the family (div <= 0) or groups of div matrices (div > 0); 0 if not known.
-    // Launches whose operands all have a count stream them with tensor copies (narrow tiles).
-    long long count = 0;
+    long long count = 0;   // matrices of the family
 };
-// C_t = C0_t + sum_u sign_u A_{t,u} Bt_{t,u}^T for every task t of tasks[n_tasks][8]
-// (a_idx[3], b_idx[3], c0_idx, c_idx); a term with a negative A index is absent from its task.  A: M x K, Bt: N x K (row-major); C, C0: M x N, row-major or (c_col) column-major.
+// C_t = C0_t + sign A_t Bt_t^T for every task t of tasks[n_tasks][4] (the matrices' numbers in A, B, C0
+// and C).  A: M x K, Bt: N x K, C, C0: M x N, all row-major.
 struct ZGemmArgs {
     int M = 0, N = 0, K = 0;
-    int nterms = 1;
-    ZOperand A[3], B[3];
-    float sign[3] = {1.f, 1.f, 1.f};
+    ZOperand A, B;
+    float sign = 1.f;
     ZOperand C0;          // base == nullptr: no C0
     float2 *C = nullptr;
-    long long c_stride = 0, c_stride_hi = 0;
-    int c_div = 0;
+    long long c_stride = 0;
     int ldc = 0;
-    int c_col = 0;
     const int *tasks = nullptr;
     int *status = nullptr;
-    const int *skip = nullptr;
     uint32_t tries = 0;
-    double flops = 0.0;   // useful flops of the launch (8 M N K per complex term of every task), for tracing
+    double flops = 0.0;   // useful flops of the launch (8 M N K per task), for tracing
     // split-K: with part != nullptr a launch that fills less than a wave of CTAs splits each
     // task's K chunks over ksplit CTAs, which write partial tiles into part (at most part_cap
     // complex elements; laid out like C, without C0); a second kernel sums them in a fixed order
@@ -141,10 +134,6 @@ struct ZGemmArgs {
     int ksplit = 1;
     float2 *part = nullptr;
     size_t part_cap = 0;
-    // per-system skip (refinement): a task whose system (C index / sys_div) has
-    // sys_frozen[2 * system] set does nothing
-    const int *sys_frozen = nullptr;
-    int sys_div = 1;
 };
 cudaError_t launch_zgemm(const ZGemmArgs &a, int n_tasks, cudaStream_t st);
 

@@ -1,8 +1,8 @@
 // Batched complex-FP32 GEMM on the fifth-generation tensor cores (tcgen05, accumulator in
 // tensor memory), with the 3xTF32 split that keeps the products near FP32 accuracy:
-//     C_t = C0_t + sum_u s_u A_{t,u} Bt_{t,u}^T      (t: task, u <= 3 terms, s_u = +-1)
-// A (M x K) and Bt (N x K) are row-major complex matrices (interleaved re, im); C and C0 are
-// row-major or column-major.  This is the library's product of FP32 blocks: helm_zgemm_batched,
+//     C_t = C0_t + s A_t Bt_t^T      (t: task, s = +-1)
+// A (M x K), Bt (N x K), C and C0 are row-major complex matrices (interleaved re, im).
+// This is the library's product of FP32 blocks: helm_zgemm_batched,
 // and the products of helm_zinv_batched above n = 128 (the block-cyclic-reduction factor and solve
 // have theirs on FP16 pairs, bcr_gemm.cu and bcr_solve.cu).
 //
@@ -22,7 +22,7 @@
 // the stage's empty barrier, which the operand warps wait for before they overwrite the stage
 // STAGES chunks later.  No CTA-wide barrier sits in the K loop.  The epilogue reads the
 // accumulator with tcgen05.ld into a padded tile in the (then idle) shared memory, from which
-// each warp writes whole rows (row-major C) or whole columns (column-major C), adding C0.
+// each warp writes whole rows, adding C0.
 #include <cuda.h>   // CUtensorMap and its enums (the encoder is taken from the driver at run time)
 #include <stdint.h>
 
@@ -41,10 +41,6 @@ namespace {
 constexpr int ZG_PRODUCERS = 512;                 // threads of the 16 operand warps
 constexpr int ZG_BM = 128;   // tile rows (tcgen05 M)
 constexpr int ZG_KC = 16;    // complex K per chunk: 32 floats = one 128-byte swizzle row
-
-__device__ __forceinline__ long long zop_off(int idx, int div, long long stride, long long stride_hi) {
-    return div > 0 ? (long long)(idx / div) * stride_hi + (long long)(idx % div) * stride : (long long)idx * stride;
-}
 
 constexpr int ZG_SMEM_MAX = 232448;   // dynamic + static shared memory of one CTA (227 KB)
 
@@ -75,20 +71,19 @@ template <int NT, bool RING> struct ZCfg {
 };
 
 // Tensor maps of the operands of a RING launch: each family of R x K complex matrices as a
-// rank-4 float tensor (2K floats of a row, then rows, matrices of a group and groups, ordered by
-// increasing stride); pos[u][role] is the dimension (1..3) of the row, in-group and group index.
+// rank-3 float tensor (2K floats of a row, then rows and matrices by increasing stride);
+// rows_first: dimension 1 counts rows, 2 matrices (else the other way round).
 struct ZMaps {
-    CUtensorMap a[3], b[3];
-    int8_t apos[3][3], bpos[3][3];
+    CUtensorMap a, b;
+    bool a_rows_first, b_rows_first;
 };
 
 // tiled tensor copy of one box into this CTA's shared memory, completing its bytes on the mbarrier
-__device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap *map, int c0, int c1, int c2, int c3,
-                                            uint64_t *bar) {
+__device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap *map, int c0, int c1, int c2, uint64_t *bar) {
     asm volatile(
-        "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, "
-        "%5}], [%6];" ::"r"(dst),
-        "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(smem_u32(bar))
+        "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];" ::"r"(
+            dst),
+        "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(c2), "r"(smem_u32(bar))
         : "memory");
 }
 
@@ -113,24 +108,18 @@ __global__ void __launch_bounds__(ZCfg<NT, RING>::THREADS, 1)
     __shared__ uint32_t s_tmem;
     __shared__ int s_abort;
 
-    if (a.skip && *a.skip) return;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int m0 = blockIdx.x * ZG_BM, n0 = blockIdx.y * NT;
     const int ks = a.ksplit, kpart = (int)(blockIdx.z % (unsigned)ks);   // split-K part of this CTA
-    const int* task = a.tasks + (size_t)(blockIdx.z / (unsigned)ks) * 8;
-    if (a.sys_frozen && a.sys_frozen[2 * (task[7] / a.sys_div)]) return;   // its system needs no correction
+    const int *task = a.tasks + (size_t)(blockIdx.z / (unsigned)ks) * 4;
     const uint32_t smem0 = (smem_u32(zg_smem_raw) + 1023u) & ~1023u;
     const uint32_t ring0 = smem0 + (uint32_t)(Cfg::STAGES * Cfg::STAGE);   // raw slots (RING)
 
-    // active terms (a term whose A index is negative is absent)
-    int act[3] = {0, 0, 0}, nterms = 0;
-    for (int u = 0; u < a.nterms; ++u)
-        if (task[u] >= 0) act[nterms++] = u;
     const int nkc = (a.K + ZG_KC - 1) / ZG_KC;
-    // this CTA's K chunks [cbase, cbase + nchunks) of the task's nterms * nkc (all of them
-    // unless split); the loops below count chunks locally from 0
-    const int cbase = (int)((long long)kpart * nterms * nkc / ks);
-    const int nchunks = (int)((long long)(kpart + 1) * nterms * nkc / ks) - cbase;
+    // this CTA's K chunks [cbase, cbase + nchunks) of the task's nkc (all of them unless split); the
+    // loops below count chunks locally from 0
+    const int cbase = (int)((long long)kpart * nkc / ks);
+    const int nchunks = (int)((long long)(kpart + 1) * nkc / ks) - cbase;
 
     const bool mma_warp = warp == 0;
     const int ptid = tid - 32 * Cfg::PW0;   // operand-thread index (warps PW0 .. PW0 + 15)
@@ -163,29 +152,26 @@ __global__ void __launch_bounds__(ZCfg<NT, RING>::THREADS, 1)
     // is stored, so that a load has NSETS - 1 chunks of work to arrive in)
     using RA = float4[Cfg::A_V4];
     using RB = float4[Cfg::B_V4];
-    auto term_of = [&](int c) { const int cu = c / nkc; return cu == 0 ? act[0] : (cu == 1 ? act[1] : act[2]); };
+    const float2 *A = a.A.base + task[0] * a.A.stride, *B = a.B.base + task[1] * a.B.stride;
     auto fetch = [&](int c, RA &ra, RB &rb) {
-        const int u = term_of(cbase + c), k0 = ((cbase + c) % nkc) * ZG_KC;
-        const float2 *A = a.A[u].base + zop_off(task[u], a.A[u].div, a.A[u].stride, a.A[u].stride_hi);
-        const float2 *B = a.B[u].base + zop_off(task[3 + u], a.B[u].div, a.B[u].stride, a.B[u].stride_hi);
+        const int k0 = (cbase + c) * ZG_KC;
 #pragma unroll
         for (int i = 0; i < Cfg::A_V4; ++i) {
             const int e = ptid + i * ZG_PRODUCERS, r = e >> 3, k = k0 + 2 * (e & 7);
             ra[i] = (m0 + r < a.M && k < a.K)
-                        ? __ldg(reinterpret_cast<const float4 *>(A + (long long)(m0 + r) * a.A[u].ld + k))
+                        ? __ldg(reinterpret_cast<const float4 *>(A + (long long)(m0 + r) * a.A.ld + k))
                         : make_float4(0.f, 0.f, 0.f, 0.f);
         }
 #pragma unroll
         for (int i = 0; i < Cfg::B_V4; ++i) {
             const int e = ptid + i * ZG_PRODUCERS, n = e >> 3, k = k0 + 2 * (e & 7);
             rb[i] = (e < NT * 8 && n0 + n < a.N && k < a.K)
-                        ? __ldg(reinterpret_cast<const float4 *>(B + (long long)(n0 + n) * a.B[u].ld + k))
+                        ? __ldg(reinterpret_cast<const float4 *>(B + (long long)(n0 + n) * a.B.ld + k))
                         : make_float4(0.f, 0.f, 0.f, 0.f);
         }
     };
     // ---- split and store of a fetched chunk into stage s
-    auto store = [&](int c, int s, const RA &ra, const RB &rb) {
-        const float sg = a.sign[term_of(cbase + c)];
+    auto store = [&](int s, const RA &ra, const RB &rb) {
         const uint32_t base = smem0 + (uint32_t)(s * Cfg::STAGE);
         const uint32_t a_hi = base, a_lo = base + Cfg::A_BYTES;
         const uint32_t b_hi = base + 2 * Cfg::A_BYTES, b_lo = b_hi + Cfg::B_BYTES;
@@ -193,7 +179,7 @@ __global__ void __launch_bounds__(ZCfg<NT, RING>::THREADS, 1)
         for (int i = 0; i < Cfg::A_V4; ++i) {
             const int e = ptid + i * ZG_PRODUCERS, r = e >> 3, j = e & 7;
             float4 hi, lo;
-            split4(ra[i], sg, hi, lo);
+            split4(ra[i], a.sign, hi, lo);
             st_shared_v4(a_hi + sw128(r, j), hi);
             st_shared_v4(a_lo + sw128(r, j), lo);
         }
@@ -216,7 +202,7 @@ __global__ void __launch_bounds__(ZCfg<NT, RING>::THREADS, 1)
 
     // ---- RING: the chunk from its raw slot (rows of 128 bytes as copied) into registers
     auto fetch_raw = [&](int c, RA &ra, RB &rb) {
-        const int k0 = ((cbase + c) % nkc) * ZG_KC;
+        const int k0 = (cbase + c) * ZG_KC;
         const uint32_t slot = ring0 + (uint32_t)((c % Cfg::SLOTS) * Cfg::RAW);
 #pragma unroll
         for (int i = 0; i < Cfg::A_V4; ++i) {
@@ -252,7 +238,7 @@ __global__ void __launch_bounds__(ZCfg<NT, RING>::THREADS, 1)
                 if (bad) give_up();
                 return false;
             }
-            store(c, s, ra, rb);
+            store(s, ra, rb);
             // the stores are made visible to the tensor core's (async proxy) reads before the
             // next loads are issued: a proxy fence after them would wait for those loads as well
             // and expose their latency on every chunk
@@ -291,7 +277,7 @@ __global__ void __launch_bounds__(ZCfg<NT, RING>::THREADS, 1)
             }
             float4 ra[Cfg::A_V4], rb[Cfg::B_V4];
             fetch_raw(c, ra, rb);
-            store(c, s, ra, rb);
+            store(s, ra, rb);
             fence_proxy_async_smem();   // the stores, before the tensor core reads them
             __syncwarp();               // every lane's slot reads, stores and fence before the arrivals
             if (lane == 0) {
@@ -317,19 +303,12 @@ __global__ void __launch_bounds__(ZCfg<NT, RING>::THREADS, 1)
                 }
             }
             if (lane == 0) {
-                const int u = term_of(cbase + c), k0 = ((cbase + c) % nkc) * ZG_KC;
+                const int k0 = (cbase + c) * ZG_KC, ia = task[0], ib = task[1];
                 const uint32_t slot = ring0 + (uint32_t)(q * Cfg::RAW);
                 mbar_arrive_expect_tx(&raw_full[q], (uint32_t)Cfg::RAW);
-                int ca[4] = {2 * k0, 0, 0, 0}, cb[4] = {2 * k0, 0, 0, 0};
-                const int ia = task[u], ib = task[3 + u];
-                ca[maps.apos[u][0]] = m0;
-                ca[maps.apos[u][1]] = a.A[u].div > 0 ? ia % a.A[u].div : ia;
-                ca[maps.apos[u][2]] = a.A[u].div > 0 ? ia / a.A[u].div : 0;
-                cb[maps.bpos[u][0]] = n0;
-                cb[maps.bpos[u][1]] = a.B[u].div > 0 ? ib % a.B[u].div : ib;
-                cb[maps.bpos[u][2]] = a.B[u].div > 0 ? ib / a.B[u].div : 0;
-                tma_load_4d(slot, &maps.a[u], ca[0], ca[1], ca[2], ca[3], &raw_full[q]);
-                tma_load_4d(slot + Cfg::RAW_A, &maps.b[u], cb[0], cb[1], cb[2], cb[3], &raw_full[q]);
+                tma_load_3d(slot, &maps.a, 2 * k0, maps.a_rows_first ? m0 : ia, maps.a_rows_first ? ia : m0, &raw_full[q]);
+                tma_load_3d(slot + Cfg::RAW_A, &maps.b, 2 * k0, maps.b_rows_first ? n0 : ib, maps.b_rows_first ? ib : n0,
+                            &raw_full[q]);
             }
             __syncwarp();
             issued = c + 1;
@@ -375,8 +354,8 @@ __global__ void __launch_bounds__(ZCfg<NT, RING>::THREADS, 1)
         // Epilogue through shared memory (free once every MMA is complete): the operand warps
         // copy the accumulator tile from tensor memory (warp w: lanes 32 (w % 4) .. + 31, the
         // real columns of part (w - 1) / 4) into a padded [128][NT + 1] complex tile, meet, and
-        // write C (adding C0) a row or a column per warp and step, so that every warp store
-        // covers consecutive addresses whether C is row- or column-major.
+        // write C (adding C0) a row per warp and step, so that every warp store covers consecutive
+        // addresses.
         constexpr int parts = Cfg::NR >= 64 ? 4 : Cfg::NR / 16, cpp = Cfg::NR / parts, TS = NT + 1;
         float2 *T = reinterpret_cast<float2 *>(zg_smem_raw + (smem0 - smem_u32(zg_smem_raw)));
         const int q = warp & 3, pw = warp - Cfg::PW0, h = pw >> 2;
@@ -395,41 +374,22 @@ __global__ void __launch_bounds__(ZCfg<NT, RING>::THREADS, 1)
             }
         }
         asm volatile("bar.sync 1, %0;" ::"n"(ZG_PRODUCERS) : "memory");
-        // split parts write their partial tile (C's layout, leading dimension M or N, no C0)
+        // split parts write their partial tile (rows of N, no C0)
         const bool split = ks > 1;
-        const float2 *C0 = (!split && a.C0.base)
-                               ? a.C0.base + zop_off(task[6], a.C0.div, a.C0.stride, a.C0.stride_hi)
-                               : nullptr;
-        float2 *C = split ? a.part + (size_t)blockIdx.z * ((size_t)a.M * a.N)
-                          : a.C + zop_off(task[7], a.c_div, a.c_stride, a.c_stride_hi);
-        const long long ldc = split ? (a.c_col ? a.M : a.N) : a.ldc;
-        if (!a.c_col) {
-            for (int rr = pw; rr < ZG_BM; rr += ZG_PRODUCERS / 32) {   // row-major: a row per warp
-                const int m = m0 + rr;
-                if (m >= a.M) break;
-                for (int nn = lane; nn < NT && n0 + nn < a.N; nn += 32) {
-                    float2 out = T[rr * TS + nn];
-                    if (C0) {
-                        const float2 b = C0[(long long)m * a.C0.ld + n0 + nn];
-                        out.x += b.x;
-                        out.y += b.y;
-                    }
-                    C[(long long)m * ldc + n0 + nn] = out;
+        const float2 *C0 = (!split && a.C0.base) ? a.C0.base + task[2] * a.C0.stride : nullptr;
+        float2 *C = split ? a.part + (size_t)blockIdx.z * ((size_t)a.M * a.N) : a.C + task[3] * a.c_stride;
+        const long long ldc = split ? a.N : a.ldc;
+        for (int rr = pw; rr < ZG_BM; rr += ZG_PRODUCERS / 32) {   // a row per warp
+            const int m = m0 + rr;
+            if (m >= a.M) break;
+            for (int nn = lane; nn < NT && n0 + nn < a.N; nn += 32) {
+                float2 out = T[rr * TS + nn];
+                if (C0) {
+                    const float2 b = C0[(long long)m * a.C0.ld + n0 + nn];
+                    out.x += b.x;
+                    out.y += b.y;
                 }
-            }
-        } else {
-            for (int nn = pw; nn < NT; nn += ZG_PRODUCERS / 32) {     // column-major: a column per warp
-                const int n = n0 + nn;
-                if (n >= a.N) break;
-                for (int rr = lane; rr < ZG_BM && m0 + rr < a.M; rr += 32) {
-                    float2 out = T[rr * TS + nn];
-                    if (C0) {
-                        const float2 b = C0[(long long)n * a.C0.ld + m0 + rr];
-                        out.x += b.x;
-                        out.y += b.y;
-                    }
-                    C[(long long)n * ldc + m0 + rr] = out;
-                }
+                C[(long long)m * ldc + n0 + nn] = out;
             }
         }
     }
@@ -443,14 +403,11 @@ __global__ void __launch_bounds__(ZCfg<NT, RING>::THREADS, 1)
 // C_t = C0_t + sum over the ksplit partial tiles of task t, in part order; one thread per element
 // of C, consecutive threads along C's contiguous dimension
 __global__ void zsplit_reduce_kernel(ZGemmArgs a) {
-    if (a.skip && *a.skip) return;   // the GEMM itself was skipped
-    const int *task = a.tasks + (size_t)blockIdx.y * 8;
-    if (a.sys_frozen && a.sys_frozen[2 * (task[7] / a.sys_div)]) return;
+    const int *task = a.tasks + (size_t)blockIdx.y * 4;
     const long long mn = (long long)a.M * a.N;
     const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= mn) return;
-    const int inner = a.c_col ? a.M : a.N;   // C's contiguous dimension
-    const int i = (int)(e / inner), o = (int)(e % inner);
+    const int i = (int)(e / a.N), o = (int)(e % a.N);
     const float2 *P = a.part + (size_t)blockIdx.y * a.ksplit * mn + e;
     float2 v = P[0];
     for (int p = 1; p < a.ksplit; ++p) {
@@ -458,12 +415,12 @@ __global__ void zsplit_reduce_kernel(ZGemmArgs a) {
         v.x += w.x;
         v.y += w.y;
     }
-    if (a.C0.base && task[6] >= 0) {
-        const float2 b = a.C0.base[zop_off(task[6], a.C0.div, a.C0.stride, a.C0.stride_hi) + (long long)i * a.C0.ld + o];
+    if (a.C0.base) {
+        const float2 b = a.C0.base[task[2] * a.C0.stride + (long long)i * a.C0.ld + o];
         v.x += b.x;
         v.y += b.y;
     }
-    a.C[zop_off(task[7], a.c_div, a.c_stride, a.c_stride_hi) + (long long)i * a.ldc + o] = v;
+    a.C[task[3] * a.c_stride + (long long)i * a.ldc + o] = v;
 }
 
 using EncodeTiledFn = CUresult (*)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *,
@@ -488,39 +445,32 @@ EncodeTiledFn tensor_map_encoder() {
 // Tensor map of a family of R x K complex matrices (see ZMaps) with boxes of 32 floats x
 // box_rows rows; false if the family cannot be described (unknown count, strides that are not
 // multiples of 16 bytes) or the encoder refuses it.
-bool encode_family(CUtensorMap *m, int8_t pos[3], const ZOperand &o, int R, int K, int box_rows) {
+bool encode_family(CUtensorMap *m, bool *rows_first, const ZOperand &o, int R, int K, int box_rows) {
     const EncodeTiledFn enc = tensor_map_encoder();
     if (!enc || !o.base || o.count <= 0 || o.ld < K) return false;
-    struct Dim { unsigned long long ext, stride; int role; };
-    Dim d[3];
-    d[0] = {(unsigned long long)R, (unsigned long long)o.ld * 8ull, 0};
-    if (o.div > 0) {
-        d[1] = {(unsigned long long)o.div, (unsigned long long)o.stride * 8ull, 1};
-        d[2] = {(unsigned long long)o.count, (unsigned long long)o.stride_hi * 8ull, 2};
-    } else {
-        d[1] = {(unsigned long long)o.count, (unsigned long long)o.stride * 8ull, 1};
-        d[2] = {1ull, 0ull, 2};
-    }
-    // dimensions of one element last, the others by increasing stride; a dimension of one
-    // element takes the stride that nests it after the previous one
-    std::stable_sort(d, d + 3, [](const Dim &x, const Dim &y) {
+    struct Dim { unsigned long long ext, stride; bool rows; };
+    Dim d[2] = {{(unsigned long long)R, (unsigned long long)o.ld * 8ull, true},
+                {(unsigned long long)o.count, (unsigned long long)o.stride * 8ull, false}};
+    // a dimension of one element last, else by increasing stride; a dimension of one element takes the
+    // stride that nests it after the previous one
+    std::stable_sort(d, d + 2, [](const Dim &x, const Dim &y) {
         if ((x.ext == 1) != (y.ext == 1)) return y.ext == 1;
         return x.stride < y.stride;
     });
-    cuuint64_t dims[4] = {(cuuint64_t)2 * K, 0, 0, 0}, strides[3];
-    cuuint32_t box[4] = {32, 1, 1, 1}, estr[4] = {1, 1, 1, 1};
+    cuuint64_t dims[3] = {(cuuint64_t)2 * K, 0, 0}, strides[2];
+    cuuint32_t box[3] = {32, 1, 1}, estr[3] = {1, 1, 1};
     unsigned long long prev = (unsigned long long)2 * K * 4, prev_ext = 1;
-    for (int i = 0; i < 3; ++i) {
+    for (int i = 0; i < 2; ++i) {
         unsigned long long st = d[i].ext == 1 ? prev * prev_ext : d[i].stride;
         if (st == 0 || (st & 15) || st >= (1ull << 40) || d[i].ext > (1ull << 32)) return false;
         dims[i + 1] = d[i].ext;
         strides[i] = st;
-        if (d[i].role == 0) box[i + 1] = (cuuint32_t)box_rows;
-        pos[d[i].role] = (int8_t)(i + 1);
+        if (d[i].rows) box[i + 1] = (cuuint32_t)box_rows;
         prev = st;
         prev_ext = d[i].ext;
     }
-    return enc(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, const_cast<float2 *>(o.base), dims, strides, box, estr,
+    *rows_first = d[0].rows;
+    return enc(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, const_cast<float2 *>(o.base), dims, strides, box, estr,
                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
@@ -531,7 +481,7 @@ template <int NT, bool RING> cudaError_t launch_nt(const ZGemmArgs &a, const ZMa
     cudaError_t e = ensure_dyn_smem(fn, Cfg::SMEM);
     if (e != cudaSuccess) return e;
     // split-K where the launch fills at most half of the SMs: as many parts as keep it within one
-    // wave, at most one part per K chunk of a term, within the partial buffer
+    // wave, at most one part per K chunk, within the partial buffer
     ZGemmArgs b = a;
     b.ksplit = 1;
     const long long tiles = (long long)((a.M + ZG_BM - 1) / ZG_BM) * ((a.N + NT - 1) / NT) * n_tasks;
@@ -559,10 +509,8 @@ template <int NT, bool RING> cudaError_t launch_nt(const ZGemmArgs &a, const ZMa
 // register path
 template <int NT> cudaError_t launch_narrow(const ZGemmArgs &a, int n_tasks, cudaStream_t st) {
     ZMaps maps{};
-    bool ring = true;
-    for (int u = 0; ring && u < a.nterms; ++u)
-        ring = encode_family(&maps.a[u], maps.apos[u], a.A[u], a.M, a.K, ZG_BM) &&
-               encode_family(&maps.b[u], maps.bpos[u], a.B[u], a.N, a.K, NT);
+    const bool ring = encode_family(&maps.a, &maps.a_rows_first, a.A, a.M, a.K, ZG_BM) &&
+                      encode_family(&maps.b, &maps.b_rows_first, a.B, a.N, a.K, NT);
     return ring ? launch_nt<NT, true>(a, maps, n_tasks, st) : launch_nt<NT, false>(a, maps, n_tasks, st);
 }
 
@@ -582,13 +530,11 @@ int device_sms() {
 
 cudaError_t launch_zgemm(const ZGemmArgs &a, int n_tasks, cudaStream_t st) {
     if (n_tasks <= 0) return cudaSuccess;
-    if (a.M <= 0 || a.N <= 0 || a.K <= 0 || (a.K & 1) || a.nterms < 1 || a.nterms > 3 || n_tasks > 65535)
+    if (a.M <= 0 || a.N <= 0 || a.K <= 0 || (a.K & 1) || n_tasks > 65535) return cudaErrorInvalidValue;
+    // 16-byte operand loads: even leading dimensions and offsets
+    if ((a.A.ld & 1) || (a.B.ld & 1) || (a.A.stride & 1) || (a.B.stride & 1) || ((uintptr_t)a.A.base & 15) ||
+        ((uintptr_t)a.B.base & 15))
         return cudaErrorInvalidValue;
-    for (int u = 0; u < a.nterms; ++u)   // 16-byte operand loads: even leading dimensions and offsets
-        if ((a.A[u].ld & 1) || (a.B[u].ld & 1) || (a.A[u].stride & 1) || (a.B[u].stride & 1) ||
-            (a.A[u].stride_hi & 1) || (a.B[u].stride_hi & 1) || ((uintptr_t)a.A[u].base & 15) ||
-            ((uintptr_t)a.B[u].base & 15))
-            return cudaErrorInvalidValue;
     if (a.N <= 16) return launch_narrow<16>(a, n_tasks, st);
     if (a.N <= 32) return launch_narrow<32>(a, n_tasks, st);
     if (a.N <= 64) return launch_narrow<64>(a, n_tasks, st);
