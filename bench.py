@@ -381,15 +381,15 @@ def server_session(args):
 
 # ------------------------------------------------------ tensor-core GEMM alone
 
-GEMM_SHAPES = {   # (batch, M, N, K): the two shapes of the mixed workload's block products
-    "factor_256x256x256": (256, 256, 256, 256),     # Schur updates of a factor level
-    "solve_256x64x256": (1024, 256, 64, 256),       # one level-0 pass of the solve: 8 freq x 128 lines
+GEMM_SHAPES = {   # (batch, M, N, K): one wide and one narrow shape of the size of the mixed workload's blocks
+    "factor_256x256x256": (256, 256, 256, 256),     # (whose own products are bcr_gemm's and bcr_solve's)
+    "solve_256x64x256": (1024, 256, 64, 256),
 }
 
 
 def gemm_kernel_bench(hm, torch, peaks, reps=10):
-    """helm_zgemm_batched on its own at the workload's two product shapes (operands larger
-    than L2): useful TFLOP/s (8 M N K per complex product), the tensor pipe's issued rate (three
+    """helm_zgemm_batched on its own, square and with 64 columns, on blocks of 256 (operands larger
+    than L2; the workload's products run on FP16 pairs, bcr_gemm and bcr_solve): useful TFLOP/s (8 M N K per complex product), the tensor pipe's issued rate (three
     TF32 products per useful one) against the measured tensor peak, and the operand bytes'
     GB/s against the measured HBM bandwidth."""
     out = {}

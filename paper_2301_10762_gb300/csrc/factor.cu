@@ -316,7 +316,7 @@ __device__ void polish_inverse16(const float2 *M, int ld, int kb, float2 *P, flo
 
 // FP64 inverse of the kb x kb block M (shared, row stride ld; the rest of the 16 x 16 tile taken as
 // the identity) into P (row stride NB) by the 256 threads of the CTA, thread (r, c) holding one
-// entry: Gauss-Jordan in place with partial pivoting, A (16 x 17) and B ping-pong, two barriers a
+// entry: Gauss-Jordan in place with partial pivoting, A (16 x 17) and B ping-pong, one barrier a
 // column.  Bounds: about 1100 cycles a column, half of them the FP64 pipe (8 instructions of every
 // warp at 2 lanes a cycle).  One warp holding the block in registers took 270 us a block (the
 // 128^2 factor 163 ms for three frequencies): half a lane a cycle, sixteen columns of eight
