@@ -856,17 +856,67 @@ cudaError_t launch_line_sweep(const GridGeom &g, int n_sys, int nrhs, const cx_t
     int cs = nz / 16;
     cs = cs < 1 ? 1 : (cs > 16 / teams ? 16 / teams : cs);
     const bool fp64 = sizeof(TG) == 8;
+    // threads per output (K split): as many as fit the CTA's 256 threads twice over
+    auto tpo_of = [&](int rpc, int R) {
+        int t = 1;
+        while (t < 8 && rpc * R * t * 2 <= SW_THREADS) t *= 2;
+        return t;
+    };
+    auto smem_of = [&](int rpc, int R, bool pf) {
+        const int t = tpo_of(rpc, R);
+        const size_t nzp = (size_t)padded<TG>(nz, t), kcp = (size_t)padded<TG>(SW_KC, t);
+        return (size_t)32 + vsz * 5 * (size_t)R * nzp + (pf ? vsz * 2 * (size_t)rpc * nzp : vsz * (size_t)rpc * kcp) +
+               vsz * 2 * (size_t)R * rpc;
+    };
+    // R right-hand sides a cluster, or as many as fit, with the slab where it fits with four
+    auto fit = [&](int rpc, int R) -> SweepFit {
+        R = std::max(1, std::min(R, nrhs));
+        while (R > 1 && rpc * R > SW_MAXOPT * SW_THREADS) R = (R + 1) / 2;
+        bool pf = true;
+        while (smem_of(rpc, R, pf) > SW_SMEM_MAX) {
+            if (pf && R <= 4) pf = false;
+            else if (R > 1) R = (R + 1) / 2;
+            else return SweepFit{0, false, 1, 0};
+        }
+        return SweepFit{R, pf, tpo_of(rpc, R), smem_of(rpc, R, pf)};
+    };
+    // right-hand sides per cluster (the chain is latency bound and the GPU otherwise
+    // idle, so more clusters with fewer outputs each; 128 outputs per CTA measured best)
+    auto usual_R = [&](int rpc) {
+        int R = 1;
+        while (R * 2 <= 16 && rpc * R * 2 <= 128) R *= 2;
+        return rchunk > 0 && R > rchunk ? rchunk : R;
+    };
     int fp64_R = 0;
     if (fp64) {
-        const SweepShape sh = sweep_shape_fp64(nz, teams, n_sys, nrhs, cs, [&](int c, int r) {
-            // (shared memory at the widest padding, in steps of 32 KB: few distinct queries)
-            const int rp = (nz + c - 1) / c;
-            const size_t need = 32 + vsz * (size_t)(nz + 8) * (5 * r + 2 * rp) + vsz * 2 * (size_t)r * rp;
-            return max_active_clusters((const void *)line_sweep_kernel<TG, 0, 0, false>, teams * c, SW_THREADS,
-                                       std::min(SW_SMEM_MAX, (need + 32767) / 32768 * 32768));
-        });
-        cs = sh.cs;
-        fp64_R = sh.R;
+        // (the search takes about 10 us of the host: the thread's last one is kept)
+        static thread_local struct {
+            int dev = -1, nz, teams, n_sys, nrhs;
+            SweepShape s;
+        } memo;
+        int dev = 0;
+        cudaError_t es = cudaGetDevice(&dev);
+        if (es != cudaSuccess) return es;
+        if (memo.dev != dev || memo.nz != nz || memo.teams != teams || memo.n_sys != n_sys || memo.nrhs != nrhs) {
+            const void *fn = (const void *)line_sweep_kernel<TG, 0, 0, false>;
+            if ((es = ensure_dyn_smem(fn, SW_SMEM_MAX)) != cudaSuccess) return es;   // (for the queries)
+            memo.s = sweep_shape_fp64(
+                nz, teams, n_sys, nrhs, SweepShape{cs, usual_R((nz + cs - 1) / cs)},
+                [&](int c) {   // (one, two and three CTAs per SM by their shared memory)
+                    SweepActive a;
+                    const size_t kb[kSweepMaxPerSm] = {120, 100, 60};
+                    for (int k = 0; k < kSweepMaxPerSm; ++k) a.n[k] = max_active_clusters(fn, teams * c, SW_THREADS, kb[k] * 1024);
+                    return a;
+                },
+                [&](int c, int R) { return fit((nz + c - 1) / c, R); });
+            memo.dev = dev;
+            memo.nz = nz;
+            memo.teams = teams;
+            memo.n_sys = n_sys;
+            memo.nrhs = nrhs;
+        }
+        cs = memo.s.cs;
+        fp64_R = memo.s.R;
     }
     // tuning overrides: CTAs per team and right-hand sides per cluster
     const char *env_cs = getenv("HELM_SWEEP_CS"), *env_r = getenv("HELM_SWEEP_R");
@@ -881,36 +931,14 @@ cudaError_t launch_line_sweep(const GridGeom &g, int n_sys, int nrhs, const cx_t
     for (;;) {
         cs = sweep_filled_ctas(nz, cs);
         const int rpc = (nz + cs - 1) / cs;
-        // threads per output (K split): as many as fit the CTA's 256 threads twice over
-        auto tpo_of = [&](int R) {
-            int t = 1;
-            while (t < 8 && rpc * R * t * 2 <= SW_THREADS) t *= 2;
-            return t;
-        };
-        auto smem_of = [&](int R, int pf) {
-            const size_t nzp = (size_t)padded<TG>(nz, tpo_of(R)), kcp = (size_t)padded<TG>(SW_KC, tpo_of(R));
-            return (size_t)32 + vsz * 5 * (size_t)R * nzp + (pf ? vsz * 2 * (size_t)rpc * nzp : vsz * (size_t)rpc * kcp) +
-                   vsz * 2 * (size_t)R * rpc;
-        };
-        // right-hand sides per cluster (the chain is latency bound and the GPU otherwise
-        // idle, so more clusters with fewer outputs each; 128 outputs per CTA measured best)
-        int R = 1;
-        while (R * 2 <= 16 && rpc * R * 2 <= 128) R *= 2;
-        if (rchunk > 0 && R > rchunk) R = rchunk;
-        if (fp64 && fp64_R > 0) R = fp64_R;
+        int R = fp64_R > 0 ? fp64_R : usual_R(rpc);
         if (env_r && atoi(env_r) > 0) R = atoi(env_r);
-        if (R > nrhs) R = nrhs;
-        if (R < 1) R = 1;
-        while (R > 1 && rpc * R > SW_MAXOPT * SW_THREADS) R = (R + 1) / 2;
-        int pf = 1;
-        while (smem_of(R, pf) > SW_SMEM_MAX) {
-            if (pf && R <= 4) pf = 0;
-            else if (R > 1) R = (R + 1) / 2;
-            else if (pf) pf = 0;
-            else return cudaErrorInvalidConfiguration;
-        }
-        size_t smem = smem_of(R, pf);
-        int tpo = tpo_of(R);
+        const SweepFit ft = fit(rpc, R);
+        if (ft.R == 0) return cudaErrorInvalidConfiguration;
+        R = ft.R;
+        int pf = ft.slab ? 1 : 0;
+        size_t smem = ft.smem;
+        int tpo = ft.tpo;
         SweepFn<TG> kfn = line_sweep_kernel<TG, 0, 0, false>;
         bool mma = false;
         // tensor-pipe product: complex FP32, even n_z (16-byte fragment loads), at most two m
