@@ -116,10 +116,32 @@ __global__ void split_diag_kernel(size_t n, const double2 *diag, float4 *diag2) 
     }
 }
 
-// Nodes of a column are taken by warps as groups of 32 consecutive nodes of a line (ng = ceil(nz /
-// 32) groups a line, lanes beyond the line idle), so that the group's maximum, which the block
-// cyclic reduction scales its operands by (bcr_solve.cu), is one warp reduction here instead of
-// another pass over the vector (0.05 ms of a 256^2 sweep with 512 columns).
+// Nodes of a column are taken by warps as groups of 32.  For the block cyclic reduction they are groups
+// of a line (ng = ceil(nz / 32) of them, lanes beyond the line idle), so that the group's maximum, by which
+// its solve scales its operands (bcr_solve.cu), is one warp reduction here instead of another pass over
+// the vector (0.05 ms of a 256^2 sweep with 512 columns).  For the line factor (FLAT) they run on across
+// lines: short ones would leave most lanes idle (10 nodes a line, 7 x 79 columns: a solve 473 us, 559 by
+// lines).
+struct RefineItem {
+    int line, grp, j;
+    bool on;
+};
+template <bool FLAT> __device__ __forceinline__ RefineItem refine_item(int it, int lane, int nz, int ng, int N) {
+    RefineItem r;
+    if (FLAT) {
+        const int k = 32 * it + lane;
+        r.line = k / nz;
+        r.j = k - r.line * nz;
+        r.grp = 0;
+        r.on = k < N;
+    } else {
+        r.line = it / ng;
+        r.grp = it - r.line * ng;
+        r.j = 32 * r.grp + lane;
+        r.on = r.j < nz;
+    }
+    return r;
+}
 struct RefineVec {
     float *gmax;      // maxima of r: [sys][line][ng][nrhs] (null: not wanted)
     unsigned *ctl;    // the solve's counters, zeroed for the next solve (null: none)
@@ -134,11 +156,11 @@ __device__ __forceinline__ void group_max(const RefineVec &rv, float2 r, bool on
 }
 
 // grid: (blocks of 8 * NPT groups, columns)
-template <int NPT>
+template <int NPT, bool FLAT>
 __global__ void __launch_bounds__(RF_THREADS) refine_start_kernel(GridGeom g, int nrhs, int cols, const double2 *B, int conj,
                                                                   float4 *bd, float2 *r32, double *norms, RefineVec rv) {
     __shared__ double sh[RF_THREADS / 32];
-    const int nz = g.nz, N = g.nx * nz, ng = (nz + 31) >> 5, items = g.nx * ng;
+    const int nz = g.nz, N = g.nx * nz, ng = (nz + 31) >> 5, items = FLAT ? (N + 31) >> 5 : g.nx * ng;
     const int lane = threadIdx.x & 31, i0 = blockIdx.x * (RF_THREADS / 32) * NPT + (threadIdx.x >> 5);
     if (blockIdx.x == 0 && blockIdx.y == 0 && rv.ctl)
         for (int e = threadIdx.x; e < rv.n_ctl; e += RF_THREADS) rv.ctl[e] = 0u;
@@ -148,14 +170,17 @@ __global__ void __launch_bounds__(RF_THREADS) refine_start_kernel(GridGeom g, in
         double2 b[NPT];
 #pragma unroll
         for (int q = 0; q < NPT; ++q) {   // all loads first: NPT in flight per thread
-            const int it = i0 + q * (RF_THREADS / 32), line = it / ng, j = 32 * (it - line * ng) + lane;
-            b[q] = it < items && j < nz ? __ldcs(B + base + (size_t)line * nz + j) : make_double2(0.0, 0.0);
+            const int it = i0 + q * (RF_THREADS / 32);
+            const RefineItem r = refine_item<FLAT>(it, lane, nz, ng, N);
+            b[q] = it < items && r.on ? __ldcs(B + base + (size_t)r.line * nz + r.j) : make_double2(0.0, 0.0);
         }
 #pragma unroll
         for (int q = 0; q < NPT; ++q) {
-            const int it = i0 + q * (RF_THREADS / 32), line = it / ng, grp = it - line * ng, j = 32 * grp + lane;
+            const int it = i0 + q * (RF_THREADS / 32);
             if (it >= items) break;   // (uniform in the warp)
-            const bool on = j < nz;
+            const RefineItem ri = refine_item<FLAT>(it, lane, nz, ng, N);
+            const int line = ri.line, grp = ri.grp, j = ri.j;
+            const bool on = ri.on;
             float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
             if (on) {
                 const size_t k = base + (size_t)line * nz + j;
@@ -168,9 +193,10 @@ __global__ void __launch_bounds__(RF_THREADS) refine_start_kernel(GridGeom g, in
                 // (the zeros of point sources skip the FP64 arithmetic, tested on the bits)
                 if (((ps_bits64(v2.x) | ps_bits64(v2.y)) << 1) != 0) bb += v2.x * v2.x + v2.y * v2.y;
             }
-            if (j == nz && rv.ld > nz) r32[((size_t)c * g.nx + line) * rv.ld + j] = make_float2(0.f, 0.f);
-            group_max(rv, make_float2(v.x, v.y), on,
-                      (((size_t)(c / nrhs) * g.nx + line) * ng + grp) * nrhs + c % nrhs, lane);
+            if (!FLAT && j == nz && rv.ld > nz) r32[((size_t)c * g.nx + line) * rv.ld + j] = make_float2(0.f, 0.f);
+            if (!FLAT)
+                group_max(rv, make_float2(v.x, v.y), on,
+                          (((size_t)(c / nrhs) * g.nx + line) * ng + grp) * nrhs + c % nrhs, lane);
         }
         bb = block_sum(bb, sh);
         if (threadIdx.x == 0) {
@@ -242,7 +268,7 @@ __device__ void refine_stop_test(int cols, int nrhs, double *norms, RefineStop s
 // grid: (blocks of 8 * NPT groups, columns); norms[col][0] pre-zeroed, norms[col][1] = ||b||^2
 // (the arrays are distinct: __restrict__ lets the loads of later nodes move above the stores of
 // earlier ones, so that several nodes' loads are in flight)
-template <int NPT>
+template <int NPT, bool FLAT>
 __global__ void __launch_bounds__(RF_THREADS) refine_update_kernel(GridGeom g, int nrhs, int cols,
                                                                    const float4 *__restrict__ diag2,
                                                                    const float4 *__restrict__ bd,
@@ -256,7 +282,7 @@ __global__ void __launch_bounds__(RF_THREADS) refine_update_kernel(GridGeom g, i
     __shared__ int s_last;
     __shared__ double shd[32];
     if (state && state->done) return;   // the refinement has stopped: later passes do nothing
-    const int nx = g.nx, nz = g.nz, N = nx * nz, ng = (nz + 31) >> 5, items = nx * ng;
+    const int nx = g.nx, nz = g.nz, N = nx * nz, ng = (nz + 31) >> 5, items = FLAT ? (N + 31) >> 5 : nx * ng;
     const int lane = threadIdx.x & 31, i0 = blockIdx.x * (RF_THREADS / 32) * NPT + (threadIdx.x >> 5);
     const int *sysflags = state ? refine_sys(state) : nullptr;
     for (int c = blockIdx.y; c < cols; c += gridDim.y) {
@@ -276,9 +302,11 @@ __global__ void __launch_bounds__(RF_THREADS) refine_update_kernel(GridGeom g, i
         float2 *__restrict__ rc = r32 + (size_t)c * nx * rv.ld;
 #pragma unroll (NPT < 4 ? NPT : 4)
         for (int q = 0; q < NPT; ++q) {
-            const int it = i0 + q * (RF_THREADS / 32), i = it / ng, grp = it - i * ng, j = 32 * grp + lane;
+            const int it = i0 + q * (RF_THREADS / 32);
             if (it >= items) break;   // (uniform in the warp)
-            const bool on = j < nz;
+            const RefineItem ri = refine_item<FLAT>(it, lane, nz, ng, N);
+            const int i = ri.line, grp = ri.grp, j = ri.j;
+            const bool on = ri.on;
             float2 rf = make_float2(0.f, 0.f);
             if (on) {
                 const int k = i * nz + j, kd = i * rv.ld + j;
@@ -300,8 +328,8 @@ __global__ void __launch_bounds__(RF_THREADS) refine_update_kernel(GridGeom g, i
                 const float sr = r.re.hi * scale, si = r.im.hi * scale;
                 rr = fmaf(sr, sr, fmaf(si, si, rr));
             }
-            if (j == nz && rv.ld > nz) rc[i * rv.ld + j] = make_float2(0.f, 0.f);
-            group_max(rv, rf, on, (((size_t)sys * nx + i) * ng + grp) * nrhs + (c - sys * nrhs), lane);
+            if (!FLAT && j == nz && rv.ld > nz) rc[i * rv.ld + j] = make_float2(0.f, 0.f);
+            if (!FLAT) group_max(rv, rf, on, (((size_t)sys * nx + i) * ng + grp) * nrhs + (c - sys * nrhs), lane);
         }
         rr = block_sum(rr, shf);
         if (threadIdx.x == 0) atomicAdd(norms + 2 * (size_t)c, ldexp((double)rr, 2 * ks));
@@ -377,24 +405,27 @@ cudaError_t launch_split_diag(size_t n, const double2 *diag, float4 *diag2, cuda
     return cudaGetLastError();
 }
 
-// groups per thread of the per-column kernels: 8 where that still gives several blocks per SM,
-// else 2 (128^2 with 48 columns: 384 blocks of 8 took 27 us an update, 1536 of 2 are below 20)
-static int refine_npt(const GridGeom &g, int cols) {
-    const long long items = (long long)g.nx * ((g.nz + 31) / 32);
-    return (items + 63) / 64 * cols >= 8 * 152 ? 8 : 2;
+// groups of a column (flat: they run on across lines), and groups per thread of the per-column
+// kernels: 8 where that still gives several blocks per SM, else 2 (128^2 with 48 columns: 384 blocks of 8
+// took 27 us an update, 1536 of 2 are below 20)
+static int refine_items(const GridGeom &g, bool flat) {
+    return flat ? (g.nx * g.nz + 31) / 32 : g.nx * ((g.nz + 31) / 32);
 }
-static dim3 refine_grid(const GridGeom &g, int cols, int npt) {
-    const int items = g.nx * ((g.nz + 31) / 32), per = RF_THREADS / 32 * npt;
+static int refine_npt(int items, int cols) { return (long long)((items + 63) / 64) * cols >= 8 * 152 ? 8 : 2; }
+static dim3 refine_grid(int items, int cols, int npt) {
+    const int per = RF_THREADS / 32 * npt;
     return dim3((items + per - 1) / per, std::min(cols, 65535));
 }
 
 cudaError_t launch_refine_start(const GridGeom &g, int n_sys, int nrhs, const double2 *B, int conj, float4 *bd, float2 *r32,
                                 double *norms, int ld, float *gmax, unsigned *ctl, int n_ctl, cudaStream_t st) {
-    const int cols = n_sys * nrhs, npt = refine_npt(g, cols);
-    const dim3 grid = refine_grid(g, cols, npt);
+    const bool flat = !gmax && ld == g.nz;
+    const int cols = n_sys * nrhs, items = refine_items(g, flat), npt = refine_npt(items, cols);
+    const dim3 grid = refine_grid(items, cols, npt);
     const RefineVec rv{gmax, ctl, n_ctl, ld};
-    HELM_TRACED(K_REFSTART, st, ((npt == 8 ? refine_start_kernel<8> : refine_start_kernel<2>)<<<grid, RF_THREADS, 0, st>>>(
-                                    g, nrhs, cols, B, conj, bd, r32, norms, rv)));
+    auto kern = flat ? (npt == 8 ? refine_start_kernel<8, true> : refine_start_kernel<2, true>)
+                     : (npt == 8 ? refine_start_kernel<8, false> : refine_start_kernel<2, false>);
+    HELM_TRACED(K_REFSTART, st, (kern<<<grid, RF_THREADS, 0, st>>>(g, nrhs, cols, B, conj, bd, r32, norms, rv)));
     return cudaGetLastError();
 }
 
@@ -402,13 +433,15 @@ cudaError_t launch_refine_update(const GridGeom &g, int n_sys, int nrhs, const f
                                  const float4 *x_in, const float2 *delta, float4 *x_out, float2 *r32, double *norms,
                                  int ld, float *gmax, unsigned *ctl, int n_ctl, const int *solve_status, cudaStream_t st,
                                  RefineState *state, RefineStop stop) {
-    const int cols = n_sys * nrhs, npt = refine_npt(g, cols);
-    const dim3 grid = refine_grid(g, cols, npt);
+    const bool flat = !gmax && ld == g.nz;
+    const int cols = n_sys * nrhs, items = refine_items(g, flat), npt = refine_npt(items, cols);
+    const dim3 grid = refine_grid(items, cols, npt);
     const RefineVec rv{gmax, ctl, n_ctl, ld};
+    auto kern = flat ? (npt == 8 ? refine_update_kernel<8, true> : refine_update_kernel<2, true>)
+                     : (npt == 8 ? refine_update_kernel<8, false> : refine_update_kernel<2, false>);
     StencilPairs cp{pair_of(coup_x(g, 1)), pair_of(coup_x(g, 0)), pair_of(coup_z(g, 1)), pair_of(coup_z(g, 0))};
-    HELM_TRACED(K_REFUPDATE, st, ((npt == 8 ? refine_update_kernel<8> : refine_update_kernel<2>)<<<grid, RF_THREADS, 0, st>>>(
-                                     g, nrhs, cols, diag2, bd, x_in, delta, x_out, r32, norms, cp, state, stop, rv,
-                                     solve_status)));
+    HELM_TRACED(K_REFUPDATE, st, (kern<<<grid, RF_THREADS, 0, st>>>(g, nrhs, cols, diag2, bd, x_in, delta, x_out, r32, norms, cp,
+                                                                   state, stop, rv, solve_status)));
     return cudaGetLastError();
 }
 

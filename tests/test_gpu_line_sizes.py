@@ -48,3 +48,19 @@ def test_fp64_sweep_teams_without_idle_ctas(nx, nz, nrhs, teams, monkeypatch):
     op, B, ref = _case(nx, nz, 1, nrhs)
     f = hm.helm_factor(op, hm.HELM_FP64)
     assert _error(hm.helm_solve(f, torch.tensor(B, device="cuda"))[0], ref) <= 1e-9
+
+
+@pytest.mark.parametrize("nx,nz,n_omega,nrhs", [(4, 4, 1, 1), (119, 10, 2, 79), (7, 5, 3, 2), (33, 31, 1, 40), (40, 33, 2, 3), (64, 64, 2, 64)])
+def test_refinement_runs_on_across_short_lines(nx, nz, n_omega, nrhs):
+    """The line factor's refinement takes groups of 32 nodes across lines, 2 or 8 of them a thread: columns
+    that end within a group, both thread counts, the adjoint and the working-array solve.  Mixed bar 1e-8."""
+    op, B, ref = _case(nx, nz, n_omega, nrhs)
+    f = hm.helm_factor(op, hm.HELM_MIXED, method=hm.HELM_FACTOR_LINE)
+    Bd = torch.tensor(B, device="cuda")
+    assert _error(hm.helm_solve(f, Bd, rtol=1e-12, max_iter=20)[0], ref) <= 1e-8
+    X = hm.helm_adjoint_solve(f, Bd.conj().resolve_conj(), rtol=1e-12, max_iter=20)[0]   # A^H conj(x) = conj(b)
+    assert _error(X.conj().resolve_conj(), ref) <= 1e-8
+    one = Bd[:, :1].contiguous()
+    Y = torch.empty_like(one)
+    hm.helm_solve_noalloc(f, one, Y, rtol=1e-12, max_iter=20)
+    assert _error(Y, ref[:, :1]) <= 1e-8
