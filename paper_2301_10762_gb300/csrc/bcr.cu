@@ -357,11 +357,19 @@ struct InvArgs {
 // The chain of pivot blocks is what bounds it, so it runs ahead of the rest: warps 0 to 7 update the
 // next pivot block W[K1, K1] first and warp 0 inverts it while the other warps form R',
 // the tensor core multiplies and W is updated.
-constexpr int ZT_THREADS = 512;
-constexpr int ZT_WS = 129, ZT_PS = 17;   // row strides (complex) of the pivot rows and of the 16 x 16 blocks
-constexpr int ZT_TS = 65;                // row stride (complex) of half a block on its way in or out
-constexpr uint32_t ZT_A = 0, ZT_B = 32768, ZT_WK = 98304, ZT_P = ZT_WK + 8 * PIV * ZT_WS, ZT_BLK = ZT_P + 2 * 8 * PIV * PIV;
-constexpr size_t ZT_SMEM = ZT_BLK + 4 * 8 * PIV * ZT_PS + 1024;
+// H groups of 32 columns: four, or two for n <= 64 (256 threads and 86 KB, so that two CTAs share an SM and
+// hide each other's chain: 1000 blocks of 16 take 44 us, of 30 81, of 64 143; with four groups 80, 142 and
+// 233; a wave of them 14, 23 and 34 us against 16, 25 and 38).
+constexpr int ZT_PS = 17;   // row stride (complex) of the 16 x 16 blocks
+constexpr int ZT_TS = 65;   // row stride (complex) of 64 columns on their way in or out
+template <int H> struct ZtCfg {
+    static constexpr int WARPS = 4 * H, THREADS = 32 * WARPS;
+    static constexpr int WS = 32 * H + 1;   // row stride (complex) of the pivot rows
+    static constexpr uint32_t A = 0, B = 32768, B_BYTES = 8192 * H, WK = B + 2 * B_BYTES, P = WK + 8 * PIV * WS,
+                              BLK = P + 2 * 8 * PIV * PIV;
+    static constexpr size_t SMEM = BLK + 4 * 8 * PIV * ZT_PS + 1024;
+    static constexpr uint32_t TMEM = 64 * H;
+};
 
 // 16 x 16 inverse in place by one warp: lane (r, h) holds row r, columns 8 h .. + 7 of M (shared, row
 // stride ZT_PS); P row stride 16.  Gauss-Jordan with partial pivoting without row swaps: at step
@@ -411,7 +419,9 @@ __device__ bool warp_invert16_inplace(const float2 *M, float2 *P) {
     return ok;
 }
 
-__global__ void __launch_bounds__(ZT_THREADS, 1) zinv_kernel(InvArgs a) {
+template <int H> __global__ void __launch_bounds__(ZtCfg<H>::THREADS, 4 / H) zinv_kernel(InvArgs a) {
+    using Cfg = ZtCfg<H>;
+    constexpr int ZT_WS = Cfg::WS;
     extern __shared__ __align__(16) unsigned char zt_smem[];
     __shared__ __align__(8) uint64_t mma_bar;
     __shared__ uint32_t s_tmem;
@@ -421,12 +431,12 @@ __global__ void __launch_bounds__(ZT_THREADS, 1) zinv_kernel(InvArgs a) {
     const int q = warp & 3, h = warp >> 2, r = 32 * q + lane, lr = lane & 15, lh = lane >> 4;
     const uint32_t base = (smem_u32(zt_smem) + 1023u) & ~1023u;
     unsigned char *gbase = zt_smem + (base - smem_u32(zt_smem));
-    float2 *Wk = reinterpret_cast<float2 *>(gbase + ZT_WK);      // [16][ZT_WS]: the pivot rows
-    float2 *Pb = reinterpret_cast<float2 *>(gbase + ZT_P);       // [2][16][16]: the pivot block's inverse, of even and odd steps
-    float2 *Nd = reinterpret_cast<float2 *>(gbase + ZT_BLK);     // [16][ZT_PS] each: W[K1, K1],
+    float2 *Wk = reinterpret_cast<float2 *>(gbase + Cfg::WK);      // [16][ZT_WS]: the pivot rows
+    float2 *Pb = reinterpret_cast<float2 *>(gbase + Cfg::P);       // [2][16][16]: the pivot block's inverse, of even and odd steps
+    float2 *Nd = reinterpret_cast<float2 *>(gbase + Cfg::BLK);     // [16][ZT_PS] each: W[K1, K1],
     float2 *Un = Nd + PIV * ZT_PS, *Rn = Un + PIV * ZT_PS;       // W[K1, K] and R'[:, K1] of the next block,
     float2 *Sn = Rn + PIV * ZT_PS;                               // and the next pivot block
-    const uint32_t a_hi = base + ZT_A, a_lo = a_hi + 16384, b_hi = base + ZT_B, b_lo = b_hi + 32768;
+    const uint32_t a_hi = base + Cfg::A, a_lo = a_hi + 16384, b_hi = base + Cfg::B, b_lo = b_hi + Cfg::B_BYTES;
     float2 *X = a.X + a.idx[blockIdx.x] * a.stride;
     if (tid == 0) {
         s_bad = 0;
@@ -435,7 +445,7 @@ __global__ void __launch_bounds__(ZT_THREADS, 1) zinv_kernel(InvArgs a) {
     }
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&s_tmem)),
-                     "r"(256u)
+                     "r"(Cfg::TMEM)
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
@@ -443,10 +453,10 @@ __global__ void __launch_bounds__(ZT_THREADS, 1) zinv_kernel(InvArgs a) {
     float2 *T = reinterpret_cast<float2 *>(gbase);
     float2 w[32];
 #pragma unroll 1
-    for (int half = 0; half < 2; ++half) {
+    for (int half = 0; half < H / 2; ++half) {
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            const int rr = 8 * warp + i;
+        for (int i = 0; i < 128 / Cfg::WARPS; ++i) {
+            const int rr = 128 / Cfg::WARPS * warp + i;
 #pragma unroll
             for (int e = 0; e < 2; ++e) {
                 const int c = 64 * half + 32 * e + lane;
@@ -545,8 +555,8 @@ __global__ void __launch_bounds__(ZT_THREADS, 1) zinv_kernel(InvArgs a) {
             // (c) R' and the expanded B tiles: 32 columns c and u = 2j, 2j + 1 at a time; B row 2c = (Re,
             // -Im), row 2c + 1 = (Im, Re) of R'[u][c], split into hi and lo
 #pragma unroll 1
-            for (int it = warp - 1; it < 32; it += 15) {
-                const int c = 32 * (it & 3) + lane, j = it >> 2;
+            for (int it = warp - 1; it < 8 * H; it += Cfg::WARPS - 1) {
+                const int c = 32 * (it % H) + lane, j = it / H;
                 if (c >= np) continue;
                 float2 x0, x1;
                 const float2 *p0 = P + 2 * j * PIV;
@@ -578,9 +588,9 @@ __global__ void __launch_bounds__(ZT_THREADS, 1) zinv_kernel(InvArgs a) {
             }
             fence_proxy_async_smem();   // the operand tiles, before the tensor core reads them
             tc_fence_before();
-            asm volatile("bar.sync 2, 480;" ::: "memory");
+            asm volatile("bar.sync 2, %0;" ::"n"(Cfg::THREADS - 32) : "memory");
             // (d) A' R' into tensor memory, the cross terms first
-            if (warp == 15 && elect_one()) {
+            if (warp == Cfg::WARPS - 1 && elect_one()) {
                 tc_fence_after();
 #pragma unroll
                 for (int p = 0; p < 3; ++p) {   // lo*hi, hi*lo, hi*hi
@@ -619,15 +629,15 @@ __global__ void __launch_bounds__(ZT_THREADS, 1) zinv_kernel(InvArgs a) {
     }
     if (!aborted) {
 #pragma unroll 1
-        for (int half = 0; half < 2; ++half) {
+        for (int half = 0; half < H / 2; ++half) {
             if ((h >> 1) == half) {
 #pragma unroll
                 for (int i = 0; i < 32; ++i) T[r * ZT_TS + 32 * (h & 1) + i] = w[i];
             }
             __syncthreads();
 #pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                const int rr = 8 * warp + i;
+            for (int i = 0; i < 128 / Cfg::WARPS; ++i) {
+                const int rr = 128 / Cfg::WARPS * warp + i;
 #pragma unroll
                 for (int e = 0; e < 2; ++e) {
                     const int c = 64 * half + 32 * e + lane;
@@ -643,7 +653,7 @@ __global__ void __launch_bounds__(ZT_THREADS, 1) zinv_kernel(InvArgs a) {
     tc_fence_before();
     __syncthreads();
     if (warp == 0)
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(s_tmem), "r"(256u) : "memory");
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(s_tmem), "r"(Cfg::TMEM) : "memory");
 }
 
 // *out = largest of n words
@@ -765,13 +775,16 @@ helm_status invert_blocks(int n, Fam X, const std::vector<int> &blocks, int *sta
     helm_status s;
     if (n <= INV_MAX) {
         const int off = pl.add(blocks);
-        cudaError_t e = ensure_dyn_smem((const void *)zinv_kernel, ZT_SMEM);
+        const bool small = n <= 64;
+        const size_t smem = small ? ZtCfg<2>::SMEM : ZtCfg<4>::SMEM;
+        cudaError_t e = ensure_dyn_smem(small ? (const void *)zinv_kernel<2> : (const void *)zinv_kernel<4>, smem);
         if (e != cudaSuccess) { helm_set_error("bcr: block inversion", e); return HELM_ECUDA; }
         InvArgs a{n, X.base, X.stride, X.ld, nullptr, status};
         a.tries = wait_tries();
-        pl.ops.push_back([a, off, count, st](const int *dev) mutable -> helm_status {
+        pl.ops.push_back([a, off, count, st, small, smem](const int *dev) mutable -> helm_status {
             a.idx = dev + off;
-            HELM_TRACED(K_ZINV, st, (zinv_kernel<<<count, ZT_THREADS, ZT_SMEM, st>>>(a)));
+            if (small) HELM_TRACED(K_ZINV, st, (zinv_kernel<2><<<count, ZtCfg<2>::THREADS, smem, st>>>(a)));
+            else HELM_TRACED(K_ZINV, st, (zinv_kernel<4><<<count, ZtCfg<4>::THREADS, smem, st>>>(a)));
             const cudaError_t e2 = cudaGetLastError();
             if (e2 != cudaSuccess) { helm_set_error("bcr: block inversion", e2); return HELM_ECUDA; }
             return HELM_OK;

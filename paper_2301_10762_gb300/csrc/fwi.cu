@@ -351,7 +351,8 @@ __global__ void regR_kernel(GridGeom g, const double *v, double *out) {
 //     the operand instead, it doubled the time of every sum (512^2: 1272 us a call against 589);
 //   - the symmetry C[a][n-1-j] = (-1)^a C[a][j] halves the multiply-adds: a line is folded into its
 //     even and odd parts first, or the even and odd sums are unfolded after;
-//   - a CTA per line (column) puts 128 of them on a 128^2 problem.
+//   - a CTA per line (column) puts 128 of them on a 128^2 problem; few long lines are shared by several
+//     CTAs (P2Solver::split), their columns in two launches.
 // One vector, us a call: with the matrices formed (2 launches), four tiled products and a scaling (5
 // launches) 84 at 64^2, 101 at 128^2, 113 at 160^2, 196 at 256^2, 1072 at 512^2; three passes and
 // the table 57, 64, 83, 123, 589 (64 to 512, square and not, odd and even: the least gain is 1.36, just
@@ -374,15 +375,15 @@ __device__ __forceinline__ int dct_parts(int outputs) {
     while (s < 8 && 2 * s * outputs <= 2 * DCT_THREADS) s *= 2;
     return s;
 }
-// out(a, sum_j cos(pi a (2j+1) / (2n)) v_j) for every a, v folded: F[j] = v_j + v_{n-1-j} for even a,
+// out(a, sum_j cos(pi a (2j+1) / (2n)) v_j) for a in [a0, a1), v folded: F[j] = v_j + v_{n-1-j} for even a,
 // F[h + j] = v_j - v_{n-1-j} for odd a, h = (n + 1) / 2 (the middle of an odd n once, and 0)
-template <typename Out> __device__ void dct_forward(const double *T, int n, const double *F, Out out) {
-    const int h = (n + 1) / 2, S = dct_parts(n), part = threadIdx.x % S;
-    const int rounds = (n * S + DCT_THREADS - 1) / DCT_THREADS;
+template <typename Out> __device__ void dct_forward(const double *T, int n, const double *F, int a0, int a1, Out out) {
+    const int h = (n + 1) / 2, S = dct_parts(a1 - a0), part = threadIdx.x % S;
+    const int rounds = ((a1 - a0) * S + DCT_THREADS - 1) / DCT_THREADS;
     for (int q = 0; q < rounds; ++q) {   // (uniform trip count: the shuffles need whole warps)
-        const int a = (q * DCT_THREADS + (int)threadIdx.x) / S;
+        const int a = a0 + (q * DCT_THREADS + (int)threadIdx.x) / S;
         double acc = 0.0, acc1 = 0.0;
-        if (a < n) {
+        if (a < a1) {
             const double *v = F + (a & 1) * h;
             const int step = (int)((2ll * a * S) % (4 * n));
             int idx = (int)(((long long)a * (2 * part + 1)) % (4 * n));
@@ -399,17 +400,18 @@ template <typename Out> __device__ void dct_forward(const double *T, int n, cons
             acc += acc1;
         }
         for (int o = 1; o < S; o *= 2) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-        if (a < n && part == 0) out(a, acc);
+        if (a < a1 && part == 0) out(a, acc);
     }
 }
-// out(j, sum_a cos(pi a (2j+1) / (2n)) t_a) for every j: the even and the odd a apart
-template <typename Out> __device__ void dct_backward(const double *T, int n, const double *t, Out out) {
-    const int h = (n + 1) / 2, S = dct_parts(h), part = threadIdx.x % S;
-    const int rounds = (h * S + DCT_THREADS - 1) / DCT_THREADS;
+// out(j, sum_a cos(pi a (2j+1) / (2n)) t_a) for j in [j0, j1) of the first h = (n + 1) / 2 and their mirror
+// images: the even and the odd a apart
+template <typename Out> __device__ void dct_backward(const double *T, int n, const double *t, int j0, int j1, Out out) {
+    const int S = dct_parts(j1 - j0), part = threadIdx.x % S;
+    const int rounds = ((j1 - j0) * S + DCT_THREADS - 1) / DCT_THREADS;
     for (int q = 0; q < rounds; ++q) {
-        const int j = (q * DCT_THREADS + (int)threadIdx.x) / S;
+        const int j = j0 + (q * DCT_THREADS + (int)threadIdx.x) / S;
         double ev = 0.0, od = 0.0;
-        if (j < h) {
+        if (j < j1) {
             const int w = 2 * j + 1, step2 = (int)((2ll * w * S) % (4 * n));
             int ie = (int)((2ll * part * w) % (4 * n)), io = (int)(((2ll * part + 1) * w) % (4 * n));
             for (int a = 2 * part; a < n; a += 2 * S) {
@@ -425,7 +427,7 @@ template <typename Out> __device__ void dct_backward(const double *T, int n, con
             ev += __shfl_xor_sync(0xffffffffu, ev, o);
             od += __shfl_xor_sync(0xffffffffu, od, o);
         }
-        if (j < h && part == 0) {
+        if (j < j1 && part == 0) {
             out(j, ev + od);
             if (n - 1 - j != j) out(n - 1 - j, ev - od);
         }
@@ -453,9 +455,21 @@ struct DctBuf {
     double *u;
 };
 __device__ __forceinline__ DctBuf dct_buf(int n, int vectors, const double *table, double *big, double *smem) {
-    if (big) return DctBuf{table, big + dct_vec_elems(n, vectors) * (blockIdx.x + (size_t)gridDim.x * blockIdx.y)};
+    if (big) {
+        const size_t cta = blockIdx.x + (size_t)gridDim.x * (blockIdx.y + (size_t)gridDim.y * blockIdx.z);
+        return DctBuf{table, big + dct_vec_elems(n, vectors) * cta};
+    }
     for (int k = threadIdx.x; k <= 2 * n; k += DCT_THREADS) smem[k] = table[k];
     return DctBuf{smem, smem + 2 * n + 1};
+}
+// this CTA's share of n outputs (gridDim.z CTAs to a line)
+__device__ __forceinline__ int dct_share(int n, int z) { return (int)((long long)n * z / gridDim.z); }
+
+// scale of the x transform's output a in column e: s_a^2, s_e^2 and the division
+__device__ __forceinline__ double dct_scaled(double x, int a, int nx, const double *Tx, double sx, double lz, double s2,
+                                             double alpha0, double mu) {
+    const double lx = sx * (2.0 - 2.0 * dct_cos(Tx, nx, 2 * a));
+    return x * (s2 * (a == 0 ? 1.0 : 2.0)) / (nx * (alpha0 * (lx + lz) + mu));
 }
 
 // z transforms of the lines (blockIdx.x) of the vectors (blockIdx.y): out = in C_z^T without s_b, or
@@ -466,14 +480,15 @@ __global__ void __launch_bounds__(DCT_THREADS) dct_lines_kernel(int nx, int nz, 
     const size_t off = ((size_t)blockIdx.y * nx + blockIdx.x) * nz;
     const DctBuf b = dct_buf(nz, DCT_LINE_VECS, tz, big, dct_smem);
     double *o = out + off;
+    const int z = blockIdx.z, h = (nz + 1) / 2;
     if (back) {
         for (int k = threadIdx.x; k < nz; k += DCT_THREADS) b.u[k] = in[off + k];
         __syncthreads();
-        dct_backward(b.T, nz, b.u, [&](int j, double x) { o[j] = x; });
+        dct_backward(b.T, nz, b.u, dct_share(h, z), dct_share(h, z + 1), [&](int j, double x) { o[j] = x; });
     } else {
         dct_fold(nz, in + off, 1, b.u);
         __syncthreads();
-        dct_forward(b.T, nz, b.u, [&](int a, double x) { o[a] = x; });
+        dct_forward(b.T, nz, b.u, dct_share(nz, z), dct_share(nz, z + 1), [&](int a, double x) { o[a] = x; });
     }
 }
 
@@ -486,19 +501,40 @@ __global__ void __launch_bounds__(DCT_THREADS) dct_columns_kernel(int nx, int nz
     double *t = b.u + nx + 1;
     dct_fold(nx, col, nz, b.u);
     __syncthreads();
-    dct_forward(b.T, nx, b.u, [&](int a, double x) { t[a] = x; });
+    dct_forward(b.T, nx, b.u, 0, nx, [&](int a, double x) { t[a] = x; });
     __syncthreads();
     // (once per output with all threads: in dct_forward's lanes it cost the FP64 pipe as much as the sums)
     const int e = blockIdx.x;
     const double sx = (double)(nx - 1) * (nx - 1), sz = (double)(nz - 1) * (nz - 1);
-    const double lz = sz * (2.0 - 2.0 * dct_cos(tz, nz, 2 * e));
-    const double s2 = (e == 0 ? 1.0 : 2.0) / nz;
-    for (int a = threadIdx.x; a < nx; a += DCT_THREADS) {
-        const double lx = sx * (2.0 - 2.0 * dct_cos(b.T, nx, 2 * a));
-        t[a] = t[a] * (s2 * (a == 0 ? 1.0 : 2.0)) / (nx * (alpha0 * (lx + lz) + mu));
-    }
+    const double lz = sz * (2.0 - 2.0 * dct_cos(tz, nz, 2 * e)), s2 = (e == 0 ? 1.0 : 2.0) / nz;
+    for (int a = threadIdx.x; a < nx; a += DCT_THREADS) t[a] = dct_scaled(t[a], a, nx, b.T, sx, lz, s2, alpha0, mu);
     __syncthreads();
-    dct_backward(b.T, nx, t, [&](int j, double x) { col[(size_t)j * nz] = x; });
+    dct_backward(b.T, nx, t, 0, (nx + 1) / 2, [&](int j, double x) { col[(size_t)j * nz] = x; });
+}
+
+// The same in two launches, several CTAs to a column: transforms and division, and (back) the
+// transforms back; in and out are distinct
+__global__ void __launch_bounds__(DCT_THREADS) dct_column_parts_kernel(int nx, int nz, const double *tx, const double *tz,
+                                                                       double alpha0, double mu, int back, const double *in,
+                                                                       double *out, double *big) {
+    extern __shared__ double dct_smem[];
+    const size_t off = (size_t)blockIdx.y * nx * nz + blockIdx.x;
+    const DctBuf b = dct_buf(nx, DCT_LINE_VECS, tx, big, dct_smem);
+    double *col = out + off;
+    const int z = blockIdx.z, h = (nx + 1) / 2;
+    if (back) {
+        for (int k = threadIdx.x; k < nx; k += DCT_THREADS) b.u[k] = in[off + (size_t)k * nz];
+        __syncthreads();
+        dct_backward(b.T, nx, b.u, dct_share(h, z), dct_share(h, z + 1), [&](int j, double x) { col[(size_t)j * nz] = x; });
+    } else {
+        dct_fold(nx, in + off, nz, b.u);
+        __syncthreads();
+        const int e = blockIdx.x;
+        const double sx = (double)(nx - 1) * (nx - 1), sz = (double)(nz - 1) * (nz - 1);
+        const double lz = sz * (2.0 - 2.0 * dct_cos(tz, nz, 2 * e)), s2 = (e == 0 ? 1.0 : 2.0) / nz;
+        dct_forward(b.T, nx, b.u, dct_share(nx, z), dct_share(nx, z + 1),
+                    [&](int a, double x) { col[(size_t)a * nz] = dct_scaled(x, a, nx, b.T, sx, lz, s2, alpha0, mu); });
+    }
 }
 
 }  // namespace helm
@@ -597,7 +633,7 @@ struct Dotter {
 struct P2Solver {
     int nx = 0, nz = 0, batch = 1;
     double alpha0 = 0, mu = 0;
-    double *tx = nullptr, *tz = nullptr, *T1 = nullptr, *big_z = nullptr, *big_x = nullptr;
+    double *tx = nullptr, *tz = nullptr, *T1 = nullptr, *T2 = nullptr, *big_z = nullptr, *big_x = nullptr;
     helm_status init(Ws &ws, const GridGeom &g, double a0, double m0, cudaStream_t st, int n_batch = 1) {
         nx = g.nx;
         nz = g.nz;
@@ -607,12 +643,14 @@ struct P2Solver {
         helm_status s = HELM_OK;
         tx = ws.get<double>(2 * ((size_t)nx + nz) + 2, &s);
         T1 = ws.get<double>((size_t)nx * nz * batch, &s);
-        if (nz > DCT_SMEM_N) big_z = ws.get<double>(dct_vec_elems(nz, DCT_LINE_VECS) * nx * batch, &s);
-        if (nx > DCT_SMEM_N) big_x = ws.get<double>(dct_vec_elems(nx, DCT_COL_VECS) * nz * batch, &s);
+        if (split(nz, nx) > 1) T2 = ws.get<double>((size_t)nx * nz * batch, &s);
+        if (nz > DCT_SMEM_N) big_z = ws.get<double>(big_elems(nz, DCT_LINE_VECS, nx, batch), &s);
+        if (nx > DCT_SMEM_N) big_x = ws.get<double>(big_elems(nx, DCT_COL_VECS, nz, batch), &s);
         if (s != HELM_OK) return s;
         tz = tx + 2 * nx + 1;
         if (smem(nz, DCT_LINE_VECS) > 48 * 1024) HK(ensure_dyn_smem((const void *)dct_lines_kernel, smem(nz, DCT_LINE_VECS)));
         if (smem(nx, DCT_COL_VECS) > 48 * 1024) HK(ensure_dyn_smem((const void *)dct_columns_kernel, smem(nx, DCT_COL_VECS)));
+        if (smem(nx, DCT_LINE_VECS) > 48 * 1024) HK(ensure_dyn_smem((const void *)dct_column_parts_kernel, smem(nx, DCT_LINE_VECS)));
         HELM_TRACED(K_DCTMAT, st, (dct_table_kernel<<<nblk(2 * ((size_t)nx + nz) + 2, 32), 32, 0, st>>>(nx, nz, tx, tz)));
         HL();
         return HELM_OK;
@@ -620,20 +658,38 @@ struct P2Solver {
     static size_t smem(int n, int vectors) {
         return n > DCT_SMEM_N ? 0 : (2 * (size_t)n + 1 + dct_vec_elems(n, vectors)) * sizeof(double);
     }
-    // vectors at a time: 16 while their scratch stays within 64 MB (one vector's is 1 to 4 N values)
+    // CTAs to a line of n nodes where `lines` of them leave SMs idle: 128 outputs each at least (us, one
+    // CTA / split: 4 x 6500 10920 / 616, 30 x 2000 1109 / 331, 3 x 900 298 / 104; the tiled products 5060, 874, 275)
+    static int split(int lines, int n) { return std::max(1, std::min(device_sms() / lines, (n + 127) / 128)); }
+    // global scratch: a CTA's vectors, one per line or as many as split() makes
+    static size_t big_elems(int n, int vectors, int lines, int n_batch) {
+        return dct_vec_elems(n, vectors) * std::max<size_t>((size_t)lines * n_batch, (size_t)device_sms());
+    }
+    // vectors at a time: 16 while their scratch stays within 64 MB (one vector's is 1 to 5 N values)
     static int max_batch(const GridGeom &g) {
-        const size_t v = sizeof(double) * ((size_t)g.nx * g.nz + (g.nz > DCT_SMEM_N ? dct_vec_elems(g.nz, DCT_LINE_VECS) * g.nx : 0) +
+        const size_t v = sizeof(double) * ((size_t)g.nx * g.nz * (split(g.nz, g.nx) > 1 ? 2 : 1) +
+                                           (g.nz > DCT_SMEM_N ? dct_vec_elems(g.nz, DCT_LINE_VECS) * g.nx : 0) +
                                            (g.nx > DCT_SMEM_N ? dct_vec_elems(g.nx, DCT_COL_VECS) * g.nz : 0));
         return (int)std::max<size_t>(1, std::min<size_t>(16, ((size_t)64 << 20) / v));
     }
     // out may be r
     helm_status apply(const double *r, double *out, cudaStream_t st, int count = 1) {
-        HELM_TRACED(K_DGEMM, st, (dct_lines_kernel<<<dim3(nx, count), DCT_THREADS, smem(nz, DCT_LINE_VECS), st>>>(nx, nz, tz, 0, r, T1, big_z)));
+        const int pz = split(nx * count, nz), px = split(nz * count, nx);
+        const size_t sz = smem(nz, DCT_LINE_VECS), sx = smem(nx, DCT_LINE_VECS);
+        HELM_TRACED(K_DGEMM, st, (dct_lines_kernel<<<dim3(nx, count, pz), DCT_THREADS, sz, st>>>(nx, nz, tz, 0, r, T1, big_z)));
         HL();
-        HELM_TRACED(K_DGEMM, st, (dct_columns_kernel<<<dim3(nz, count), DCT_THREADS, smem(nx, DCT_COL_VECS), st>>>(nx, nz, tx, tz, alpha0, mu,
-                                                                                                    T1, big_x)));
-        HL();
-        HELM_TRACED(K_DGEMM, st, (dct_lines_kernel<<<dim3(nx, count), DCT_THREADS, smem(nz, DCT_LINE_VECS), st>>>(nx, nz, tz, 1, T1, out, big_z)));
+        if (px > 1) {
+            for (int back = 0; back < 2; ++back) {
+                HELM_TRACED(K_DGEMM, st, (dct_column_parts_kernel<<<dim3(nz, count, px), DCT_THREADS, sx, st>>>(
+                                             nx, nz, tx, tz, alpha0, mu, back, back ? T2 : T1, back ? T1 : T2, big_x)));
+                HL();
+            }
+        } else {
+            HELM_TRACED(K_DGEMM, st, (dct_columns_kernel<<<dim3(nz, count), DCT_THREADS, smem(nx, DCT_COL_VECS), st>>>(
+                                         nx, nz, tx, tz, alpha0, mu, T1, big_x)));
+            HL();
+        }
+        HELM_TRACED(K_DGEMM, st, (dct_lines_kernel<<<dim3(nx, count, pz), DCT_THREADS, sz, st>>>(nx, nz, tz, 1, T1, out, big_z)));
         HL();
         return HELM_OK;
     }
