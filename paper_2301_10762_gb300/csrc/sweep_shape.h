@@ -56,7 +56,7 @@ inline double sweep_time_fp64(int nz, int cs, long clusters, const SweepActive &
 // was, 249 spread out).  active(c): of clusters of teams * c CTAs; fit(c, R): the launch.
 // Measured on 60 lines of 48 to 160 nodes, 1 to 8 systems of 1 to 64 right-hand sides, every shape (25000
 // points, which the model meets to 8 %): 1.43 times as fast as the given shape on average and 2 % above
-// the best, 5 % slower than the given one in 3 of 498 calls.  64^2 with 8 right-hand sides: 649 -> 278 us.  Counting
+// the best, 5 % slower than the given one in 3 of 498 calls.  64^2 with 8 right-hand sides: a call 770 -> 324 us.  Counting
 // CTAs that share an SM as free took 60 to 72 nodes with 24 to 64 right-hand sides twice as long.
 template <typename Active, typename Fit>
 SweepShape sweep_shape_fp64(int nz, int teams, int n_sys, int nrhs, SweepShape s, Active active, Fit fit) {
